@@ -13,7 +13,7 @@
 #include "gc_threshold.cuh"
 #include "gc_thr_single.cuh"
 #include "gc_thr_multi.cuh"
-#include "gc_decode.cuh"
+#include "gc_decode_rings.cuh"
 
 using namespace gc;
 
@@ -48,10 +48,8 @@ struct gc_plan_s {
            control_bytes = 0, off_tinfo = 0, off_cidx = 0, ws_bytes = 0;
     int sm_count = 0;
     int grid_thr = 0, grid_decode[2] = {0, 0};
-    int grid_decode8 = 0, grid_decode8_apply = 0;      // k_decode_tiles with eight pre-loaded entries per thread (one tile buffer)
     int grid_decode_seg[2] = {0, 0}, grid_decode_seg_apply = 0;    // k_decode_segments: one / two tile buffers; with optimizer
-    bool wide_ok = false;                         // k_decode_wide may use up to 64 KB of dynamic shared memory
-    std::vector<std::pair<size_t, int>> wide_occ[2];      // (shared-memory bytes -> CTAs per SM), plain / with optimizer
+    bool rings_ok = false;                        // k_decode_rings may use up to kRingSmem2 of dynamic shared memory
     int grid_hist = 0, grid_compact = 0, grid_fold = 0, grid_sample = 0, grid_chist = 0, grid_ccompact = 0;
     int grid_fused = 0;                     // CTAs of the cooperative launch (0 = not available)
     // single-tensor shared-memory-pool kernel
@@ -494,61 +492,48 @@ int blocks_per_sm(K kernel, int threads) {
 
 }  // namespace
 
-// Which decode kernel a call takes.  The narrow kernel pre-loads 4 x (256 / W) entries per worker
-// and tile in registers; lists that are expected to hold more per tile than that (many workers,
-// or dense lists) go to the wide kernel, which keeps `win` entries per worker in shared memory.
-struct DecodeRoute {
-    bool wide = false;
-    bool any = false;           // (with wide) the kernel that adds without a fixed worker order
-    uint32_t win = 0;
-    size_t smem = 0;
-    int grid = 0;
-    int rounds = kDecRounds;    // (narrow) entries a thread pre-loads per tile: kDecRounds or twice that
-};
-template <bool APPLY>
-static DecodeRoute decode_route(gc_plan_t* p, uint32_t W, bool zero_first) {
-    DecodeRoute r;
-    if (W == 0 || p->total_n == 0) return r;
-    const uint64_t avg = (p->total_cap * (uint64_t)kDecTile + p->total_n - 1) / p->total_n;     // per worker and tile
-    const uint64_t need = avg + avg / 2 + 16;
-    uint32_t Wp = 1;
-    while (Wp < W && Wp < 64) Wp <<= 1;
-    uint64_t narrow_window = (uint64_t)kDecRounds * (kDecBlock / Wp);
-    r.any = p->decode_order == GC_ORDER_ANY;
-    // Tiles that start at +0 take the narrow kernel's counted route from a few workers on; there a
-    // window of twice the size (eight pre-loaded entries per thread) still beats the rings, so
-    // lists up to that density stay with the narrow kernel (16 workers at 1 %: measured below).
-    if (!r.any && zero_first && W >= kDecCountedFrom && avg + avg / 4 > narrow_window &&
-        avg + avg / 4 <= 2 * narrow_window && p->grid_decode8 > 0) {
-        r.rounds = 2 * kDecRounds;
-        narrow_window *= 2;
-    }
-    // measured: the narrow kernel wins as long as most tiles fit its window
-    r.wide = r.any || (p->decode_route == GC_DECODE_AUTO ? avg + avg / 4 > narrow_window
-                                                          : p->decode_route == GC_DECODE_WIDE);
-    if (!p->wide_ok) r.wide = false;
-    if (!r.wide) return r;
-    uint32_t win = 32;
-    while (win < need && win < 1024) win <<= 1;
-    while ((uint64_t)W * win > kDecWideEntries && win > 32) win >>= 1;
-    r.win = win;
-    r.smem = kDecTileBytes + 8 * (size_t)W * win;
-    int nb = -1;
-    const size_t key = r.smem + (r.any ? 1 : 0);          // (shared-memory sizes are multiples of 256)
-    for (auto& e : p->wide_occ[APPLY ? 1 : 0]) if (e.first == key) nb = e.second;
-    if (nb < 0) {
-        const cudaError_t eo = r.any
-            ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_decode_any<APPLY>, kDecBlock, r.smem)
-            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_decode_wide<APPLY>, kDecBlock, r.smem);
-        if (eo != cudaSuccess) {
-            (void)cudaGetLastError();
-            nb = 0;
+// Geometry of k_decode_rings for W lists of this plan, and whether a call takes it or k_decode_tiles.
+// Shared memory decides how many of its CTAs fit an SM: three up to kRingSmem3 bytes, two up to kRingSmem2.
+constexpr size_t kRingSmem3 = 74 * 1024 - 512, kRingSmem2 = 111 * 1024;
+struct RingGeom { uint32_t T = 0, RS = 0; size_t smem = 0; int ctas = 0; };
+static size_t ring_smem(uint32_t W, uint32_t T, uint32_t RS, bool apply) {
+    const size_t Wb = (W + kRingBatch - 1) / kRingBatch * kRingBatch;
+    return 8 * Wb * RS + sizeof(float) * 8 * (size_t)(T + kRingPad + (apply ? 2 * T : 0)) + 8 * 8 * (size_t)(W > 32 ? 64 : 32);
+}
+static RingGeom ring_geometry(const gc_plan_s* p, uint32_t W, bool apply) {
+    const double dens = (double)p->total_cap / (double)p->total_n;
+    // a warp adds a worker's share of its sub-tile in rounds of 32 entries: one round for nearly all
+    // shares where that leaves a sub-tile worth its fixed cost, two rounds for denser lists
+    const double per_sub = dens * 1152.0 <= 17.0 ? 17.0 : 51.0;
+    auto largest = [&](size_t budget) {
+        RingGeom g;
+        for (uint32_t T = apply ? 1024 : 2048; T >= 128; T -= 128) {
+            const double avg = dens * 8.0 * T;
+            uint32_t RS = std::max(32u, ((uint32_t)(avg + 3.2 * std::sqrt(avg)) + 12u) / 4u * 4u);
+            size_t b = ring_smem(W, T, RS, apply);
+            if (T > 128 && (b > budget || dens * T > per_sub)) continue;
+            while (RS > 32 && b > budget) { RS -= 4; b = ring_smem(W, T, RS, apply); }      // (then steps end at a full ring)
+            g.T = T; g.RS = RS; g.smem = b;
+            break;
         }
-        p->wide_occ[APPLY ? 1 : 0].emplace_back(key, nb);
-    }
-    r.grid = p->sm_count * nb;
-    if (r.grid <= 0) r.wide = false;
-    return r;
+        return g;
+    };
+    // 24 warps per SM unless 16 get sub-tiles a third larger (110M elements, 1 %: W = 16 149 us with
+    // T = 1408 and three CTAs against 156 us with 1664 and two; W = 32 241 us with 1152 against 217 us)
+    RingGeom g3 = largest(kRingSmem3), g2 = largest(kRingSmem2);
+    g3.ctas = 3; g2.ctas = 2;
+    return 4u * g3.T > 3u * g2.T ? g3 : g2;
+}
+static bool takes_rings(const gc_plan_s* p, uint32_t W) {
+    if (W == 0 || !p->rings_ok) return false;
+    if (p->decode_route != GC_DECODE_AUTO) return p->decode_route == GC_DECODE_WIDE;
+    // k_decode_tiles pre-loads 4 x (256 / W) entries per worker and 8192-element tile: denser lists go
+    // through the rings, and so do lists whose entries add up to more than 4.5 % of the elements (the
+    // block-wide steps of the tile kernel then cost more than the rings' fixed work per sub-tile)
+    uint32_t Wp = 1;
+    while (Wp < W) Wp <<= 1;
+    const uint64_t avg = (p->total_cap * (uint64_t)kDecTile + p->total_n - 1) / p->total_n;
+    return avg + avg / 4 > (uint64_t)kDecRounds * (kDecBlock / Wp) || (double)W * (double)p->total_cap > 0.045 * (double)p->total_n;
 }
 
 extern "C" {
@@ -701,23 +686,16 @@ int gc_plan(gc_plan_t** out, int device, uint32_t n_tensors, const uint64_t* siz
     }
     p->grid_thr = p->sm_count * blocks_per_sm(k_threshold_emit, kBlock);
     {
-        cudaError_t ed = cudaFuncSetAttribute(k_decode_tiles<false, kDecRounds>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t ed = cudaFuncSetAttribute(k_decode_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)(2 * kDecTileBytes));
         for (int nbuf = 1; nbuf <= 2; ++nbuf) {
             int nb = 0;
             if (ed == cudaSuccess)
-                ed = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_decode_tiles<false, kDecRounds>, kDecBlock,
+                ed = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_decode_tiles, kDecBlock,
                                                                    nbuf * kDecTileBytes);
             if (ed != cudaSuccess || nb < 1) { (void)cudaGetLastError(); nb = 0; }
             p->grid_decode[nbuf - 1] = p->sm_count * nb;     // 0: fall back to one launch per worker
         }
-        int nb8 = 0, nb8a = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb8, k_decode_tiles<false, 2 * kDecRounds>, kDecBlock,
-                                                          kDecTileBytes) != cudaSuccess || nb8 < 1) { (void)cudaGetLastError(); nb8 = 0; }
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb8a, k_decode_tiles<true, 2 * kDecRounds>, kDecBlock,
-                                                          kDecTileBytes) != cudaSuccess || nb8a < 1) { (void)cudaGetLastError(); nb8a = 0; }
-        p->grid_decode8 = p->sm_count * nb8;
-        p->grid_decode8_apply = p->sm_count * nb8a;
     }
     {
         // lists with per-tensor counts (plans of several tensors): the segment-walking tile kernel
@@ -736,14 +714,11 @@ int gc_plan(gc_plan_t** out, int device, uint32_t n_tensors, const uint64_t* siz
                 cudaSuccess || nb < 1) { (void)cudaGetLastError(); nb = 0; }
         p->grid_decode_seg_apply = p->sm_count * nb;
     }
-    p->wide_ok = cudaFuncSetAttribute(k_decode_wide<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)(kDecTileBytes + 8 * kDecWideEntries)) == cudaSuccess &&
-                 cudaFuncSetAttribute(k_decode_wide<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)(kDecTileBytes + 8 * kDecWideEntries)) == cudaSuccess &&
-                 cudaFuncSetAttribute(k_decode_any<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)(kDecTileBytes + 8 * kDecWideEntries)) == cudaSuccess &&
-                 cudaFuncSetAttribute(k_decode_any<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)(kDecTileBytes + 8 * kDecWideEntries)) == cudaSuccess;
+    p->rings_ok = true;
+    for (const void* fn : {(const void*)k_decode_rings<false, false, false>, (const void*)k_decode_rings<false, false, true>,
+                           (const void*)k_decode_rings<false, true, false>, (const void*)k_decode_rings<false, true, true>,
+                           (const void*)k_decode_rings<true, false, false>, (const void*)k_decode_rings<true, false, true>})
+        p->rings_ok = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRingSmem2) == cudaSuccess && p->rings_ok;
     (void)cudaGetLastError();
     p->grid_sample = p->sm_count * blocks_per_sm(k_hist<0, SRC_SAMPLE>, kBlock);
     p->grid_chist = p->sm_count * blocks_per_sm(k_cand_hist<1>, kBlock);
@@ -1275,24 +1250,17 @@ int gc_decompress_accumulate(gc_plan_t* p, uint32_t W, const uint32_t* const* id
         const int grid = (int)std::min<uint32_t>(ntl, (uint32_t)p->grid_decode[nbuf - 1]);
         const int use_bulk = (reinterpret_cast<uintptr_t>(dense_out) & 15u) == 0 ? 1 : 0;
         Timed tm(p, s, GC_K_DECODE_TILES);
-        const DecodeRoute rt = decode_route<false>(p, W, zero_first != 0);
-        if (rt.wide) {
-            auto kw = rt.any ? k_decode_any<false> : k_decode_wide<false>;
-            kw<<<(int)std::min<uint32_t>(ntl, (uint32_t)rt.grid), kDecBlock, rt.smem, s>>>(
-                ls, W, (uint32_t)p->total_cap, (uint32_t)p->total_n, dense_out, zero_first ? 1 : 0, use_bulk, rt.win,
-                ws.hdr, ApplyArgs{});
-            GC_CUDA(p, cudaGetLastError());
-            return GC_OK;
+        if (takes_rings(p, W)) {
+            const RingGeom g = ring_geometry(p, W, false);
+            const uint32_t nt8 = (uint32_t)((p->total_n + 8u * g.T - 1) / (8u * g.T));
+            auto kr = zero_first ? (W > 32 ? k_decode_rings<false, false, true> : k_decode_rings<false, false, false>)
+                                 : (W > 32 ? k_decode_rings<false, true, true> : k_decode_rings<false, true, false>);
+            kr<<<std::min<uint32_t>(nt8, (uint32_t)(p->sm_count * g.ctas)), kDecBlock, g.smem, s>>>(
+                ls, W, (uint32_t)p->total_cap, (uint32_t)p->total_n, g.T, g.RS, dense_out, use_bulk, ws.hdr, ApplyArgs{});
+        } else {
+            k_decode_tiles<<<grid, kDecBlock, nbuf * kDecTileBytes, s>>>(
+                ls, W, (uint32_t)p->total_cap, (uint32_t)p->total_n, dense_out, zero_first ? 1 : 0, use_bulk, nbuf, ws.hdr);
         }
-        if (rt.rounds != kDecRounds)
-            k_decode_tiles<false, 2 * kDecRounds><<<(int)std::min<uint32_t>(ntl, (uint32_t)p->grid_decode8), kDecBlock,
-                                                    kDecTileBytes, s>>>(ls, W, (uint32_t)p->total_cap, (uint32_t)p->total_n,
-                                                                        dense_out, zero_first ? 1 : 0, use_bulk, 1, ws.hdr,
-                                                                        ApplyArgs{});
-        else
-            k_decode_tiles<false, kDecRounds><<<grid, kDecBlock, nbuf * kDecTileBytes, s>>>(
-                ls, W, (uint32_t)p->total_cap, (uint32_t)p->total_n, dense_out, zero_first ? 1 : 0, use_bulk, nbuf, ws.hdr,
-                ApplyArgs{});
         GC_CUDA(p, cudaGetLastError());
         return GC_OK;
     }
@@ -1348,7 +1316,7 @@ int gc_decompress_apply_momentum(gc_plan_t* p, uint32_t W, const uint32_t* const
         (reinterpret_cast<uintptr_t>(velocity) & 15u))
         return GC_E_INVALID;
     const bool segmented = count != nullptr && p->T != 1;              // lists with unused slots between tensors
-    if ((segmented ? p->grid_decode_seg_apply : p->grid_decode[0]) <= 0) return GC_E_UNSUPPORTED;
+    if (segmented ? p->grid_decode_seg_apply <= 0 : !p->rings_ok) return GC_E_UNSUPPORTED;
     if (segmented && p->d_dectile == nullptr) return GC_E_UNSUPPORTED;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     WsView ws = view(p, workspace);
@@ -1359,7 +1327,6 @@ int gc_decompress_apply_momentum(gc_plan_t* p, uint32_t W, const uint32_t* const
         ls.len[w] = (W && count != nullptr) ? count[q] : nullptr;
     }
     const uint32_t ntl = (uint32_t)((p->total_n + kDecTile - 1) / kDecTile);
-    const int grid = (int)std::min<uint32_t>(ntl, (uint32_t)p->grid_decode[0]);
     ApplyArgs ap{param, velocity, lr, momentum, scale};
     Timed tm(p, s, GC_K_DECODE_TILES);
     if (segmented && W > 0) {
@@ -1369,21 +1336,11 @@ int gc_decompress_apply_momentum(gc_plan_t* p, uint32_t W, const uint32_t* const
         GC_CUDA(p, cudaGetLastError());
         return GC_OK;
     }
-    const DecodeRoute rt = decode_route<true>(p, W, true);
-    if (rt.wide) {
-        auto kw = rt.any ? k_decode_any<true> : k_decode_wide<true>;
-        kw<<<(int)std::min<uint32_t>(ntl, (uint32_t)rt.grid), kDecBlock, rt.smem, s>>>(
-            ls, W, (uint32_t)p->total_cap, (uint32_t)p->total_n, nullptr, 1, 0, rt.win, ws.hdr, ap);
-        GC_CUDA(p, cudaGetLastError());
-        return GC_OK;
-    }
-    if (rt.rounds != kDecRounds && p->grid_decode8_apply > 0)
-        k_decode_tiles<true, 2 * kDecRounds><<<(int)std::min<uint32_t>(ntl, (uint32_t)p->grid_decode8_apply), kDecBlock,
-                                               kDecTileBytes, s>>>(ls, W, (uint32_t)p->total_cap, (uint32_t)p->total_n,
-                                                                   nullptr, 1, 0, 1, ws.hdr, ap);
-    else
-        k_decode_tiles<true, kDecRounds><<<grid, kDecBlock, kDecTileBytes, s>>>(
-            ls, W, (uint32_t)p->total_cap, (uint32_t)p->total_n, nullptr, 1, 0, 1, ws.hdr, ap);
+    const RingGeom g = ring_geometry(p, W, true);
+    const uint32_t nt8 = (uint32_t)((p->total_n + 8u * g.T - 1) / (8u * g.T));
+    auto kr = W > 32 ? k_decode_rings<true, false, true> : k_decode_rings<true, false, false>;
+    kr<<<std::min<uint32_t>(nt8, (uint32_t)(p->sm_count * g.ctas)), kDecBlock, g.smem, s>>>(
+        ls, W, (uint32_t)p->total_cap, (uint32_t)p->total_n, g.T, g.RS, nullptr, 0, ws.hdr, ap);
     GC_CUDA(p, cudaGetLastError());
     return GC_OK;
 }

@@ -18,7 +18,6 @@ namespace gc {
 constexpr int kDecTile = 8192;               // floats per CTA tile
 constexpr int kDecBlock = 256;
 constexpr int kDecRounds = 4;                // entries a thread pre-loads per tile
-constexpr size_t kDecWideEntries = 4096;     // ring entries (8 bytes each) the wide kernel keeps in shared memory, all workers together
 constexpr size_t kDecTileBytes = kDecTile * sizeof(float);
 
 struct DecodeLists {
@@ -43,6 +42,13 @@ template <int N>
 __device__ __forceinline__ void bulk_wait_read() {
     asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
 }
+
+// 4-byte asynchronous copy global -> shared, and the wait for all such copies of this thread.
+__device__ __forceinline__ void cp_async_4(void* sdst, const void* gsrc) {
+    const uint32_t sa = (uint32_t)__cvta_generic_to_shared(sdst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sa), "l"(gsrc) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // First position p in idx[0..cnt) with idx[p] >= key; all 32 lanes of a warp cooperate
 // (33-way split per round, about four rounds for a million entries).
@@ -131,36 +137,28 @@ __device__ __forceinline__ void stage_tile(float* s_tile, const float* out, uint
 // back at +0 and the caller applies the entries on the ordered route.  Called by the whole CTA.
 constexpr uint32_t kDecCountedFrom = 4;      // workers from which the counted route is taken
 constexpr int kDecConfCap = 128;             // colliding entries (three and more hits) a tile may hold
-template <int R>
 __device__ __forceinline__ bool counted_apply(float* s_tile, uint32_t lo, uint32_t seg_lo, uint32_t seg_hi,
-                                              uint32_t (&ix)[R], const float (&v)[R], uint32_t my_w,
+                                              uint32_t (&ix)[kDecRounds], const float (&v)[kDecRounds], uint32_t my_w,
                                               uint32_t c0, WsHeader* hdr, uint4* s_conf, uint32_t* s_nconf, int tid) {
     int* const t_cnt = reinterpret_cast<int*>(s_tile);
-    // per entry one byte: arrival number (6 bits) | min(hits, 3) << 6.  Four entries: a register
-    // each (packing them cost registers and 5 % of the time); eight entries: packed into 64 bits,
-    // which keeps that form at 64 registers and four CTAs per SM.
-    constexpr bool kPacked = R > 4;
-    uint32_t oh_a[kPacked ? 1 : R] = {};
-    unsigned long long oh_p = 0ull;
-    auto put = [&](int rd, uint32_t bits) { if constexpr (kPacked) oh_p |= (unsigned long long)bits << (8 * rd); else oh_a[rd] |= bits; };
-    auto get = [&](int rd) -> uint32_t { if constexpr (kPacked) return (uint32_t)(oh_p >> (8 * rd)) & 255u; else return oh_a[rd]; };
+    uint32_t oh[kDecRounds] = {};                          // per entry: arrival number (6 bits) | min(hits, 3) << 6
 #pragma unroll
-    for (int rd = 0; rd < R; ++rd) {
+    for (int rd = 0; rd < kDecRounds; ++rd) {
         if (ix[rd] < seg_hi) {
-            if (ix[rd] >= seg_lo) put(rd, (uint32_t)atomicAdd(&t_cnt[ix[rd] - lo], 1) & 63u);
+            if (ix[rd] >= seg_lo) oh[rd] = (uint32_t)atomicAdd(&t_cnt[ix[rd] - lo], 1) & 63u;
             else { record_status(hdr, -1 /*GC_E_INVALID*/, c0); ix[rd] = 0xFFFFFFFFu; }     // list not ascending: skipped
         }
     }
     __syncthreads();
 #pragma unroll
-    for (int rd = 0; rd < R; ++rd)
-        if (ix[rd] < seg_hi) put(rd, min((uint32_t)t_cnt[ix[rd] - lo], 3u) << 6);
+    for (int rd = 0; rd < kDecRounds; ++rd)
+        if (ix[rd] < seg_hi) oh[rd] |= min((uint32_t)t_cnt[ix[rd] - lo], 3u) << 6;
     __syncthreads();                                       // every count has been read
     bool conflict = false;
 #pragma unroll
-    for (int rd = 0; rd < R; ++rd) {
+    for (int rd = 0; rd < kDecRounds; ++rd) {
         if (ix[rd] >= seg_hi) continue;
-        const uint32_t b8 = get(rd);
+        const uint32_t b8 = oh[rd];
         if ((b8 >> 6) <= 2u) {
             if ((b8 & 63u) == 0u) s_tile[ix[rd] - lo] = __fadd_rn(0.0f, v[rd]);
         } else {
@@ -176,7 +174,7 @@ __device__ __forceinline__ bool counted_apply(float* s_tile, uint32_t lo, uint32
             // more colliding entries than the list holds: every touched element goes back to +0
             __syncthreads();
 #pragma unroll
-            for (int rd = 0; rd < R; ++rd) if (ix[rd] < seg_hi) s_tile[ix[rd] - lo] = 0.0f;
+            for (int rd = 0; rd < kDecRounds; ++rd) if (ix[rd] < seg_hi) s_tile[ix[rd] - lo] = 0.0f;
             done = false;
         } else if ((uint32_t)tid < nc) {
             // one thread per element with three or more hits: the entry of the lowest worker sums them all
@@ -202,22 +200,17 @@ __device__ __forceinline__ bool counted_apply(float* s_tile, uint32_t lo, uint32
     }
     if (done) {
 #pragma unroll
-        for (int rd = 0; rd < R; ++rd)
-            if (ix[rd] < seg_hi && get(rd) == ((2u << 6) | 1u))
+        for (int rd = 0; rd < kDecRounds; ++rd)
+            if (ix[rd] < seg_hi && oh[rd] == ((2u << 6) | 1u))
                 s_tile[ix[rd] - lo] = __fadd_rn(s_tile[ix[rd] - lo], v[rd]);
     }
     __syncthreads();
     return done;
 }
 
-// R = entries a thread pre-loads per tile (R, or twice that for lists that are denser
-// than four per thread and worker but still fit eight).
-template <bool APPLY, int R>
-// (the eight-entry form is held to 64 registers: four CTAs per SM measured better than three;
-// holding the four-entry form to 40 registers for six CTAs per SM measured worse than five)
-static __global__ void __launch_bounds__(kDecBlock, R == kDecRounds ? 0 : 4)
+static __global__ void __launch_bounds__(kDecBlock)
 k_decode_tiles(DecodeLists ls, uint32_t W, uint32_t cnt, uint32_t total_n, float* __restrict__ out,
-               int zero_first, int use_bulk, int nbuf, WsHeader* hdr, ApplyArgs ap) {
+               int zero_first, int use_bulk, int nbuf, WsHeader* hdr) {
     // nbuf tile buffers: with two, one fills while the other drains (pays off when there are few
     // workers per tile; with many workers more resident CTAs are worth more than the overlap)
     extern __shared__ __align__(128) float s_tiles[];
@@ -255,30 +248,30 @@ k_decode_tiles(DecodeLists ls, uint32_t W, uint32_t cnt, uint32_t total_n, float
         const uint32_t hi = min(total_n, lo + (uint32_t)kDecTile);
         const bool full = hi - lo == (uint32_t)kDecTile;
         stage_tile(s_tile, out, lo, hi, full, zero_first, use_bulk, tid);
-        // pre-load the next R * E entries of every worker
+        // pre-load the next kDecRounds * E entries of every worker
         const uint32_t c0 = live ? s_cur[my_w] : 0u;
-        uint32_t ix[R];
-        float v[R];
+        uint32_t ix[kDecRounds];
+        float v[kDecRounds];
         uint32_t nin = 0;
 #pragma unroll
-        for (int rd = 0; rd < R; ++rd) {
+        for (int rd = 0; rd < kDecRounds; ++rd) {
             const uint32_t p = c0 + (uint32_t)(rd * E + sub);
             ix[rd] = 0xFFFFFFFFu; v[rd] = 0.f;
             if (live && p < my_len) { ix[rd] = __ldg(ls.idx[my_w] + p); v[rd] = __ldg(ls.val[my_w] + p); }
         }
 #pragma unroll
-        for (int rd = 0; rd < R; ++rd) nin += ix[rd] < hi;       // sorted lists: the ins are a prefix
+        for (int rd = 0; rd < kDecRounds; ++rd) nin += ix[rd] < hi;       // sorted lists: the ins are a prefix
         // a worker whose pre-loaded entries all fall inside may have more: then the tile takes
         // the strictly sequential path so that worker order is kept for every element
-        const bool maybe_more = (ix[R - 1] < hi) && sub == E - 1;
+        const bool maybe_more = (ix[kDecRounds - 1] < hi) && sub == E - 1;
         if (tid == 0) s_nconf = 0u;
         if (!__syncthreads_or(maybe_more ? 1 : 0)) {                      // (also: tile staged, cursors read)
             const bool counted = zero_first && W >= kDecCountedFrom &&
-                                 counted_apply<R>(s_tile, lo, lo, hi, ix, v, my_w, c0, hdr, s_conf, &s_nconf, tid);
+                                 counted_apply(s_tile, lo, lo, hi, ix, v, my_w, c0, hdr, s_conf, &s_nconf, tid);
             for (uint32_t q = 0; q < W && !counted; ++q) {                 // apply in worker order
                 if (my_w == q) {
 #pragma unroll
-                    for (int rd = 0; rd < R; ++rd) {
+                    for (int rd = 0; rd < kDecRounds; ++rd) {
                         if (ix[rd] < hi) {
                             if (ix[rd] >= lo) s_tile[ix[rd] - lo] = __fadd_rn(s_tile[ix[rd] - lo], v[rd]);
                             else record_status(hdr, -1 /*GC_E_INVALID*/, c0);      // list not ascending
@@ -311,11 +304,6 @@ k_decode_tiles(DecodeLists ls, uint32_t W, uint32_t cnt, uint32_t total_n, float
             }
         }
         __syncthreads();
-        if (APPLY) {
-            apply_tile(ap, s_tile, lo, hi, full, tid);
-            __syncthreads();
-            continue;
-        }
         // the tile leaves shared memory
         if (full && use_bulk) {
             if (tid == 0) bulk_store_tile(out + lo, s_tile, (uint32_t)(kDecTile * sizeof(float)));
@@ -407,7 +395,7 @@ k_decode_segments(DecodeLists ls, uint32_t W, const TensorDesc* __restrict__ des
             if (tid == 0) s_nconf = 0u;
             if (!__syncthreads_or(maybe_more ? 1 : 0)) {                  // (also: tile staged, cursors read)
                 const bool counted = zero_first && W >= kDecCountedFrom &&
-                                     counted_apply<kDecRounds>(s_tile, lo, seg_lo, seg_hi, ix, v, my_w, c0, hdr, s_conf, &s_nconf, tid);
+                                     counted_apply(s_tile, lo, seg_lo, seg_hi, ix, v, my_w, c0, hdr, s_conf, &s_nconf, tid);
                 for (uint32_t q = 0; q < W && !counted; ++q) {             // apply in worker order
                     if (my_w == q) {
 #pragma unroll
@@ -474,242 +462,6 @@ k_decode_segments(DecodeLists ls, uint32_t W, const TensorDesc* __restrict__ des
         __syncthreads();
     }
     if (use_bulk && tid == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-}
-
-// 4-byte asynchronous copy global -> shared, and the wait for all such copies of this thread.
-__device__ __forceinline__ void cp_async_4(void* sdst, const void* gsrc) {
-    const uint32_t sa = (uint32_t)__cvta_generic_to_shared(sdst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sa), "l"(gsrc) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-// Decode for many workers or dense lists.  Every worker's next `win` entries sit in a ring in
-// shared memory that is topped up with asynchronous copies as entries are consumed, so every
-// list entry is fetched once and the fetch for the next tile overlaps with this tile's way out.
-// The workers are applied one after the other, each by the whole CTA (one ring entry per
-// thread), so a worker's share of a tile may be as large as the ring whatever the number of
-// workers, and the block-wide count that separates two workers also yields how far the cursor
-// moves.  If some worker has more than `win` entries in the tile, the pass ends at the smallest
-// index up to which every worker's ring is complete and the rest of the tile takes another
-// pass.  One tile buffer; `win` is a power of two.
-template <bool APPLY>
-static __global__ void __launch_bounds__(kDecBlock)
-k_decode_wide(DecodeLists ls, uint32_t W, uint32_t cnt, uint32_t total_n, float* __restrict__ out,
-              int zero_first, int use_bulk, uint32_t win, WsHeader* hdr, ApplyArgs ap) {
-    extern __shared__ __align__(128) float s_tiles[];
-    float* const s_tile = s_tiles;
-    uint32_t* const rg_idx = reinterpret_cast<uint32_t*>(s_tiles + kDecTile);      // [W][win]
-    float* const rg_val = reinterpret_cast<float*>(rg_idx + W * win);              // [W][win]
-    __shared__ uint32_t s_cur[64], s_len[64], s_adv[64], s_bound;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint32_t ntl = (total_n + kDecTile - 1) / kDecTile;
-    const uint32_t per = (ntl + gridDim.x - 1) / gridDim.x;
-    const uint32_t t0 = blockIdx.x * per, t1 = min(ntl, t0 + per);
-    if (t0 >= t1) return;
-    const uint32_t mask = win - 1u;
-    // E consecutive threads top up one worker's ring
-    int Wp = 1;
-    while (Wp < (int)W && Wp < 64) Wp <<= 1;
-    const int E = kDecBlock / Wp;
-    const uint32_t my_w = (uint32_t)(tid / E);
-    const int sub = tid % E;
-
-    for (uint32_t w = warp; w < W; w += kDecBlock / 32) {
-        const uint32_t len = ls.len[w] != nullptr ? min(__ldg(ls.len[w]), cnt) : cnt;
-        const uint32_t c = warp_lower_bound(ls.idx[w], len, t0 * (uint32_t)kDecTile, lane);
-        if (lane == 0) { s_cur[w] = c; s_len[w] = len; s_adv[w] = 0u; }
-    }
-    __syncthreads();
-    // list positions [from, to) of worker my_w go to their ring slots
-    auto top_up = [&](uint32_t from, uint32_t to) {
-        for (uint32_t p = from + (uint32_t)sub; p < to; p += (uint32_t)E) {
-            cp_async_4(rg_idx + my_w * win + (p & mask), ls.idx[my_w] + p);
-            cp_async_4(rg_val + my_w * win + (p & mask), ls.val[my_w] + p);
-        }
-    };
-    if (my_w < W) top_up(s_cur[my_w], min(s_len[my_w], s_cur[my_w] + win));
-
-    for (uint32_t tl = t0; tl < t1; ++tl) {
-        const uint32_t lo = tl * (uint32_t)kDecTile;
-        const uint32_t hi = min(total_n, lo + (uint32_t)kDecTile);
-        const bool full = hi - lo == (uint32_t)kDecTile;
-        if (use_bulk && !APPLY && tid == 0) bulk_wait_read<0>();     // the previous tile has left the buffer
-        cp_async_wait_all();
-        if (tid == 0) s_bound = hi;
-        __syncthreads();                                 // rings complete, cursors settled, buffer free
-        stage_tile(s_tile, out, lo, hi, full, zero_first, use_bulk, tid);
-        uint32_t sub_lo = lo;
-        while (true) {
-            // a worker whose ring is full and ends inside the tile may have more entries there
-            if ((uint32_t)tid < W) {
-                const uint32_t cur = s_cur[tid];
-                if (s_len[tid] - cur >= win) {
-                    const uint32_t last = rg_idx[tid * win + ((cur + win - 1u) & mask)];
-                    if (last < hi) atomicMin(&s_bound, last + 1u);
-                }
-            }
-            __syncthreads();                             // (also: the staged tile is visible)
-            uint32_t bound = s_bound;
-            if (bound <= sub_lo) {                       // no progress: a list is not ascending
-                if (tid == 0) record_status(hdr, -1 /*GC_E_INVALID*/, sub_lo);
-                bound = hi;
-            }
-            for (uint32_t q = 0; q < W; ++q) {           // worker order
-                const uint32_t cur = s_cur[q];
-                const uint32_t avail = min(s_len[q] - cur, win);
-                uint32_t adv = 0;
-                for (uint32_t i0 = 0; i0 < win; i0 += kDecBlock) {
-                    const uint32_t i = i0 + (uint32_t)tid;
-                    const uint32_t slot = q * win + ((cur + i) & mask);
-                    const uint32_t ix = i < avail ? rg_idx[slot] : 0xFFFFFFFFu;
-                    const bool in = ix < bound;
-                    if (in) {
-                        if (ix >= sub_lo) s_tile[ix - lo] = __fadd_rn(s_tile[ix - lo], rg_val[slot]);
-                        else record_status(hdr, -1 /*GC_E_INVALID*/, ix);      // behind the cursor: skipped
-                    }
-                    const uint32_t c = (uint32_t)__syncthreads_count(in ? 1 : 0);   // next worker may start
-                    adv += c;
-                    if (c < (uint32_t)kDecBlock) break;                          // ascending: nothing more below the bound
-                }
-                if (tid == 0) { s_cur[q] = cur + adv; s_adv[q] = adv; }
-            }
-            if (tid == 0) s_bound = hi;
-            __syncthreads();                             // cursors moved
-            if (my_w < W) {                              // the consumed slots are topped up
-                const uint32_t cur = s_cur[my_w], len = s_len[my_w];
-                top_up(min(len, cur - s_adv[my_w] + win), min(len, cur + win));
-            }
-            if (bound >= hi) break;
-            cp_async_wait_all();
-            __syncthreads();
-            sub_lo = bound;
-        }
-        if (APPLY) {
-            apply_tile(ap, s_tile, lo, hi, full, tid);
-            continue;                                    // (the barrier at the top of the loop orders the reuse)
-        }
-        if (full && use_bulk) {
-            if (tid == 0) bulk_store_tile(out + lo, s_tile, (uint32_t)(kDecTile * sizeof(float)));
-        } else {
-            for (uint32_t q = tid; q < hi - lo; q += kDecBlock) out[lo + q] = s_tile[q];
-        }
-    }
-    cp_async_wait_all();
-    __syncthreads();
-    if (t1 == ntl && tid < (int)W && s_cur[tid] < s_len[tid])
-        record_status(hdr, -1 /*GC_E_INVALID*/, s_cur[tid]);   // leftovers point at or beyond total_n
-    if (use_bulk && !APPLY && tid == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-}
-
-// Decode without a fixed order among the workers (GC_OPT_DECODE_ORDER = GC_ORDER_ANY): the rings
-// of k_decode_wide, but all entries of a pass are added at once with shared-memory atomics, so
-// a tile costs a constant number of block-wide steps whatever W is.  The sum of an element that
-// several workers hit is then rounded in an order that may change from run to run: every result
-// is within (hits - 1) x 2^-24 x sum |values| of the fixed-order one, and equal to it for
-// elements hit once.
-template <bool APPLY>
-static __global__ void __launch_bounds__(kDecBlock)
-k_decode_any(DecodeLists ls, uint32_t W, uint32_t cnt, uint32_t total_n, float* __restrict__ out,
-             int zero_first, int use_bulk, uint32_t win, WsHeader* hdr, ApplyArgs ap) {
-    extern __shared__ __align__(128) float s_tiles[];
-    float* const s_tile = s_tiles;
-    uint32_t* const rg_idx = reinterpret_cast<uint32_t*>(s_tiles + kDecTile);      // [W][win]
-    float* const rg_val = reinterpret_cast<float*>(rg_idx + W * win);              // [W][win]
-    __shared__ uint32_t s_cur[64], s_len[64], s_adv[64], s_bound;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint32_t ntl = (total_n + kDecTile - 1) / kDecTile;
-    const uint32_t per = (ntl + gridDim.x - 1) / gridDim.x;
-    const uint32_t t0 = blockIdx.x * per, t1 = min(ntl, t0 + per);
-    if (t0 >= t1) return;
-    const uint32_t mask = win - 1u;
-    // E consecutive threads serve one worker: they top up its ring and add its entries
-    int Wp = 1;
-    while (Wp < (int)W && Wp < 64) Wp <<= 1;
-    const int E = kDecBlock / Wp;
-    const uint32_t my_w = (uint32_t)(tid / E);
-    const int sub = tid % E;
-
-    for (uint32_t w = warp; w < W; w += kDecBlock / 32) {
-        const uint32_t len = ls.len[w] != nullptr ? min(__ldg(ls.len[w]), cnt) : cnt;
-        const uint32_t c = warp_lower_bound(ls.idx[w], len, t0 * (uint32_t)kDecTile, lane);
-        if (lane == 0) { s_cur[w] = c; s_len[w] = len; s_adv[w] = 0u; }
-    }
-    __syncthreads();
-    auto top_up = [&](uint32_t from, uint32_t to) {      // list positions [from, to) of worker my_w go to their ring slots
-        for (uint32_t p = from + (uint32_t)sub; p < to; p += (uint32_t)E) {
-            cp_async_4(rg_idx + my_w * win + (p & mask), ls.idx[my_w] + p);
-            cp_async_4(rg_val + my_w * win + (p & mask), ls.val[my_w] + p);
-        }
-    };
-    if (my_w < W) top_up(s_cur[my_w], min(s_len[my_w], s_cur[my_w] + win));
-
-    for (uint32_t tl = t0; tl < t1; ++tl) {
-        const uint32_t lo = tl * (uint32_t)kDecTile;
-        const uint32_t hi = min(total_n, lo + (uint32_t)kDecTile);
-        const bool full = hi - lo == (uint32_t)kDecTile;
-        if (use_bulk && !APPLY && tid == 0) bulk_wait_read<0>();     // the previous tile has left the buffer
-        cp_async_wait_all();
-        if (tid == 0) s_bound = hi;
-        __syncthreads();                                 // rings complete, cursors settled, buffer free
-        stage_tile(s_tile, out, lo, hi, full, zero_first, use_bulk, tid);
-        uint32_t sub_lo = lo;
-        while (true) {
-            if ((uint32_t)tid < W) {                     // a full ring that ends inside the tile may hide more entries
-                const uint32_t cur = s_cur[tid];
-                s_adv[tid] = 0u;
-                if (s_len[tid] - cur >= win) {
-                    const uint32_t last = rg_idx[tid * win + ((cur + win - 1u) & mask)];
-                    if (last < hi) atomicMin(&s_bound, last + 1u);
-                }
-            }
-            __syncthreads();                             // (also: the staged tile is visible)
-            uint32_t bound = s_bound;
-            if (bound <= sub_lo) {                       // no progress: a list is not ascending
-                if (tid == 0) record_status(hdr, -1 /*GC_E_INVALID*/, sub_lo);
-                bound = hi;
-            }
-            if (my_w < W) {
-                const uint32_t cur = s_cur[my_w];
-                const uint32_t avail = min(s_len[my_w] - cur, win);
-                uint32_t below = 0;
-                for (uint32_t i = (uint32_t)sub; i < avail; i += (uint32_t)E) {
-                    const uint32_t slot = my_w * win + ((cur + i) & mask);
-                    const uint32_t ix = rg_idx[slot];
-                    if (ix >= bound) break;                                      // ascending: the rest lies above
-                    ++below;
-                    if (ix < sub_lo) { record_status(hdr, -1 /*GC_E_INVALID*/, ix); continue; }   // behind the cursor: skipped
-                    atomicAdd(&s_tile[ix - lo], rg_val[slot]);
-                }
-                if (below) atomicAdd(&s_adv[my_w], below);
-            }
-            __syncthreads();                             // the tile is complete up to the bound
-            if ((uint32_t)tid < W) s_cur[tid] += s_adv[tid];
-            if (tid == 0) s_bound = hi;
-            __syncthreads();                             // cursors moved
-            if (my_w < W) {                              // the consumed slots are topped up
-                const uint32_t nc = s_cur[my_w], len = s_len[my_w];
-                top_up(min(len, nc - s_adv[my_w] + win), min(len, nc + win));
-            }
-            if (bound >= hi) break;
-            cp_async_wait_all();
-            __syncthreads();
-            sub_lo = bound;
-        }
-        if (APPLY) {
-            apply_tile(ap, s_tile, lo, hi, full, tid);
-            continue;                                    // (the barrier at the top of the loop orders the reuse)
-        }
-        if (full && use_bulk) {
-            if (tid == 0) bulk_store_tile(out + lo, s_tile, (uint32_t)(kDecTile * sizeof(float)));
-        } else {
-            for (uint32_t q = tid; q < hi - lo; q += kDecBlock) out[lo + q] = s_tile[q];
-        }
-    }
-    cp_async_wait_all();
-    __syncthreads();
-    if (t1 == ntl && tid < (int)W && s_cur[tid] < s_len[tid])
-        record_status(hdr, -1 /*GC_E_INVALID*/, s_cur[tid]);   // leftovers point at or beyond total_n
-    if (use_bulk && !APPLY && tid == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
 }  // namespace gc
