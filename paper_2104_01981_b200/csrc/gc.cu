@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <initializer_list>
 #include <new>
 #include <utility>
 #include <vector>
@@ -97,7 +98,7 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 constexpr size_t kSingleMidCap = 65536;      // short list of k_topk_single (candidates in the band bin of the threshold)
 constexpr uint64_t kSampleMax = 131072;       // most sampled elements per tensor
 constexpr uint64_t kSampleMaxSingle = 262144;   // ... when the plan holds one tensor (the sample is read in one step)
-constexpr uint32_t kSinglePoolMax = 16384;   // most candidates one CTA of k_topk_single may hold
+constexpr uint32_t kSinglePoolMax = 98304;   // most candidates one CTA of the fused top-k kernels may hold
 // Share of the oldest CTA of an SM above (and of the youngest below) the middle one's: measured
 // best between 6 and 10 % on the 110M-element workload at 1 % density.  At 0.1 % density the
 // fold loop has fewer candidates to handle, competes less for issue slots, and 4 % did better
@@ -105,7 +106,7 @@ constexpr uint32_t kSinglePoolMax = 16384;   // most candidates one CTA of k_top
 constexpr double kSingleSkew = 0.08, kSingleSkewSparse = 0.04;
 constexpr size_t kSingleRowBytes = (2 * kWarps + 3) * sizeof(uint32_t);   // shared memory per owned tile
 constexpr uint32_t kMultiMaxTab = 1024;      // tensors whose tile tables k_topk_multi keeps in shared memory
-constexpr size_t kMultiMaxPer = 160;         // most tiles one CTA of k_topk_multi may own
+constexpr size_t kMultiMaxPer = 224;         // most tiles one CTA of k_topk_multi may own
 constexpr size_t kMultiRowBytes = (2 * kWarps + kSegWords) * sizeof(uint32_t);   // shared memory per owned tile
 constexpr size_t kSingleMaxT = 341;          // most tiles one CTA of k_topk_single may own
 
@@ -170,6 +171,10 @@ void sample_params(TensorDesc& d, double density, uint32_t rank_permille, uint64
     *ccap = n;
     *nsg_if_sampled = 0;
     if (d.ntiles <= 1) { d.kind = kKindSmall; *ccap = 0; return; }   // fits one tile: one CTA does the whole tensor
+    // Several tensors: a sample the kernel can rank a second time (kRefineTiles sample tiles) gives tau
+    // 22 bits instead of a bin edge (12 % in value).  From 1 % on that is worth more than a larger sample:
+    // the margin of 32,000 samples is a third of k at 1 % and 15 % at 5 %, a bin edge costs up to as much again.
+    if (target_max == kSampleMax && density >= 0.01) target_max = 32000;
     uint64_t target = std::min<uint64_t>(target_max, std::max<uint64_t>(n / 128, std::min<uint64_t>(8192, n / 2)));
     uint64_t stride = std::max<uint64_t>(1, n / target);
     uint64_t groups = (n + 3) / 4;
@@ -201,7 +206,7 @@ void finish_layout(gc_plan_s* p) {
             // (many tensors: the bracket is a histogram bin edge, up to twice the candidates)
             uint64_t nsg_w = 0;
             sample_params(d, p->density, p->rank_permille, &ccap, p->T == 1 ? kSampleMaxSingle : kSampleMax,
-                          p->T == 1 ? 1.0 : 2.0, &nsg_w);
+                          p->T == 1 ? (p->density <= 0.1 ? 1.3 : 1.0) : 2.0, &nsg_w);
             stiles_worst += (nsg_w + (uint64_t)kSampleTile - 1) / (uint64_t)kSampleTile;
         } else {
             // threshold mode: the sample is part of the definition -- one 4-element group out of
@@ -413,7 +418,7 @@ MultiGeom multi_geometry(const gc_plan_s* p, uint32_t G, bool age_skew) {
     const uint32_t per = (p->ntiles + G - 1) / G;
     if (per > kMultiMaxPer) return mg;
     const uint32_t pool = std::min<uint32_t>(p->cand_cap_alloc / G, kSinglePoolMax);
-    // expected candidates of the busiest CTA (bracket rank over sample size, times two for the
+    // expected candidates of the busiest CTA (bracket rank over sample size, times two where tau is a
     // bin edge), with head-room
     std::vector<double> per_tile(p->T, 0.0);
     for (uint32_t t = 0; t < p->T; ++t) {
@@ -421,7 +426,8 @@ MultiGeom multi_geometry(const gc_plan_s* p, uint32_t G, bool age_skew) {
         if (d.kind == kKindSmall || d.ntiles == 0) continue;
         if (d.sstride == 0) { per_tile[t] = (double)kTile; continue; }
         const uint64_t groups = ((uint64_t)d.n + 3) / 4, nsg = (groups + d.sstride - 1) / d.sstride;
-        per_tile[t] = std::min<double>(kTile, 2.0 * (double)kTile * (double)d.srank / (4.0 * (double)nsg));
+        const double edge = d.nstiles <= kRefineTiles ? 1.02 : 2.0;      // tau is exact to 22 bits, or a bin edge
+        per_tile[t] = std::min<double>(kTile, edge * (double)kTile * (double)d.srank / (4.0 * (double)nsg));
     }
     // runs: `per` tiles for the first two thirds of a full grid, the rest spread over the last third
     // (the youngest CTAs of their SMs, which advance the slowest); every CTA `per` tiles otherwise
@@ -488,6 +494,13 @@ int blocks_per_sm(K kernel, int threads) {
         nb = 1;
     }
     return nb;
+}
+
+// Lets every kernel of the list be launched with up to `bytes` of dynamic shared memory.
+bool allow_smem(std::initializer_list<const void*> kernels, size_t bytes) {
+    for (const void* fn : kernels)
+        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) return false;
+    return true;
 }
 
 }  // namespace
@@ -638,8 +651,9 @@ int gc_plan(gc_plan_t** out, int device, uint32_t n_tensors, const uint64_t* siz
         p->grid_single_max = 0;
         if (coop) {
             int nb = 0;       // sized for the largest chunk-record block the kernel may be given
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_topk_single<GradF32>, kBlock, kSingleMaxT * kSingleRowBytes + kSinglePoolMax / 8) ==
-                    cudaSuccess && nb >= 1)
+            const size_t smem_max = kSingleMaxT * kSingleRowBytes + kSinglePoolMax / 8;
+            if (allow_smem({(const void*)k_topk_single<GradF32>, (const void*)k_topk_single<GradBF16>}, smem_max) &&
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_topk_single<GradF32>, kBlock, smem_max) == cudaSuccess && nb >= 1)
                 p->grid_single_max = p->sm_count * nb;
         }
         (void)cudaGetLastError();
@@ -660,7 +674,8 @@ int gc_plan(gc_plan_t** out, int device, uint32_t n_tensors, const uint64_t* siz
             int nb = 0;
             p->thrm_smem_max = kMultiMaxPer * kMultiRowBytes + 8 * kMultiMaxTab;
             int nbw = 0;          // (the several-workers form of the kernel must be as resident as the kernel itself)
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_threshold_multi, kBlock, p->thrm_smem_max) ==
+            if (allow_smem({(const void*)k_threshold_multi, (const void*)k_threshold_workers}, p->thrm_smem_max) &&
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_threshold_multi, kBlock, p->thrm_smem_max) ==
                     cudaSuccess && nb >= 1 &&
                 cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nbw, k_threshold_workers, kBlock, p->thrm_smem_max) ==
                     cudaSuccess && nbw >= 1)
@@ -674,7 +689,9 @@ int gc_plan(gc_plan_t** out, int device, uint32_t n_tensors, const uint64_t* siz
             int nb = 0;
             p->multi_smem_max = kMultiMaxPer * kMultiRowBytes + kSinglePoolMax / 8 + 8 * kMultiMaxTab;
             int nbw = 0;          // (the several-workers form of the kernel must be as resident as the kernel itself)
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_topk_multi<GradF32>, kBlock, p->multi_smem_max) ==
+            if (allow_smem({(const void*)k_topk_multi<GradF32>, (const void*)k_topk_multi<GradBF16>,
+                            (const void*)k_topk_workers<GradF32>}, p->multi_smem_max) &&
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_topk_multi<GradF32>, kBlock, p->multi_smem_max) ==
                     cudaSuccess && nb >= 1 &&
                 cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nbw, k_topk_workers<GradF32>, kBlock, p->multi_smem_max) ==
                     cudaSuccess && nbw >= 1)
@@ -714,11 +731,9 @@ int gc_plan(gc_plan_t** out, int device, uint32_t n_tensors, const uint64_t* siz
                 cudaSuccess || nb < 1) { (void)cudaGetLastError(); nb = 0; }
         p->grid_decode_seg_apply = p->sm_count * nb;
     }
-    p->rings_ok = true;
-    for (const void* fn : {(const void*)k_decode_rings<false, false, false>, (const void*)k_decode_rings<false, false, true>,
-                           (const void*)k_decode_rings<false, true, false>, (const void*)k_decode_rings<false, true, true>,
-                           (const void*)k_decode_rings<true, false, false>, (const void*)k_decode_rings<true, false, true>})
-        p->rings_ok = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRingSmem2) == cudaSuccess && p->rings_ok;
+    p->rings_ok = allow_smem({(const void*)k_decode_rings<false, false, false>, (const void*)k_decode_rings<false, false, true>,
+                              (const void*)k_decode_rings<false, true, false>, (const void*)k_decode_rings<false, true, true>,
+                              (const void*)k_decode_rings<true, false, false>, (const void*)k_decode_rings<true, false, true>}, kRingSmem2);
     (void)cudaGetLastError();
     p->grid_sample = p->sm_count * blocks_per_sm(k_hist<0, SRC_SAMPLE>, kBlock);
     p->grid_chist = p->sm_count * blocks_per_sm(k_cand_hist<1>, kBlock);

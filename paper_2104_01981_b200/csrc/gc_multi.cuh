@@ -26,7 +26,7 @@
 
 namespace gc {
 
-constexpr uint32_t kMultiMidCap = kMidFast;      // short list per tensor (entries stay in registers)
+constexpr uint32_t kMultiMidCap = 4u * kMidFast; // short list per tensor (the first kMidFast entries stay in registers)
 constexpr uint32_t kSegWords = 16;               // shared-memory words per segment record
 constexpr uint32_t kRefineTiles = 32;            // samples of up to this many sample tiles are ranked a second time
 constexpr uint32_t kWarpMid = 128;               // short lists up to this length are settled by one warp
@@ -258,10 +258,10 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
                 block_select_multi<(1 << level_bits(0)), 3>(sm, a.shist + (size_t)cur * kHistBins, want, pk);
                 if (pk[0].ok) tau = pk[0].bin << level_shift(0);
                 if (pk[0].ok && d.nstiles <= kRefineTiles) {
-                    // second radix level of the lower bracket over the kept sample keys:
-                    // tau gets 22 significant bits
+                    // second radix level of the lower bracket and of the guess over the kept sample keys:
+                    // tau and tau_z get 21 significant bits
                     const uint4* sk = a.skeys + (size_t)d.stile0 * kBlock;
-                    const uint32_t nk = d.nstiles * kBlock, bin0 = pk[0].bin;
+                    const uint32_t nk = d.nstiles * kBlock, bin0 = pk[0].bin, bin2 = pk[2].ok ? pk[2].bin : bin0;
                     for (uint32_t q0 = tid; q0 < nk; q0 += 4 * kBlock) {
                         uint4 kv[4];
 #pragma unroll
@@ -272,20 +272,25 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
                         for (int u = 0; u < 4; ++u) {
                             const uint32_t kk[4] = {kv[u].x, kv[u].y, kv[u].z, kv[u].w};
 #pragma unroll
-                            for (int e = 0; e < 4; ++e)
-                                if ((kk[e] >> level_shift(0)) == bin0)
-                                    atomicAdd(&sm.hist[(kk[e] >> (level_shift(0) - 11)) & 2047u], 1u);
+                            for (int e = 0; e < 4; ++e) {
+                                const uint32_t c = kk[e] >> level_shift(0);
+                                if (c == bin0 || c == bin2)
+                                    atomicAdd(&sm.hist[((kk[e] >> (level_shift(0) - 10)) & 1023u) + (c == bin0 ? 0u : 1024u)], 1u);
+                            }
                         }
                     }
                     __syncthreads();
-                    uint32_t bin1, above1;
-                    const bool ok1 = block_select<2048, true>(sm, sm.hist, d.srank - pk[0].above, bin1, above1);
+                    uint32_t bin1, above1, bin3, above3;
+                    const bool ok1 = block_select<1024, true>(sm, sm.hist, d.srank - pk[0].above, bin1, above1);
+                    const bool ok3 = pk[2].ok && block_select<1024, true>(sm, sm.hist + (bin2 == bin0 ? 0 : 1024),
+                                                                          want[2] - pk[2].above, bin3, above3);
                     for (int i2 = tid; i2 < 2048; i2 += kBlock) sm.hist[i2] = 0u;
                     __syncthreads();
-                    if (ok1) tau |= bin1 << (level_shift(0) - 11);
+                    if (ok1) tau |= bin1 << (level_shift(0) - 10);
+                    if (ok3) tau_z = (bin2 << level_shift(0)) | (bin3 << (level_shift(0) - 10));
                 }
                 if (pk[1].ok) tau_hi = (pk[1].bin + 1u) << level_shift(0);
-                if (pk[2].ok) {
+                if (pk[2].ok && tau_z == 0u) {
                     const float pos = ((float)(want[2] - pk[2].above) - 0.5f) / (float)pk[2].count;   // from the top of the bin
                     tau_z = (pk[2].bin << level_shift(0)) +
                             (uint32_t)((1.0f - pos) * (float)((1u << level_shift(0)) - 1u));
@@ -461,7 +466,7 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
         return (s[SG_TILE0] + (rel >> 12)) * kWarps + ((rel >> 9) & (kWarps - 1u));
     };
 
-    const bool overflowed = ld_cg(&hdr->overflow) != 0u;
+    const bool overflowed = ld_cg(&hdr->overflow) != 0u, by_chunk = used >= kChunkWalk * ntl * kWarps;
     if (!overflowed && nseg != 0u) {
         // ------------------------------------------------------------ band bin per segment, counts above it
         for (uint32_t sidx = (uint32_t)warp; sidx < nseg; sidx += kWarps) {      // a warp per segment, all at once
@@ -623,14 +628,16 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
                 // sent short-list entries: before the segment they shift its first slot, inside it
                 // they join the count of their chunk
                 const uint32_t seg_end = s[SG_BASE0] + s[SG_NTILE] * (uint32_t)kTile;
+                auto settle = [&](const uint2& pr) {
+                    const uint32_t key = pr.y & kKeyMask;
+                    if (!(key > Tkey || (key == Tkey && pr.x <= idx_cut))) return;
+                    if (pr.x < s[SG_BEGIN]) atomicAdd(&s_cnt, 1u);
+                    else if (pr.x < seg_end) atomicAdd(&rec2[chunk_of(s, pr.x)], 1u);
+                };
 #pragma unroll
-                for (uint32_t u = 0; u < kMidRegs; ++u) {
-                    if (!(good && u * kBlock + tid < m)) continue;
-                    const uint32_t key = e[u].y & kKeyMask;
-                    if (!(key > Tkey || (key == Tkey && e[u].x <= idx_cut))) continue;
-                    if (e[u].x < s[SG_BEGIN]) atomicAdd(&s_cnt, 1u);
-                    else if (e[u].x < seg_end) atomicAdd(&rec2[chunk_of(s, e[u].x)], 1u);
-                }
+                for (uint32_t u = 0; u < kMidRegs; ++u)
+                    if (good && u * kBlock + tid < m) settle(e[u]);
+                for (uint32_t i = kMidFast + tid; good && i < m; i += kBlock) settle(ld_cg(mid + i));
                 __syncthreads();
                 if (tid == 0) {
                     s[SG_TKEY] = Tkey; s[SG_CUT] = idx_cut;
@@ -666,21 +673,45 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
             const uint32_t key = pr.y & kKeyMask;
             return s[SG_OK] != 0u && (key > s[SG_TKEY] || (key == s[SG_TKEY] && pr.x <= s[SG_CUT]));
         };
-        const uint32_t nwords = (used + 31u) >> 5;
-        for (uint32_t i0 = 0; i0 < nwords * 32u; i0 += kBlock) {
-            const uint32_t i = i0 + tid;
-            if (i0 + (tid & ~31) >= nwords * 32u) continue;          // whole warp past the end
-            bool sent = false;
-            if (i < used) {
-                const uint2 pr = pool[i];
-                sent = sent_of(seg_of(pr.x), pr);
+        if (by_chunk) {                        // see for_chunks
+            const uint32_t* s = seg;
+            for_chunks(rec, ntl * kWarps, pool, warp, lane, [&](uint32_t c, uint32_t off, uint32_t cnt, const uint2 (&p)[2]) {
+                while (c / kWarps >= s[SG_TILE0] + s[SG_NTILE]) s += kSegWords;
+                uint32_t slot = rec2[c];
+                for (uint32_t q0 = 0; q0 < cnt; q0 += 32u) {
+                    const bool in = q0 + lane < cnt;
+                    const uint2 pr = q0 == 0u ? p[0] : q0 == 32u ? p[1] : in ? pool[off + q0 + lane] : make_uint2(0u, 0u);
+                    const bool sent = in && sent_of(s, pr), zeroed = (pr.y & kKeyMask) >= s[SG_TAUZ];
+                    const unsigned sb = __ballot_sync(0xFFFFFFFFu, sent);
+                    if (in && sent != zeroed) a.r[pr.x] = sent ? 0.0f : __uint_as_float(pr.y);
+                    if (sent) {
+                        const uint32_t at = slot + (uint32_t)__popc(sb & ((1u << lane) - 1u));
+                        __stcs(a.out_idx + at, pr.x);
+                        __stcs(a.out_val + at, __uint_as_float(pr.y));
+                    }
+                    slot += (uint32_t)__popc(sb);
+                }
+            });
+        }
+        const uint32_t nwords = by_chunk ? 0u : (used + 31u) >> 5;
+        for (uint32_t i0 = 0; i0 < nwords * 32u; i0 += 4 * kBlock) {      // four loads in flight per thread
+            uint2 pr[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const uint32_t i = i0 + u * kBlock + tid;
+                pr[u] = i < used ? pool[i] : make_uint2(0u, 0u);
             }
-            const unsigned sb = __ballot_sync(0xFFFFFFFFu, sent);
-            if (lane == 0) sent_bits[i >> 5] = sb;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const uint32_t i = i0 + u * kBlock + tid;
+                if (i0 + u * kBlock + (tid & ~31) >= nwords * 32u) continue;          // whole warp past the end
+                const unsigned sb = __ballot_sync(0xFFFFFFFFu, i < used && sent_of(seg_of(pr[u].x), pr[u]));
+                if (lane == 0) sent_bits[i >> 5] = sb;
+            }
         }
         __syncthreads();
         // emission: slot = first slot of the chunk + sent candidates before this one in the chunk
-        for (uint32_t i0 = tid; i0 < used; i0 += 4 * kBlock) {
+        for (uint32_t i0 = by_chunk ? used : tid; i0 < used; i0 += 4 * kBlock) {
             uint2 pr[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
