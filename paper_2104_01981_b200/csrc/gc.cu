@@ -98,13 +98,13 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 constexpr size_t kSingleMidCap = 65536;      // short list of k_topk_single (candidates in the band bin of the threshold)
 constexpr uint64_t kSampleMax = 131072;       // most sampled elements per tensor
 constexpr uint64_t kSampleMaxSingle = 262144;   // ... when the plan holds one tensor (the sample is read in one step)
-constexpr uint32_t kSinglePoolMax = 98304;   // most candidates one CTA of the fused top-k kernels may hold
+constexpr uint32_t kSinglePoolMax = 65536, kMultiPoolMax = 98304;   // most candidates one CTA of the fused kernels may hold
 // Share of the oldest CTA of an SM above (and of the youngest below) the middle one's: measured
 // best between 6 and 10 % on the 110M-element workload at 1 % density.  At 0.1 % density the
 // fold loop has fewer candidates to handle, competes less for issue slots, and 4 % did better
 // than 8 % (with 8 % the oldest CTAs of the 355M-element workload finished last).
 constexpr double kSingleSkew = 0.08, kSingleSkewSparse = 0.04;
-constexpr size_t kSingleRowBytes = (2 * kWarps + 3) * sizeof(uint32_t);   // shared memory per owned tile
+constexpr size_t kSingleRowBytes = (2 * kWarps + 4) * sizeof(uint32_t);   // shared memory per owned tile
 constexpr uint32_t kMultiMaxTab = 1024;      // tensors whose tile tables k_topk_multi keeps in shared memory
 constexpr size_t kMultiMaxPer = 224;         // most tiles one CTA of k_topk_multi may own
 constexpr size_t kMultiRowBytes = (2 * kWarps + kSegWords) * sizeof(uint32_t);   // shared memory per owned tile
@@ -267,7 +267,7 @@ void finish_layout(gc_plan_s* p) {
     p->off_hist5 = align_up(p->off_gstate + sizeof(unsigned long long) * (size_t)p->ngroups, 256);
     // one-tensor kernels: six 2048-bin histogram slots, then 32-CTA segment totals
     p->off_rowseg = align_up(p->off_hist5 + (T == 1 ? sizeof(uint32_t) * 6 * (size_t)kHistBins : 0), 256);
-    p->control_bytes = align_up(p->off_rowseg + (T == 1 ? sizeof(uint32_t) * kSingleMaxT * 20 : 0), 256);
+    p->control_bytes = align_up(p->off_rowseg + (T == 1 ? sizeof(uint32_t) * kSingleMaxT * 20 * 2 : 0), 256);
     p->off_fine = p->control_bytes;
     p->control_bytes = align_up(p->off_fine + (T == 1 ? sizeof(uint32_t) * (size_t)kFineBins : 0), 256);
     p->off_age = p->control_bytes;                                   // CTAs arrived per SM (one-tensor kernels)
@@ -417,7 +417,7 @@ MultiGeom multi_geometry(const gc_plan_s* p, uint32_t G, bool age_skew) {
     G = std::min<uint32_t>(G, p->ntiles);
     const uint32_t per = (p->ntiles + G - 1) / G;
     if (per > kMultiMaxPer) return mg;
-    const uint32_t pool = std::min<uint32_t>(p->cand_cap_alloc / G, kSinglePoolMax);
+    const uint32_t pool = std::min<uint32_t>(p->cand_cap_alloc / G, kMultiPoolMax);
     // expected candidates of the busiest CTA (bracket rank over sample size, times two where tau is a
     // bin edge), with head-room
     std::vector<double> per_tile(p->T, 0.0);
@@ -650,10 +650,16 @@ int gc_plan(gc_plan_t** out, int device, uint32_t n_tensors, const uint64_t* siz
         p->grid_fused = coop ? p->sm_count * blocks_per_sm(k_compress_fused, kBlock) : 0;
         p->grid_single_max = 0;
         if (coop) {
-            int nb = 0;       // sized for the largest chunk-record block the kernel may be given
+            // sized for the largest chunk-record block the kernel may be given; the form that fits least counts
             const size_t smem_max = kSingleMaxT * kSingleRowBytes + kSinglePoolMax / 8;
-            if (allow_smem({(const void*)k_topk_single<GradF32>, (const void*)k_topk_single<GradBF16>}, smem_max) &&
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_topk_single<GradF32>, kBlock, smem_max) == cudaSuccess && nb >= 1)
+            int nb = 1 << 20;
+            for (const void* fn : {(const void*)k_topk_single<GradF32, false>, (const void*)k_topk_single<GradF32, true>,
+                                   (const void*)k_topk_single<GradBF16, false>, (const void*)k_topk_single<GradBF16, true>}) {
+                int n1 = 0;
+                if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n1, fn, kBlock, smem_max) != cudaSuccess) n1 = 0;
+                nb = std::min(nb, n1);
+            }
+            if (nb >= 1)
                 p->grid_single_max = p->sm_count * nb;
         }
         (void)cudaGetLastError();
@@ -687,7 +693,7 @@ int gc_plan(gc_plan_t** out, int device, uint32_t n_tensors, const uint64_t* siz
         p->grid_multi_max = 0;
         if (coop) {
             int nb = 0;
-            p->multi_smem_max = kMultiMaxPer * kMultiRowBytes + kSinglePoolMax / 8 + 8 * kMultiMaxTab;
+            p->multi_smem_max = kMultiMaxPer * kMultiRowBytes + kMultiPoolMax / 8 + 8 * kMultiMaxTab;
             int nbw = 0;          // (the several-workers form of the kernel must be as resident as the kernel itself)
             if (allow_smem({(const void*)k_topk_multi<GradF32>, (const void*)k_topk_multi<GradBF16>,
                             (const void*)k_topk_workers<GradF32>}, p->multi_smem_max) &&
@@ -1034,12 +1040,15 @@ static int compress_impl(gc_plan_t* p, const void* grad_any, bool bf16, float* r
         sa.age = reinterpret_cast<uint32_t*>(wb + p->off_age);
         sa.tile_cnt = reinterpret_cast<uint32_t*>(wb + p->off_tinfo);
         sa.seg_tot = reinterpret_cast<uint32_t*>(wb + p->off_rowseg);
+        sa.tile_eq = sa.tile_cnt + nt; sa.seg_eq = sa.seg_tot + kSingleMaxT * 20;
         sa.ws = ws; sa.gws = gws;
         sa.cl = clean_args(p, workspace, GC_ROUTE_TOPK_ONE, kept_clean);
         note_clean(p, workspace);
         void* args[] = {&sa};
         Timed tm(p, s, GC_K_FUSED);
-        const void* kfn = bf16 ? (const void*)k_topk_single<GradBF16> : (const void*)k_topk_single<GradF32>;
+        const bool dense = p->density >= 0.02;
+        const void* kfn = bf16 ? (dense ? (const void*)k_topk_single<GradBF16, true> : (const void*)k_topk_single<GradBF16, false>)
+                               : (dense ? (const void*)k_topk_single<GradF32, true> : (const void*)k_topk_single<GradF32, false>);
         GC_CUDA(p, cudaLaunchCooperativeKernel(kfn, dim3(p->single_grid), dim3(kBlock), args, p->single_smem, s));
         return GC_OK;
     }

@@ -122,6 +122,7 @@ __device__ __forceinline__ unsigned long long ld_cg(const unsigned long long* p)
 // How the gradient is stored.  The kernels that read g are templates on one of these; the
 // arithmetic is fp32 either way (a bf16 value is an fp32 value with 16 zero bits appended).
 struct GradF32 {
+    static constexpr bool kManyTies = false;       // values with 24 significant bits
     static __device__ __forceinline__ float ld1(const void* g, uint32_t i) {
         return __ldg(reinterpret_cast<const float*>(g) + i);
     }
@@ -133,6 +134,7 @@ struct GradF32 {
     }
 };
 struct GradBF16 {
+    static constexpr bool kManyTies = true;        // 8 significant bits: equal magnitudes by the thousands
     static __device__ __forceinline__ float ld1(const void* g, uint32_t i) {
         return __uint_as_float((uint32_t)__ldg(reinterpret_cast<const unsigned short*>(g) + i) << 16);
     }

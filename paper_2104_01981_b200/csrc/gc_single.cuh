@@ -46,6 +46,9 @@ constexpr uint32_t kFineBins = 1u << (11 + kFineBits);
 __device__ __forceinline__ uint32_t fine_slot(uint32_t bin) { return (bin * 40503u) & (kFineBins - 1u); }
 constexpr uint32_t kMidRegs = 4;                       // short-list entries a thread keeps in registers
 constexpr uint32_t kMidFast = kMidRegs * kBlock;       // short lists up to this size are read once
+// Band bins with more candidates than this are not listed but counted (k_topk_single, "counted band"):
+// ranking a list costs every CTA five passes over it, counting costs one more grid barrier.
+constexpr uint32_t kMidCounted = 4096;
 
 // Rows of tiles.  A column is one CTA's share of the tensor: row i of column c is one tile, and
 // the tiles are numbered row by row.  The three CTAs that share an SM do not advance at the same
@@ -106,11 +109,13 @@ struct SingleArgs {
     uint2* cand;                     // [gridDim.x * pool_cap] candidate list, one region per CTA
     uint2* mid;                      // [mid_cap] candidates inside the band bin of the threshold
     uint32_t* hist5;                 // [0] coarse sample histogram, [2] band histogram,
-                                     // [3][0] short-list length (all zeroed)
+                                     // [3][0] short-list length, [4] keys inside a counted band (all zeroed)
     uint32_t* age;                   // [1024] CTAs that have arrived on every SM (zeroed)
     uint32_t* fine;                  // [kFineBins] fine sample histogram (zeroed)
     uint32_t* tile_cnt;              // [ntiles] candidates above the band bin, per tile
     uint32_t* seg_tot;               // [maxt][ceil(G/32)] the same summed over each run of 32 CTAs of a row (zeroed)
+    uint32_t* tile_eq;               // [ntiles], [maxt][ceil(G/32)] (zeroed): counted band, candidates that equal the
+    uint32_t* seg_eq;                // threshold key, per tile and per run of 32 CTAs of a row
     WsView ws, gws;
     CleanArgs cl;                    // the control block is left clean for the next launch
 };
@@ -289,7 +294,10 @@ __device__ __forceinline__ void for_chunks(const uint32_t* rec, uint32_t nchunks
 
 // Three CTAs per SM (80 registers, no spills): measured 15 us faster on the 110M-element workload
 // than four CTAs at 64 registers with spills, and than two.
-template <typename GL>
+// DENSE (plans of 2 % and more) has the emission by chunk, the bfloat16 form the counted band: the other
+// forms do without their code (a tensor of 1M elements runs every phase from a cold instruction cache:
+// 37.0 against 38.7 us for compress and decode).
+template <typename GL, bool DENSE>
 static __global__ void __launch_bounds__(kBlock, 3)
 k_topk_single(const __grid_constant__ SingleArgs a) {
     __shared__ BlockSmem sm;
@@ -301,7 +309,8 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
     uint32_t* const tile_base = rec2 + (size_t)a.maxt * kWarps;                // [maxt]
     uint32_t* const row_sum = tile_base + a.maxt;                              // [maxt]
     uint32_t* const row_mid = row_sum + a.maxt;                                // [maxt]
-    uint32_t* const sent_bits = row_mid + a.maxt;                              // [ceil(pool_cap / 32)]
+    uint32_t* const row_eq = row_mid + a.maxt;                                 // [maxt] (counted band)
+    uint32_t* const sent_bits = row_eq + a.maxt;                               // [ceil(pool_cap / 32)]
     // This CTA's region.  Only this CTA (hence only this SM) ever writes or reads it, and it is
     // never read before it is written, so the later phases may read it through L1.
     uint2* const pool = a.cand + (size_t)blockIdx.x * a.pool_cap;
@@ -568,9 +577,16 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
     Picked pa[1];
     block_select_multi<2048, 1>(sm, a.hist5 + 2 * kHistBins, want_k, pa);
     const uint32_t A = pa[0].bin, aboveA = pa[0].above, m = pa[0].count;      // m = candidates inside the band bin
-    bool good = overflowed == 0u && pa[0].ok && m <= a.mid_cap;
+    // A band bin with thousands of candidates (bfloat16 gradients tie by the thousands at the threshold)
+    // is counted: its keys are histogrammed one by one (at most 2048 of them), which gives the threshold
+    // key after the barrier; then every CTA counts its candidates above and at that key per tile, and
+    // after one more barrier the candidates at the key in the tiles before a tile say how many of its own
+    // are sent.  110M elements, bfloat16, 60,000 ties: counts + threshold + slots 15 + 41 us as a list.
+    const bool counted = GL::kManyTies && overflowed == 0u && pa[0].ok && m > kMidCounted && A < 2047u && shift <= 11;
+    bool good = overflowed == 0u && pa[0].ok && (m <= a.mid_cap || counted);
+    const uint32_t binlo = tau + (A << shift);
 
-    const bool by_chunk = used >= kChunkWalk * n_own * kWarps;
+    const bool by_chunk = DENSE && used >= kChunkWalk * n_own * kWarps;
     if (good) {
         // ------------------------------------------------------------ counts above the band bin
         // One linear pass over the CTA's candidates: those above the bin are counted per chunk
@@ -582,6 +598,7 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
                 const uint32_t rel = pr.x - base0;
                 atomicAdd(&rec2[rm.row_of(rel >> 12) * kWarps + ((rel >> 9) & (kWarps - 1u))], 1u);
             } else if (bin == A) {
+                if (counted) { atomicAdd(&sm.hist[(pr.y & kKeyMask) - binlo], 1u); return; }
                 const uint32_t slot = atomicAdd(a.hist5 + 3 * kHistBins, 1u);
                 if (slot < a.mid_cap) a.mid[slot] = pr;
             }
@@ -600,13 +617,40 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
             for (int u = 0; u < 4; ++u)
                 if (i0 + u * kBlock < used) classify(pr[u]);
         }
+        uint32_t Tkey = 0, m_eq = 0;
+        if (counted) {
+            flush_hist(sm, a.hist5 + 4 * kHistBins, 2048);
+            if (!grid_barrier(hdr, passed, &sm.ok)) return;
+            phase_stamp(hdr, n_stamp);
+            const uint32_t want_in[1] = {d.k - aboveA};
+            Picked pt[1];
+            block_select_multi<2048, 1>(sm, a.hist5 + 4 * kHistBins, want_in, pt);
+            Tkey = binlo + pt[0].bin; m_eq = d.k - aboveA - pt[0].above;
+            // per chunk: candidates above the threshold key in the low half, those at it in the high half
+            for (uint32_t i0 = tid; i0 < used; i0 += 8 * kBlock) {
+                uint2 pr[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) pr[u] = i0 + u * kBlock < used ? pool[i0 + u * kBlock] : make_uint2(0u, 0u);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const uint32_t key = pr[u].y & kKeyMask;
+                    if (i0 + u * kBlock >= used || key < Tkey || min((key - tau) >> shift, 2047u) != A) continue;
+                    const uint32_t rel = pr[u].x - base0;
+                    atomicAdd(&rec2[rm.row_of(rel >> 12) * kWarps + ((rel >> 9) & (kWarps - 1u))], key == Tkey ? 1u << 16 : 1u);
+                }
+            }
+        }
         __syncthreads();
         for (uint32_t i = tid; i < n_own; i += kBlock) {
-            uint32_t tot = 0;
+            uint32_t tot = 0, eq = 0;
 #pragma unroll
-            for (int w = 0; w < kWarps; ++w) tot += rec2[i * kWarps + w];
+            for (int w = 0; w < kWarps; ++w) { tot += rec2[i * kWarps + w] & 0xFFFFu; eq += rec2[i * kWarps + w] >> 16; }
             a.tile_cnt[rm.tile_of(i, col)] = tot;
             atomicAdd(a.seg_tot + (size_t)i * nseg + myseg, tot);
+            if (counted) {
+                a.tile_eq[rm.tile_of(i, col)] = eq;
+                atomicAdd(a.seg_eq + (size_t)i * nseg + myseg, eq);
+            }
         }
         if (!grid_barrier(hdr, passed, &sm.ok)) return;
         phase_stamp(hdr, n_stamp);
@@ -618,7 +662,7 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
         uint2 e[kMidRegs];
 #pragma unroll
         for (uint32_t u = 0; u < kMidRegs; ++u)
-            e[u] = u * kBlock + tid < m ? ld_cg(a.mid + u * kBlock + tid) : make_uint2(0u, 0u);
+            e[u] = !counted && u * kBlock + tid < m ? ld_cg(a.mid + u * kBlock + tid) : make_uint2(0u, 0u);
         // while those loads fly: per row, the candidates above the bin in the whole row and in
         // the tiles of lower CTAs (whole 32-CTA segments below this CTA's + the lower CTAs of
         // its own segment): two loads per lane and row, two rows per step
@@ -637,13 +681,24 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
                 if (lane == 0 && i0 + u < n_own) { row_sum[i0 + u] = row; tile_base[i0 + u] = low; }
             }
         }
-        const uint32_t binlo = tau + (A << shift);
-        uint32_t v_sel, mid_gt, n_eq, idx_cut = 0xFFFFFFFFu;
+        if (counted) {                                    // the same for the candidates at the threshold key
+            for (uint32_t i = warp; i < n_own; i += kWarps) {
+                const uint32_t q = myseg * 32u + (uint32_t)lane;
+                const uint32_t sv = (uint32_t)lane < nseg ? ld_cg(a.seg_eq + (size_t)i * nseg + lane) : 0u;
+                const uint32_t tv = q < col ? ld_cg(a.tile_eq + rm.tile_of(i, q)) : 0u;
+                const uint32_t row = __reduce_add_sync(0xFFFFFFFFu, sv);
+                const uint32_t low = __reduce_add_sync(0xFFFFFFFFu, tv + ((uint32_t)lane < myseg ? sv : 0u));
+                if (lane == 0) { row_eq[i] = low; row_mid[i] = row; }
+            }
+        }
+        uint32_t v_sel, mid_gt, n_eq = 0, cut_end = 0xFFFFFFFFu;      // candidates at Tkey are sent below index cut_end
+        if (!counted) {
         good = short_list_select(sm, e, a.mid, m, A == 2047u ? 31 : max(shift, 1), d.k - aboveA,
                                  [&](const uint2& pr, uint32_t& v) { v = (pr.y & kKeyMask) - binlo; return true; },
                                  v_sel, mid_gt, n_eq);
-        const uint32_t Tkey = binlo + v_sel;
-        const uint32_t m_eq = d.k - aboveA - mid_gt;      // entries equal to Tkey that are sent
+        Tkey = binlo + v_sel;
+        m_eq = d.k - aboveA - mid_gt;      // entries equal to Tkey that are sent
+        }
         if (good && n_eq > m_eq && n_eq <= (uint32_t)kBlock) {
             // a few entries tie at the threshold: list their indices, rank them directly
             auto note = [&](const uint2& pr) {
@@ -661,7 +716,7 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
                 if (lower == m_eq - 1u) sm.scratch[0] = mine;
             }
             __syncthreads();
-            idx_cut = sm.scratch[0];
+            cut_end = sm.scratch[0] + 1u;
             __syncthreads();
             if ((uint32_t)tid < n_eq) sm.hist[tid] = 0u;
             if (tid == 0) sm.hist[2047] = 0u;
@@ -671,7 +726,7 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
             good = short_list_select(sm, e, a.mid, m, 32, m_eq,
                                      [&](const uint2& pr, uint32_t& v) { v = ~pr.x; return (pr.y & kKeyMask) == Tkey; },
                                      v_idx, x0, x1);
-            idx_cut = ~v_idx;
+            cut_end = ~v_idx + 1u;
         }
         // (a failure here would mean the short list changed under us; all CTAs see the same)
         if (good) {
@@ -681,7 +736,7 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
             // tile it also raises the count of its chunk.
             auto sent_key = [&](const uint2& pr) {
                 const uint32_t key = pr.y & kKeyMask;
-                return key > Tkey || (key == Tkey && pr.x <= idx_cut);
+                return key > Tkey || (key == Tkey && pr.x < cut_end);
             };
             auto below = [&](const uint2& pr) {
                 if (!sent_key(pr)) return;
@@ -694,22 +749,65 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
             };
 #pragma unroll
             for (uint32_t u = 0; u < kMidRegs; ++u)
-                if (u * kBlock + tid < m) below(e[u]);
-            for (uint32_t i = kMidFast + tid; i < m; i += kBlock) below(ld_cg(a.mid + i));
+                if (!counted && u * kBlock + tid < m) below(e[u]);
+            for (uint32_t i = kMidFast + tid; !counted && i < m; i += kBlock) below(ld_cg(a.mid + i));
+            if (tid == 0) { sm.scratch[0] = 0u; sm.scratch[1] = 0xFFFFFFFFu; }
             __syncthreads();
             if (warp == 0) {
                 // tile_base[i] = rows before i + lower CTAs of row i + sent short-list entries before the tile
-                uint32_t run = 0;
+                // (counted band: + the candidates at the threshold key in the tiles before it, as far as sent)
+                uint32_t run = 0, run_eq = 0;
                 for (uint32_t i0 = 0; i0 < n_own; i0 += 32) {
                     const uint32_t i = i0 + lane;
                     const uint32_t v = i < n_own ? row_sum[i] : 0u;
                     const uint32_t w = i < n_own ? row_mid[i] : 0u;
-                    const uint32_t inc = warp_incl_scan(v + w, lane);
-                    if (i < n_own) tile_base[i] += run + inc - v;
-                    run += __shfl_sync(0xFFFFFFFFu, inc, 31);
+                    if (counted) {
+                        const uint32_t inc = warp_incl_scan(v, lane), inc_eq = warp_incl_scan(w, lane);
+                        if (i < n_own) {
+                            const uint32_t eq = row_eq[i] + run_eq + inc_eq - w;
+                            row_eq[i] = eq;
+                            tile_base[i] += run + inc - v + min(eq, m_eq);
+                        }
+                        run += __shfl_sync(0xFFFFFFFFu, inc, 31);
+                        run_eq += __shfl_sync(0xFFFFFFFFu, inc_eq, 31);
+                    } else {
+                        const uint32_t inc = warp_incl_scan(v + w, lane);
+                        if (i < n_own) tile_base[i] += run + inc - v;
+                        run += __shfl_sync(0xFFFFFFFFu, inc, 31);
+                    }
                 }
             }
             __syncthreads();
+            if (counted) {
+                // what every chunk sends; this CTA's cut: the end of its last chunk that sends all its
+                // candidates at the key, or a place inside the one chunk (of the whole tensor) that sends some
+                for (uint32_t i = tid; i < n_own; i += kBlock) {
+                    uint32_t left = m_eq - min(row_eq[i], m_eq);
+                    const uint32_t tile_lo = base0 + rm.tile_of(i, col) * (uint32_t)kTile;
+#pragma unroll
+                    for (uint32_t w = 0; w < (uint32_t)kWarps; ++w) {
+                        const uint32_t c = rec2[i * kWarps + w], eq = c >> 16, take = min(eq, left);
+                        rec2[i * kWarps + w] = (c & 0xFFFFu) + take;
+                        left -= take;
+                        if (take != 0u && take == eq) atomicMax(&sm.scratch[0], tile_lo + (w + 1u) * kWarpChunk);
+                        if (take != 0u && take != eq) { sm.scratch[1] = i * kWarps + w; sm.scratch[2] = take; }
+                    }
+                }
+                __syncthreads();
+                if (warp == 0 && sm.scratch[1] != 0xFFFFFFFFu) {
+                    const uint32_t rc = rec[sm.scratch[1]], cnt = rc & 1023u, take = sm.scratch[2];
+                    uint32_t seen = 0;                     // (a chunk's candidates are in index order)
+                    for (uint32_t q0 = 0; q0 < cnt && seen < take; q0 += 32u) {
+                        const uint2 pr = q0 + lane < cnt ? pool[(rc >> 10) + q0 + lane] : make_uint2(0u, 0u);
+                        const bool at = q0 + lane < cnt && (pr.y & kKeyMask) == Tkey;
+                        const unsigned b32 = __ballot_sync(0xFFFFFFFFu, at);
+                        if (at && seen + (uint32_t)__popc(b32 & ((1u << lane) - 1u)) == take - 1u) sm.scratch[0] = pr.x + 1u;
+                        seen += (uint32_t)__popc(b32);
+                    }
+                }
+                __syncthreads();
+                cut_end = sm.scratch[0];
+            }
             // rec2[c] = output slot of the first sent candidate of chunk c
             for (uint32_t i = tid; i < n_own; i += kBlock) {
                 uint32_t pos = tile_base[i];
