@@ -236,9 +236,10 @@ void finish_layout(gc_plan_s* p) {
     }
     p->nstiles = (uint32_t)stile0;
     p->ngroups = (uint32_t)group0;
-    // tiny tensors (one warp each in the many-tensor top-k kernel) first in the list of small ones
+    // tiny tensors (one warp each in the many-tensor kernels) first in the list of small ones
     {
-        auto tiny = [&](uint32_t t) { return p->mode == GC_TOPK && is_tiny(p->desc[t].n, p->desc[t].k); };
+        // (threshold mode: a tensor of that size is sampled in full, its rank is k)
+        auto tiny = [&](uint32_t t) { return is_tiny(p->desc[t].n, p->desc[t].k); };
         std::stable_partition(p->small_ids.begin(), p->small_ids.end(), tiny);
         p->n_tiny = (uint32_t)std::count_if(p->small_ids.begin(), p->small_ids.end(), tiny);
     }
@@ -898,7 +899,7 @@ static ThrMultiArgs thr_multi_args(const gc_plan_s* p, const MultiGeom& mg, cons
     ThrMultiArgs ta;
     ta.desc = p->d_desc; ta.T = p->T; ta.ntiles = p->ntiles; ta.nstiles = p->nstiles;
     ta.per = mg.per; ta.pool_cap = mg.pool; ta.ntab = mg.ntab;
-    ta.small_ids = p->d_small; ta.n_small = (uint32_t)p->small_ids.size();
+    ta.small_ids = p->d_small; ta.n_small = (uint32_t)p->small_ids.size(); ta.n_tiny = p->n_tiny;
     ta.reg_ids = p->d_small + p->T; ta.n_reg = (uint32_t)p->reg_ids.size();
     ta.g = grad; ta.r = residual; ta.out_idx = out_idx; ta.out_val = out_val; ta.out_count = out_count;
     ta.cand = reinterpret_cast<uint2*>(wb + p->off_cidx);

@@ -27,7 +27,7 @@ struct ThrMultiArgs {
     uint32_t pool_cap;               // hit slots per CTA
     uint32_t ntab;                   // T if the tile tables fit in shared memory, else 0
     const uint32_t* small_ids;       // tensors that fit one tile
-    uint32_t n_small;
+    uint32_t n_small, n_tiny;        // (the tiny ones, a warp each, first)
     const uint32_t* reg_ids;         // the others (with elements)
     uint32_t n_reg;
     const float* g;
@@ -42,6 +42,54 @@ struct ThrMultiArgs {
     TensorSel* tsel;                 // [T] .T receives tau
     WsView ws;
 };
+
+// A tiny tensor (at most kTinyMaxN elements, sampled in full, rank at most kTinyMaxK) by one warp:
+// tau by rounds of a warp-wide maximum over the keys below the last one, each with its multiplicity.
+static __device__ __noinline__ void tiny_threshold_warp(const TensorDesc& d, uint32_t t, uint32_t T, const float* __restrict__ g,
+                                                        float* __restrict__ r, uint32_t* __restrict__ out_idx,
+                                                        float* __restrict__ out_val, uint32_t* __restrict__ out_count,
+                                                        WsHeader* hdr, int lane) {
+    constexpr int kU = (int)kTinyMaxN / 32;               // element i sits in lane i % 32, slot i / 32
+    float av[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+        const uint32_t i = (uint32_t)lane + 32u * u;
+        av[u] = i < d.n ? __fadd_rn(__ldg(g + d.off + i), r[d.off + i]) : 0.f;
+    }
+    uint32_t tau = 0x80000000u, left = d.srank;
+    while (true) {
+        uint32_t best = 0u, same = 0u;                    // largest key below the last one, plus 1
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const uint32_t key = key_of(av[u]);
+            if ((uint32_t)lane + 32u * u < d.n && key < tau) best = max(best, key + 1u);
+        }
+        best = __reduce_max_sync(0xFFFFFFFFu, best);
+        if (best == 0u) break;                            // (the rank never exceeds the number of elements)
+        tau = best - 1u;
+#pragma unroll
+        for (int u = 0; u < kU; ++u) same += ((uint32_t)lane + 32u * u < d.n && key_of(av[u]) == tau) ? 1u : 0u;
+        same = __reduce_add_sync(0xFFFFFFFFu, same);
+        if (same >= left) break;
+        left -= same;
+    }
+    uint32_t hits = 0;
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+        const uint32_t i = (uint32_t)lane + 32u * u;
+        const bool hit = i < d.n && key_of(av[u]) >= tau;
+        const unsigned b = __ballot_sync(0xFFFFFFFFu, hit);
+        const uint32_t slot = hits + (uint32_t)__popc(b & ((1u << lane) - 1u));
+        const bool sent = hit && slot < d.cap;
+        if (sent) { out_idx[d.out_off + slot] = d.off + i; out_val[d.out_off + slot] = av[u]; }
+        if (i < d.n) r[d.off + i] = sent ? 0.0f : av[u];
+        hits += (uint32_t)__popc(b);
+    }
+    if (lane == 0) {
+        if (out_count != nullptr) { out_count[t] = min(hits, d.cap); out_count[T + t] = hits; }
+        if (hits > d.cap) record_status(hdr, 1 /*GC_W_TRUNCATED*/, t);
+    }
+}
 
 // A tensor that fits one tile, start to finish by one CTA: exact k_s-th largest key of its own
 // sample (three shared-memory radix levels over registers), then every element at or above it
@@ -64,6 +112,36 @@ static __device__ __noinline__ void small_threshold_body(BlockSmem& sm, const Te
             if (((tl.valid >> (4 * j + e)) & 1u) && (((f - d.off) >> 2) % d.sstride) == 0u) smask |= 1u << (4 * j + e);
         }
     uint32_t prefix = 0, krem = d.srank;
+    if (d.srank <= kFewK) {
+        // a small rank: rounds of a block-wide maximum over the keys below the last one, each with its
+        // multiplicity (two barriers a round; the histogram levels take some twenty)
+        uint32_t upper = 0x80000000u;
+        while (true) {
+            uint32_t best = 0u, same = 0u;
+#pragma unroll
+            for (int q = 0; q < 4 * kVpt; ++q) {
+                const uint32_t key = key_of(tl.a[q / 4][q % 4]);
+                if (((smask >> q) & 1u) && key < upper) best = max(best, key + 1u);
+            }
+            best = __reduce_max_sync(0xFFFFFFFFu, best);
+            if (lane == 0) sm.scratch[warp] = best;
+            __syncthreads();
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) best = max(best, sm.scratch[w]);
+            if (best == 0u) break;                         // (the rank never exceeds the size of the sample)
+            prefix = upper = best - 1u;
+#pragma unroll
+            for (int q = 0; q < 4 * kVpt; ++q) same += (((smask >> q) & 1u) && key_of(tl.a[q / 4][q % 4]) == upper) ? 1u : 0u;
+            same = __reduce_add_sync(0xFFFFFFFFu, same);
+            if (lane == 0) sm.gt_tot[warp] = same;
+            __syncthreads();
+            same = 0u;
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) same += sm.gt_tot[w];
+            if (same >= krem) break;
+            krem -= same;
+        }
+    } else
 #pragma unroll 1
     for (int level = 0; level < kLevels; ++level) {
         const int bits = level_bits(level), sh = level_shift(level);
@@ -173,42 +251,73 @@ static __device__ __forceinline__ void threshold_multi_body(const ThrMultiArgs& 
         const uint32_t sfirst = min(a.nstiles, b * sper), slast = min(a.nstiles, sfirst + sper);
         uint32_t t = 0xFFFFFFFFu;
         TensorDesc d;
-        for (uint32_t st = sfirst; st < slast; ++st) {
+        for (uint32_t st = sfirst; st < slast;) {
             if (t == 0xFFFFFFFFu || st >= d.stile0 + d.nstiles) {
                 if (t != 0xFFFFFFFFu) flush_hist(sm, a.shist + (size_t)t * kHistBins, 1 << level_bits(0));
                 __syncthreads();
                 t = a.ntab ? owner(tab_stile0, st) : find_tensor<SampleSpace>(a.desc, a.T, st);
                 d = a.desc[t];
             }
-            if (d.kind == kKindSmall) continue;           // sampled by the CTA that finishes it
+            // up to kSampleBatch sample tiles at once, a group per thread in one 16-byte load each: a CTA
+            // of an eight-worker launch has some twenty-five of them and pays a round trip per batch
+            // (sample phase of eight 161-tensor workers: 80 us one tile at a time, with scalar loads)
+            constexpr uint32_t kSampleBatch = 4;
+            const uint32_t nb = min(kSampleBatch, min(slast, d.stile0 + d.nstiles) - st);
+            if (d.kind == kKindSmall) { st += nb; continue; }         // sampled by the CTA that finishes it
             const uint32_t ngroups = (d.n + 3u) >> 2;
             const uint32_t nsg = (ngroups + d.sstride - 1) / d.sstride;
-            const uint64_t sg = (uint64_t)(st - d.stile0) * kBlock + tid;
-            const uint64_t gi = sg * d.sstride;
-            uint32_t key[4] = {0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu};     // = not a sample
-            if (sg < nsg && gi < ngroups) {
-                const uint32_t i0 = (uint32_t)gi * 4u;
-                float gv[4], rv[4];
+            const bool vec_ok = (d.off & 3u) == 0u;       // the tensor's groups are 16-byte aligned in the flat buffers
+            float gv[kSampleBatch][4], rv[kSampleBatch][4];
+            uint32_t i0[kSampleBatch];
+            bool live[kSampleBatch];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const bool v = i0 + e < d.n;
-                    const uint32_t f = d.off + (v ? i0 + e : 0u);
-                    gv[e] = v ? __ldg(a.g + f) : 0.f;
-                    rv[e] = v ? ld_cg(a.r + f) : 0.f;
+            for (uint32_t u = 0; u < kSampleBatch; ++u) {
+                const uint64_t sg = (uint64_t)(st + u - d.stile0) * kBlock + tid;
+                const uint64_t gi = sg * d.sstride;
+                live[u] = u < nb && sg < nsg && gi < ngroups;
+                i0[u] = live[u] ? (uint32_t)gi * 4u : 0u;
+                if (vec_ok && live[u] && i0[u] + 3u < d.n) {
+                    const float4 g4 = __ldg(reinterpret_cast<const float4*>(a.g + d.off + i0[u]));
+                    const float4 r4 = ld_cg(reinterpret_cast<const float4*>(a.r + d.off + i0[u]));
+                    gv[u][0] = g4.x; gv[u][1] = g4.y; gv[u][2] = g4.z; gv[u][3] = g4.w;
+                    rv[u][0] = r4.x; rv[u][1] = r4.y; rv[u][2] = r4.z; rv[u][3] = r4.w;
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const bool v = live[u] && i0[u] + e < d.n;
+                        const uint32_t f = d.off + (v ? i0[u] + e : 0u);
+                        gv[u][e] = v ? __ldg(a.g + f) : 0.f;
+                        rv[u][e] = v ? ld_cg(a.r + f) : 0.f;
+                    }
                 }
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    if (i0 + e < d.n) key[e] = key_of(__fadd_rn(gv[e], rv[e]));
             }
 #pragma unroll
-            for (int e = 0; e < 4; ++e)          // (all lanes: the coarse counts are aggregated over the warp)
-                hist_add_warp(sm.hist, key[e] == 0xFFFFFFFFu ? 0xFFFFFFFFu : key[e] >> level_shift(0), lane);
-            a.skeys[(size_t)st * kBlock + tid] = make_uint4(key[0], key[1], key[2], key[3]);
+            for (uint32_t u = 0; u < kSampleBatch; ++u) {
+                if (u < nb) {                             // (uniform over the CTA)
+                    uint32_t key[4] = {0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu};     // = not a sample
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {         // (all lanes: the coarse counts are aggregated over the warp)
+                        if (live[u] && i0[u] + e < d.n) key[e] = key_of(__fadd_rn(gv[u][e], rv[u][e]));
+                        hist_add_warp(sm.hist, key[e] == 0xFFFFFFFFu ? 0xFFFFFFFFu : key[e] >> level_shift(0), lane);
+                    }
+                    a.skeys[(size_t)(st + u) * kBlock + tid] = make_uint4(key[0], key[1], key[2], key[3]);
+                }
+            }
+            st += nb;
         }
         if (t != 0xFFFFFFFFu) flush_hist(sm, a.shist + (size_t)t * kHistBins, 1 << level_bits(0));
     }
     grid_arrive(hdr);
-    for (uint32_t q = G - 1u - b; q < a.n_small; q += G) {
+    for (uint32_t q8 = G - 1u - b; q8 * kWarps < a.n_tiny; q8 += G) {        // tiny tensors: a warp each, eight at a time
+        const uint32_t q = q8 * kWarps + (uint32_t)warp;
+        if (q < a.n_tiny) {
+            const uint32_t t = a.small_ids[q];
+            const TensorDesc d = a.desc[t];
+            tiny_threshold_warp(d, t, a.T, a.g, a.r, a.out_idx, a.out_val, a.out_count, hdr, lane);
+        }
+    }
+    // (the other small ones start with the CTAs next to those that took the tiny ones)
+    for (uint32_t q = a.n_tiny + (2u * G - 1u - b - ((a.n_tiny + kWarps - 1u) / kWarps) % G) % G; q < a.n_small; q += G) {
         const uint32_t t = a.small_ids[q];
         const TensorDesc d = a.desc[t];
         small_threshold_body(sm, d, t, a.T, a.g, a.r, a.out_idx, a.out_val, a.out_count, hdr);
@@ -222,15 +331,17 @@ static __device__ __forceinline__ void threshold_multi_body(const ThrMultiArgs& 
     for (uint32_t q = b; q < a.n_reg; q += G) {
         const uint32_t t = a.reg_ids[q];
         const TensorDesc d = a.desc[t];
-        uint32_t bin0 = 0, above0 = 0, tau = 0xFFFFFFFFu;
-        bool ok = block_select<(1 << level_bits(0)), false>(sm, a.shist + (size_t)t * kHistBins, d.srank, bin0, above0);
+        uint32_t tau = 0xFFFFFFFFu;
+        const uint32_t want[1] = {d.srank};
+        Picked p0[1];
+        block_select_multi<(1 << level_bits(0)), 1>(sm, a.shist + (size_t)t * kHistBins, want, p0);
+        bool ok = p0[0].ok;
         const uint4* sk = a.skeys + (size_t)d.stile0 * kBlock;
         const uint32_t nk = d.nstiles * kBlock;
-        uint32_t prefix = bin0, krem = d.srank - above0;
+        uint32_t prefix = p0[0].bin, krem = d.srank - p0[0].above;
         int have = level_bits(0);                          // key bits fixed so far
-        while (ok && have < 31) {
-            const int w = min(11, 31 - have), sh = 31 - have - w;       // this level: bits [sh, sh + w)
-            constexpr int kKeyBatch = 8;                   // loads in flight per thread: one CTA walks a whole tensor's keys
+        constexpr int kKeyBatch = 8;                       // loads in flight per thread: one CTA walks a whole tensor's keys
+        auto walk = [&](auto f) {
             for (uint32_t q0 = tid; q0 < nk; q0 += kKeyBatch * kBlock) {
                 uint4 kv[kKeyBatch];
 #pragma unroll
@@ -238,13 +349,26 @@ static __device__ __forceinline__ void threshold_multi_body(const ThrMultiArgs& 
                     kv[u] = q0 + u * kBlock < nk ? ld_cg(sk + q0 + u * kBlock)
                                                  : make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
 #pragma unroll
-                for (int u = 0; u < kKeyBatch; ++u) {
-                    const uint32_t kk[4] = {kv[u].x, kv[u].y, kv[u].z, kv[u].w};
-#pragma unroll
-                    for (int e = 0; e < 4; ++e)
-                        if ((kk[e] >> (sh + w)) == prefix) atomicAdd(&sm.hist[(kk[e] >> sh) & ((1u << w) - 1u)], 1u);
-                }
+                for (int u = 0; u < kKeyBatch; ++u) { f(kv[u].x); f(kv[u].y); f(kv[u].z); f(kv[u].w); }
             }
+        };
+        // the keys inside the coarse bin go to a list in shared memory if they fit (they are read once
+        // from memory then), and the remaining levels run on the list
+        constexpr uint32_t kListCap = kWarps * kEmitStage * 2;
+        uint32_t* const list = reinterpret_cast<uint32_t*>(sm.emit);
+        const uint32_t n_in = p0[0].count;
+        const bool listed = ok && n_in <= kListCap;
+        if (listed) {
+            if (tid == 0) s_cnt = 0u;
+            __syncthreads();
+            walk([&](uint32_t k) { if ((k >> level_shift(0)) == prefix) list[min(atomicAdd(&s_cnt, 1u), kListCap - 1u)] = k; });
+            __syncthreads();
+        }
+        while (ok && have < 31) {
+            const int w = min(11, 31 - have), sh = 31 - have - w;       // this level: bits [sh, sh + w)
+            auto count = [&](uint32_t k) { if ((k >> (sh + w)) == prefix) atomicAdd(&sm.hist[(k >> sh) & ((1u << w) - 1u)], 1u); };
+            if (listed) { for (uint32_t i = tid; i < n_in; i += kBlock) count(list[i]); }
+            else walk(count);
             __syncthreads();
             uint32_t bin, above;
             ok = block_select<2048, true>(sm, sm.hist, krem, bin, above);
