@@ -374,7 +374,7 @@ const char *gc_kernel_name(int kernel_id);
  * cudaMalloc can fail, and would in any case stall every stream of the device while it
  * runs), or a latency-bound loop that may not touch the allocator.  Such callers cannot use
  * gc_plan, which allocates its tensor table.  Here the scratch the kernels need (histograms,
- * tile words, selection record; 41,728 bytes, about 41 KB) is a fixed array inside the library image, so
+ * list of near-ties; 29,184 bytes, about 29 KB) is a fixed array inside the library image, so
  * every GPU that loads libgc carries it until the process exits.
  *
  *   grad, residual  device, fp32[n], 16-byte aligned; residual is in/out exactly as in gc_compress
@@ -387,10 +387,11 @@ const char *gc_kernel_name(int kernel_id);
  *                   (on every path that returns GC_OK, n = 0 and k = 0 included)
  *   stream          cudaStream_t; the call is asynchronous
  * The current device is used.  The first call on each device resolves the device address of
- * the array (cudaGetSymbolAddress) and sizes its grids; make that first call outside any
- * stream capture.  All calls on a device share the one array: each call clears what it
- * needs, so back-to-back calls on one stream are fine, but two calls whose kernels can
- * overlap on the GPU (different streams, different threads) race on it -- serialise them.
+ * the array (cudaGetSymbolAddress) and sets the kernel's shared-memory limit; make that first call
+ * outside any stream capture.  One cooperative launch per call.  All calls on a device share the one
+ * array: each call leaves it as it found it, so back-to-back calls on one stream are fine, but two calls
+ * whose kernels can overlap on the GPU (different streams, different threads) race on it -- serialise
+ * them.
  * Calls no cudaMalloc/cudaFree and no allocating library routine.
  */
 #define GC_NOALLOC_MAX_N (1u << 24)

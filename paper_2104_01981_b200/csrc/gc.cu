@@ -3,6 +3,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <initializer_list>
 #include <new>
@@ -10,6 +11,7 @@
 #include <vector>
 
 #include "gc_single.cuh"
+#include "gc_direct.cuh"
 #include "gc_multi.cuh"
 #include "gc_threshold.cuh"
 #include "gc_thr_single.cuh"
@@ -55,6 +57,7 @@ struct gc_plan_s {
     int grid_fused = 0;                     // CTAs of the cooperative launch (0 = not available)
     // single-tensor shared-memory-pool kernel
     int grid_single_max = 0;                // resident CTAs (0 = not available)
+    bool direct_ok = false;                 // k_topk_direct may be launched as deep as direct_geometry says
     uint32_t single_grid = 0, single_maxt = 0, single_pool = 0;   // 0 = plan does not qualify
     RowMap single_rows = {};
     size_t single_smem = 0;
@@ -664,6 +667,18 @@ int gc_plan(gc_plan_t** out, int device, uint32_t n_tensors, const uint64_t* siz
                 p->grid_single_max = p->sm_count * nb;
         }
         (void)cudaGetLastError();
+        p->direct_ok = coop != 0;
+        for (const void* fn : {(const void*)k_topk_direct<GradF32, true>, (const void*)k_topk_direct<GradBF16, true>}) {
+            int nb = 0;
+            if (!allow_smem({fn}, kDirectResident) ||
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kBlock, kDirectResident) != cudaSuccess || nb < 2)
+                p->direct_ok = false;
+        }
+        for (const void* fn : {(const void*)k_topk_direct<GradF32, false>, (const void*)k_topk_direct<GradBF16, false>}) {
+            int nb = 0;
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kBlock, 0) != cudaSuccess || nb < 3) p->direct_ok = false;
+        }
+        (void)cudaGetLastError();
         plan_single(p);
         p->grid_thr_single_max = 0;
         if (coop) {
@@ -761,6 +776,7 @@ int gc_plan_set_option(gc_plan_t* p, int option, uint64_t value) {
             if (value < 1 || value > 100000) return GC_E_INVALID;
             if (p->device >= 0 && !on_plan_device(p)) return GC_E_INVALID;      // (the table is uploaded again)
             p->rank_permille = (uint32_t)value;
+            p->clean_ws.clear();                       // (another kernel may take the plan now)
             p->wk_W = 0;
             finish_layout(p);                          // workspace size stays as planned (see skeys_tiles_alloc)
             plan_single(p);
@@ -769,6 +785,7 @@ int gc_plan_set_option(gc_plan_t* p, int option, uint64_t value) {
         case GC_OPT_CANDIDATE_CAPACITY:
             if (value > p->cand_cap_alloc) return GC_E_INVALID;
             p->cand_cap = (uint32_t)value;
+            p->clean_ws.clear();                       // (another kernel may take the plan now)
             p->wk_W = 0;
             return GC_OK;
         case GC_OPT_WORKSPACE_PRIVATE:
@@ -813,6 +830,13 @@ int gc_plan_query(const gc_plan_t* p, int what, uint32_t tensor, uint64_t* value
         case GC_Q_TENSOR_STRIDE: *value = d.stride; return GC_OK;
         default: return GC_E_INVALID;
     }
+}
+
+// One-tensor plans of up to kDirectMaxPlan elements take k_topk_direct (with the testing options at their
+// defaults: those steer the candidate path).
+static bool takes_direct(const gc_plan_s* p) {
+    return p->direct_ok && p->single_grid > 0 && p->total_n <= kDirectMaxPlan && p->rank_permille == 1000 &&
+           p->cand_cap == p->cand_cap_alloc;
 }
 
 // The control block as the self-cleaning kernels see it (see CleanArgs): up to three early sections.
@@ -936,10 +960,11 @@ static int compress_impl(gc_plan_t* p, const void* grad_any, bool bf16, float* r
     // for a workspace that kernel ran on last (the kernel checks a mark in the header and leaves
     // with GC_E_INVALID if the promise was broken).
     const bool self_cleaning = route == GC_ROUTE_TOPK_ONE || route == GC_ROUTE_TOPK_MANY;
+    const bool direct = route == GC_ROUTE_TOPK_ONE && takes_direct(p);
     const bool kept_clean = take_clean(p, workspace) && p->ws_private && self_cleaning;
     if (!kept_clean) {
         Timed tm(p, s, GC_K_CLEAR_CTRL);
-        const size_t n16 = p->control_bytes / 16;             // control_bytes is a multiple of 256
+        const size_t n16 = (direct ? offsetof(DirectScratch, list) : p->control_bytes) / 16;             // (multiples of 256)
         const int gc = (int)std::min<size_t>((n16 + kBlock - 1) / kBlock, (size_t)p->sm_count * 8);
         k_clear<<<gc, kBlock, 0, s>>>(reinterpret_cast<uint4*>(workspace), n16);
     }
@@ -1027,6 +1052,20 @@ static int compress_impl(gc_plan_t* p, const void* grad_any, bool bf16, float* r
     cv.group_cnt = reinterpret_cast<unsigned long long*>(wb + p->off_gstate);
     cv.cap = p->cand_cap;
     cv.ssel = sws.sel;
+    if (direct) {
+        DirectArgs da{};
+        da.g = grad_any; da.r = residual; da.n = (uint32_t)p->total_n; da.k = p->desc[0].k; da.out_idx = out_idx; da.out_val = out_val;
+        da.out_count = out_count; da.s = reinterpret_cast<DirectScratch*>(workspace);
+        da.mark = clean_args(p, workspace, GC_ROUTE_TOPK_ONE, false).mark + 1u; da.expect_clean = kept_clean ? 1u : 0u;
+        const DirectGeom dg = direct_geometry(da.n, p->sm_count);
+        note_clean(p, workspace);
+        void* args[] = {&da};
+        Timed tm(p, s, GC_K_FUSED);
+        const void* kfn = dg.resident ? (bf16 ? (const void*)k_topk_direct<GradBF16, true> : (const void*)k_topk_direct<GradF32, true>)
+                                      : (bf16 ? (const void*)k_topk_direct<GradBF16, false> : (const void*)k_topk_direct<GradF32, false>);
+        GC_CUDA(p, cudaLaunchCooperativeKernel(kfn, dim3(dg.G), dim3(kBlock), args, dg.smem, s));
+        return GC_OK;
+    }
     if (route == GC_ROUTE_TOPK_ONE) {
         // one large tensor: candidates stay in shared memory
         SingleArgs sa;
