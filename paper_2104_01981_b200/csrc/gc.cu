@@ -6,6 +6,7 @@
 #include <cstddef>
 #include <cstring>
 #include <initializer_list>
+#include <mutex>
 #include <new>
 #include <utility>
 #include <vector>
@@ -22,7 +23,24 @@ using namespace gc;
 
 struct MultiGeom { uint32_t G = 0, per = 0, pool = 0, full = 0, ntab = 0; size_t smem = 0; };   // see multi_geometry
 
-struct gc_plan_s {
+// How many CTAs of every kernel are resident on a device (the dynamic shared memory raised where a kernel
+// needs it): asked once per device, copied into every plan.
+struct DeviceFacts {
+    int sm_count = 0;
+    int grid_thr = 0, grid_decode[2] = {0, 0};
+    int grid_decode_seg[2] = {0, 0}, grid_decode_seg_apply = 0;    // k_decode_segments: one / two tile buffers; with optimizer
+    bool rings_ok = false;                        // k_decode_rings may use up to kRingSmem2 of dynamic shared memory
+    int grid_hist = 0, grid_compact = 0, grid_fold = 0, grid_sample = 0, grid_chist = 0, grid_ccompact = 0;
+    int grid_fused = 0;                     // CTAs of the cooperative launch (0 = not available)
+    int grid_single_max = 0;                // k_topk_single: resident CTAs (0 = not available)
+    bool direct_ok = false;                 // k_topk_direct may be launched as deep as direct_geometry says
+    int grid_thr_single_max = 0;
+    int grid_thr_multi_max = 0;
+    int grid_multi_max = 0;                 // resident CTAs of k_topk_multi (0 = not available)
+    size_t multi_smem_max = 0, thrm_smem_max = 0;   // dynamic shared memory those occupancy figures were taken with
+};
+
+struct gc_plan_s : DeviceFacts {
     int device = 0;
     int mode = GC_TOPK;
     double density = 0.0;
@@ -49,28 +67,16 @@ struct gc_plan_s {
     // workspace layout (byte offsets)
     size_t off_sel = 0, off_ssel = 0, off_gsel = 0, off_hist = 0, off_state = 0, off_gstate = 0,
            control_bytes = 0, off_tinfo = 0, off_cidx = 0, ws_bytes = 0;
-    int sm_count = 0;
-    int grid_thr = 0, grid_decode[2] = {0, 0};
-    int grid_decode_seg[2] = {0, 0}, grid_decode_seg_apply = 0;    // k_decode_segments: one / two tile buffers; with optimizer
-    bool rings_ok = false;                        // k_decode_rings may use up to kRingSmem2 of dynamic shared memory
-    int grid_hist = 0, grid_compact = 0, grid_fold = 0, grid_sample = 0, grid_chist = 0, grid_ccompact = 0;
-    int grid_fused = 0;                     // CTAs of the cooperative launch (0 = not available)
     // single-tensor shared-memory-pool kernel
-    int grid_single_max = 0;                // resident CTAs (0 = not available)
-    bool direct_ok = false;                 // k_topk_direct may be launched as deep as direct_geometry says
     uint32_t single_grid = 0, single_maxt = 0, single_pool = 0;   // 0 = plan does not qualify
     RowMap single_rows = {};
     size_t single_smem = 0;
     size_t off_hist5 = 0, off_rowseg = 0, off_mid = 0, off_fine = 0, off_age = 0;
     uint32_t single_srank_hi = 0, single_srank_mid = 0;
-    int grid_thr_single_max = 0;
     uint32_t thr_grid = 0, thr_maxt = 0, thr_pool = 0, thr_rounds = 0;    // one-tensor threshold kernel (0 = no)
     size_t thr_smem = 0;
-    int grid_thr_multi_max = 0;
     uint32_t thrm_grid = 0, thrm_per = 0, thrm_pool = 0, thrm_ntab = 0;   // many-tensor threshold kernel (0 = no)
     size_t thrm_smem = 0;
-    int grid_multi_max = 0;                 // resident CTAs of k_topk_multi (0 = not available)
-    size_t multi_smem_max = 0, thrm_smem_max = 0;   // dynamic shared memory those occupancy figures were taken with
     bool ws_private = false;                // GC_OPT_WORKSPACE_PRIVATE
     std::vector<const void*> clean_ws;      // workspaces the one-tensor top-k kernel ran on last (and left clean), if private
     uint32_t wk_W = 0, wk_batch = 0;        // gc_compress_workers: workers per launch chosen for the last W seen
@@ -108,6 +114,7 @@ constexpr uint32_t kSinglePoolMax = 65536, kMultiPoolMax = 98304;   // most cand
 // than 8 % (with 8 % the oldest CTAs of the 355M-element workload finished last).
 constexpr double kSingleSkew = 0.08, kSingleSkewSparse = 0.04;
 constexpr size_t kSingleRowBytes = (2 * kWarps + 4) * sizeof(uint32_t);   // shared memory per owned tile
+constexpr double kDenseFrom = 0.02;          // density from which the forms with emission by chunk are taken (12 candidates per chunk)
 constexpr uint32_t kMultiMaxTab = 1024;      // tensors whose tile tables k_topk_multi keeps in shared memory
 constexpr size_t kMultiMaxPer = 224;         // most tiles one CTA of k_topk_multi may own
 constexpr size_t kMultiRowBytes = (2 * kWarps + kSegWords) * sizeof(uint32_t);   // shared memory per owned tile
@@ -553,6 +560,156 @@ static bool takes_rings(const gc_plan_s* p, uint32_t W) {
     return avg + avg / 4 > (uint64_t)kDecRounds * (kDecBlock / Wp) || (double)W * (double)p->total_cap > 0.045 * (double)p->total_n;
 }
 
+static bool ask_device(int device, DeviceFacts* p) {
+    if (cudaDeviceGetAttribute(&p->sm_count, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    p->grid_hist = p->sm_count * blocks_per_sm(k_hist<0, SRC_FOLD>, kBlock);
+    p->grid_compact = p->sm_count * blocks_per_sm(k_compact, kBlock);
+    p->grid_fold = p->sm_count * blocks_per_sm(k_fold_cand, kBlock);
+    {
+        int coop = 0;
+        if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device) != cudaSuccess) {
+            (void)cudaGetLastError();
+            coop = 0;
+        }
+        p->grid_fused = coop ? p->sm_count * blocks_per_sm(k_compress_fused, kBlock) : 0;
+        p->grid_single_max = 0;
+        if (coop) {
+            // sized for the largest chunk-record block the kernel may be given; the form that fits least counts
+            const size_t smem_max = kSingleMaxT * kSingleRowBytes + kSinglePoolMax / 8;
+            int nb = 1 << 20;
+            for (const void* fn : {(const void*)k_topk_single<GradF32, false>, (const void*)k_topk_single<GradF32, true>,
+                                   (const void*)k_topk_single<GradBF16, false>, (const void*)k_topk_single<GradBF16, true>}) {
+                int n1 = 0;
+                if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n1, fn, kBlock, smem_max) != cudaSuccess) n1 = 0;
+                nb = std::min(nb, n1);
+            }
+            if (nb >= 1)
+                p->grid_single_max = p->sm_count * nb;
+        }
+        (void)cudaGetLastError();
+        p->direct_ok = coop != 0;
+        for (const void* fn : {(const void*)k_topk_direct<GradF32, true>, (const void*)k_topk_direct<GradBF16, true>}) {
+            int nb = 0;
+            if (!allow_smem({fn}, kDirectResident) ||
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kBlock, kDirectResident) != cudaSuccess || nb < 2)
+                p->direct_ok = false;
+        }
+        for (const void* fn : {(const void*)k_topk_direct<GradF32, false>, (const void*)k_topk_direct<GradBF16, false>}) {
+            int nb = 0;
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kBlock, 0) != cudaSuccess || nb < 3) p->direct_ok = false;
+        }
+        (void)cudaGetLastError();
+        p->grid_thr_single_max = 0;
+        if (coop) {
+            int nb = 0;
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_threshold_single, kBlock,
+                                                              kSingleMaxT * (2 * kWarps + 2) * sizeof(uint32_t)) ==
+                    cudaSuccess && nb >= 1)
+                p->grid_thr_single_max = p->sm_count * nb;
+            else
+                (void)cudaGetLastError();
+        }
+        p->grid_thr_multi_max = 0;
+        if (coop) {
+            int nb = 0;
+            p->thrm_smem_max = kMultiMaxPer * kMultiRowBytes + 8 * kMultiMaxTab;
+            int nbw = 0;          // (the several-workers form of the kernel must be as resident as the kernel itself)
+            if (allow_smem({(const void*)k_threshold_multi, (const void*)k_threshold_workers}, p->thrm_smem_max) &&
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_threshold_multi, kBlock, p->thrm_smem_max) ==
+                    cudaSuccess && nb >= 1 &&
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nbw, k_threshold_workers, kBlock, p->thrm_smem_max) ==
+                    cudaSuccess && nbw >= 1)
+                p->grid_thr_multi_max = p->sm_count * std::min(nb, nbw);
+            else
+                (void)cudaGetLastError();
+        }
+        p->grid_multi_max = 0;
+        if (coop) {
+            int nb = 0;
+            p->multi_smem_max = kMultiMaxPer * kMultiRowBytes + kMultiPoolMax / 8 + 8 * kMultiMaxTab;
+            int nbw = 0;          // (the several-workers form of the kernel must be as resident as the kernel itself)
+            const std::initializer_list<const void*> forms = {
+                (const void*)k_topk_multi<GradF32, false>, (const void*)k_topk_multi<GradF32, true>,
+                (const void*)k_topk_multi<GradBF16, false>, (const void*)k_topk_multi<GradBF16, true>,
+                (const void*)k_topk_workers<GradF32, false>, (const void*)k_topk_workers<GradF32, true>};
+            if (allow_smem(forms, p->multi_smem_max)) {
+                nb = 1 << 20;
+                for (const void* fn : forms) {
+                    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nbw, fn, kBlock, p->multi_smem_max) != cudaSuccess) nbw = 0;
+                    nb = std::min(nb, nbw);
+                }
+            }
+            if (nb >= 1)
+                p->grid_multi_max = p->sm_count * nb;
+            else
+                (void)cudaGetLastError();
+        }
+    }
+    p->grid_thr = p->sm_count * blocks_per_sm(k_threshold_emit, kBlock);
+    {
+        cudaError_t ed = cudaFuncSetAttribute(k_decode_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)(2 * kDecTileBytes));
+        for (int nbuf = 1; nbuf <= 2; ++nbuf) {
+            int nb = 0;
+            if (ed == cudaSuccess)
+                ed = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_decode_tiles, kDecBlock,
+                                                                   nbuf * kDecTileBytes);
+            if (ed != cudaSuccess || nb < 1) { (void)cudaGetLastError(); nb = 0; }
+            p->grid_decode[nbuf - 1] = p->sm_count * nb;     // 0: fall back to one launch per worker
+        }
+    }
+    {
+        // lists with per-tensor counts (plans of several tensors): the segment-walking tile kernel
+        cudaError_t ed = cudaFuncSetAttribute(k_decode_segments<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)(2 * kDecTileBytes));
+        for (int nbuf = 1; nbuf <= 2; ++nbuf) {
+            int nb = 0;
+            if (ed == cudaSuccess)
+                ed = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_decode_segments<false>, kDecBlock,
+                                                                   nbuf * kDecTileBytes);
+            if (ed != cudaSuccess || nb < 1) { (void)cudaGetLastError(); nb = 0; }
+            p->grid_decode_seg[nbuf - 1] = p->sm_count * nb;
+        }
+        int nb = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_decode_segments<true>, kDecBlock, kDecTileBytes) !=
+                cudaSuccess || nb < 1) { (void)cudaGetLastError(); nb = 0; }
+        p->grid_decode_seg_apply = p->sm_count * nb;
+    }
+    p->rings_ok = allow_smem({(const void*)k_decode_rings<false, false, false>, (const void*)k_decode_rings<false, false, true>,
+                              (const void*)k_decode_rings<false, true, false>, (const void*)k_decode_rings<false, true, true>,
+                              (const void*)k_decode_rings<true, false, false>, (const void*)k_decode_rings<true, false, true>}, kRingSmem2);
+    (void)cudaGetLastError();
+    p->grid_sample = p->sm_count * blocks_per_sm(k_hist<0, SRC_SAMPLE>, kBlock);
+    p->grid_chist = p->sm_count * blocks_per_sm(k_cand_hist<1>, kBlock);
+    p->grid_ccompact = p->sm_count * blocks_per_sm(k_cand_compact<true>, kBlock);
+    return true;
+}
+
+// The facts of a device, asked on its first plan (some forty driver calls, a millisecond) and again if the
+// device was reset since (the kernels' shared-memory limits are gone then).  The device is current.
+static bool device_facts(int device, DeviceFacts& out) {
+    static std::mutex mu;
+    static std::vector<std::pair<int, DeviceFacts>> known;
+    std::lock_guard<std::mutex> lock(mu);
+    for (auto& e : known) {
+        if (e.first != device) continue;
+        cudaFuncAttributes fa;
+        const bool valid = cudaFuncGetAttributes(&fa, k_topk_workers<GradF32, true>) == cudaSuccess &&
+                           (size_t)fa.maxDynamicSharedSizeBytes >= e.second.multi_smem_max;
+        if (!valid) { (void)cudaGetLastError(); if (!ask_device(device, &e.second)) return false; }
+        out = e.second;
+        return true;
+    }
+    DeviceFacts f;
+    if (!ask_device(device, &f)) return false;
+    known.emplace_back(device, f);
+    out = f;
+    return true;
+}
+
 extern "C" {
 
 static int compress_route(const gc_plan_s* p);
@@ -614,7 +771,6 @@ int gc_plan(gc_plan_t** out, int device, uint32_t n_tensors, const uint64_t* siz
         ~RestoreDevice() { if (dev >= 0) (void)cudaSetDevice(dev); }
     } restore_device{caller_device};
     cudaError_t e = cudaSetDevice(device);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&p->sm_count, cudaDevAttrMultiProcessorCount, device);
     if (e == cudaSuccess && n_tensors > 0) {
         e = cudaMalloc(reinterpret_cast<void**>(&p->d_desc), sizeof(TensorDesc) * (size_t)n_tensors);
         if (e == cudaSuccess)
@@ -642,124 +798,17 @@ int gc_plan(gc_plan_t** out, int device, uint32_t n_tensors, const uint64_t* siz
         delete p;
         return GC_E_CUDA;
     }
-    p->grid_hist = p->sm_count * blocks_per_sm(k_hist<0, SRC_FOLD>, kBlock);
-    p->grid_compact = p->sm_count * blocks_per_sm(k_compact, kBlock);
-    p->grid_fold = p->sm_count * blocks_per_sm(k_fold_cand, kBlock);
-    {
-        int coop = 0;
-        if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device) != cudaSuccess) {
-            (void)cudaGetLastError();
-            coop = 0;
-        }
-        p->grid_fused = coop ? p->sm_count * blocks_per_sm(k_compress_fused, kBlock) : 0;
-        p->grid_single_max = 0;
-        if (coop) {
-            // sized for the largest chunk-record block the kernel may be given; the form that fits least counts
-            const size_t smem_max = kSingleMaxT * kSingleRowBytes + kSinglePoolMax / 8;
-            int nb = 1 << 20;
-            for (const void* fn : {(const void*)k_topk_single<GradF32, false>, (const void*)k_topk_single<GradF32, true>,
-                                   (const void*)k_topk_single<GradBF16, false>, (const void*)k_topk_single<GradBF16, true>}) {
-                int n1 = 0;
-                if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n1, fn, kBlock, smem_max) != cudaSuccess) n1 = 0;
-                nb = std::min(nb, n1);
-            }
-            if (nb >= 1)
-                p->grid_single_max = p->sm_count * nb;
-        }
-        (void)cudaGetLastError();
-        p->direct_ok = coop != 0;
-        for (const void* fn : {(const void*)k_topk_direct<GradF32, true>, (const void*)k_topk_direct<GradBF16, true>}) {
-            int nb = 0;
-            if (!allow_smem({fn}, kDirectResident) ||
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kBlock, kDirectResident) != cudaSuccess || nb < 2)
-                p->direct_ok = false;
-        }
-        for (const void* fn : {(const void*)k_topk_direct<GradF32, false>, (const void*)k_topk_direct<GradBF16, false>}) {
-            int nb = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kBlock, 0) != cudaSuccess || nb < 3) p->direct_ok = false;
-        }
-        (void)cudaGetLastError();
-        plan_single(p);
-        p->grid_thr_single_max = 0;
-        if (coop) {
-            int nb = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_threshold_single, kBlock,
-                                                              kSingleMaxT * (2 * kWarps + 2) * sizeof(uint32_t)) ==
-                    cudaSuccess && nb >= 1)
-                p->grid_thr_single_max = p->sm_count * nb;
-            else
-                (void)cudaGetLastError();
-        }
-        plan_thr_single(p);
-        p->grid_thr_multi_max = 0;
-        if (coop) {
-            int nb = 0;
-            p->thrm_smem_max = kMultiMaxPer * kMultiRowBytes + 8 * kMultiMaxTab;
-            int nbw = 0;          // (the several-workers form of the kernel must be as resident as the kernel itself)
-            if (allow_smem({(const void*)k_threshold_multi, (const void*)k_threshold_workers}, p->thrm_smem_max) &&
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_threshold_multi, kBlock, p->thrm_smem_max) ==
-                    cudaSuccess && nb >= 1 &&
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nbw, k_threshold_workers, kBlock, p->thrm_smem_max) ==
-                    cudaSuccess && nbw >= 1)
-                p->grid_thr_multi_max = p->sm_count * std::min(nb, nbw);
-            else
-                (void)cudaGetLastError();
-        }
-        plan_thr_multi(p);
-        p->grid_multi_max = 0;
-        if (coop) {
-            int nb = 0;
-            p->multi_smem_max = kMultiMaxPer * kMultiRowBytes + kMultiPoolMax / 8 + 8 * kMultiMaxTab;
-            int nbw = 0;          // (the several-workers form of the kernel must be as resident as the kernel itself)
-            if (allow_smem({(const void*)k_topk_multi<GradF32>, (const void*)k_topk_multi<GradBF16>,
-                            (const void*)k_topk_workers<GradF32>}, p->multi_smem_max) &&
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_topk_multi<GradF32>, kBlock, p->multi_smem_max) ==
-                    cudaSuccess && nb >= 1 &&
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nbw, k_topk_workers<GradF32>, kBlock, p->multi_smem_max) ==
-                    cudaSuccess && nbw >= 1)
-                p->grid_multi_max = p->sm_count * std::min(nb, nbw);
-            else
-                (void)cudaGetLastError();
-        }
-        plan_multi(p);
+    if (!device_facts(device, *p)) {
+        if (p->d_desc) cudaFree(p->d_desc);
+        if (p->d_small) cudaFree(p->d_small);
+        if (p->d_dectile) cudaFree(p->d_dectile);
+        delete p;
+        return GC_E_CUDA;
     }
-    p->grid_thr = p->sm_count * blocks_per_sm(k_threshold_emit, kBlock);
-    {
-        cudaError_t ed = cudaFuncSetAttribute(k_decode_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)(2 * kDecTileBytes));
-        for (int nbuf = 1; nbuf <= 2; ++nbuf) {
-            int nb = 0;
-            if (ed == cudaSuccess)
-                ed = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_decode_tiles, kDecBlock,
-                                                                   nbuf * kDecTileBytes);
-            if (ed != cudaSuccess || nb < 1) { (void)cudaGetLastError(); nb = 0; }
-            p->grid_decode[nbuf - 1] = p->sm_count * nb;     // 0: fall back to one launch per worker
-        }
-    }
-    {
-        // lists with per-tensor counts (plans of several tensors): the segment-walking tile kernel
-        cudaError_t ed = cudaFuncSetAttribute(k_decode_segments<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)(2 * kDecTileBytes));
-        for (int nbuf = 1; nbuf <= 2; ++nbuf) {
-            int nb = 0;
-            if (ed == cudaSuccess)
-                ed = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_decode_segments<false>, kDecBlock,
-                                                                   nbuf * kDecTileBytes);
-            if (ed != cudaSuccess || nb < 1) { (void)cudaGetLastError(); nb = 0; }
-            p->grid_decode_seg[nbuf - 1] = p->sm_count * nb;
-        }
-        int nb = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_decode_segments<true>, kDecBlock, kDecTileBytes) !=
-                cudaSuccess || nb < 1) { (void)cudaGetLastError(); nb = 0; }
-        p->grid_decode_seg_apply = p->sm_count * nb;
-    }
-    p->rings_ok = allow_smem({(const void*)k_decode_rings<false, false, false>, (const void*)k_decode_rings<false, false, true>,
-                              (const void*)k_decode_rings<false, true, false>, (const void*)k_decode_rings<false, true, true>,
-                              (const void*)k_decode_rings<true, false, false>, (const void*)k_decode_rings<true, false, true>}, kRingSmem2);
-    (void)cudaGetLastError();
-    p->grid_sample = p->sm_count * blocks_per_sm(k_hist<0, SRC_SAMPLE>, kBlock);
-    p->grid_chist = p->sm_count * blocks_per_sm(k_cand_hist<1>, kBlock);
-    p->grid_ccompact = p->sm_count * blocks_per_sm(k_cand_compact<true>, kBlock);
+    plan_single(p);
+    plan_thr_single(p);
+    plan_thr_multi(p);
+    plan_multi(p);
     *out = p;
     return GC_OK;
 }
@@ -1086,7 +1135,7 @@ static int compress_impl(gc_plan_t* p, const void* grad_any, bool bf16, float* r
         note_clean(p, workspace);
         void* args[] = {&sa};
         Timed tm(p, s, GC_K_FUSED);
-        const bool dense = p->density >= 0.02;
+        const bool dense = p->density >= kDenseFrom;
         const void* kfn = bf16 ? (dense ? (const void*)k_topk_single<GradBF16, true> : (const void*)k_topk_single<GradBF16, false>)
                                : (dense ? (const void*)k_topk_single<GradF32, true> : (const void*)k_topk_single<GradF32, false>);
         GC_CUDA(p, cudaLaunchCooperativeKernel(kfn, dim3(p->single_grid), dim3(kBlock), args, p->single_smem, s));
@@ -1101,7 +1150,9 @@ static int compress_impl(gc_plan_t* p, const void* grad_any, bool bf16, float* r
         note_clean(p, workspace);
         void* args[] = {&ma};
         Timed tm(p, s, GC_K_FUSED);
-        const void* kfn = bf16 ? (const void*)k_topk_multi<GradBF16> : (const void*)k_topk_multi<GradF32>;
+        const bool dense = p->density >= kDenseFrom;
+        const void* kfn = bf16 ? (dense ? (const void*)k_topk_multi<GradBF16, true> : (const void*)k_topk_multi<GradBF16, false>)
+                               : (dense ? (const void*)k_topk_multi<GradF32, true> : (const void*)k_topk_multi<GradF32, false>);
         GC_CUDA(p, cudaLaunchCooperativeKernel(kfn, dim3(p->multi_grid), dim3(kBlock), args, p->multi_smem, s));
         return GC_OK;
     }
@@ -1272,7 +1323,8 @@ int gc_compress_workers(gc_plan_t* p, uint32_t W, const float* const* grads, flo
         }
         void* args[] = {topk_multi ? (void*)&wa : (void*)&ta};
         Timed tm(p, s, GC_K_FUSED);
-        GC_CUDA(p, cudaLaunchCooperativeKernel(topk_multi ? (const void*)k_topk_workers<GradF32> : (const void*)k_threshold_workers,
+        GC_CUDA(p, cudaLaunchCooperativeKernel(topk_multi ? (p->density >= kDenseFrom ? (const void*)k_topk_workers<GradF32, true> : (const void*)k_topk_workers<GradF32, false>)
+                                                          : (const void*)k_threshold_workers,
                                                dim3(mg.G * wn), dim3(kBlock), args, mg.smem, s));
     }
     return GC_OK;

@@ -100,7 +100,8 @@ __device__ __forceinline__ bool grid_wait(WsHeader* hdr, uint32_t& passed, int* 
 
 // The whole compress of one worker by the G CTAs of one group (this CTA is number b of them);
 // the group's barriers count on the worker's own workspace header.
-template <typename GL>
+// (DENSE: see k_topk_single)
+template <typename GL, bool DENSE>
 __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32_t G, const uint32_t b, BlockSmem& sm,
                                                 uint32_t& s_used, uint32_t& s_cnt, unsigned char* s_dyn) {
     uint32_t* const rec = reinterpret_cast<uint32_t*>(s_dyn);                  // [per*kWarps] off<<10 | cnt
@@ -466,7 +467,7 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
         return (s[SG_TILE0] + (rel >> 12)) * kWarps + ((rel >> 9) & (kWarps - 1u));
     };
 
-    const bool overflowed = ld_cg(&hdr->overflow) != 0u, by_chunk = used >= kChunkWalk * ntl * kWarps;
+    const bool overflowed = ld_cg(&hdr->overflow) != 0u, by_chunk = DENSE && used >= kChunkWalk * ntl * kWarps;
     if (!overflowed && nseg != 0u) {
         // ------------------------------------------------------------ band bin per segment, counts above it
         for (uint32_t sidx = (uint32_t)warp; sidx < nseg; sidx += kWarps) {      // a warp per segment, all at once
@@ -774,14 +775,14 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
     leave_clean(a.cl, hdr, G, tid);
 }
 
-template <typename GL>
+template <typename GL, bool DENSE>
 // (three CTAs per SM: 80 registers and no spills beat four at 64 registers, see k_topk_single)
 static __global__ void __launch_bounds__(kBlock, 3)
 k_topk_multi(const __grid_constant__ MultiArgs a) {
     __shared__ BlockSmem sm;
     __shared__ uint32_t s_used, s_cnt;
     extern __shared__ __align__(16) unsigned char s_dyn[];
-    topk_multi_body<GL>(a, gridDim.x, blockIdx.x, sm, s_used, s_cnt, s_dyn);
+    topk_multi_body<GL, DENSE>(a, gridDim.x, blockIdx.x, sm, s_used, s_cnt, s_dyn);
 }
 
 // Several workers' compress calls in ONE cooperative launch: the grid is cut into one group of
@@ -797,7 +798,7 @@ struct WorkersArgs {
 };
 static_assert(sizeof(WorkersArgs) <= 4000, "kernel parameters stay below 4 KB");
 
-template <typename GL>
+template <typename GL, bool DENSE>
 static __global__ void __launch_bounds__(kBlock, 3)
 k_topk_workers(const __grid_constant__ WorkersArgs wa) {
     __shared__ BlockSmem sm;
@@ -811,7 +812,7 @@ k_topk_workers(const __grid_constant__ WorkersArgs wa) {
         for (uint32_t i = threadIdx.x; i < sizeof(MultiArgs) / 4; i += kBlock) dst[i] = src[i];
     }
     __syncthreads();
-    topk_multi_body<GL>(s_args, wa.G, b, sm, s_used, s_cnt, s_dyn);
+    topk_multi_body<GL, DENSE>(s_args, wa.G, b, sm, s_used, s_cnt, s_dyn);
 }
 
 }  // namespace gc
