@@ -829,6 +829,7 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
                 }
             };
             if (by_chunk) {
+                __syncthreads();                           // (every chunk's first slot is written)
                 for_chunks(rec, n_own * kWarps, pool, warp, lane, [&](uint32_t c, uint32_t off, uint32_t cnt, const uint2 (&p)[2]) {
                     uint32_t slot = rec2[c];
                     for (uint32_t q0 = 0; q0 < cnt; q0 += 32u) {
