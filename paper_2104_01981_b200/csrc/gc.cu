@@ -21,6 +21,8 @@
 
 using namespace gc;
 
+// Geometry of k_topk_single; votes: see its template argument.
+struct SingleGeom { uint32_t G = 0, maxt = 0, pool = 0; size_t smem = 0; RowMap rows = {}; bool votes = false; };
 struct MultiGeom { uint32_t G = 0, per = 0, pool = 0, full = 0, ntab = 0; size_t smem = 0; };   // see multi_geometry
 
 // How many CTAs of every kernel are resident on a device (the dynamic shared memory raised where a kernel
@@ -68,9 +70,8 @@ struct gc_plan_s : DeviceFacts {
     size_t off_sel = 0, off_ssel = 0, off_gsel = 0, off_hist = 0, off_state = 0, off_gstate = 0,
            control_bytes = 0, off_tinfo = 0, off_cidx = 0, ws_bytes = 0;
     // single-tensor shared-memory-pool kernel
-    uint32_t single_grid = 0, single_maxt = 0, single_pool = 0;   // 0 = plan does not qualify
-    RowMap single_rows = {};
-    size_t single_smem = 0;
+    SingleGeom single[2];                   // k_topk_single for fp32 and for bfloat16 gradients
+    uint32_t single_grid = 0;               // CTAs of the first (0 = plan does not qualify)
     size_t off_hist5 = 0, off_rowseg = 0, off_mid = 0, off_fine = 0, off_age = 0;
     uint32_t single_srank_hi = 0, single_srank_mid = 0;
     uint32_t thr_grid = 0, thr_maxt = 0, thr_pool = 0, thr_rounds = 0;    // one-tensor threshold kernel (0 = no)
@@ -114,6 +115,7 @@ constexpr uint32_t kSinglePoolMax = 65536, kMultiPoolMax = 98304;   // most cand
 // than 8 % (with 8 % the oldest CTAs of the 355M-element workload finished last).
 constexpr double kSingleSkew = 0.08, kSingleSkewSparse = 0.04;
 constexpr size_t kSingleRowBytes = (2 * kWarps + 4) * sizeof(uint32_t);   // shared memory per owned tile
+constexpr double kSparseUpTo = 0.002;        // density up to which the fold is bound by memory alone (see VOTES of k_topk_single)
 constexpr double kDenseFrom = 0.02;          // density from which the forms with emission by chunk are taken (12 candidates per chunk)
 constexpr uint32_t kMultiMaxTab = 1024;      // tensors whose tile tables k_topk_multi keeps in shared memory
 constexpr size_t kMultiMaxPer = 224;         // most tiles one CTA of k_topk_multi may own
@@ -325,37 +327,41 @@ static RowMap make_row_map(const gc_plan_s* p, uint32_t ntiles, uint32_t G, uint
     return rm;
 }
 
-// Decides whether the plan can use the single-tensor kernel and with which geometry.
+// Decides whether the plan can use the single-tensor kernel and with which geometries.
 void plan_single(gc_plan_s* p) {
     p->single_grid = 0;
     if (p->mode != GC_TOPK || p->T != 1 || p->grid_single_max <= 0) return;
     const TensorDesc& d = p->desc[0];
     if (d.sstride == 0 || d.ntiles == 0 || d.off != 0) return;
-    uint32_t G = std::min<uint32_t>((uint32_t)p->grid_single_max, d.ntiles);
-    // Small tensors are all latency (a CTA has a handful of tiles and five phases to walk through):
-    // there two CTAs per SM get through the phases sooner than three (2M-10M elements: 31-49 us
-    // against 37-51 us).  From about 12M elements on the third CTA pays for itself; below 300
-    // tiles there is a CTA per tile anyway (fewer were no faster).
-    if (d.ntiles <= 3000u) G = std::min<uint32_t>(G, 2u * (uint32_t)p->sm_count);
-    uint32_t maxt = (d.ntiles + G - 1) / G;
-    const RowMap rm = make_row_map(p, d.ntiles, G, maxt, p->density >= 0.005 ? kSingleSkew : kSingleSkewSparse);
-    if (maxt > kSingleMaxT || G > 640) return;                       // chunk records and totals must stay small
     if (d.ntiles >= (1u << 20)) return;                              // (the row arithmetic divides by multiplication)
-    // region per CTA; one bit per slot has to fit in shared memory beside the chunk records
-    const uint32_t pool = std::min<uint32_t>(p->cand_cap_alloc / G, kSinglePoolMax);
-    const size_t rec_bytes = (size_t)maxt * kSingleRowBytes + sizeof(uint32_t) * ((pool + 31) / 32);
-    // expected candidates per CTA (sample rank over sample size, times n), with head-room
     const uint64_t groups = ((uint64_t)d.n + 3) / 4, nsg = (groups + d.sstride - 1) / d.sstride;
-    if (nsg > (uint64_t)2 * G * kBlock) return;                     // a thread owns at most two sample groups
-    const double expect = (double)d.n * (double)d.srank / (4.0 * (double)nsg) / (double)G;
-    if ((double)pool < 1.5 * expect + 512.0) return;
+    for (int bf16 = 0; bf16 < 2; ++bf16) {
+        SingleGeom g;
+        g.votes = bf16 != 0 || p->density <= kSparseUpTo;
+        g.G = std::min<uint32_t>((uint32_t)p->grid_single_max, d.ntiles);
+        // Small tensors are all latency (a CTA has a handful of tiles and five phases to walk through):
+        // there two CTAs per SM get through the phases sooner than three (2M-10M elements: 31-49 us
+        // against 37-51 us).  From about 12M elements on the third CTA pays for itself, except on sparse
+        // plans (see VOTES); below 300 tiles there is a CTA per tile anyway (fewer were no faster).
+        if (d.ntiles <= 3000u || p->density <= kSparseUpTo) g.G = std::min<uint32_t>(g.G, 2u * (uint32_t)p->sm_count);
+        g.maxt = (d.ntiles + g.G - 1) / g.G;
+        g.rows = make_row_map(p, d.ntiles, g.G, g.maxt, g.votes ? 0.0 : p->density >= 0.005 ? kSingleSkew : kSingleSkewSparse);
+        if (g.maxt > kSingleMaxT || g.G > 640) return;               // chunk records and totals must stay small
+        // region per CTA; one bit per slot has to fit in shared memory beside the chunk records
+        g.pool = std::min<uint32_t>(p->cand_cap_alloc / g.G, kSinglePoolMax);
+        g.smem = (size_t)g.maxt * kSingleRowBytes + sizeof(uint32_t) * ((g.pool + 31) / 32);
+        // expected candidates per CTA (sample rank over sample size, times n), with head-room
+        if (nsg > (uint64_t)2 * g.G * kBlock) return;                // a thread owns at most two sample groups
+        const double expect = (double)d.n * (double)d.srank / (4.0 * (double)nsg) / (double)g.G;
+        if ((double)g.pool < 1.5 * expect + 512.0) return;
+        p->single[bf16] = g;
+    }
     // upper bracket: the sample rank that stays below the expected one by the same margin
     const double ks = p->density * 4.0 * (double)nsg;
     const double hi = std::floor(ks - 6.0 * std::sqrt(ks) - 8.0);
     p->single_srank_hi = hi >= 1.0 ? (uint32_t)hi : 1u;    // small sample: the largest sampled key bounds the band
     p->single_srank_mid = (uint32_t)std::max(1.0, std::ceil(ks));
-    p->single_grid = G; p->single_maxt = maxt; p->single_pool = pool; p->single_smem = rec_bytes;
-    p->single_rows = rm;
+    p->single_grid = p->single[0].G;
 }
 
 // Decides whether a threshold plan can use the one-tensor kernel and with which geometry.
@@ -580,8 +586,9 @@ static bool ask_device(int device, DeviceFacts* p) {
             // sized for the largest chunk-record block the kernel may be given; the form that fits least counts
             const size_t smem_max = kSingleMaxT * kSingleRowBytes + kSinglePoolMax / 8;
             int nb = 1 << 20;
-            for (const void* fn : {(const void*)k_topk_single<GradF32, false>, (const void*)k_topk_single<GradF32, true>,
-                                   (const void*)k_topk_single<GradBF16, false>, (const void*)k_topk_single<GradBF16, true>}) {
+            for (const void* fn : {(const void*)k_topk_single<GradF32, false, false>, (const void*)k_topk_single<GradF32, true, false>,
+                                   (const void*)k_topk_single<GradF32, false, true>, (const void*)k_topk_single<GradBF16, false, true>,
+                                   (const void*)k_topk_single<GradBF16, true, true>}) {
                 int n1 = 0;
                 if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n1, fn, kBlock, smem_max) != cudaSuccess) n1 = 0;
                 nb = std::min(nb, n1);
@@ -1117,9 +1124,10 @@ static int compress_impl(gc_plan_t* p, const void* grad_any, bool bf16, float* r
     }
     if (route == GC_ROUTE_TOPK_ONE) {
         // one large tensor: candidates stay in shared memory
+        const SingleGeom& sg = p->single[bf16 ? 1 : 0];
         SingleArgs sa;
-        sa.d = p->desc[0]; sa.desc = p->d_desc; sa.ntiles = nt; sa.maxt = p->single_maxt; sa.rows = p->single_rows;
-        sa.pool_cap = std::min<uint32_t>(p->single_pool, p->cand_cap);
+        sa.d = p->desc[0]; sa.desc = p->d_desc; sa.ntiles = nt; sa.maxt = sg.maxt; sa.rows = sg.rows;
+        sa.pool_cap = std::min<uint32_t>(sg.pool, p->cand_cap);
         sa.cand = reinterpret_cast<uint2*>(wb + p->off_cidx);
         sa.g = grad_any; sa.r = residual; sa.out_idx = out_idx; sa.out_val = out_val; sa.out_count = out_count;
         sa.hist5 = reinterpret_cast<uint32_t*>(wb + p->off_hist5);
@@ -1136,9 +1144,10 @@ static int compress_impl(gc_plan_t* p, const void* grad_any, bool bf16, float* r
         void* args[] = {&sa};
         Timed tm(p, s, GC_K_FUSED);
         const bool dense = p->density >= kDenseFrom;
-        const void* kfn = bf16 ? (dense ? (const void*)k_topk_single<GradBF16, true> : (const void*)k_topk_single<GradBF16, false>)
-                               : (dense ? (const void*)k_topk_single<GradF32, true> : (const void*)k_topk_single<GradF32, false>);
-        GC_CUDA(p, cudaLaunchCooperativeKernel(kfn, dim3(p->single_grid), dim3(kBlock), args, p->single_smem, s));
+        const void* kfn = bf16 ? (dense ? (const void*)k_topk_single<GradBF16, true, true> : (const void*)k_topk_single<GradBF16, false, true>)
+                        : sg.votes ? (const void*)k_topk_single<GradF32, false, true>
+                                   : (dense ? (const void*)k_topk_single<GradF32, true, false> : (const void*)k_topk_single<GradF32, false, false>);
+        GC_CUDA(p, cudaLaunchCooperativeKernel(kfn, dim3(sg.G), dim3(kBlock), args, sg.smem, s));
         return GC_OK;
     }
     if (route == GC_ROUTE_TOPK_MANY) {

@@ -292,12 +292,41 @@ __device__ __forceinline__ void for_chunks(const uint32_t* rec, uint32_t nchunks
     }
 }
 
+// Ranks of a warp chunk's candidates in element order (vector j, then lane, then element), from one mask
+// of 16 bits per thread.  Where no lane has two candidates in one vector -- nearly always at densities of
+// about 1 % -- a vote per vector gives them; otherwise the packed shuffle scan does.
+struct ChunkRanks { uint32_t lanes[kVpt], rank[kVpt], total; };
+__device__ __forceinline__ void chunk_ranks(uint32_t cm, int lane, ChunkRanks& c) {
+    static_assert(kVpt == 4, "16 elements per thread");
+    const uint32_t twice = (cm & (cm >> 1) & 0x7777u) | (cm & (cm >> 2) & 0x3333u) | (cm & (cm >> 3) & 0x1111u);
+    c.total = 0u;
+#pragma unroll
+    for (int j = 0; j < kVpt; ++j) {
+        c.lanes[j] = __ballot_sync(0xFFFFFFFFu, ((cm >> (4 * j)) & 15u) != 0u);
+        c.rank[j] = c.total + (uint32_t)__popc(c.lanes[j] & ((1u << lane) - 1u));
+        c.total += (uint32_t)__popc(c.lanes[j]);
+    }
+    if (__any_sync(0xFFFFFFFFu, twice != 0u)) {
+        uint32_t cnt[kVpt];
+#pragma unroll
+        for (int j = 0; j < kVpt; ++j) cnt[j] = (uint32_t)__popc((cm >> (4 * j)) & 15u);
+        warp_rank(cnt, lane, c.rank, c.total);
+    }
+}
+
 // Three CTAs per SM (80 registers, no spills): measured 15 us faster on the 110M-element workload
 // than four CTAs at 64 registers with spills, and than two.
+// VOTES: how the fold ranks a chunk's candidates -- votes, the residual stored first, chunks without
+// candidates left early, equal shares -- or the shuffle scan.  The votes are a fifth fewer instructions,
+// which pays where instructions bound the loop (bfloat16, 110M elements at 1 %: 241 -> 224 us) and where
+// most chunks are empty (up to 0.2 %; with two CTAs per SM, since a loop that hardly waits for itself keeps
+// the memory busier than it likes with three: 110M elements at 0.1 % 252 -> 231 us, 355M 710 -> 680 us).
+// Between, fp32 is bound by memory and the slower loop with unequal shares does better (0.5 %: 245 against
+// 249-254 us; 355M at 0.3 %: 697 against 714).
 // DENSE (plans of 2 % and more) has the emission by chunk, the bfloat16 form the counted band: the other
 // forms do without their code (a tensor of 1M elements runs every phase from a cold instruction cache:
 // 37.0 against 38.7 us for compress and decode).
-template <typename GL, bool DENSE>
+template <typename GL, bool DENSE, bool VOTES>
 static __global__ void __launch_bounds__(kBlock, 3)
 k_topk_single(const __grid_constant__ SingleArgs a) {
     __shared__ BlockSmem sm;
@@ -476,80 +505,144 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
                 }
             }
         }
-        uint32_t cnt[kVpt], cm = 0, hm = 0;      // candidates; candidates that are zeroed right away
-#pragma unroll
-        for (int j = 0; j < kVpt; ++j) {
-            cnt[j] = 0;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const uint32_t key = key_of(av[j][e]);
-                bool c = key >= tau;
-                if (!interior) c = c && ((valid >> (4 * j + e)) & 1u);
-                cnt[j] += c;
-                cm |= (uint32_t)c << (4 * j + e);
-                if (!interior) hm |= (uint32_t)(key >= tau_z) << (4 * j + e);      // tau_z >= tau > 0: implies c
+        if constexpr (VOTES) {
+            uint32_t cm = 0;                         // candidates of this thread, one bit per element
+    #pragma unroll
+            for (int q = 0; q < 4 * kVpt; ++q) cm |= key_of(av[q / 4][q % 4]) >= tau ? 1u << q : 0u;
+            if (!interior) cm &= valid;
+            // the residual goes out at once: +0 where the key reaches tau_z (implies a candidate: tau_z >= tau), a elsewhere
+            if (interior) {
+    #pragma unroll
+                for (int j = 0; j < kVpt; ++j) {
+                    float4 o;
+                    o.x = key_of(av[j][0]) >= tau_z ? 0.0f : av[j][0];
+                    o.y = key_of(av[j][1]) >= tau_z ? 0.0f : av[j][1];
+                    o.z = key_of(av[j][2]) >= tau_z ? 0.0f : av[j][2];
+                    o.w = key_of(av[j][3]) >= tau_z ? 0.0f : av[j][3];
+                    __stcs(reinterpret_cast<float4*>(a.r + tg.base + my_off + j * 128), o);    // streaming: evict first
+                }
+            } else {
+    #pragma unroll
+                for (int q = 0; q < 4 * kVpt; ++q)
+                    if ((valid >> q) & 1u)
+                        a.r[tg.base + my_off + (q / 4) * 128 + q % 4] = key_of(av[q / 4][q % 4]) >= tau_z ? 0.0f : av[q / 4][q % 4];
             }
-        }
-        uint32_t rk[kVpt], wtot;
-        warp_rank(cnt, lane, rk, wtot);
-        uint32_t off = 0;
-        if (lane == 0 && wtot) off = atomicAdd(&s_used, wtot);
-        off = __shfl_sync(0xFFFFFFFFu, off, 0);
-        const bool fits = off + wtot <= a.pool_cap;
-        if (!fits) block_overflow = true;
-        if (lane == 0) rec[i * kWarps + warp] = fits ? ((off << 10) | wtot) : 0u;
-        const uint32_t em = fits ? cm : 0u;      // goes to the candidate list
-        const uint32_t zm = fits ? (hm & cm) : 0u;      // ... and leaves +0 in the residual (probably sent)
-        if (interior) {
-            // +0 where the key reaches tau_z (implies a candidate: tau_z >= tau), a elsewhere; a chunk that
-            // did not fit keeps all its values (no key reaches 2^31)
-            const uint32_t tz = fits ? tau_z : 0x80000000u;
-#pragma unroll
-            for (int j = 0; j < kVpt; ++j) {
-                float4 o;
-                o.x = key_of(av[j][0]) >= tz ? 0.0f : av[j][0];
-                o.y = key_of(av[j][1]) >= tz ? 0.0f : av[j][1];
-                o.z = key_of(av[j][2]) >= tz ? 0.0f : av[j][2];
-                o.w = key_of(av[j][3]) >= tz ? 0.0f : av[j][3];
-                __stcs(reinterpret_cast<float4*>(a.r + tg.base + my_off + j * 128), o);    // streaming: evict first
+            ChunkRanks cr;
+            chunk_ranks(cm, lane, cr);
+            if (cr.total == 0u) {                    // (uniform: most chunks at densities of 0.1 %)
+                if (lane == 0) rec[i * kWarps + warp] = 0u;
+                continue;
             }
-        } else {
-#pragma unroll
+            uint32_t off = 0;
+            if (lane == 0) off = atomicAdd(&s_used, cr.total);
+            off = __shfl_sync(0xFFFFFFFFu, off, 0);
+            const bool fits = off + cr.total <= a.pool_cap;
+            if (lane == 0) rec[i * kWarps + warp] = fits ? ((off << 10) | cr.total) : 0u;
+            if (!fits) {                             // the chunk keeps all its values (and everything is redone)
+                block_overflow = true;
+    #pragma unroll
+                for (int q = 0; q < 4 * kVpt; ++q)
+                    if ((cm >> q) & 1u) a.r[tg.base + my_off + (q / 4) * 128 + q % 4] = av[q / 4][q % 4];
+                continue;
+            }
+            // candidates are ranked into the warp's shared staging row, then written out as one
+            // contiguous run of 8-byte pairs
+            const bool staged = cr.total <= (uint32_t)kEmitStage;
+            uint2* const to = staged ? sm.emit[warp] : pool + off;
+    #pragma unroll
             for (int j = 0; j < kVpt; ++j) {
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    if ((valid >> (4 * j + e)) & 1u)
-                        a.r[tg.base + my_off + j * 128 + e] = ((zm >> (4 * j + e)) & 1u) ? 0.0f : av[j][e];
+                if (cr.lanes[j] == 0u) continue;     // (uniform)
+                const uint32_t nib = (cm >> (4 * j)) & 15u;
+                uint32_t pos = cr.rank[j];
+                for (uint32_t m = nib; m != 0u; m &= m - 1u, ++pos) {
+                    const float v01 = (m & 1u) ? av[j][0] : av[j][1], v23 = (m & 4u) ? av[j][2] : av[j][3];
+                    const float v = (m & 3u) ? v01 : v23;
+                    const uint32_t e = (uint32_t)__ffs((int)m) - 1u;
+                    to[pos] = make_uint2(tg.base + my_off + j * 128u + e, __float_as_uint(v));
+                    atomicAdd(&sm.hist[min((key_of(v) - tau) >> shift, 2047u)], 1u);
                 }
             }
-        }
-        // candidates are ranked into the warp's shared staging row, then written out as one
-        // contiguous run of 8-byte pairs
-        const bool staged = wtot <= (uint32_t)kEmitStage;
-        if (fits && wtot != 0u) {
-            // one round per candidate of the lane that has the most (one or two at densities around
-            // 1 %), instead of sixteen predicated blocks that every warp walks through
-            for (uint32_t m = em; m != 0u; m &= m - 1u) {
-                const uint32_t bq = (uint32_t)__ffs((int)m) - 1u, j = bq >> 2;      // element 4 j + e of this thread
-                // its value by a select tree (no dynamic register indexing)
-                float s8[8], s4[4];
-#pragma unroll
-                for (int q = 0; q < 8; ++q) s8[q] = (bq & 8u) ? av[2 + q / 4][q % 4] : av[q / 4][q % 4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) s4[q] = (bq & 4u) ? s8[4 + q] : s8[q];
-                const float s20 = (bq & 2u) ? s4[2] : s4[0], s21 = (bq & 2u) ? s4[3] : s4[1];
-                const float v = (bq & 1u) ? s21 : s20;
-                const uint32_t rkj = (bq & 8u) ? ((bq & 4u) ? rk[3] : rk[2]) : ((bq & 4u) ? rk[1] : rk[0]);
-                const uint32_t pos = rkj + (uint32_t)__popc(em & ((1u << bq) - 1u) & (0xFu << (4u * j)));
-                const uint2 pr = make_uint2(tg.base + my_off + j * 128u + (bq & 3u), __float_as_uint(v));
-                if (staged) sm.emit[warp][pos] = pr; else pool[off + pos] = pr;
-                atomicAdd(&sm.hist[min((key_of(v) - tau) >> shift, 2047u)], 1u);
-            }
-
             if (staged) {
                 __syncwarp();
-                for (uint32_t q = lane; q < wtot; q += 32) pool[off + q] = sm.emit[warp][q];
+                for (uint32_t q = lane; q < cr.total; q += 32) pool[off + q] = sm.emit[warp][q];
                 __syncwarp();
+            }
+        } else {
+            uint32_t cnt[kVpt], cm = 0, hm = 0;      // candidates; candidates that are zeroed right away
+    #pragma unroll
+            for (int j = 0; j < kVpt; ++j) {
+                cnt[j] = 0;
+    #pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const uint32_t key = key_of(av[j][e]);
+                    bool c = key >= tau;
+                    if (!interior) c = c && ((valid >> (4 * j + e)) & 1u);
+                    cnt[j] += c;
+                    cm |= (uint32_t)c << (4 * j + e);
+                    if (!interior) hm |= (uint32_t)(key >= tau_z) << (4 * j + e);      // tau_z >= tau > 0: implies c
+                }
+            }
+            uint32_t rk[kVpt], wtot;
+            warp_rank(cnt, lane, rk, wtot);
+            uint32_t off = 0;
+            if (lane == 0 && wtot) off = atomicAdd(&s_used, wtot);
+            off = __shfl_sync(0xFFFFFFFFu, off, 0);
+            const bool fits = off + wtot <= a.pool_cap;
+            if (!fits) block_overflow = true;
+            if (lane == 0) rec[i * kWarps + warp] = fits ? ((off << 10) | wtot) : 0u;
+            const uint32_t em = fits ? cm : 0u;      // goes to the candidate list
+            const uint32_t zm = fits ? (hm & cm) : 0u;      // ... and leaves +0 in the residual (probably sent)
+            if (interior) {
+                // +0 where the key reaches tau_z (implies a candidate: tau_z >= tau), a elsewhere; a chunk that
+                // did not fit keeps all its values (no key reaches 2^31)
+                const uint32_t tz = fits ? tau_z : 0x80000000u;
+    #pragma unroll
+                for (int j = 0; j < kVpt; ++j) {
+                    float4 o;
+                    o.x = key_of(av[j][0]) >= tz ? 0.0f : av[j][0];
+                    o.y = key_of(av[j][1]) >= tz ? 0.0f : av[j][1];
+                    o.z = key_of(av[j][2]) >= tz ? 0.0f : av[j][2];
+                    o.w = key_of(av[j][3]) >= tz ? 0.0f : av[j][3];
+                    __stcs(reinterpret_cast<float4*>(a.r + tg.base + my_off + j * 128), o);    // streaming: evict first
+                }
+            } else {
+    #pragma unroll
+                for (int j = 0; j < kVpt; ++j) {
+    #pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        if ((valid >> (4 * j + e)) & 1u)
+                            a.r[tg.base + my_off + j * 128 + e] = ((zm >> (4 * j + e)) & 1u) ? 0.0f : av[j][e];
+                    }
+                }
+            }
+            // candidates are ranked into the warp's shared staging row, then written out as one
+            // contiguous run of 8-byte pairs
+            const bool staged = wtot <= (uint32_t)kEmitStage;
+            if (fits && wtot != 0u) {
+                // one round per candidate of the lane that has the most (one or two at densities around
+                // 1 %), instead of sixteen predicated blocks that every warp walks through
+                for (uint32_t m = em; m != 0u; m &= m - 1u) {
+                    const uint32_t bq = (uint32_t)__ffs((int)m) - 1u, j = bq >> 2;      // element 4 j + e of this thread
+                    // its value by a select tree (no dynamic register indexing)
+                    float s8[8], s4[4];
+    #pragma unroll
+                    for (int q = 0; q < 8; ++q) s8[q] = (bq & 8u) ? av[2 + q / 4][q % 4] : av[q / 4][q % 4];
+    #pragma unroll
+                    for (int q = 0; q < 4; ++q) s4[q] = (bq & 4u) ? s8[4 + q] : s8[q];
+                    const float s20 = (bq & 2u) ? s4[2] : s4[0], s21 = (bq & 2u) ? s4[3] : s4[1];
+                    const float v = (bq & 1u) ? s21 : s20;
+                    const uint32_t rkj = (bq & 8u) ? ((bq & 4u) ? rk[3] : rk[2]) : ((bq & 4u) ? rk[1] : rk[0]);
+                    const uint32_t pos = rkj + (uint32_t)__popc(em & ((1u << bq) - 1u) & (0xFu << (4u * j)));
+                    const uint2 pr = make_uint2(tg.base + my_off + j * 128u + (bq & 3u), __float_as_uint(v));
+                    if (staged) sm.emit[warp][pos] = pr; else pool[off + pos] = pr;
+                    atomicAdd(&sm.hist[min((key_of(v) - tau) >> shift, 2047u)], 1u);
+                }
+
+                if (staged) {
+                    __syncwarp();
+                    for (uint32_t q = lane; q < wtot; q += 32) pool[off + q] = sm.emit[warp][q];
+                    __syncwarp();
+                }
             }
         }
     }
