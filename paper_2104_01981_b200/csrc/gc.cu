@@ -184,9 +184,11 @@ void sample_params(TensorDesc& d, double density, uint32_t rank_permille, uint64
     *nsg_if_sampled = 0;
     if (d.ntiles <= 1) { d.kind = kKindSmall; *ccap = 0; return; }   // fits one tile: one CTA does the whole tensor
     // Several tensors: a sample the kernel can rank a second time (kRefineTiles sample tiles) gives tau
-    // 22 bits instead of a bin edge (12 % in value).  From 1 % on that is worth more than a larger sample:
-    // the margin of 32,000 samples is a third of k at 1 % and 15 % at 5 %, a bin edge costs up to as much again.
-    if (target_max == kSampleMax && density >= 0.01) target_max = 32000;
+    // 21 bits instead of a bin edge (12 % in value).  Its larger margin (15 % of k at 5 %, a third at 1 %,
+    // as much again as k at 0.1 %) is the smaller evil: under error feedback magnitudes pile up just below
+    // the threshold, and a bin edge can admit enough of them to overflow the candidate regions -- the exact
+    // redo then runs (110M elements in 199 tensors at 0.5 %, repeated gradient: 600-1250 us against 300).
+    if (target_max == kSampleMax && density >= 0.0005) target_max = 32000;
     uint64_t target = std::min<uint64_t>(target_max, std::max<uint64_t>(n / 128, std::min<uint64_t>(8192, n / 2)));
     uint64_t stride = std::max<uint64_t>(1, n / target);
     uint64_t groups = (n + 3) / 4;
@@ -639,8 +641,8 @@ static bool ask_device(int device, DeviceFacts* p) {
             p->multi_smem_max = kMultiMaxPer * kMultiRowBytes + kMultiPoolMax / 8 + 8 * kMultiMaxTab;
             int nbw = 0;          // (the several-workers form of the kernel must be as resident as the kernel itself)
             const std::initializer_list<const void*> forms = {
-                (const void*)k_topk_multi<GradF32, false>, (const void*)k_topk_multi<GradF32, true>,
-                (const void*)k_topk_multi<GradBF16, false>, (const void*)k_topk_multi<GradBF16, true>,
+                (const void*)k_topk_multi<GradF32, false, true>, (const void*)k_topk_multi<GradF32, true, true>,
+                (const void*)k_topk_multi<GradBF16, false, true>, (const void*)k_topk_multi<GradBF16, true, true>,
                 (const void*)k_topk_workers<GradF32, false>, (const void*)k_topk_workers<GradF32, true>};
             if (allow_smem(forms, p->multi_smem_max)) {
                 nb = 1 << 20;
@@ -1160,8 +1162,8 @@ static int compress_impl(gc_plan_t* p, const void* grad_any, bool bf16, float* r
         void* args[] = {&ma};
         Timed tm(p, s, GC_K_FUSED);
         const bool dense = p->density >= kDenseFrom;
-        const void* kfn = bf16 ? (dense ? (const void*)k_topk_multi<GradBF16, true> : (const void*)k_topk_multi<GradBF16, false>)
-                               : (dense ? (const void*)k_topk_multi<GradF32, true> : (const void*)k_topk_multi<GradF32, false>);
+        const void* kfn = bf16 ? (dense ? (const void*)k_topk_multi<GradBF16, true, true> : (const void*)k_topk_multi<GradBF16, false, true>)
+                               : (dense ? (const void*)k_topk_multi<GradF32, true, true> : (const void*)k_topk_multi<GradF32, false, true>);
         GC_CUDA(p, cudaLaunchCooperativeKernel(kfn, dim3(p->multi_grid), dim3(kBlock), args, p->multi_smem, s));
         return GC_OK;
     }

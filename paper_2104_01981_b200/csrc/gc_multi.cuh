@@ -100,8 +100,8 @@ __device__ __forceinline__ bool grid_wait(WsHeader* hdr, uint32_t& passed, int* 
 
 // The whole compress of one worker by the G CTAs of one group (this CTA is number b of them);
 // the group's barriers count on the worker's own workspace header.
-// (DENSE: see k_topk_single)
-template <typename GL, bool DENSE>
+// (DENSE, VOTES: see k_topk_single)
+template <typename GL, bool DENSE, bool VOTES>
 __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32_t G, const uint32_t b, BlockSmem& sm,
                                                 uint32_t& s_used, uint32_t& s_cnt, unsigned char* s_dyn) {
     uint32_t* const rec = reinterpret_cast<uint32_t*>(s_dyn);                  // [per*kWarps] off<<10 | cnt
@@ -373,76 +373,81 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
                     }
                 }
             }
-            uint32_t cnt[kVpt], cm = 0, hm = 0;      // candidates; candidates that are zeroed right away
-#pragma unroll
-            for (int j = 0; j < kVpt; ++j) {
-                cnt[j] = 0;
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const uint32_t key = key_of(av[j][e]);
-                    bool c = key >= tau;
-                    if (!interior) c = c && ((valid >> (4 * j + e)) & 1u);
-                    cnt[j] += c;
-                    cm |= (uint32_t)c << (4 * j + e);
-                    if (!interior) hm |= (uint32_t)(key >= tau_z) << (4 * j + e);
-                }
-            }
-            uint32_t rk[kVpt], wtot;
-            warp_rank(cnt, lane, rk, wtot);
-            uint32_t off = 0;
-            if (lane == 0 && wtot) off = atomicAdd(&s_used, wtot);
-            off = __shfl_sync(0xFFFFFFFFu, off, 0);
-            const bool fits = off + wtot <= a.pool_cap;
-            if (!fits) block_overflow = true;
-            if (lane == 0) rec[i * kWarps + warp] = fits ? ((off << 10) | wtot) : 0u;
-            const uint32_t em = fits ? cm : 0u;             // goes to the candidate list
-            const uint32_t zm = fits ? (hm & cm) : 0u;      // ... and leaves +0 in the residual (probably sent)
-            if (interior) {
-                // +0 where the key reaches tau_z (implies a candidate: tau_z >= tau), a elsewhere; a chunk
-                // that did not fit keeps all its values (no key reaches 2^31)
-                const uint32_t tz = fits ? tau_z : 0x80000000u;
-#pragma unroll
-                for (int j = 0; j < kVpt; ++j) {
-                    float4 o;
-                    o.x = key_of(av[j][0]) >= tz ? 0.0f : av[j][0];
-                    o.y = key_of(av[j][1]) >= tz ? 0.0f : av[j][1];
-                    o.z = key_of(av[j][2]) >= tz ? 0.0f : av[j][2];
-                    o.w = key_of(av[j][3]) >= tz ? 0.0f : av[j][3];
-                    __stcs(reinterpret_cast<float4*>(a.r + tg.base + my_off + j * 128), o);    // streaming: evict first
-                }
+            if constexpr (VOTES) {
+                block_overflow |= !fold_tail_votes(sm, av, interior, valid, tau, tau_z, shift, tg.base + my_off, a.r, s_used, a.pool_cap, pool,
+                                                   rec[i * kWarps + warp], lane, warp);
             } else {
+                uint32_t cnt[kVpt], cm = 0, hm = 0;      // candidates; candidates that are zeroed right away
 #pragma unroll
                 for (int j = 0; j < kVpt; ++j) {
+                    cnt[j] = 0;
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
-                        if ((valid >> (4 * j + e)) & 1u)
-                            a.r[tg.base + my_off + j * 128 + e] = ((zm >> (4 * j + e)) & 1u) ? 0.0f : av[j][e];
+                        const uint32_t key = key_of(av[j][e]);
+                        bool c = key >= tau;
+                        if (!interior) c = c && ((valid >> (4 * j + e)) & 1u);
+                        cnt[j] += c;
+                        cm |= (uint32_t)c << (4 * j + e);
+                        if (!interior) hm |= (uint32_t)(key >= tau_z) << (4 * j + e);
                     }
                 }
-            }
-            const bool staged = wtot <= (uint32_t)kEmitStage;
-            if (fits && wtot != 0u) {
-                // one round per candidate of the lane that has the most, instead of sixteen predicated
-                // blocks that every warp walks through (see the one-tensor kernel)
-                for (uint32_t m = em; m != 0u; m &= m - 1u) {
-                    const uint32_t bq = (uint32_t)__ffs((int)m) - 1u, j = bq >> 2;      // element 4 j + e of this thread
-                    float s8[8], s4[4];                                                 // its value by a select tree
+                uint32_t rk[kVpt], wtot;
+                warp_rank(cnt, lane, rk, wtot);
+                uint32_t off = 0;
+                if (lane == 0 && wtot) off = atomicAdd(&s_used, wtot);
+                off = __shfl_sync(0xFFFFFFFFu, off, 0);
+                const bool fits = off + wtot <= a.pool_cap;
+                if (!fits) block_overflow = true;
+                if (lane == 0) rec[i * kWarps + warp] = fits ? ((off << 10) | wtot) : 0u;
+                const uint32_t em = fits ? cm : 0u;             // goes to the candidate list
+                const uint32_t zm = fits ? (hm & cm) : 0u;      // ... and leaves +0 in the residual (probably sent)
+                if (interior) {
+                    // +0 where the key reaches tau_z (implies a candidate: tau_z >= tau), a elsewhere; a chunk
+                    // that did not fit keeps all its values (no key reaches 2^31)
+                    const uint32_t tz = fits ? tau_z : 0x80000000u;
 #pragma unroll
-                    for (int q = 0; q < 8; ++q) s8[q] = (bq & 8u) ? av[2 + q / 4][q % 4] : av[q / 4][q % 4];
+                    for (int j = 0; j < kVpt; ++j) {
+                        float4 o;
+                        o.x = key_of(av[j][0]) >= tz ? 0.0f : av[j][0];
+                        o.y = key_of(av[j][1]) >= tz ? 0.0f : av[j][1];
+                        o.z = key_of(av[j][2]) >= tz ? 0.0f : av[j][2];
+                        o.w = key_of(av[j][3]) >= tz ? 0.0f : av[j][3];
+                        __stcs(reinterpret_cast<float4*>(a.r + tg.base + my_off + j * 128), o);    // streaming: evict first
+                    }
+                } else {
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) s4[q] = (bq & 4u) ? s8[4 + q] : s8[q];
-                    const float s20 = (bq & 2u) ? s4[2] : s4[0], s21 = (bq & 2u) ? s4[3] : s4[1];
-                    const float v = (bq & 1u) ? s21 : s20;
-                    const uint32_t rkj = (bq & 8u) ? ((bq & 4u) ? rk[3] : rk[2]) : ((bq & 4u) ? rk[1] : rk[0]);
-                    const uint32_t pos = rkj + (uint32_t)__popc(em & ((1u << bq) - 1u) & (0xFu << (4u * j)));
-                    const uint2 pr = make_uint2(tg.base + my_off + j * 128u + (bq & 3u), __float_as_uint(v));
-                    if (staged) sm.emit[warp][pos] = pr; else pool[off + pos] = pr;
-                    atomicAdd(&sm.hist[min((key_of(v) - tau) >> shift, 2047u)], 1u);
+                    for (int j = 0; j < kVpt; ++j) {
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            if ((valid >> (4 * j + e)) & 1u)
+                                a.r[tg.base + my_off + j * 128 + e] = ((zm >> (4 * j + e)) & 1u) ? 0.0f : av[j][e];
+                        }
+                    }
                 }
-                if (staged) {
-                    __syncwarp();
-                    for (uint32_t q = lane; q < wtot; q += 32) pool[off + q] = sm.emit[warp][q];
-                    __syncwarp();
+                const bool staged = wtot <= (uint32_t)kEmitStage;
+                if (fits && wtot != 0u) {
+                    // one round per candidate of the lane that has the most, instead of sixteen predicated
+                    // blocks that every warp walks through (see the one-tensor kernel)
+                    for (uint32_t m = em; m != 0u; m &= m - 1u) {
+                        const uint32_t bq = (uint32_t)__ffs((int)m) - 1u, j = bq >> 2;      // element 4 j + e of this thread
+                        float s8[8], s4[4];                                                 // its value by a select tree
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) s8[q] = (bq & 8u) ? av[2 + q / 4][q % 4] : av[q / 4][q % 4];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) s4[q] = (bq & 4u) ? s8[4 + q] : s8[q];
+                        const float s20 = (bq & 2u) ? s4[2] : s4[0], s21 = (bq & 2u) ? s4[3] : s4[1];
+                        const float v = (bq & 1u) ? s21 : s20;
+                        const uint32_t rkj = (bq & 8u) ? ((bq & 4u) ? rk[3] : rk[2]) : ((bq & 4u) ? rk[1] : rk[0]);
+                        const uint32_t pos = rkj + (uint32_t)__popc(em & ((1u << bq) - 1u) & (0xFu << (4u * j)));
+                        const uint2 pr = make_uint2(tg.base + my_off + j * 128u + (bq & 3u), __float_as_uint(v));
+                        if (staged) sm.emit[warp][pos] = pr; else pool[off + pos] = pr;
+                        atomicAdd(&sm.hist[min((key_of(v) - tau) >> shift, 2047u)], 1u);
+                    }
+                    if (staged) {
+                        __syncwarp();
+                        for (uint32_t q = lane; q < wtot; q += 32) pool[off + q] = sm.emit[warp][q];
+                        __syncwarp();
+                    }
                 }
             }
         }
@@ -775,14 +780,15 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
     leave_clean(a.cl, hdr, G, tid);
 }
 
-template <typename GL, bool DENSE>
+// Votes: 25.6M elements in 161 tensors at 0.1 % 99 -> 97 us, 110M in 199 at 1 % 302 -> 289 us.
+template <typename GL, bool DENSE, bool VOTES>
 // (three CTAs per SM: 80 registers and no spills beat four at 64 registers, see k_topk_single)
 static __global__ void __launch_bounds__(kBlock, 3)
 k_topk_multi(const __grid_constant__ MultiArgs a) {
     __shared__ BlockSmem sm;
     __shared__ uint32_t s_used, s_cnt;
     extern __shared__ __align__(16) unsigned char s_dyn[];
-    topk_multi_body<GL, DENSE>(a, gridDim.x, blockIdx.x, sm, s_used, s_cnt, s_dyn);
+    topk_multi_body<GL, DENSE, VOTES>(a, gridDim.x, blockIdx.x, sm, s_used, s_cnt, s_dyn);
 }
 
 // Several workers' compress calls in ONE cooperative launch: the grid is cut into one group of
@@ -798,6 +804,8 @@ struct WorkersArgs {
 };
 static_assert(sizeof(WorkersArgs) <= 4000, "kernel parameters stay below 4 KB");
 
+// (The scan stays here: with several workers per launch the fold is bound by memory, 475 against 484 us
+// for eight 161-tensor workers.)
 template <typename GL, bool DENSE>
 static __global__ void __launch_bounds__(kBlock, 3)
 k_topk_workers(const __grid_constant__ WorkersArgs wa) {
@@ -812,7 +820,7 @@ k_topk_workers(const __grid_constant__ WorkersArgs wa) {
         for (uint32_t i = threadIdx.x; i < sizeof(MultiArgs) / 4; i += kBlock) dst[i] = src[i];
     }
     __syncthreads();
-    topk_multi_body<GL, DENSE>(s_args, wa.G, b, sm, s_used, s_cnt, s_dyn);
+    topk_multi_body<GL, DENSE, false>(s_args, wa.G, b, sm, s_used, s_cnt, s_dyn);
 }
 
 }  // namespace gc

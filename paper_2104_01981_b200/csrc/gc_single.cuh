@@ -314,6 +314,74 @@ __device__ __forceinline__ void chunk_ranks(uint32_t cm, int lane, ChunkRanks& c
     }
 }
 
+// The rest of the fold of one warp chunk in the form with votes: residual, list entries, band histogram.
+// `at0` = flat index of this thread's first element.  Returns false if the candidate region is full.
+__device__ __forceinline__ bool fold_tail_votes(BlockSmem& sm, const float (&av)[kVpt][4], bool interior, uint32_t valid, uint32_t tau,
+                                                uint32_t tau_z, int shift, uint32_t at0, float* r, uint32_t& s_used, uint32_t pool_cap,
+                                                uint2* pool, uint32_t& rec, int lane, int warp) {
+    uint32_t cm = 0;                         // candidates of this thread, one bit per element
+#pragma unroll
+    for (int q = 0; q < 4 * kVpt; ++q) cm |= key_of(av[q / 4][q % 4]) >= tau ? 1u << q : 0u;
+    if (!interior) cm &= valid;
+    // the residual goes out at once: +0 where the key reaches tau_z (implies a candidate: tau_z >= tau), a elsewhere
+    if (interior) {
+#pragma unroll
+        for (int j = 0; j < kVpt; ++j) {
+            float4 o;
+            o.x = key_of(av[j][0]) >= tau_z ? 0.0f : av[j][0];
+            o.y = key_of(av[j][1]) >= tau_z ? 0.0f : av[j][1];
+            o.z = key_of(av[j][2]) >= tau_z ? 0.0f : av[j][2];
+            o.w = key_of(av[j][3]) >= tau_z ? 0.0f : av[j][3];
+            __stcs(reinterpret_cast<float4*>(r + at0 + j * 128), o);    // streaming: evict first
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < 4 * kVpt; ++q)
+            if ((valid >> q) & 1u)
+                r[at0 + (q / 4) * 128 + q % 4] = key_of(av[q / 4][q % 4]) >= tau_z ? 0.0f : av[q / 4][q % 4];
+    }
+    ChunkRanks cr;
+    chunk_ranks(cm, lane, cr);
+    if (cr.total == 0u) {                    // (uniform: most chunks at densities of 0.1 %)
+        if (lane == 0) rec = 0u;
+        return true;
+    }
+    uint32_t off = 0;
+    if (lane == 0) off = atomicAdd(&s_used, cr.total);
+    off = __shfl_sync(0xFFFFFFFFu, off, 0);
+    const bool fits = off + cr.total <= pool_cap;
+    if (lane == 0) rec = fits ? ((off << 10) | cr.total) : 0u;
+    if (!fits) {                             // the chunk keeps all its values (and everything is redone)
+#pragma unroll
+        for (int q = 0; q < 4 * kVpt; ++q)
+            if ((cm >> q) & 1u) r[at0 + (q / 4) * 128 + q % 4] = av[q / 4][q % 4];
+        return false;
+    }
+    // candidates are ranked into the warp's shared staging row, then written out as one
+    // contiguous run of 8-byte pairs
+    const bool staged = cr.total <= (uint32_t)kEmitStage;
+    uint2* const to = staged ? sm.emit[warp] : pool + off;
+#pragma unroll
+    for (int j = 0; j < kVpt; ++j) {
+        if (cr.lanes[j] == 0u) continue;     // (uniform)
+        const uint32_t nib = (cm >> (4 * j)) & 15u;
+        uint32_t pos = cr.rank[j];
+        for (uint32_t m = nib; m != 0u; m &= m - 1u, ++pos) {
+            const float v01 = (m & 1u) ? av[j][0] : av[j][1], v23 = (m & 4u) ? av[j][2] : av[j][3];
+            const float v = (m & 3u) ? v01 : v23;
+            const uint32_t e = (uint32_t)__ffs((int)m) - 1u;
+            to[pos] = make_uint2(at0 + j * 128u + e, __float_as_uint(v));
+            atomicAdd(&sm.hist[min((key_of(v) - tau) >> shift, 2047u)], 1u);
+        }
+    }
+    if (staged) {
+        __syncwarp();
+        for (uint32_t q = lane; q < cr.total; q += 32) pool[off + q] = sm.emit[warp][q];
+        __syncwarp();
+    }
+    return true;
+}
+
 // Three CTAs per SM (80 registers, no spills): measured 15 us faster on the 110M-element workload
 // than four CTAs at 64 registers with spills, and than two.
 // VOTES: how the fold ranks a chunk's candidates -- votes, the residual stored first, chunks without
@@ -506,73 +574,14 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
             }
         }
         if constexpr (VOTES) {
-            uint32_t cm = 0;                         // candidates of this thread, one bit per element
-    #pragma unroll
-            for (int q = 0; q < 4 * kVpt; ++q) cm |= key_of(av[q / 4][q % 4]) >= tau ? 1u << q : 0u;
-            if (!interior) cm &= valid;
-            // the residual goes out at once: +0 where the key reaches tau_z (implies a candidate: tau_z >= tau), a elsewhere
-            if (interior) {
-    #pragma unroll
-                for (int j = 0; j < kVpt; ++j) {
-                    float4 o;
-                    o.x = key_of(av[j][0]) >= tau_z ? 0.0f : av[j][0];
-                    o.y = key_of(av[j][1]) >= tau_z ? 0.0f : av[j][1];
-                    o.z = key_of(av[j][2]) >= tau_z ? 0.0f : av[j][2];
-                    o.w = key_of(av[j][3]) >= tau_z ? 0.0f : av[j][3];
-                    __stcs(reinterpret_cast<float4*>(a.r + tg.base + my_off + j * 128), o);    // streaming: evict first
-                }
-            } else {
-    #pragma unroll
-                for (int q = 0; q < 4 * kVpt; ++q)
-                    if ((valid >> q) & 1u)
-                        a.r[tg.base + my_off + (q / 4) * 128 + q % 4] = key_of(av[q / 4][q % 4]) >= tau_z ? 0.0f : av[q / 4][q % 4];
-            }
-            ChunkRanks cr;
-            chunk_ranks(cm, lane, cr);
-            if (cr.total == 0u) {                    // (uniform: most chunks at densities of 0.1 %)
-                if (lane == 0) rec[i * kWarps + warp] = 0u;
-                continue;
-            }
-            uint32_t off = 0;
-            if (lane == 0) off = atomicAdd(&s_used, cr.total);
-            off = __shfl_sync(0xFFFFFFFFu, off, 0);
-            const bool fits = off + cr.total <= a.pool_cap;
-            if (lane == 0) rec[i * kWarps + warp] = fits ? ((off << 10) | cr.total) : 0u;
-            if (!fits) {                             // the chunk keeps all its values (and everything is redone)
-                block_overflow = true;
-    #pragma unroll
-                for (int q = 0; q < 4 * kVpt; ++q)
-                    if ((cm >> q) & 1u) a.r[tg.base + my_off + (q / 4) * 128 + q % 4] = av[q / 4][q % 4];
-                continue;
-            }
-            // candidates are ranked into the warp's shared staging row, then written out as one
-            // contiguous run of 8-byte pairs
-            const bool staged = cr.total <= (uint32_t)kEmitStage;
-            uint2* const to = staged ? sm.emit[warp] : pool + off;
-    #pragma unroll
-            for (int j = 0; j < kVpt; ++j) {
-                if (cr.lanes[j] == 0u) continue;     // (uniform)
-                const uint32_t nib = (cm >> (4 * j)) & 15u;
-                uint32_t pos = cr.rank[j];
-                for (uint32_t m = nib; m != 0u; m &= m - 1u, ++pos) {
-                    const float v01 = (m & 1u) ? av[j][0] : av[j][1], v23 = (m & 4u) ? av[j][2] : av[j][3];
-                    const float v = (m & 3u) ? v01 : v23;
-                    const uint32_t e = (uint32_t)__ffs((int)m) - 1u;
-                    to[pos] = make_uint2(tg.base + my_off + j * 128u + e, __float_as_uint(v));
-                    atomicAdd(&sm.hist[min((key_of(v) - tau) >> shift, 2047u)], 1u);
-                }
-            }
-            if (staged) {
-                __syncwarp();
-                for (uint32_t q = lane; q < cr.total; q += 32) pool[off + q] = sm.emit[warp][q];
-                __syncwarp();
-            }
+            block_overflow |= !fold_tail_votes(sm, av, interior, valid, tau, tau_z, shift, tg.base + my_off, a.r, s_used, a.pool_cap, pool,
+                                               rec[i * kWarps + warp], lane, warp);
         } else {
             uint32_t cnt[kVpt], cm = 0, hm = 0;      // candidates; candidates that are zeroed right away
-    #pragma unroll
+#pragma unroll
             for (int j = 0; j < kVpt; ++j) {
                 cnt[j] = 0;
-    #pragma unroll
+#pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const uint32_t key = key_of(av[j][e]);
                     bool c = key >= tau;
@@ -596,7 +605,7 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
                 // +0 where the key reaches tau_z (implies a candidate: tau_z >= tau), a elsewhere; a chunk that
                 // did not fit keeps all its values (no key reaches 2^31)
                 const uint32_t tz = fits ? tau_z : 0x80000000u;
-    #pragma unroll
+#pragma unroll
                 for (int j = 0; j < kVpt; ++j) {
                     float4 o;
                     o.x = key_of(av[j][0]) >= tz ? 0.0f : av[j][0];
@@ -606,9 +615,9 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
                     __stcs(reinterpret_cast<float4*>(a.r + tg.base + my_off + j * 128), o);    // streaming: evict first
                 }
             } else {
-    #pragma unroll
+#pragma unroll
                 for (int j = 0; j < kVpt; ++j) {
-    #pragma unroll
+#pragma unroll
                     for (int e = 0; e < 4; ++e) {
                         if ((valid >> (4 * j + e)) & 1u)
                             a.r[tg.base + my_off + j * 128 + e] = ((zm >> (4 * j + e)) & 1u) ? 0.0f : av[j][e];
@@ -625,9 +634,9 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
                     const uint32_t bq = (uint32_t)__ffs((int)m) - 1u, j = bq >> 2;      // element 4 j + e of this thread
                     // its value by a select tree (no dynamic register indexing)
                     float s8[8], s4[4];
-    #pragma unroll
+#pragma unroll
                     for (int q = 0; q < 8; ++q) s8[q] = (bq & 8u) ? av[2 + q / 4][q % 4] : av[q / 4][q % 4];
-    #pragma unroll
+#pragma unroll
                     for (int q = 0; q < 4; ++q) s4[q] = (bq & 4u) ? s8[4 + q] : s8[q];
                     const float s20 = (bq & 2u) ? s4[2] : s4[0], s21 = (bq & 2u) ? s4[3] : s4[1];
                     const float v = (bq & 1u) ? s21 : s20;
