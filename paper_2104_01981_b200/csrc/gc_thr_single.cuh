@@ -2,7 +2,8 @@
 //
 //   sample   one 4-element group out of `sstride` is folded on the fly; its keys are kept (16 B
 //            per group).  Coarse histogram (top 11 key bits, shared memory) + fine histogram
-//            (top 18 bits, global atomics into scattered slots)          | grid barrier
+//            (top 18 bits, global atomics into scattered slots; only for keys that can matter)
+//                                                                        | grid barrier
 //   level 2  every CTA derives the 18-bit prefix of the k_s-th largest sampled key, then puts the
 //            kept keys under that prefix (a handful) on a short list and counts their low 13
 //            bits in 8192 global bins                                    | grid barrier
@@ -35,7 +36,7 @@ struct ThrSingleArgs {
     uint32_t* out_count;
     uint2* cand;                     // [gridDim.x * pool_cap] hit list, one region per CTA
     uint4* skeys;                    // [sample groups] the sampled keys
-    uint32_t* hist5;                 // [0] coarse sample histogram, [1][0] short-list length (zeroed)
+    uint32_t* hist5;                 // [0] coarse sample histogram, [1][0] short-list length, [1][1] highest floor (zeroed)
     uint32_t* hist13;                // [8192] low 13 bits of the sampled keys under the prefix (zeroed)
     uint2* mid;                      // [mid_cap] those keys (second word), as a short list
     uint32_t mid_cap;
@@ -72,31 +73,79 @@ k_threshold_single(const __grid_constant__ ThrSingleArgs a) {
     // ---------------------------------------------------------------- sample, level 1
     const uint32_t ngroups = (d.n + 3u) >> 2;
     const uint32_t nsg = (ngroups + d.sstride - 1) / d.sstride;
-    for (uint32_t q = 0; q < a.sample_rounds; ++q) {
-        const uint64_t sg = (uint64_t)q * G * kBlock + (uint64_t)b * kBlock + tid;
-        const bool mine = sg < nsg;                         // (every lane stays in the loop: the coarse counts are
-        const uint64_t gi = sg * d.sstride;                 //  aggregated over the warp)  gi < ngroups by the definition of nsg
-        const uint32_t i0 = mine ? (uint32_t)gi * 4u : 0u;
-        float gv[4], rv[4];
+    // Scattered 16-byte reads bound this phase (1.1M keys of 110M elements: 31 us, 37 before), so four rounds
+    // of groups are in flight per thread.  Counting is plain: aggregating equal bins over the warp costs 4 us
+    // on spread data, and a sample in one single bin costs less than that in serialised adds.
+    const bool vec_ok = (d.off & 3u) == 0u;
+    for (uint32_t q0 = 0; q0 < a.sample_rounds; q0 += 4u) {
+        float gv[4][4], rv[4][4];
+        uint32_t i0[4];
+        bool mine[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const bool v = mine && i0 + e < d.n;
-            const uint32_t f = d.off + (v ? i0 + e : 0u);
-            gv[e] = v ? __ldg(a.g + f) : 0.f;
-            rv[e] = v ? ld_cg(a.r + f) : 0.f;
-        }
-        uint32_t key[4];
+        for (uint32_t u = 0; u < 4; ++u) {
+            const uint64_t sg = (uint64_t)(q0 + u) * G * kBlock + (uint64_t)b * kBlock + tid;
+            mine[u] = q0 + u < a.sample_rounds && sg < nsg;
+            i0[u] = mine[u] ? (uint32_t)(sg * d.sstride) * 4u : 0u;      // (below n by the definition of nsg)
+            if (vec_ok && mine[u] && i0[u] + 3u < d.n) {
+                const float4 g4 = __ldg(reinterpret_cast<const float4*>(a.g + d.off + i0[u]));
+                const float4 r4 = ld_cg(reinterpret_cast<const float4*>(a.r + d.off + i0[u]));
+                gv[u][0] = g4.x; gv[u][1] = g4.y; gv[u][2] = g4.z; gv[u][3] = g4.w;
+                rv[u][0] = r4.x; rv[u][1] = r4.y; rv[u][2] = r4.z; rv[u][3] = r4.w;
+            } else {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            key[e] = 0xFFFFFFFFu;                           // = not a sample
-            if (mine && i0 + e < d.n) {
-                key[e] = key_of(__fadd_rn(gv[e], rv[e]));
-                atomicAdd(a.fine + fine_slot(key[e] >> kFineShift), 1u);
+                for (int e = 0; e < 4; ++e) {
+                    const bool v = mine[u] && i0[u] + e < d.n;
+                    const uint32_t f = d.off + (v ? i0[u] + e : 0u);
+                    gv[u][e] = v ? __ldg(a.g + f) : 0.f;
+                    rv[u][e] = v ? ld_cg(a.r + f) : 0.f;
+                }
             }
-            hist_add_warp(sm.hist, key[e] == 0xFFFFFFFFu ? 0xFFFFFFFFu : key[e] >> level_shift(0), lane);
         }
-        if (mine) a.skeys[sg] = make_uint4(key[0], key[1], key[2], key[3]);
+#pragma unroll
+        for (uint32_t u = 0; u < 4; ++u) {
+            uint32_t key[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                key[e] = mine[u] && i0[u] + e < d.n ? key_of(__fadd_rn(gv[u][e], rv[u][e])) : 0xFFFFFFFFu;      // = not a sample
+                if (key[e] != 0xFFFFFFFFu) atomicAdd(&sm.hist[key[e] >> level_shift(0)], 1u);
+            }
+            if (mine[u]) a.skeys[(uint64_t)(q0 + u) * G * kBlock + (uint64_t)b * kBlock + tid] = make_uint4(key[0], key[1], key[2], key[3]);
+        }
     }
+    // The fine histogram takes one global atomic per key, and only the cells of one coarse bin matter: a CTA
+    // counts what lies in the bin of its own sample that holds four times the rank's share, or above (with
+    // every key counted the phase takes 10 us longer on 110M elements).  Should the rank's bin turn out to
+    // lie below the highest floor of any CTA, what the CTAs left out of that bin is counted after the barrier.
+    uint32_t floor_bin = 0;
+    {
+        __syncthreads();
+        const uint64_t own = ((uint64_t)a.sample_rounds * kBlock) * 4u;
+        const uint32_t share = (uint32_t)((float)own * (float)d.srank / (4.0f * (float)nsg));
+        uint32_t bin, above;
+        if (block_select<(1 << level_bits(0)), true>(sm, sm.hist, 4u * share + 64u, bin, above)) floor_bin = bin;
+        if (tid == 0 && floor_bin != 0u) atomicMax(a.hist5 + kHistBins + 1, floor_bin);
+    }
+    auto count_fine = [&](uint32_t lo_bin, uint32_t hi_bin) {          // own keys with lo_bin <= coarse bin < hi_bin
+        for (uint32_t q0 = 0; q0 < a.sample_rounds; q0 += 4u) {
+            uint4 kv[4];
+#pragma unroll
+            for (uint32_t u = 0; u < 4; ++u) {
+                const uint64_t sg = (uint64_t)(q0 + u) * G * kBlock + (uint64_t)b * kBlock + tid;
+                kv[u] = q0 + u < a.sample_rounds && sg < nsg ? a.skeys[sg]           // written by this very thread
+                                                             : make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
+            }
+#pragma unroll
+            for (uint32_t u = 0; u < 4; ++u) {
+                const uint32_t kk[4] = {kv[u].x, kv[u].y, kv[u].z, kv[u].w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const uint32_t c = kk[e] >> level_shift(0);
+                    if (c >= lo_bin && c < hi_bin) atomicAdd(a.fine + fine_slot(kk[e] >> kFineShift), 1u);
+                }
+            }
+        }
+    };
+    count_fine(floor_bin, 2048u);
     flush_hist(sm, a.hist5 + 0 * kHistBins, 1 << level_bits(0));
     if (!grid_barrier(hdr, passed, &sm.ok)) return;
     phase_stamp(hdr, n_stamp);
@@ -108,6 +157,10 @@ k_threshold_single(const __grid_constant__ ThrSingleArgs a) {
         const uint32_t want[1] = {d.srank};
         Picked pk[1];
         block_select_multi<(1 << level_bits(0)), 1>(sm, a.hist5 + 0 * kHistBins, want, pk);
+        if (pk[0].ok && pk[0].bin < ld_cg(a.hist5 + kHistBins + 1)) {        // (the same in every CTA)
+            if (pk[0].bin < floor_bin) count_fine(pk[0].bin, pk[0].bin + 1u);
+            if (!grid_barrier(hdr, passed, &sm.ok)) return;
+        }
         if (warp == 0) {
             uint32_t res = 0xFFFFFFFFu, rk = 0;
             if (pk[0].ok) {
