@@ -838,7 +838,7 @@ def run_decode_sweep(args, w: synth.Workload, rank: int, world: int, local_rank:
             us = e0.elapsed_time(e1) / args.steps * 1e3
             row[name + "_us"] = us
             row[name + "_frac_of_measured_peak"] = row["bytes"] / us / 1e3 / peak
-        # no fixed order among the workers (within 1e-6 relative of the fixed-order sum up to 16 workers)
+        # the caller would accept any order among the workers
         plan.set_option(api.GC_OPT_DECODE_ROUTE, api.GC_DECODE_AUTO)
         plan.set_option(api.GC_OPT_DECODE_ORDER, api.GC_ORDER_ANY)
         for _ in range(max(args.warmup, 3)):
