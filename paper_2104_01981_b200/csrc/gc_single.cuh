@@ -469,7 +469,7 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const bool okq = (sok >> (4 * q + e)) & 1u;
-                hist_add_warp(sm.hist, okq ? skey[q][e] >> level_shift(0) : 0xFFFFFFFFu, lane);
+                if (okq) atomicAdd(&sm.hist[skey[q][e] >> level_shift(0)], 1u);
                 if (okq) atomicAdd(a.fine + fine_slot(skey[q][e] >> kFineShift), 1u);
             }
         // the first own tile is asked into L2 while the sample is being settled

@@ -296,9 +296,9 @@ static __device__ __forceinline__ void threshold_multi_body(const ThrMultiArgs& 
                 if (u < nb) {                             // (uniform over the CTA)
                     uint32_t key[4] = {0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu};     // = not a sample
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {         // (all lanes: the coarse counts are aggregated over the warp)
+                    for (int e = 0; e < 4; ++e) {
                         if (live[u] && i0[u] + e < d.n) key[e] = key_of(__fadd_rn(gv[u][e], rv[u][e]));
-                        hist_add_warp(sm.hist, key[e] == 0xFFFFFFFFu ? 0xFFFFFFFFu : key[e] >> level_shift(0), lane);
+                        if (key[e] != 0xFFFFFFFFu) atomicAdd(&sm.hist[key[e] >> level_shift(0)], 1u);
                     }
                     a.skeys[(size_t)(st + u) * kBlock + tid] = make_uint4(key[0], key[1], key[2], key[3]);
                 }

@@ -74,8 +74,7 @@ k_threshold_single(const __grid_constant__ ThrSingleArgs a) {
     const uint32_t ngroups = (d.n + 3u) >> 2;
     const uint32_t nsg = (ngroups + d.sstride - 1) / d.sstride;
     // Scattered 16-byte reads bound this phase (1.1M keys of 110M elements: 31 us, 37 before), so four rounds
-    // of groups are in flight per thread.  Counting is plain: aggregating equal bins over the warp costs 4 us
-    // on spread data, and a sample in one single bin costs less than that in serialised adds.
+    // of groups are in flight per thread.  Counting is plain: aggregating equal bins over the warp costs 4 us.
     const bool vec_ok = (d.off & 3u) == 0u;
     for (uint32_t q0 = 0; q0 < a.sample_rounds; q0 += 4u) {
         float gv[4][4], rv[4][4];
@@ -117,7 +116,7 @@ k_threshold_single(const __grid_constant__ ThrSingleArgs a) {
     // every key counted the phase takes 10 us longer on 110M elements).  Should the rank's bin turn out to
     // lie below the highest floor of any CTA, what the CTAs left out of that bin is counted after the barrier.
     uint32_t floor_bin = 0;
-    {
+    if (a.sample_rounds > 1u) {                            // (a short sample: finding the floor takes longer than it saves)
         __syncthreads();
         const uint64_t own = ((uint64_t)a.sample_rounds * kBlock) * 4u;
         const uint32_t share = (uint32_t)((float)own * (float)d.srank / (4.0f * (float)nsg));
