@@ -89,6 +89,24 @@ k_decode_rings(const __grid_constant__ DecodeLists ls, uint32_t W, uint32_t cnt,
     const uint32_t t1 = (uint32_t)(((unsigned long long)(blockIdx.x + 1u) * ntl) / gridDim.x);
     if (t0 >= t1) return;
 
+    auto fetch = [&](uint32_t tl) {                        // what this warp's sub-tile of tile tl needs besides the lists
+        const uint32_t a = tl * tile + warp * T, span = a < total_n ? min(T, total_n - a) : 0u;
+        if (APPLY) {                                       // (the buffer's last words with zeros behind them)
+            for (uint32_t q = lane; 4 * q < span; q += 32) {
+                const uint32_t bytes = min(4u, span - 4 * q) * 4u;
+                cp_async_16(s_par + 4 * q, ap.param + a + 4 * q, bytes);
+                cp_async_16(s_par + T + 4 * q, ap.vel + a + 4 * q, bytes);
+            }
+        }
+        if (ADD) {
+            if (span == T && aligned) for (uint32_t q = lane; q < T / 4; q += 32) cp_async_16(s_tile + 4 * q, out + a + 4 * q);
+            else for (uint32_t q = lane; q < span; q += 32) cp_async_4(s_tile + q, out + a + q);
+        }
+    };
+    fetch(t0);                                             // (under the search below)
+    if (!ADD)
+        for (uint32_t q = lane; q < T / 4; q += 32) reinterpret_cast<float4*>(s_tile)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+
     // where every list enters this CTA's run of tiles
     if (tid < 64) s_len[tid] = (uint32_t)tid >= W ? 0u : ls.len[tid] != nullptr ? min(__ldg(ls.len[tid]), cnt) : cnt;
     __syncthreads();
@@ -135,23 +153,7 @@ k_decode_rings(const __grid_constant__ DecodeLists ls, uint32_t W, uint32_t cnt,
         if (to > my_fill) { my_slot = wrap(my_slot + (to - my_fill)); my_fill = to; }
         if (top && sub == 0u) s_fill[my_w] = min(my_fill, my_len);
     };
-    auto fetch = [&](uint32_t tl) {                        // what this warp's sub-tile of tile tl needs besides the lists
-        const uint32_t a = tl * tile + warp * T, span = a < total_n ? min(T, total_n - a) : 0u;
-        if (APPLY && span == T) {
-            for (uint32_t q = lane; q < T / 4; q += 32) {
-                cp_async_16(s_par + 4 * q, ap.param + a + 4 * q);
-                cp_async_16(s_par + T + 4 * q, ap.vel + a + 4 * q);
-            }
-        }
-        if (ADD) {
-            if (span == T && aligned) for (uint32_t q = lane; q < T / 4; q += 32) cp_async_16(s_tile + 4 * q, out + a + 4 * q);
-            else for (uint32_t q = lane; q < span; q += 32) cp_async_4(s_tile + q, out + a + q);
-        }
-    };
     if (top) top_up(s_cur[0][my_w]);
-    fetch(t0);
-    if (!ADD)
-        for (uint32_t q = lane; q < T / 4; q += 32) reinterpret_cast<float4*>(s_tile)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
 
     uint32_t top_step = 1;                                 // largest power of two <= RS
     while (2u * top_step <= RS) top_step *= 2u;
@@ -250,27 +252,28 @@ k_decode_rings(const __grid_constant__ DecodeLists ls, uint32_t W, uint32_t cnt,
         // the sub-tile leaves; its words are zero again
         const uint32_t n_out = a < total_n ? min(T, total_n - a) : 0u;
         if (APPLY) {
-            if (n_out == T) {
+            // (the sub-tile at the buffer's end as well: its loads one after the other from global memory took
+            //  longer than all the rest of a 1.5M-element call)
 #pragma unroll 2
-                for (uint32_t q = lane; q < T / 4; q += 32) {
-                    float4 vv = reinterpret_cast<const float4*>(s_par + T)[q];
-                    float4 pp = reinterpret_cast<const float4*>(s_par)[q];
-                    const float4 gs = reinterpret_cast<const float4*>(s_tile)[q];
-                    reinterpret_cast<float4*>(s_tile)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    vv.x = __fadd_rn(__fmul_rn(ap.mu, vv.x), __fmul_rn(ap.scale, gs.x));
-                    vv.y = __fadd_rn(__fmul_rn(ap.mu, vv.y), __fmul_rn(ap.scale, gs.y));
-                    vv.z = __fadd_rn(__fmul_rn(ap.mu, vv.z), __fmul_rn(ap.scale, gs.z));
-                    vv.w = __fadd_rn(__fmul_rn(ap.mu, vv.w), __fmul_rn(ap.scale, gs.w));
-                    pp.x = __fsub_rn(pp.x, __fmul_rn(ap.lr, vv.x)); pp.y = __fsub_rn(pp.y, __fmul_rn(ap.lr, vv.y));
-                    pp.z = __fsub_rn(pp.z, __fmul_rn(ap.lr, vv.z)); pp.w = __fsub_rn(pp.w, __fmul_rn(ap.lr, vv.w));
+            for (uint32_t q = lane; 4 * q < n_out; q += 32) {
+                float4 vv = reinterpret_cast<const float4*>(s_par + T)[q];
+                float4 pp = reinterpret_cast<const float4*>(s_par)[q];
+                const float4 gs = reinterpret_cast<const float4*>(s_tile)[q];
+                reinterpret_cast<float4*>(s_tile)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+                vv.x = __fadd_rn(__fmul_rn(ap.mu, vv.x), __fmul_rn(ap.scale, gs.x));
+                vv.y = __fadd_rn(__fmul_rn(ap.mu, vv.y), __fmul_rn(ap.scale, gs.y));
+                vv.z = __fadd_rn(__fmul_rn(ap.mu, vv.z), __fmul_rn(ap.scale, gs.z));
+                vv.w = __fadd_rn(__fmul_rn(ap.mu, vv.w), __fmul_rn(ap.scale, gs.w));
+                pp.x = __fsub_rn(pp.x, __fmul_rn(ap.lr, vv.x)); pp.y = __fsub_rn(pp.y, __fmul_rn(ap.lr, vv.y));
+                pp.z = __fsub_rn(pp.z, __fmul_rn(ap.lr, vv.z)); pp.w = __fsub_rn(pp.w, __fmul_rn(ap.lr, vv.w));
+                if (4 * q + 4u <= n_out) {
                     __stcs(reinterpret_cast<float4*>(ap.vel + a) + q, vv);
                     __stcs(reinterpret_cast<float4*>(ap.param + a) + q, pp);
-                }
-            } else {
-                for (uint32_t q = lane; q < n_out; q += 32) {
-                    const float vn = __fadd_rn(__fmul_rn(ap.mu, ap.vel[a + q]), __fmul_rn(ap.scale, s_tile[q]));
-                    ap.vel[a + q] = vn;
-                    ap.param[a + q] = __fsub_rn(ap.param[a + q], __fmul_rn(ap.lr, vn));
+                } else {
+                    const float ve[3] = {vv.x, vv.y, vv.z}, pe[3] = {pp.x, pp.y, pp.z};
+#pragma unroll
+                    for (uint32_t e = 0; e < 3u; ++e)
+                        if (4 * q + e < n_out) { ap.vel[a + 4 * q + e] = ve[e]; ap.param[a + 4 * q + e] = pe[e]; }
                 }
             }
         } else if (n_out == T && aligned) {

@@ -51,3 +51,25 @@ def test_ring_decode_matches_the_oracle(n, W, density, offset):
     assert np.array_equal(to_np_u32(d_p), bits(p0)) and np.array_equal(to_np_u32(d_v), bits(v0))
     st, det = plan.last_status(ws)
     assert st == api.GC_OK, (st, det)
+
+
+@pytest.mark.parametrize("n", [2, 131, 1026, 700_003, 3_000_002])
+@pytest.mark.parametrize("W", [1, 40])
+def test_momentum_at_the_buffers_end(n, W):
+    """The last sub-tile takes the optimizer step like the others, and nothing behind the buffer is written;
+    the longer buffers give every CTA one or a few even tiles."""
+    plan = api.Plan([n], 0.004, device=0)
+    ws = plan.alloc_workspace()
+    k = plan.total_cap
+    pairs = [synth.sparse_set([n], [k], 40 + w) for w in range(W)]
+    d_idx = [torch.from_numpy(i.view(np.int32)).cuda() for i, _ in pairs]
+    d_val = [torch.from_numpy(v).cuda() for _, v in pairs]
+    p0 = np.random.default_rng(n).standard_normal(n).astype(np.float32)
+    v0 = (p0 * np.float32(0.1)).astype(np.float32)
+    d_p, d_v = (torch.full((n + 8,), 7.0, device="cuda") for _ in range(2))
+    d_p[:n].copy_(torch.from_numpy(p0)); d_v[:n].copy_(torch.from_numpy(v0))
+    plan.decompress_apply_momentum(d_idx, d_val, None, d_p[:n], d_v[:n], 0.05, 0.9, 0.25, ws)
+    oracle.decode_apply_momentum(pairs, p0, v0, 0.05, 0.9, 0.25)
+    assert np.array_equal(to_np_u32(d_p[:n]), bits(p0)) and np.array_equal(to_np_u32(d_v[:n]), bits(v0))
+    assert bool((d_p[n:] == 7.0).all()) and bool((d_v[n:] == 7.0).all())
+    assert plan.last_status(ws)[0] == api.GC_OK
