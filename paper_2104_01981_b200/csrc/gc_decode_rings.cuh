@@ -195,10 +195,17 @@ k_decode_rings(const __grid_constant__ DecodeLists ls, uint32_t W, uint32_t cnt,
                 if (m0 <= have[u] && ring[wrap(slot[u] + m0 - 1u)] < k0) b0 = m0;
                 if (m1 <= have[u] && ring[wrap(slot[u] + m1 - 1u)] < k1) b1 = m1;
             }
+            // (an ascending list has nothing in front of the first sub-tile's range; what another list has
+            //  there is looked at all the same, so that no entry goes by unreported)
+            if (warp == 0) b0 = 0u;
             const uint32_t n = b1 > b0 ? b1 - b0 : 0u;
             s_rng[w] = make_uint2(wrap(slot[u] + b0), n);
             longest = max(longest, n);
-            if (warp == kW8 - 1 && w < W) { s_cur[par ^ 1u][w] = cur[u] + b1; s_slot[par ^ 1u][w] = wrap(slot[u] + b1); }      // (k1 = the bound)
+            if (warp == kW8 - 1 && w < W) {                // (k1 = the bound)
+                s_cur[par ^ 1u][w] = cur[u] + b1; s_slot[par ^ 1u][w] = wrap(slot[u] + b1);
+                // two entries that changed places across the bound: the next CTA's search may step over both
+                disorder = disorder || (b1 + 1u < have[u] && ring[wrap(slot[u] + b1 + 1u)] < bound);
+            }
         }
         const bool small = __reduce_max_sync(0xFFFFFFFFu, longest) <= 32u;
         __syncwarp();

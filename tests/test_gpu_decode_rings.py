@@ -73,3 +73,39 @@ def test_momentum_at_the_buffers_end(n, W):
     assert np.array_equal(to_np_u32(d_p[:n]), bits(p0)) and np.array_equal(to_np_u32(d_v[:n]), bits(v0))
     assert bool((d_p[n:] == 7.0).all()) and bool((d_v[n:] == 7.0).all())
     assert plan.last_status(ws)[0] == api.GC_OK
+
+
+@pytest.mark.parametrize("n,density,every", [(300_000, 0.01, 128), (8_000_000, 0.001, 2048)])
+@pytest.mark.parametrize("fused", [False, True], ids=["decode", "momentum"])
+def test_neighbours_out_of_order_are_reported_or_added(n, density, every, fused):
+    """Two neighbouring entries change places across a multiple of `every` (sub-tiles, tiles and the runs of
+    the CTAs begin at such places): either both are added all the same, or GC_E_INVALID is recorded."""
+    plan = api.Plan([n], density, device=0)
+    plan.set_option(api.GC_OPT_DECODE_ROUTE, api.GC_DECODE_WIDE)
+    ws = plan.alloc_workspace()
+    host, val = synth.sparse_set([n], [plan.total_cap], 5)
+    idx, val = torch.from_numpy(host.view(np.int32)).cuda(), torch.from_numpy(val).cuda()
+    outs = [torch.zeros(n, device="cuda") for _ in range(2)]
+
+    def call():
+        if not fused:
+            plan.decompress_accumulate([idx], [val], None, outs[0], True, ws)
+            return outs[0]
+        for o in outs:
+            o.zero_()
+        plan.decompress_apply_momentum([idx], [val], None, outs[1], outs[0], 1.0, 0.0, 1.0, ws)
+        return outs[0]                                     # the velocity: momentum 0, so the sum itself
+
+    want = call().clone()
+    assert plan.last_status(ws)[0] == api.GC_OK
+    lost = []
+    for p in np.nonzero(np.diff(host // every))[0]:
+        for t in (idx, val):
+            t[p:p + 2] = t[p:p + 2].flip(0)
+        ws[:256].zero_()
+        same = torch.equal(call(), want)
+        if plan.last_status(ws)[0] != api.GC_E_INVALID and not same:
+            lost.append(int(host[p]))
+        for t in (idx, val):
+            t[p:p + 2] = t[p:p + 2].flip(0)
+    assert not lost, lost
