@@ -173,14 +173,13 @@ k_decode_rings(const __grid_constant__ DecodeLists ls, uint32_t W, uint32_t cnt,
             if (w < W) {
                 const uint32_t fill = s_fill[w];
                 cur[u] = s_cur[par][w]; slot[u] = s_slot[par][w]; have[u] = fill - cur[u];
-                if (fill < s_len[w]) bound = min(bound, rings[2u * w * RS + wrap(slot[u] + have[u] - 1u)] + 1u);
+                // (a ring that ends below this step, or with an index no buffer has, belongs to a list that is
+                //  not ascending: it must not hold up the others)
+                const uint32_t end = fill < s_len[w] ? rings[2u * w * RS + wrap(slot[u] + have[u] - 1u)] : hi;
+                if (end >= sub_lo && end < hi) bound = min(bound, end + 1u);
             }
         }
-        bound = __reduce_min_sync(0xFFFFFFFFu, bound);
-        if (bound <= sub_lo) {                             // no progress: a list is not ascending
-            disorder = true;
-            bound = hi;
-        }
+        bound = __reduce_min_sync(0xFFFFFFFFu, bound);     // (above sub_lo: every step makes progress)
         // this warp's range of every ring
         const uint32_t a = lo + warp * T;
         const uint32_t k0 = min(max(a, sub_lo), bound), k1 = min(max(a + T, sub_lo), bound), span = k1 - k0;

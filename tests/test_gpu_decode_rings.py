@@ -109,3 +109,32 @@ def test_neighbours_out_of_order_are_reported_or_added(n, density, every, fused)
         for t in (idx, val):
             t[p:p + 2] = t[p:p + 2].flip(0)
     assert not lost, lost
+
+
+@pytest.mark.parametrize("bad", [400_000, 0xFFFFFFFF], ids=["one_beyond", "largest_word"])
+@pytest.mark.parametrize("fused", [False, True], ids=["decode", "momentum"])
+def test_a_list_with_invalid_entries_does_not_cost_the_others_theirs(bad, fused):
+    """The second half of one list is filled with an index beyond the buffer; the other lists crowd into a few
+    places, so that their rings end inside a tile.  The bad entries are skipped and reported, everything else
+    is added."""
+    n, k = 400_000, 4000
+    plan = api.Plan([n], k / n, device=0)
+    plan.set_option(api.GC_OPT_DECODE_ROUTE, api.GC_DECODE_WIDE)
+    assert plan.total_cap == k
+    ws = plan.alloc_workspace()
+    rng = np.random.default_rng(3)
+    crowd = np.concatenate([np.arange(a, a + 1000, dtype=np.uint32) for a in (20_000, 150_000, 200_500, 390_000)])
+    spread = np.sort(rng.choice(n // 2, k // 2, replace=False)).astype(np.uint32) + np.uint32(1)
+    lists = [crowd, np.concatenate([spread, np.full(k // 2, bad, np.uint32)]), crowd + np.uint32(7)]
+    vals = [rng.standard_normal(k).astype(np.float32) for _ in lists]
+    pairs = [(i[:k // 2] if w == 1 else i, v[:k // 2] if w == 1 else v) for w, (i, v) in enumerate(zip(lists, vals))]
+    d_idx = [torch.from_numpy(i.view(np.int32)).cuda() for i in lists]
+    d_val = [torch.from_numpy(v).cuda() for v in vals]
+    want = oracle.decode_accumulate(pairs, np.zeros(n, np.float32), True)
+    out, other = torch.zeros(n, device="cuda"), torch.zeros(n, device="cuda")
+    if fused:
+        plan.decompress_apply_momentum(d_idx, d_val, None, other, out, 1.0, 0.0, 1.0, ws)       # the velocity: the sum
+    else:
+        plan.decompress_accumulate(d_idx, d_val, None, out, True, ws)
+    assert plan.last_status(ws)[0] == api.GC_E_INVALID
+    assert np.array_equal(to_np_u32(out), bits(want))
