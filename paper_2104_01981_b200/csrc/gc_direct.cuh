@@ -73,9 +73,10 @@ struct DirectSmem {
     int ok;
 };
 
-// Rank `k` (1 = largest) in a histogram of NB bins: the bin, the count above it and in it.
+// Rank `k` (1 = largest) in a histogram of NB bins: the bin, the count above it and in it.  Returns the number
+// of entries in the histogram.
 template <int NB, bool IN_SMEM = false>
-__device__ __forceinline__ void direct_select(DirectSmem& sm, const uint32_t* hist, uint32_t k, int tid, int lane, int warp) {
+__device__ __forceinline__ uint32_t direct_select(DirectSmem& sm, const uint32_t* hist, uint32_t k, int tid, int lane, int warp) {
     constexpr int PER = NB / kBlock;
     uint32_t c[PER], sum = 0;
 #pragma unroll
@@ -88,9 +89,9 @@ __device__ __forceinline__ void direct_select(DirectSmem& sm, const uint32_t* hi
     const uint32_t inc = warp_incl_scan(sum, lane);
     if (lane == 31) sm.wsum[warp] = inc;
     __syncthreads();
-    uint32_t above = 0;                                    // entries in higher bins than this thread's
+    uint32_t above = 0, total = 0;                         // entries in higher bins than this thread's, in all
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) above += w >= warp ? sm.wsum[w] : 0u;
+    for (int w = 0; w < kWarps; ++w) { above += w >= warp ? sm.wsum[w] : 0u; total += sm.wsum[w]; }
     above -= inc;
 #pragma unroll
     for (int q = PER - 1; q >= 0; --q) {
@@ -98,6 +99,7 @@ __device__ __forceinline__ void direct_select(DirectSmem& sm, const uint32_t* hi
         above += c[q];
     }
     __syncthreads();
+    return total;
 }
 
 // RES: the share of a CTA stays in (dynamic) shared memory; otherwise it is read back from r.
@@ -206,8 +208,16 @@ k_topk_direct(const __grid_constant__ DirectArgs a) {
     uint32_t prefix = 0, krem = 0, T = 0, m_eq = 0, gt_before = 0, eq_before = 0;
     if (live) {
         phase_stamp(hdr, n_stamp);
+        if (b == 0 && tid == 0) hdr->clean_mark = 0ull;    // (every CTA has read it)
         // ------------------------------------------------------------ next 10 bits
-        direct_select<2048>(sm, a.s->hist0, a.k, tid, lane, warp);
+        // Somebody else's counts in the scratch: nothing is sent (the residual keeps g + r), the scratch is
+        // cleaned on the way out.  Every CTA sees the same sum.
+        if (direct_select<2048>(sm, a.s->hist0, a.k, tid, lane, warp) != a.n) {
+            if (b == 0 && tid == 0) { record_status(hdr, -1 /*GC_E_INVALID*/, 0xC1EA0001ull); atomicExch(&hdr->abort, 1u); }
+            live = false;
+        }
+    }
+    if (live) {
         prefix = sm.bin; krem = a.k - sm.above;
         for_keys([&](uint32_t key, uint32_t, float) { if ((key >> 20) == prefix) atomicAdd(&sm.hist[(key >> 10) & 1023u], 1u); });
         flush(a.s->hist1, 1024);
@@ -298,8 +308,8 @@ k_topk_direct(const __grid_constant__ DirectArgs a) {
         unsigned long long at = 0;
         for (int w = 0; w < kWarps; ++w) { at += sm.part[w]; if (w < warp) at += (unsigned long long)sm.weq[w] << 32 | sm.wgt[w]; }
         uint32_t gt_at = (uint32_t)at, eq_at = (uint32_t)(at >> 32);
-        const uint32_t lt = (1u << lane) - 1u;
-        if ((sm.wgt[warp] | sm.weq[warp]) != 0u) {
+        const uint32_t lt = (1u << lane) - 1u, gt_end = gt_at + sm.wgt[warp], eq_end = eq_at + sm.weq[warp];
+        if (gt_at != gt_end || eq_at != eq_end) {
             for (uint32_t q0 = w0; q0 < w1; q0 += 32u) {
                 const uint32_t q = q0 + lane;
                 const float4 x = q < w1 ? value(q) : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -327,19 +337,28 @@ k_topk_direct(const __grid_constant__ DirectArgs a) {
                     const bool sent = ((gm >> e) & 1u) || (((em >> e) & 1u) && ee < m_eq);
                     if (sent) {
                         const uint32_t slot = ge + min(ee, m_eq), i = 4u * (v0 + q) + e;
-                        a.out_idx[slot] = i;
-                        a.out_val[slot] = xe[e];
-                        a.r[i] = 0.0f;
+                        if (slot < a.k) {
+                            a.out_idx[slot] = i;
+                            a.out_val[slot] = xe[e];
+                            a.r[i] = 0.0f;
+                        } else {
+                            record_status(hdr, -1 /*GC_E_INVALID*/, i);
+                        }
                     }
                 }
                 gt_at += gall; eq_at += eall;
             }
         }
+        // (counted and emitted entries agree and add up to k, unless others wrote to the scratch)
+        if (lane == 0 && (gt_at != gt_end || eq_at != eq_end ||
+                          (b == G - 1u && warp == kWarps - 1 && gt_at + min(eq_at, m_eq) != a.k)))
+            record_status(hdr, -1 /*GC_E_INVALID*/, 0xC1EA0002ull);
         if (a.out_count != nullptr && b == 0 && tid == 0) { a.out_count[0] = a.k; a.out_count[1] = a.k; }
         phase_stamp(hdr, n_stamp);
     }
     // The CTA that leaves last resets what the others may still have been reading; after a wait that ran
-    // out it cleans everything (and sets no mark).
+    // out, or counts that do not add up, it cleans everything and sets no mark (the next call on a private
+    // workspace ends with GC_E_INVALID until the status has been read, see CleanArgs).
     __syncthreads();
     if (tid == 0) {
         __threadfence();

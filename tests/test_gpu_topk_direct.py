@@ -71,3 +71,33 @@ def test_bfloat16_and_a_private_workspace():
         assert np.array_equal(to_np_u32(r), bits(r_cpu))
     assert plan.launches() - before == 5                  # one clearing launch, then one launch per call
     assert plan.last_status(ws) == (api.GC_OK, 0)
+
+
+# word ranges of the scratch behind its header: the three histograms, the length of the list
+@pytest.mark.parametrize("words,value", [((64, 64 + 2048), 40), ((64 + 2047, 64 + 2048), 1), ((64, 65), 1 << 20),
+                                         ((2112, 2112 + 1024), 500), ((4160, 4161), 40), ((4160, 4161), 1 << 30)])
+def test_scratch_that_others_wrote_to_is_reported_and_writes_stay_in_bounds(words, value):
+    """A private workspace in which somebody raised counts and left the header's mark alone: the call ends with
+    GC_E_INVALID, nothing is written behind the k entries, and after the status has been read the next call is
+    exact again."""
+    n, k, slack = 1_000_003, 10_001, 4096
+    plan = api.Plan([n], 0.01, device=0)
+    plan.set_option(api.GC_OPT_WORKSPACE_PRIVATE, 1)
+    assert plan.total_cap == k
+    ws = plan.alloc_workspace()
+    idx = torch.full((k + slack,), -7, dtype=torch.int32, device="cuda")
+    val = torch.full((k + slack,), -7.0, device="cuda")
+    gen = torch.Generator(device="cuda").manual_seed(value & 0xFFFF)
+    r = torch.zeros(n, device="cuda")
+    for step in range(3):
+        g = torch.randn(n, device="cuda", generator=gen)
+        if step == 1:
+            ws.view(torch.int32)[words[0]:words[1]] += value
+        r_cpu = r.cpu().numpy().copy()
+        plan.compress(g, r, idx, val, None, ws)
+        assert plan.last_status(ws)[0] == (api.GC_E_INVALID if step == 1 else api.GC_OK)
+        assert bool((idx[k:] == -7).all()) and bool((val[k:] == -7.0).all())
+        if step != 1:
+            oi, ov = oracle.topk_compress_tensors([n], [k], g.cpu().numpy(), r_cpu)
+            assert np.array_equal(to_np_u32(idx[:k]), oi) and np.array_equal(to_np_u32(val[:k]), bits(ov))
+            assert np.array_equal(to_np_u32(r), bits(r_cpu))
