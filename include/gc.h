@@ -383,15 +383,18 @@ const char *gc_kernel_name(int kernel_id);
  *                   same output order and same residual rule as gc_compress in top-k mode.
  *                   k = 0 sends nothing and still folds: the residual becomes g + r
  *   out_idx/out_val device, uint32/fp32[k] (may be NULL when k = 0)
- *   device_status   device int32 or NULL: receives GC_OK or GC_E_TIMEOUT when the work is done
- *                   (on every path that returns GC_OK, n = 0 and k = 0 included)
+ *   device_status   device int32 or NULL: receives GC_OK, GC_E_TIMEOUT or GC_E_INVALID (counts in the
+ *                   scratch that do not add up, see below) when the work is done (on every path that
+ *                   returns GC_OK, n = 0 and k = 0 included)
  *   stream          cudaStream_t; the call is asynchronous
  * The current device is used.  The first call on each device resolves the device address of
  * the array (cudaGetSymbolAddress) and sets the kernel's shared-memory limit; make that first call
- * outside any stream capture.  One cooperative launch per call.  All calls on a device share the one
- * array: each call leaves it as it found it, so back-to-back calls on one stream are fine, but two calls
- * whose kernels can overlap on the GPU (different streams, different threads) race on it -- serialise
- * them.
+ * outside any stream capture.  One cooperative launch per call, of up to two (beyond 7.2M elements
+ * three) CTAs per SM; it starts when its whole grid fits beside what other streams run.  All calls on
+ * a device share the one array: back-to-back calls on one stream are fine, but two calls whose kernels
+ * can overlap on the GPU (different streams, different threads) race on it -- serialise them.  If two
+ * do overlap, their results are undefined (GC_E_INVALID or GC_E_TIMEOUT is likely, writes stay within
+ * the given arrays); each call starts from a scratch it has cleared, so the next one is exact again.
  * Calls no cudaMalloc/cudaFree and no allocating library routine.
  */
 #define GC_NOALLOC_MAX_N (1u << 24)

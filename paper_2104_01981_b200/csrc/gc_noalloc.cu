@@ -14,9 +14,8 @@ constexpr uint32_t kMaxN = GC_NOALLOC_MAX_N;
 static_assert(sizeof(DirectScratch) == 29184, "the documented size of the fixed scratch (about 29 KB)");
 
 // The scratch itself.  Every GPU that loads this library carries these 29,184 bytes until the
-// process exits; they start at zero and every launch leaves them as it found them.  In host code this
-// name is only a handle for cudaGetSymbolAddress; it is not a device address and must never be handed
-// to a kernel directly.
+// process exits; every launch clears what it needs of them.  In host code this name is only a handle
+// for cudaGetSymbolAddress; it is not a device address and must never be handed to a kernel directly.
 static __device__ __align__(256) DirectScratch g_noalloc_scratch;
 
 struct PerDevice {
@@ -92,6 +91,9 @@ extern "C" int gc_compress_noalloc(const float* grad, float* residual, uint32_t 
     da.g = grad; da.r = residual; da.n = n; da.k = k; da.out_idx = out_idx; da.out_val = out_val;
     da.status_out = device_status; da.s = pd.scratch;
     const DirectGeom dg = direct_geometry(n, pd.sms);
+    // The kernel leaves the scratch clean, but no caller can replace this array: what two calls that
+    // overlapped against the rules left in it must not outlive them.
+    da.clear_first = 1u;
     void* args[] = {&da};
     const void* fn = dg.resident ? (const void*)k_topk_direct<GradF32, true> : (const void*)k_topk_direct<GradF32, false>;
     if (cudaLaunchCooperativeKernel(fn, dim3(dg.G), dim3(kBlock), args, dg.smem, s) != cudaSuccess) {

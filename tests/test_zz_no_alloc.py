@@ -9,6 +9,8 @@ meets the first call's leftovers in the shared array -- and to what the oracle g
 file name keeps it last in collection order, so a failure here cannot hide the other tests
 from a stop-at-first run.
 """
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -156,3 +158,47 @@ def test_sizes_beyond_the_fixed_scratch_are_refused():
     assert api.compress_noalloc(g, g.clone(), 8, 9, i, g.clone()) == api.GC_E_INVALID
     assert api.compress_noalloc(g, g.clone(), 0, 0, i, g.clone()) == api.GC_OK
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("fill", [0x5A, 0xFF])
+def test_whatever_is_left_in_the_scratch_does_not_reach_the_next_call(fill):
+    """No caller can replace the library's array, so a call has to start from a cleared one whatever is in it
+    (two calls that overlapped, say).  A captured call tells where the array is: the kernel's argument block
+    begins with the caller's pointers and sizes, and the array's address follows them."""
+    from cuda.bindings import driver, runtime
+
+    class Args(ctypes.Structure):
+        _fields_ = [("grad", ctypes.c_uint64), ("residual", ctypes.c_uint64), ("n", ctypes.c_uint32), ("k", ctypes.c_uint32),
+                    ("out_idx", ctypes.c_uint64), ("out_val", ctypes.c_uint64), ("out_count", ctypes.c_uint64),
+                    ("status", ctypes.c_uint64), ("scratch", ctypes.c_uint64)]
+
+    torch.cuda.set_device(0)
+    n, k = 300_007, 3001
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    r = torch.zeros(n, device="cuda")
+    idx, val = torch.zeros(k, dtype=torch.int32, device="cuda"), torch.zeros(k, device="cuda")
+    status = torch.full((1,), 77, dtype=torch.int32, device="cuda")
+    g = torch.randn(n, device="cuda", generator=gen)
+    assert api.compress_noalloc(g, r, n, k, idx, val, status) == api.GC_OK      # set-up happens here
+    torch.cuda.synchronize()
+    graph, side = torch.cuda.CUDAGraph(keep_graph=True), torch.cuda.Stream()
+    with torch.cuda.graph(graph, stream=side):
+        assert api.compress_noalloc(g, r, n, k, idx, val, status, side) == api.GC_OK
+    err, nodes, count = driver.cuGraphGetRootNodes(driver.CUgraph(graph.raw_cuda_graph()), 1)
+    assert err == driver.CUresult.CUDA_SUCCESS and count == 1
+    err, params = driver.cuGraphKernelNodeGetParams(nodes[0])
+    assert err == driver.CUresult.CUDA_SUCCESS
+    a = ctypes.cast(ctypes.cast(int(params.kernelParams), ctypes.POINTER(ctypes.c_void_p))[0], ctypes.POINTER(Args))[0]
+    assert (a.grad, a.residual, a.n, a.k) == (g.data_ptr(), r.data_ptr(), n, k)
+    assert (a.out_idx, a.out_val, a.out_count, a.status) == (idx.data_ptr(), val.data_ptr(), 0, status.data_ptr())
+    address, length = a.scratch, 29_184
+    for _ in range(2):
+        g = torch.randn(n, device="cuda", generator=gen)
+        o_idx, o_val, o_r = oracle_compress(n, k, g, r)
+        torch.cuda.synchronize()
+        assert runtime.cudaMemset(address, fill, length)[0] == runtime.cudaError_t.cudaSuccess
+        torch.cuda.synchronize()
+        assert api.compress_noalloc(g, r, n, k, idx, val, status) == api.GC_OK
+        torch.cuda.synchronize()
+        assert status.item() == api.GC_OK
+        assert np.array_equal(u32(idx), o_idx) and np.array_equal(u32(val), o_val) and np.array_equal(u32(r), o_r)
