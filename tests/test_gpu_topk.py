@@ -321,6 +321,34 @@ def test_which_plans_take_which_route():
     assert api.Plan([100], 0.1, device=-1).query(api.GC_Q_COMPRESS_ROUTE) == api.GC_ROUTE_NONE
 
 
+@pytest.mark.parametrize("density", [0.001, 0.002, 0.0021])
+@pytest.mark.parametrize("n", [413_433_856, 413_433_857, 560_000_000])
+def test_large_sparse_one_tensor_plans_stay_on_the_one_tensor_kernel(n, density):
+    """On both sides of the most tiles that two CTAs per SM may own (and of the density up to which there are
+    two): the route that bfloat16 gradients need."""
+    assert api.Plan([n], density, device=0).query(api.GC_Q_COMPRESS_ROUTE) == api.GC_ROUTE_TOPK_ONE
+
+
+def test_large_sparse_bfloat16_gradient():
+    """A bfloat16 gradient of 414M elements at 0.1 %, on a residual with few ties, against torch.topk."""
+    n = 414_000_000
+    plan = api.Plan([n], 0.001, device=0)
+    k, ws = plan.total_cap, plan.alloc_workspace()
+    idx, val, cnt = plan.alloc_outputs()
+    gen = torch.Generator(device="cuda").manual_seed(6)
+    g = torch.empty(n, dtype=torch.bfloat16, device="cuda").normal_(generator=gen)
+    r = torch.empty(n, device="cuda").normal_(generator=gen)
+    a = r + g.float()
+    plan.compress_bf16(g, r, idx, val, cnt, ws)
+    assert plan.last_status(ws)[0] == api.GC_OK and plan.last_counters(ws)[1:] == (0, 0)
+    i = idx.to(torch.int64)
+    assert bool((i[1:] > i[:-1]).all()) and torch.equal(val, a[i]) and not r[i].any()
+    cut = a.abs().topk(k, sorted=False).values.min()
+    assert bool((val.abs() >= cut).all())
+    r[i] = val
+    assert torch.equal(r, a)
+
+
 @pytest.mark.parametrize("options", [{}, {api.GC_OPT_SAMPLE_RANK_PERMILLE: 30}, {api.GC_OPT_CANDIDATE_CAPACITY: 4}],
                          ids=["plain", "starved", "overflow"])
 def test_private_workspace_skips_the_clearing_launch_and_stays_exact(options):
