@@ -344,11 +344,11 @@ void plan_single(gc_plan_s* p) {
         // Small tensors are all latency (a CTA has a handful of tiles and five phases to walk through):
         // there two CTAs per SM get through the phases sooner than three (2M-10M elements: 31-49 us
         // against 37-51 us).  From about 12M elements on the third CTA pays for itself, except on sparse
-        // plans (see VOTES); below 300 tiles there is a CTA per tile anyway (fewer were no faster).
-        // Sparse plans of more tiles than two CTAs per SM may own (413M elements) keep the third: 420M at
-        // 0.1 % 836 us against 1103 us on the general kernel, which reads no bfloat16 gradient at all.
+        // plans of fp32 gradients (see VOTES); below 300 tiles there is a CTA per tile anyway (fewer were
+        // no faster).  Sparse plans of more tiles than two CTAs per SM may own (413M elements) keep the
+        // third: 420M at 0.1 % 836 us against 1103 us on the general kernel, which reads no bfloat16 at all.
         const uint32_t two = 2u * (uint32_t)p->sm_count;
-        if (d.ntiles <= 3000u || (p->density <= kSparseUpTo && d.ntiles <= two * (uint32_t)kSingleMaxT)) g.G = std::min(g.G, two);
+        if (d.ntiles <= 3000u || (bf16 == 0 && p->density <= kSparseUpTo && d.ntiles <= two * (uint32_t)kSingleMaxT)) g.G = std::min(g.G, two);
         g.maxt = (d.ntiles + g.G - 1) / g.G;
         g.rows = make_row_map(p, d.ntiles, g.G, g.maxt, g.votes ? 0.0 : p->density >= 0.005 ? kSingleSkew : kSingleSkewSparse);
         if (g.maxt > kSingleMaxT || g.G > 640) return;               // chunk records and totals must stay small

@@ -387,8 +387,9 @@ __device__ __forceinline__ bool fold_tail_votes(BlockSmem& sm, const float (&av)
 // VOTES: how the fold ranks a chunk's candidates -- votes, the residual stored first, chunks without
 // candidates left early, equal shares -- or the shuffle scan.  The votes are a fifth fewer instructions,
 // which pays where instructions bound the loop (bfloat16, 110M elements at 1 %: 241 -> 224 us) and where
-// most chunks are empty (up to 0.2 %; with two CTAs per SM, since a loop that hardly waits for itself keeps
-// the memory busier than it likes with three: 110M elements at 0.1 % 252 -> 231 us, 355M 710 -> 680 us).
+// most chunks are empty (fp32 up to 0.2 %, with two CTAs per SM, since a loop that hardly waits for itself
+// keeps the memory busier than it likes with three: 110M elements at 0.1 % 252 -> 231 us, 355M 710 -> 680 us;
+// bfloat16 at five sixths of the bytes wants the third: 0.2 % 227 -> 208 us and 655 -> 598 us).
 // Between, fp32 is bound by memory and the slower loop with unequal shares does better (0.5 %: 245 against
 // 249-254 us; 355M at 0.3 %: 697 against 714).
 // DENSE (plans of 2 % and more) has the emission by chunk, the bfloat16 form the counted band: the other
