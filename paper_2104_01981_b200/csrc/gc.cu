@@ -637,15 +637,19 @@ static bool ask_device(int device, DeviceFacts* p) {
         }
         p->grid_thr_multi_max = 0;
         if (coop) {
-            int nb = 0;
+            int nb = 1 << 20;
             p->thrm_smem_max = kMultiMaxPer * kMultiRowBytes + 8 * kMultiMaxTab;
-            int nbw = 0;          // (the several-workers form of the kernel must be as resident as the kernel itself)
-            if (allow_smem({(const void*)k_threshold_multi, (const void*)k_threshold_workers}, p->thrm_smem_max) &&
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_threshold_multi, kBlock, p->thrm_smem_max) ==
-                    cudaSuccess && nb >= 1 &&
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nbw, k_threshold_workers, kBlock, p->thrm_smem_max) ==
-                    cudaSuccess && nbw >= 1)
-                p->grid_thr_multi_max = p->sm_count * std::min(nb, nbw);
+            // (the form that fits least counts)
+            const std::initializer_list<const void*> forms = {(const void*)k_threshold_multi<false>, (const void*)k_threshold_multi<true>,
+                                                              (const void*)k_threshold_workers<false>, (const void*)k_threshold_workers<true>};
+            if (!allow_smem(forms, p->thrm_smem_max)) nb = 0;
+            for (const void* fn : forms) {
+                int n1 = 0;
+                if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n1, fn, kBlock, p->thrm_smem_max) != cudaSuccess) n1 = 0;
+                nb = std::min(nb, n1);
+            }
+            if (nb >= 1)
+                p->grid_thr_multi_max = p->sm_count * nb;
             else
                 (void)cudaGetLastError();
         }
@@ -988,6 +992,9 @@ static MultiArgs multi_args(const gc_plan_s* p, const MultiGeom& mg, const void*
     return ma;
 }
 
+// Which form of the many-tensor threshold kernel a plan takes.
+static bool thr_list(const gc_plan_s* p) { return p->density < kThrListBelow; }
+
 // Argument block of the many-tensor threshold kernel for one worker's buffers and a given geometry.
 static ThrMultiArgs thr_multi_args(const gc_plan_s* p, const MultiGeom& mg, const float* grad, float* residual,
                                    uint32_t* out_idx, float* out_val, uint32_t* out_count, void* workspace) {
@@ -1076,7 +1083,7 @@ static int compress_impl(gc_plan_t* p, const void* grad_any, bool bf16, float* r
         ThrMultiArgs ta = thr_multi_args(p, mg, grad, residual, out_idx, out_val, out_count, workspace);
         void* args[] = {&ta};
         Timed tm(p, s, GC_K_FUSED);
-        GC_CUDA(p, cudaLaunchCooperativeKernel((const void*)k_threshold_multi, dim3(p->thrm_grid), dim3(kBlock),
+        GC_CUDA(p, cudaLaunchCooperativeKernel(thr_list(p) ? (const void*)k_threshold_multi<true> : (const void*)k_threshold_multi<false>, dim3(p->thrm_grid), dim3(kBlock),
                                                args, p->thrm_smem, s));
         return GC_OK;
     }
@@ -1349,7 +1356,7 @@ int gc_compress_workers(gc_plan_t* p, uint32_t W, const float* const* grads, flo
         void* args[] = {topk_multi ? (void*)&wa : (void*)&ta};
         Timed tm(p, s, GC_K_FUSED);
         GC_CUDA(p, cudaLaunchCooperativeKernel(topk_multi ? (p->density >= kDenseFrom ? (const void*)k_topk_workers<GradF32, true> : (const void*)k_topk_workers<GradF32, false>)
-                                                          : (const void*)k_threshold_workers,
+                                                          : thr_list(p) ? (const void*)k_threshold_workers<true> : (const void*)k_threshold_workers<false>,
                                                dim3(mg.G * wn), dim3(kBlock), args, mg.smem, s));
     }
     return GC_OK;

@@ -210,8 +210,14 @@ static __device__ __noinline__ void small_threshold_body(BlockSmem& sm, const Te
     __syncthreads();
 }
 
+// LIST pays where few keys share the coarse bin; where they are many the walk over memory is the shorter way,
+// and it takes 2 us longer in a form that holds the list's code as well.  0.1 %: 161 tensors 98.9 us without, 98.1
+// with it, eight workers 504 and 501, a dozen tensors (4M elements) 44.4 and 42.8; 0.3 %: the same dozen 45.4 and
+// 45.5, with 1M elements 41.9 both; 5 %: 47.3 and 49.3, four workers of 1M elements 54.2 and 58.3.
+constexpr double kThrListBelow = 0.002;
 // The whole threshold compress of one worker by the G CTAs of one group (this CTA is number b of
 // them); the group's barriers count on the worker's own workspace header.
+template <bool LIST>
 static __device__ __forceinline__ void threshold_multi_body(const ThrMultiArgs& a, const uint32_t G, const uint32_t b,
                                                             BlockSmem& sm, uint32_t& s_used, uint32_t& s_cnt,
                                                             unsigned char* s_dyn) {
@@ -352,12 +358,12 @@ static __device__ __forceinline__ void threshold_multi_body(const ThrMultiArgs& 
                 for (int u = 0; u < kKeyBatch; ++u) { f(kv[u].x); f(kv[u].y); f(kv[u].z); f(kv[u].w); }
             }
         };
-        // the keys inside the coarse bin go to a list in shared memory if they fit (they are read once
+        // LIST: the keys inside the coarse bin go to a list in shared memory if they fit (they are read once
         // from memory then), and the remaining levels run on the list
         constexpr uint32_t kListCap = kWarps * kEmitStage * 2;
         uint32_t* const list = reinterpret_cast<uint32_t*>(sm.emit);
         const uint32_t n_in = p0[0].count;
-        const bool listed = ok && n_in <= kListCap;
+        const bool listed = LIST && ok && n_in <= kListCap;
         if (listed) {
             if (tid == 0) s_cnt = 0u;
             __syncthreads();
@@ -611,12 +617,13 @@ static __device__ __forceinline__ void threshold_multi_body(const ThrMultiArgs& 
 }
 
 // (three CTAs per SM: 80 registers and no spills beat four at 64 registers, see k_topk_single)
+template <bool LIST>
 static __global__ void __launch_bounds__(kBlock, 3)
 k_threshold_multi(const __grid_constant__ ThrMultiArgs a) {
     __shared__ BlockSmem sm;
     __shared__ uint32_t s_used, s_cnt;
     extern __shared__ __align__(16) unsigned char s_dyn[];
-    threshold_multi_body(a, gridDim.x, blockIdx.x, sm, s_used, s_cnt, s_dyn);
+    threshold_multi_body<LIST>(a, gridDim.x, blockIdx.x, sm, s_used, s_cnt, s_dyn);
 }
 
 // Several workers' threshold compress calls in one cooperative launch, one group of CTAs per
@@ -627,6 +634,7 @@ struct ThrWorkersArgs {
 };
 static_assert(sizeof(ThrWorkersArgs) <= 4000, "kernel parameters stay below 4 KB");
 
+template <bool LIST>
 static __global__ void __launch_bounds__(kBlock, 3)
 k_threshold_workers(const __grid_constant__ ThrWorkersArgs wa) {
     __shared__ BlockSmem sm;
@@ -640,7 +648,7 @@ k_threshold_workers(const __grid_constant__ ThrWorkersArgs wa) {
         for (uint32_t i = threadIdx.x; i < sizeof(ThrMultiArgs) / 4; i += kBlock) dst[i] = src[i];
     }
     __syncthreads();
-    threshold_multi_body(s_args, wa.G, b, sm, s_used, s_cnt, s_dyn);
+    threshold_multi_body<LIST>(s_args, wa.G, b, sm, s_used, s_cnt, s_dyn);
 }
 
 }  // namespace gc
