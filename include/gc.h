@@ -136,12 +136,12 @@ int gc_plan(gc_plan_t **out, int device, uint32_t n_tensors, const uint64_t *siz
  *                                and so exercise the safety net -- a testing aid).  The workspace
  *                                size reported at plan creation stays sufficient.
  *   GC_OPT_CANDIDATE_CAPACITY    lowers the candidate-list capacity (testing aid for overflow)
- *   GC_OPT_DECODE_ROUTE          which tiled decode kernel gc_decompress_accumulate takes:
- *                                GC_DECODE_AUTO (default) picks by the expected number of pairs --
- *                                GC_DECODE_NARROW pre-loads 4 x (256 / W) pairs per worker and
- *                                8192-element tile in registers, GC_DECODE_WIDE moves the lists through
- *                                rings in shared memory (many workers, dense lists;
- *                                gc_decompress_apply_momentum always does).  Same result.
+ *   GC_OPT_DECODE_ROUTE          which tiled decode kernel gc_decompress_accumulate and
+ *                                gc_decompress_apply_momentum take: GC_DECODE_AUTO (default) picks by
+ *                                size and expected number of pairs -- GC_DECODE_NARROW pre-loads
+ *                                4 x (256 / W) pairs per worker and 8192-element tile in registers,
+ *                                GC_DECODE_WIDE moves the lists through rings in shared memory (many
+ *                                workers, dense lists).  Same result.
  *   GC_OPT_DECODE_ORDER          GC_ORDER_FIXED (default): every element's contributions are added in
  *                                worker order 0..W-1, so the result is bit-reproducible.
  *                                GC_ORDER_ANY: the caller would accept any order, i.e. results within

@@ -30,6 +30,7 @@ struct MultiGeom { uint32_t G = 0, per = 0, pool = 0, full = 0, ntab = 0; size_t
 struct DeviceFacts {
     int sm_count = 0;
     int grid_thr = 0, grid_decode[2] = {0, 0};
+    int grid_decode_apply = 0;                    // k_decode_tiles with the optimizer (one tile buffer)
     int grid_decode_seg[2] = {0, 0}, grid_decode_seg_apply = 0;    // k_decode_segments: one / two tile buffers; with optimizer
     bool rings_ok = false;                        // k_decode_rings may use up to kRingSmem2 of dynamic shared memory
     int grid_hist = 0, grid_compact = 0, grid_fold = 0, grid_sample = 0, grid_chist = 0, grid_ccompact = 0;
@@ -532,14 +533,15 @@ bool allow_smem(std::initializer_list<const void*> kernels, size_t bytes) {
 constexpr size_t kRingSmem3 = 74 * 1024 - 512, kRingSmem2 = 111 * 1024;
 struct RingGeom { uint32_t T = 0, RS = 0; size_t smem = 0; int ctas = 0; };
 static size_t ring_smem(uint32_t W, uint32_t T, uint32_t RS, bool apply) {
-    const size_t Wb = (W + kRingBatch - 1) / kRingBatch * kRingBatch;
-    return 8 * Wb * RS + sizeof(float) * 8 * (size_t)(T + kRingPad + (apply ? 2 * T : 0)) + 8 * 8 * (size_t)(W > 32 ? 64 : 32);
+    return 8 * (size_t)W * RS + sizeof(float) * 8 * (size_t)(T + kRingPad + (apply ? 2 * T : 0)) + 8 * 8 * (size_t)(W > 32 ? 64 : 32);
 }
 static RingGeom ring_geometry(const gc_plan_s* p, uint32_t W, bool apply) {
     const double dens = (double)p->total_cap / (double)p->total_n;
     // a warp adds a worker's share of its sub-tile in rounds of 32 entries: one round for nearly all
-    // shares where that leaves a sub-tile worth its fixed cost, two rounds for denser lists
-    const double per_sub = dens * 1152.0 <= 17.0 ? 17.0 : 51.0;
+    // shares where that leaves a sub-tile worth its fixed cost, two rounds for more than eight lists of up
+    // to 5 % (50M elements, 12 lists at 5 %: 138 against 150 us); otherwise the sub-tile is as large as the
+    // rings allow (one list, 5 %: 61 -> 48 us, 20 %: 326 -> 70; eight lists, 20 %: 411 -> 238)
+    const double per_sub = dens * 1152.0 <= 17.0 ? 17.0 : W > 8 && dens <= 0.051 ? 51.0 : 1e9;
     auto slots = [](double avg) { return std::max(32u, ((uint32_t)(avg + 3.2 * std::sqrt(avg)) + 12u) / 4u * 4u); };
     auto largest = [&](size_t budget) {
         RingGeom g;
@@ -570,16 +572,37 @@ static RingGeom ring_geometry(const gc_plan_s* p, uint32_t W, bool apply) {
     }
     return g;
 }
-static bool takes_rings(const gc_plan_s* p, uint32_t W) {
-    if (W == 0 || !p->rings_ok) return false;
+// The lines below were drawn with lists whose indices are independent of each other ("ind") and with lists
+// that agree on a fifth of their entries, as gradients of one model do ("corr"; tiles / rings in us):
+//  - k_decode_tiles pre-loads 4 x (256 / W) entries per worker and 8192-element tile.  Denser lists go through
+//    the rings; one or two lists on a buffer that lies in L2 may be twice as dense (10M elements at 20 %, one
+//    list: 16.7 / 20.7; 50M: 120 / 70).
+//  - Inside that window the tile kernel wins as long as hardly any element has three hits, whose sums it
+//    orders by worker.  W x density > 4.5 % is where the two kinds of lists leave the least to lose: 50M, W = 24
+//    at 0.2 %: ind 55 / 70, corr 96 / 64; W = 32 at 0.3 %: ind 69 / 94, corr 208 / 83; W = 24 at 0.1 %: corr
+//    58 / 62.  It counts from four lists on (50M at 2 %: ind 50 / 54, corr 60 / 54), in L2 from six (10M at 2 %,
+//    W = 4: 14.6 / 16.5 either way).  Sums that continue the buffer's content have no such ordering step: there
+//    the rings' two barriers per step pay from a dozen lists on (0.5 %: W = 8 80 / 82, W = 12 97 / 85), and for
+//    one or two beyond L2 (50M at 5 %, W = 2: 97 / 87).
+//  - With the optimizer the rings fetch parameters and velocities under the additions: better below 1M and
+//    from 11M elements on (W = 1: 0.3M 12.4 / 10.6, 4M 12.6 / 14.7, 10M 27 / 31, 12M 41 / 39, 50M 162 / 143),
+//    but not for more than 32 sparse lists, whose rings leave little room for sub-tiles (W = 64 at 0.05 %, 25M:
+//    109 / 156).  Between, the line of 4.5 % counts from eight lists on (5M at 1 %, W = 6: ind 16.5 / 20.6;
+//    W = 8: ind 16.7 / 20.7, corr 22.8 / 20.7; W = 16: corr 49 / 23).
+constexpr uint64_t kTilesInL2 = 12u << 20, kApplyTilesFrom = 1u << 20, kApplyRingsFrom = 11u << 20;
+static bool takes_rings(const gc_plan_s* p, uint32_t W, bool zero_first, bool apply) {
+    if (!p->rings_ok) return false;
+    if ((apply ? p->grid_decode_apply : p->grid_decode[0]) <= 0) return true;
     if (p->decode_route != GC_DECODE_AUTO) return p->decode_route == GC_DECODE_WIDE;
-    // k_decode_tiles pre-loads 4 x (256 / W) entries per worker and 8192-element tile: denser lists go
-    // through the rings, and so do lists whose entries add up to more than 4.5 % of the elements (the
-    // block-wide steps of the tile kernel then cost more than the rings' fixed work per sub-tile)
     uint32_t Wp = 1;
     while (Wp < W) Wp <<= 1;
+    const bool in_l2 = p->total_n <= kTilesInL2;
     const uint64_t avg = (p->total_cap * (uint64_t)kDecTile + p->total_n - 1) / p->total_n;
-    return avg + avg / 4 > (uint64_t)kDecRounds * (kDecBlock / Wp) || (double)W * (double)p->total_cap > 0.045 * (double)p->total_n;
+    const uint64_t window = (uint64_t)kDecRounds * (kDecBlock / Wp) * (W <= 2 && in_l2 ? 2u : 1u);
+    if (avg + avg / 4 > window) return true;
+    const bool from = apply ? W >= 8u : zero_first ? W >= (in_l2 ? 6u : 4u) : W >= 12u || (W <= 2u && !in_l2);
+    if (from && (double)W * (double)p->total_cap > 0.045 * (double)p->total_n) return true;
+    return apply && W <= 32 && (p->total_n < kApplyTilesFrom || p->total_n > kApplyRingsFrom);
 }
 
 static bool ask_device(int device, DeviceFacts* p) {
@@ -677,16 +700,20 @@ static bool ask_device(int device, DeviceFacts* p) {
     }
     p->grid_thr = p->sm_count * blocks_per_sm(k_threshold_emit, kBlock);
     {
-        cudaError_t ed = cudaFuncSetAttribute(k_decode_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t ed = cudaFuncSetAttribute(k_decode_tiles<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)(2 * kDecTileBytes));
         for (int nbuf = 1; nbuf <= 2; ++nbuf) {
             int nb = 0;
             if (ed == cudaSuccess)
-                ed = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_decode_tiles, kDecBlock,
+                ed = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_decode_tiles<false>, kDecBlock,
                                                                    nbuf * kDecTileBytes);
             if (ed != cudaSuccess || nb < 1) { (void)cudaGetLastError(); nb = 0; }
             p->grid_decode[nbuf - 1] = p->sm_count * nb;     // 0: fall back to one launch per worker
         }
+        int nb = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_decode_tiles<true>, kDecBlock, kDecTileBytes) != cudaSuccess ||
+            nb < 1) { (void)cudaGetLastError(); nb = 0; }
+        p->grid_decode_apply = p->sm_count * nb;
     }
     {
         // lists with per-tensor counts (plans of several tensors): the segment-walking tile kernel
@@ -1398,7 +1425,7 @@ int gc_decompress_accumulate(gc_plan_t* p, uint32_t W, const uint32_t* const* id
         const int grid = (int)std::min<uint32_t>(ntl, (uint32_t)p->grid_decode[nbuf - 1]);
         const int use_bulk = (reinterpret_cast<uintptr_t>(dense_out) & 15u) == 0 ? 1 : 0;
         Timed tm(p, s, GC_K_DECODE_TILES);
-        if (takes_rings(p, W)) {
+        if (takes_rings(p, W, zero_first != 0, false)) {
             const RingGeom g = ring_geometry(p, W, false);
             const uint32_t nt8 = (uint32_t)((p->total_n + 8u * g.T - 1) / (8u * g.T));
             auto kr = zero_first ? (W > 32 ? k_decode_rings<false, false, true> : k_decode_rings<false, false, false>)
@@ -1406,8 +1433,9 @@ int gc_decompress_accumulate(gc_plan_t* p, uint32_t W, const uint32_t* const* id
             kr<<<std::min<uint32_t>(nt8, (uint32_t)(p->sm_count * g.ctas)), kDecBlock, g.smem, s>>>(
                 ls, W, (uint32_t)p->total_cap, (uint32_t)p->total_n, g.T, g.RS, dense_out, use_bulk, ws.hdr, ApplyArgs{});
         } else {
-            k_decode_tiles<<<grid, kDecBlock, nbuf * kDecTileBytes, s>>>(
-                ls, W, (uint32_t)p->total_cap, (uint32_t)p->total_n, dense_out, zero_first ? 1 : 0, use_bulk, nbuf, ws.hdr);
+            k_decode_tiles<false><<<grid, kDecBlock, nbuf * kDecTileBytes, s>>>(
+                ls, W, (uint32_t)p->total_cap, (uint32_t)p->total_n, dense_out, zero_first ? 1 : 0, use_bulk, nbuf, ws.hdr,
+                ApplyArgs{});
         }
         GC_CUDA(p, cudaGetLastError());
         return GC_OK;
@@ -1464,7 +1492,7 @@ int gc_decompress_apply_momentum(gc_plan_t* p, uint32_t W, const uint32_t* const
         (reinterpret_cast<uintptr_t>(velocity) & 15u))
         return GC_E_INVALID;
     const bool segmented = count != nullptr && p->T != 1;              // lists with unused slots between tensors
-    if (segmented ? p->grid_decode_seg_apply <= 0 : !p->rings_ok) return GC_E_UNSUPPORTED;
+    if (segmented ? p->grid_decode_seg_apply <= 0 : p->grid_decode_apply <= 0 && !p->rings_ok) return GC_E_UNSUPPORTED;
     if (segmented && p->d_dectile == nullptr) return GC_E_UNSUPPORTED;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     WsView ws = view(p, workspace);
@@ -1481,6 +1509,12 @@ int gc_decompress_apply_momentum(gc_plan_t* p, uint32_t W, const uint32_t* const
         k_decode_segments<true><<<(int)std::min<uint32_t>(ntl, (uint32_t)p->grid_decode_seg_apply), kDecBlock,
                                   kDecTileBytes, s>>>(ls, W, p->d_desc, p->T, p->d_dectile, (uint32_t)p->total_n,
                                                       nullptr, 1, 0, 1, ws.hdr, ap);
+        GC_CUDA(p, cudaGetLastError());
+        return GC_OK;
+    }
+    if (!takes_rings(p, W, true, true)) {
+        k_decode_tiles<true><<<(int)std::min<uint32_t>(ntl, (uint32_t)p->grid_decode_apply), kDecBlock, kDecTileBytes, s>>>(
+            ls, W, (uint32_t)p->total_cap, (uint32_t)p->total_n, nullptr, 1, 0, 1, ws.hdr, ap);
         GC_CUDA(p, cudaGetLastError());
         return GC_OK;
     }

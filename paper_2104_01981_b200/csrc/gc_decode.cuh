@@ -208,9 +208,10 @@ __device__ __forceinline__ bool counted_apply(float* s_tile, uint32_t lo, uint32
     return done;
 }
 
+template <bool APPLY>
 static __global__ void __launch_bounds__(kDecBlock)
 k_decode_tiles(DecodeLists ls, uint32_t W, uint32_t cnt, uint32_t total_n, float* __restrict__ out,
-               int zero_first, int use_bulk, int nbuf, WsHeader* hdr) {
+               int zero_first, int use_bulk, int nbuf, WsHeader* hdr, ApplyArgs ap) {
     // nbuf tile buffers: with two, one fills while the other drains (pays off when there are few
     // workers per tile; with many workers more resident CTAs are worth more than the overlap)
     extern __shared__ __align__(128) float s_tiles[];
@@ -305,6 +306,11 @@ k_decode_tiles(DecodeLists ls, uint32_t W, uint32_t cnt, uint32_t total_n, float
         }
         __syncthreads();
         // the tile leaves shared memory
+        if (APPLY) {
+            apply_tile(ap, s_tile, lo, hi, full, tid);
+            __syncthreads();
+            continue;
+        }
         if (full && use_bulk) {
             if (tid == 0) bulk_store_tile(out + lo, s_tile, (uint32_t)(kDecTile * sizeof(float)));
         } else {

@@ -74,10 +74,10 @@ k_decode_rings(const __grid_constant__ DecodeLists ls, uint32_t W, uint32_t cnt,
     constexpr int kW8 = kDecBlock / 32, U = WIDE ? 2 : 1;
     extern __shared__ __align__(128) float s_dyn_rings[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    // rings [W rounded up to kRingBatch][2][RS] (indices, values), then the sub-tiles
+    // rings [W][2][RS] (indices, values), then the sub-tiles
     const uint32_t Wb = (W + kRingBatch - 1u) / kRingBatch * kRingBatch;
     uint32_t* const rings = reinterpret_cast<uint32_t*>(s_dyn_rings);
-    float* const s_tiles = s_dyn_rings + 2u * Wb * RS;
+    float* const s_tiles = s_dyn_rings + 2u * W * RS;
     float* const s_tile = s_tiles + warp * (T + kRingPad);               // this warp's sub-tile
     float* const s_par = s_tiles + kW8 * (T + kRingPad) + warp * 2u * T;          // APPLY: its parameters and velocities
     uint2* const s_rng = reinterpret_cast<uint2*>(s_tiles + kW8 * (T + kRingPad) + (APPLY ? kW8 * 2u * T : 0u)) + warp * (32 * U);
@@ -223,7 +223,7 @@ k_decode_rings(const __grid_constant__ DecodeLists ls, uint32_t W, uint32_t cnt,
 #pragma unroll
                 for (uint32_t j = 0; j < kRingBatch; ++j) {
                     const uint2 r = s_rng[w0 + j];
-                    const uint32_t* const e = rings + 2u * (w0 + j) * RS + wrap(r.x + lane);
+                    const uint32_t* const e = rings + 2u * min(w0 + j, W - 1u) * RS + wrap(r.x + lane);
                     n[j] = r.y; x[j] = e[0]; v[j] = __uint_as_float(e[RS]);
                 }
 #pragma unroll

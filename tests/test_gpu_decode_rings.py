@@ -138,3 +138,37 @@ def test_a_list_with_invalid_entries_does_not_cost_the_others_theirs(bad, fused)
         plan.decompress_accumulate(d_idx, d_val, None, out, True, ws)
     assert plan.last_status(ws)[0] == api.GC_E_INVALID
     assert np.array_equal(to_np_u32(out), bits(want))
+
+
+@pytest.mark.parametrize("n,density,W", [(300_000, 0.01, 1), ((1 << 20) + 3, 0.02, 2), (2_000_001, 0.2, 2), (3_000_001, 0.003, 16),
+                                         (3_000_001, 0.3, 1), (500_001, 1.0, 3), (1_500_000, 0.001, 64), (11_600_000, 0.001, 40),
+                                         (11_600_000, 0.001, 3)])
+def test_decode_on_both_sides_of_the_route_rules(n, density, W):
+    """Sizes, densities and worker counts around the lines between the tile kernel and the rings, dense lists whose
+    sub-tiles are bounded by the rings alone, and both kernels on request: plain decode in both modes and the
+    momentum step."""
+    k = api.Plan([n], density, device=-1).total_cap
+    pairs, d_idx, d_val = [], [], []
+    for w in range(W):
+        idx, _ = synth.sparse_set([n], [k], 300 + (w // 3 if w % 2 else w))
+        _, val = synth.sparse_set([n], [k], 700 + w, scale=10.0 ** (w % 5 - 2))
+        pairs.append((idx, val))
+        d_idx.append(torch.from_numpy(idx.view(np.int32)).cuda())
+        d_val.append(torch.from_numpy(val).cuda())
+    p0 = np.random.default_rng(n).standard_normal(n).astype(np.float32)
+    sums = [oracle.decode_accumulate(pairs, p0.copy(), zero_first) for zero_first in (True, False)]
+    p1, v1 = p0.copy(), (p0 * np.float32(0.1)).astype(np.float32)
+    v0 = torch.from_numpy(v1.copy())
+    oracle.decode_apply_momentum(pairs, p1, v1, 0.05, 0.9, 0.25)
+    for route in (api.GC_DECODE_AUTO, api.GC_DECODE_NARROW, api.GC_DECODE_WIDE):
+        plan = api.Plan([n], density, device=0)
+        plan.set_option(api.GC_OPT_DECODE_ROUTE, route)
+        ws = plan.alloc_workspace()
+        for want, zero_first in zip(sums, (True, False)):
+            out = torch.from_numpy(p0.copy()).cuda()
+            plan.decompress_accumulate(d_idx, d_val, None, out, zero_first, ws)
+            assert np.array_equal(to_np_u32(out), bits(want)), (route, zero_first)
+        d_p, d_v = torch.from_numpy(p0.copy()).cuda(), v0.cuda()
+        plan.decompress_apply_momentum(d_idx, d_val, None, d_p, d_v, 0.05, 0.9, 0.25, ws)
+        assert np.array_equal(to_np_u32(d_p), bits(p1)) and np.array_equal(to_np_u32(d_v), bits(v1)), route
+        assert plan.last_status(ws)[0] == api.GC_OK
