@@ -108,6 +108,8 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 constexpr size_t kSingleMidCap = 65536;      // short list of k_topk_single (candidates in the band bin of the threshold)
 constexpr uint64_t kSampleMax = 131072;       // most sampled elements per tensor
+constexpr double kRefineFrom = 0.0005;         // plans of several tensors from this density,
+constexpr uint64_t kRefineLarge = 1u << 26;    // or this many elements on rank their sample twice (see sample_params)
 constexpr uint64_t kSampleMaxSingle = 262144;   // ... when the plan holds one tensor (the sample is read in one step)
 constexpr uint32_t kSinglePoolMax = 65536, kMultiPoolMax = 98304;   // most candidates one CTA of the fused kernels may hold
 // Share of the oldest CTA of an SM above (and of the youngest below) the middle one's: measured
@@ -178,7 +180,7 @@ WsView view(const gc_plan_s* p, void* ws) {
 // sits six standard deviations of the sampling noise above the expected rank density*m, so a
 // candidate set smaller than k is a < 1e-8 event for well-mixed data (and only costs a redo).
 void sample_params(TensorDesc& d, double density, uint32_t rank_permille, uint64_t* ccap, uint64_t target_max,
-                   double coarse_factor, uint64_t* nsg_if_sampled) {
+                   double coarse_factor, uint64_t* nsg_if_sampled, bool refine) {
     const uint64_t n = d.n;
     d.sstride = 0; d.srank = 0;
     *ccap = n;
@@ -188,8 +190,11 @@ void sample_params(TensorDesc& d, double density, uint32_t rank_permille, uint64
     // 21 bits instead of a bin edge (12 % in value).  Its larger margin (15 % of k at 5 %, a third at 1 %,
     // as much again as k at 0.1 %) is the smaller evil: under error feedback magnitudes pile up just below
     // the threshold, and a bin edge can admit enough of them to overflow the candidate regions -- the exact
-    // redo then runs (110M elements in 199 tensors at 0.5 %, repeated gradient: 600-1250 us against 300).
-    if (target_max == kSampleMax && density >= 0.0005) target_max = 32000;
+    // redo then runs (110M elements in 199 tensors at 1 %, us: one gradient again and again 784 -> 287, eight
+    // in turn 520 -> 285; a dozen tensors of 200M at 0.04 %: 1629 -> 466).  Below 0.05 % that happens to large
+    // plans only, and the second ranking costs small ones a few microseconds (9M elements in two tensors at
+    // 0.01 %: 49.5 us without, 55.7 with it; 50M: 146.5 and 149.6; 110M: 280 and 274).
+    if (refine) target_max = 32000;
     uint64_t target = std::min<uint64_t>(target_max, std::max<uint64_t>(n / 128, std::min<uint64_t>(8192, n / 2)));
     uint64_t stride = std::max<uint64_t>(1, n / target);
     uint64_t groups = (n + 3) / 4;
@@ -221,7 +226,8 @@ void finish_layout(gc_plan_s* p) {
             // (many tensors: the bracket is a histogram bin edge, up to twice the candidates)
             uint64_t nsg_w = 0;
             sample_params(d, p->density, p->rank_permille, &ccap, p->T == 1 ? kSampleMaxSingle : kSampleMax,
-                          p->T == 1 ? (p->density <= 0.1 ? 1.3 : 1.0) : 2.0, &nsg_w);
+                          p->T == 1 ? (p->density <= 0.1 ? 1.3 : 1.0) : 2.0, &nsg_w,
+                          p->T > 1 && (p->density >= kRefineFrom || p->total_n >= kRefineLarge));
             stiles_worst += (nsg_w + (uint64_t)kSampleTile - 1) / (uint64_t)kSampleTile;
         } else {
             // threshold mode: the sample is part of the definition -- one 4-element group out of

@@ -482,6 +482,26 @@ def test_candidate_path_needs_no_redo_in_error_feedback_steady_state():
     assert all(k <= c[0] <= 4 * k + 600_000 for c in seen), seen
 
 
+@pytest.mark.parametrize("density", [0.0001, 0.0004])
+def test_large_sparse_plans_of_several_tensors_need_no_redo(density):
+    """A dozen tensors of 200M elements whose unsent entries pile up below the thresholds: the brackets admit few
+    enough candidates for the regions at every step."""
+    weight = [(1 + i * 7919 % 13) ** 1.5 for i in range(12)]
+    sizes = [int(200_000_000 * x / sum(weight)) for x in weight]
+    plan = api.Plan(sizes, density, device=0)
+    n, wk = plan.total_n, GpuWorker(plan)
+    gen = torch.Generator(device="cuda").manual_seed(8)
+    scale = torch.cat([torch.full((s,), (1 + s % 977) ** -0.5, device="cuda") for s in sizes])
+    # (the residual in the middle of a run: triangular up to the threshold)
+    wk.residual.copy_(torch.rand(n, device="cuda", generator=gen) - torch.rand(n, device="cuda", generator=gen))
+    wk.residual.mul_(scale).mul_(density ** -0.5)
+    grads = [torch.empty(n, device="cuda").normal_(generator=gen).mul_(scale) for _ in range(2)]
+    for step in range(60):
+        wk.step(grads[step % 2])
+        wk.check_status()
+        assert plan.last_counters(wk.ws)[1:] == (0, 0), step
+
+
 def test_sample_blind_spot_falls_back_and_stays_exact():
     """All large values sit where the sample never looks (groups that are not a multiple of the
     stride), so the sampled threshold is far too low or too high; the result must not care."""
