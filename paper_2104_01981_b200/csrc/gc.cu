@@ -773,6 +773,8 @@ static bool device_facts(int device, DeviceFacts& out) {
 extern "C" {
 
 static int compress_route(const gc_plan_s* p);
+static int fill_plan(gc_plan_s* p, int device, uint32_t n_tensors, const uint64_t* sizes, double density, int mode,
+                     uint32_t sample_stride, double cap_factor, uint64_t total);
 
 uint32_t gc_version(void) { return 1u; }
 
@@ -793,9 +795,28 @@ int gc_plan(gc_plan_t** out, int device, uint32_t n_tensors, const uint64_t* siz
     }
     gc_plan_s* p = new (std::nothrow) gc_plan_s();
     if (p == nullptr) return GC_E_INVALID;
+    int rc;
+    try {
+        rc = fill_plan(p, device, n_tensors, sizes, density, mode, sample_stride, cap_factor, total);
+    } catch (...) {                        // out of host memory
+        rc = GC_E_INVALID;
+    }
+    if (rc != GC_OK) {
+        (void)gc_destroy(p);
+        if (device >= 0) (void)cudaGetLastError();
+        return rc;
+    }
+    *out = p;
+    return GC_OK;
+}
+
+static int fill_plan(gc_plan_s* p, int device, uint32_t n_tensors, const uint64_t* sizes, double density, int mode,
+                     uint32_t sample_stride, double cap_factor, uint64_t total) {
     p->device = device; p->mode = mode; p->density = density;
     p->cap_factor = cap_factor; p->stride = sample_stride; p->T = n_tensors;
     p->total_n = total;
+    p->clean_ws.reserve(2 * GC_MAX_WORKERS);          // (the calls add to these without allocating)
+    p->staging.reserve(8);
     p->desc.resize(n_tensors);
     uint64_t off = 0, out_off = 0, tile0 = 0;
     for (uint32_t t = 0; t < n_tensors; ++t) {
@@ -820,10 +841,7 @@ int gc_plan(gc_plan_t** out, int device, uint32_t n_tensors, const uint64_t* siz
     p->ntiles = (uint32_t)tile0;
     finish_layout(p);
 
-    if (device < 0) {            // host-only plan: answers queries, refuses compute calls
-        *out = p;
-        return GC_OK;
-    }
+    if (device < 0) return GC_OK;                     // host-only plan: answers queries, refuses compute calls
     int caller_device = -1;
     if (cudaGetDevice(&caller_device) != cudaSuccess) { (void)cudaGetLastError(); caller_device = -1; }
     struct RestoreDevice {           // the caller's current device is left as it was found
@@ -850,26 +868,14 @@ int gc_plan(gc_plan_t** out, int device, uint32_t n_tensors, const uint64_t* siz
                 e = cudaMemcpy(p->d_dectile, tt.data(), sizeof(uint32_t) * (size_t)ntl, cudaMemcpyHostToDevice);
         }
     }
-    if (e != cudaSuccess) {
+    if (e != cudaSuccess || !device_facts(device, *p)) {
         (void)cudaGetLastError();
-        if (p->d_desc) cudaFree(p->d_desc);
-        if (p->d_small) cudaFree(p->d_small);
-        if (p->d_dectile) cudaFree(p->d_dectile);
-        delete p;
-        return GC_E_CUDA;
-    }
-    if (!device_facts(device, *p)) {
-        if (p->d_desc) cudaFree(p->d_desc);
-        if (p->d_small) cudaFree(p->d_small);
-        if (p->d_dectile) cudaFree(p->d_dectile);
-        delete p;
         return GC_E_CUDA;
     }
     plan_single(p);
     plan_thr_single(p);
     plan_thr_multi(p);
     plan_multi(p);
-    *out = p;
     return GC_OK;
 }
 
@@ -887,9 +893,11 @@ int gc_plan_set_option(gc_plan_t* p, int option, uint64_t value) {
             p->rank_permille = (uint32_t)value;
             p->clean_ws.clear();                       // (another kernel may take the plan now)
             p->wk_W = 0;
-            finish_layout(p);                          // workspace size stays as planned (see skeys_tiles_alloc)
-            plan_single(p);
-            plan_multi(p);
+            try {
+                finish_layout(p);                      // workspace size stays as planned (see skeys_tiles_alloc)
+                plan_single(p);
+                plan_multi(p);
+            } catch (...) { return GC_E_INVALID; }     // out of host memory
             return upload_table(p);
         case GC_OPT_CANDIDATE_CAPACITY:
             if (value > p->cand_cap_alloc) return GC_E_INVALID;
@@ -1329,13 +1337,15 @@ int gc_compress_workers(gc_plan_t* p, uint32_t W, const float* const* grads, flo
     if ((topk_multi || thr_multi) && W >= 2) {
         if (p->wk_W != W) {                      // (kept for the next call; options that change the layout reset it)
             p->wk_W = W; p->wk_batch = 0;
-            for (uint32_t wb = std::min<uint32_t>(W, kWorkersPerLaunch); wb >= 2 && p->wk_batch == 0; --wb) {
-                const MultiGeom g2 = topk_multi ? multi_geometry(p, (uint32_t)p->grid_multi_max / wb, false)
-                                                : thr_multi_geometry(p, (uint32_t)p->grid_thr_multi_max / wb);
-                if (g2.G > 0 && g2.smem <= (topk_multi ? p->multi_smem_max : p->thrm_smem_max)) {
-                    p->wk_batch = wb; p->wk_geom = g2;
+            try {
+                for (uint32_t wb = std::min<uint32_t>(W, kWorkersPerLaunch); wb >= 2 && p->wk_batch == 0; --wb) {
+                    const MultiGeom g2 = topk_multi ? multi_geometry(p, (uint32_t)p->grid_multi_max / wb, false)
+                                                    : thr_multi_geometry(p, (uint32_t)p->grid_thr_multi_max / wb);
+                    if (g2.G > 0 && g2.smem <= (topk_multi ? p->multi_smem_max : p->thrm_smem_max)) {
+                        p->wk_batch = wb; p->wk_geom = g2;
+                    }
                 }
-            }
+            } catch (...) { p->wk_W = 0; return GC_E_INVALID; }       // out of host memory
         }
         batch = p->wk_batch; mg = p->wk_geom;
     }
@@ -1609,7 +1619,7 @@ int gc_profile_enable(gc_plan_t* p, uint32_t max_records) {
     for (auto& r : p->recs) { cudaEventDestroy(r.a); cudaEventDestroy(r.b); }
     p->recs.clear();
     p->recs_used = 0;
-    p->recs.reserve(max_records);
+    try { p->recs.reserve(max_records); } catch (...) { return GC_E_INVALID; }       // out of host memory
     for (uint32_t i = 0; i < max_records; ++i) {
         gc_plan_s::Rec r{};
         cudaError_t e = cudaEventCreate(&r.a);

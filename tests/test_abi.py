@@ -4,6 +4,8 @@ import ctypes
 import math
 import os
 import re
+import subprocess
+import sys
 
 import pytest
 
@@ -133,3 +135,24 @@ def test_ecrm_placement_matches_the_oracle_rule(lib):
         ecrm.placement(0, 1)
     with pytest.raises(ecrm.EcrmError):
         ecrm.placement(33, 1)
+
+
+def test_running_out_of_host_memory_is_an_error_code(lib):
+    """A plan whose tables do not fit the process's address space: an error code, not an exception that ends
+    the caller.  In a process of its own, which limits itself to 300 MB above what it has."""
+    code = """
+import ctypes, resource, sys
+lib = ctypes.CDLL(sys.argv[1])
+lib.gc_plan.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_uint32, ctypes.c_void_p, ctypes.c_double, ctypes.c_int,
+                        ctypes.c_uint32, ctypes.c_double]
+T = 16_000_000                                       # 1 GB of table entries
+sizes, out = (ctypes.c_uint64 * T)(), ctypes.c_void_p()
+limit = int(open('/proc/self/statm').read().split()[0]) * resource.getpagesize() + (300 << 20)
+resource.setrlimit(resource.RLIMIT_AS, (limit, limit))
+rc = lib.gc_plan(ctypes.byref(out), -1, T, sizes, 0.01, 0, 0, 0.0)
+assert rc < 0 and not out.value, (rc, out.value)
+rc = lib.gc_plan(ctypes.byref(out), -1, 1000, sizes, 0.01, 0, 0, 0.0)
+assert rc == 0 and out.value
+"""
+    r = subprocess.run([sys.executable, "-c", code, api._SO], capture_output=True, text=True)
+    assert r.returncode == 0, (r.returncode, r.stderr[-500:])
