@@ -85,7 +85,8 @@ typedef struct gc_plan_s gc_plan_t;
 #define GC_ROUTE_TOPK_MANY        2 /* one cooperative launch, many-tensor kernel                              */
 #define GC_ROUTE_TOPK_GENERAL     3 /* one cooperative launch, general candidate kernel (global histograms per
                                        level): plans the two kernels above do not take -- candidate sets too
-                                       large for a CTA's region (more than 65,536 candidates per CTA),
+                                       large for a CTA's region (more than 65,536 candidates per CTA, several
+                                       tensors 98,304),
                                        tensors beyond their tile limits, unsampled tensors                    */
 #define GC_ROUTE_TOPK_STAGED      4 /* the general candidate path as separate launches                         */
 #define GC_ROUTE_EXACT            5 /* exact multi-pass kernels only                                           */

@@ -65,7 +65,6 @@ struct gc_plan_s : DeviceFacts {
     uint32_t n_sampled = 0;                 // tensors with a sample
     int path = 0;                           // GC_PATH_AUTO or GC_PATH_EXACT
     int decode_route = 0;                   // GC_DECODE_AUTO, GC_DECODE_NARROW or GC_DECODE_WIDE
-    int decode_order = 0;                   // GC_ORDER_FIXED or GC_ORDER_ANY
     uint32_t rank_permille = 1000;          // scales the sample rank (testing aid)
     // workspace layout (byte offsets)
     size_t off_sel = 0, off_ssel = 0, off_gsel = 0, off_hist = 0, off_state = 0, off_gstate = 0,
@@ -113,12 +112,13 @@ constexpr uint64_t kRefineLarge = 1u << 26;    // or this many elements on rank 
 constexpr uint64_t kSampleMaxSingle = 262144;   // ... when the plan holds one tensor (the sample is read in one step)
 constexpr uint32_t kSinglePoolMax = 65536, kMultiPoolMax = 98304;   // most candidates one CTA of the fused kernels may hold
 // Share of the oldest CTA of an SM above (and of the youngest below) the middle one's: measured
-// best between 6 and 10 % on the 110M-element workload at 1 % density.  At 0.1 % density the
-// fold loop has fewer candidates to handle, competes less for issue slots, and 4 % did better
-// than 8 % (with 8 % the oldest CTAs of the 355M-element workload finished last).
+// best between 6 and 10 % on the 110M-element workload at 1 % density.  Sparser plans have fewer
+// candidates to handle in the fold loop and compete less for issue slots: below 0.5 % the smaller
+// one (4 % did better than 8 % at 0.1 %, where 8 % let the oldest CTAs of the 355M-element workload
+// finish last).  Forms with votes (up to kSparseUpTo, bfloat16) take equal shares.
 constexpr double kSingleSkew = 0.08, kSingleSkewSparse = 0.04;
 constexpr size_t kSingleRowBytes = (2 * kWarps + 4) * sizeof(uint32_t);   // shared memory per owned tile
-constexpr double kSparseUpTo = 0.002;        // density up to which the fold is bound by memory alone (see VOTES of k_topk_single)
+constexpr double kSparseUpTo = 0.002;        // density up to which most chunks are empty (see VOTES of k_topk_single)
 constexpr double kDenseFrom = 0.02;          // density from which the forms with emission by chunk are taken (12 candidates per chunk)
 constexpr uint32_t kMultiMaxTab = 1024;      // tensors whose tile tables k_topk_multi keeps in shared memory
 constexpr size_t kMultiMaxPer = 224;         // most tiles one CTA of k_topk_multi may own
@@ -455,7 +455,7 @@ MultiGeom multi_geometry(const gc_plan_s* p, uint32_t G, bool age_skew) {
         if (d.kind == kKindSmall || d.ntiles == 0) continue;
         if (d.sstride == 0) { per_tile[t] = (double)kTile; continue; }
         const uint64_t groups = ((uint64_t)d.n + 3) / 4, nsg = (groups + d.sstride - 1) / d.sstride;
-        const double edge = d.nstiles <= kRefineTiles ? 1.02 : 2.0;      // tau is exact to 22 bits, or a bin edge
+        const double edge = d.nstiles <= kRefineTiles ? 1.02 : 2.0;      // tau is exact to 21 bits, or a bin edge
         per_tile[t] = std::min<double>(kTile, edge * (double)kTile * (double)d.srank / (4.0 * (double)nsg));
     }
     // runs: `per` tiles for the first two thirds of a full grid, the rest spread over the last third
@@ -912,8 +912,7 @@ int gc_plan_set_option(gc_plan_t* p, int option, uint64_t value) {
             return GC_OK;
         case GC_OPT_DECODE_ORDER:
             if (value != GC_ORDER_FIXED && value != GC_ORDER_ANY) return GC_E_INVALID;
-            p->decode_order = (int)value;
-            return GC_OK;
+            return GC_OK;                              // (the fixed order serves both)
         case GC_OPT_DECODE_ROUTE:
             if (value != GC_DECODE_AUTO && value != GC_DECODE_NARROW && value != GC_DECODE_WIDE) return GC_E_INVALID;
             p->decode_route = (int)value;

@@ -134,7 +134,7 @@ struct GradF32 {
     }
 };
 struct GradBF16 {
-    static constexpr bool kManyTies = true;        // 8 significant bits: equal magnitudes by the thousands
+    static constexpr bool kManyTies = true;        // 8 significant bits: equal magnitudes by the thousands on a residual of zero or of few values
     static __device__ __forceinline__ float ld1(const void* g, uint32_t i) {
         return __uint_as_float((uint32_t)__ldg(reinterpret_cast<const unsigned short*>(g) + i) << 16);
     }

@@ -9,9 +9,10 @@
 //   * all histograms and short lists exist once per tensor in global memory; a CTA only looks
 //     at those of its own segments;
 //   * the sample is a coarse histogram (top 11 key bits) per tensor plus the kept sampled keys;
-//     after the first barrier ONE CTA per tensor computes the bracket (the kept keys give tau a
-//     second radix level; tau_hi is a bin edge; tau_z is interpolated inside its bin -- it is
-//     only a guess) and publishes it, so the fold pass of the many CTAs that share a tensor
+//     after the first barrier ONE CTA per tensor computes the bracket (short samples, see
+//     kRefineTiles: the kept keys give tau and tau_z a second radix level; long ones: tau is a
+//     bin edge and tau_z interpolated inside its bin -- it is only a guess; tau_hi always is a
+//     bin edge) and publishes it, so the fold pass of the many CTAs that share a tensor
 //     only reads three words per segment;
 //   * the slot of a segment's first entry = what the tensor's earlier tiles send: the sum of
 //     their published counts + the sent short-list entries that lie before the segment;
@@ -239,10 +240,10 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
     clean_in_use(hdr, b, tid);
 
     // ---------------------------------------------------------------- bracket per tensor, one CTA each
-    // tau = the srank-th largest sampled key (22 bits when the kept keys allow the second radix
+    // tau = the srank-th largest sampled key (21 bits when the kept keys allow the second radix
     // level, else the lower edge of its coarse bin), tau_hi = upper edge of the bin of the key
-    // that stays below the expected rank by the same margin, tau_z inside the bin of the
-    // expected rank itself; published as (tau, tau_z, shift of the band histogram).
+    // that stays below the expected rank by the same margin, tau_z = the key of the expected rank
+    // itself (21 bits, or a place inside its bin); published as (tau, tau_z, shift of the band histogram).
     for (uint32_t q = b; q < a.n_reg; q += G) {
         const uint32_t cur = a.reg_ids[q];
         const TensorDesc d = a.desc[cur];
@@ -782,7 +783,8 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
     leave_clean(a.cl, hdr, G, tid);
 }
 
-// Votes: 25.6M elements in 161 tensors at 0.1 % 99 -> 97 us, 110M in 199 at 1 % 302 -> 289 us.
+// Votes: 25.6M elements in 161 tensors at 0.1 % 99 -> 97 us, 110M in 199 at 1 % 302 -> 289 us.  (Why the
+// one-tensor kernel loses with them at 1 %, see there, was not found.)
 template <typename GL, bool DENSE, bool VOTES>
 // (three CTAs per SM: 80 registers and no spills beat four at 64 registers, see k_topk_single)
 static __global__ void __launch_bounds__(kBlock, 3)
@@ -806,8 +808,8 @@ struct WorkersArgs {
 };
 static_assert(sizeof(WorkersArgs) <= 4000, "kernel parameters stay below 4 KB");
 
-// (The scan stays here: with several workers per launch the fold is bound by memory, 475 against 484 us
-// for eight 161-tensor workers.)
+// (The scan stays here: 475 against 484 us with votes for eight 161-tensor workers at 0.1 %, the one shape
+// both were measured on.)
 template <typename GL, bool DENSE>
 static __global__ void __launch_bounds__(kBlock, 3)
 k_topk_workers(const __grid_constant__ WorkersArgs wa) {

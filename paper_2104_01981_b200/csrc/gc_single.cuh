@@ -393,8 +393,8 @@ __device__ __forceinline__ bool fold_tail_votes(BlockSmem& sm, const float (&av)
 // Between, fp32 is bound by memory and the slower loop with unequal shares does better (0.5 %: 245 against
 // 249-254 us; 355M at 0.3 %: 697 against 714).
 // DENSE (plans of 2 % and more) has the emission by chunk, the bfloat16 form the counted band: the other
-// forms do without their code (a tensor of 1M elements runs every phase from a cold instruction cache:
-// 37.0 against 38.7 us for compress and decode).
+// forms do without their code.  Many tensors, without / with DENSE: 110M elements at 2 % 305 / 310 us, 5 %
+// 359 / 346; 25.6M at 5 % 134 / 131; one tensor: 110M at 2 % 268 / 267, 5 % 312 / 311, 8M at 2 % 49 / 51.
 template <typename GL, bool DENSE, bool VOTES>
 static __global__ void __launch_bounds__(kBlock, 3)
 k_topk_single(const __grid_constant__ SingleArgs a) {
@@ -680,11 +680,11 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
     Picked pa[1];
     block_select_multi<2048, 1>(sm, a.hist5 + 2 * kHistBins, want_k, pa);
     const uint32_t A = pa[0].bin, aboveA = pa[0].above, m = pa[0].count;      // m = candidates inside the band bin
-    // A band bin with thousands of candidates (bfloat16 gradients tie by the thousands at the threshold)
-    // is counted: its keys are histogrammed one by one (at most 2048 of them), which gives the threshold
+    // A band bin with thousands of candidates (bfloat16 gradients on a residual of zero, or of few values as
+    // when one gradient is folded again and again, tie by the thousands) is counted: its keys are histogrammed one by one (at most 2048 of them), which gives the threshold
     // key after the barrier; then every CTA counts its candidates above and at that key per tile, and
     // after one more barrier the candidates at the key in the tiles before a tile say how many of its own
-    // are sent.  110M elements, bfloat16, 60,000 ties: counts + threshold + slots 15 + 41 us as a list.
+    // are sent.  110M elements, bfloat16, 60,000 ties: counts + threshold + slots 15 us, 41 us as a list.
     const bool counted = GL::kManyTies && overflowed == 0u && pa[0].ok && m > kMidCounted && A < 2047u && shift <= 11;
     bool good = overflowed == 0u && pa[0].ok && (m <= a.mid_cap || counted);
     const uint32_t binlo = tau + (A << shift);
