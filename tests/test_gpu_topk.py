@@ -45,16 +45,20 @@ def test_tie_stress_quantised_values():
         check_topk_against_oracle([100_000, 100_000, 100_000], density, grads)
 
 
+DIRECT_MAX = 1 << 22                                     # one-tensor plans up to this size: direct radix select
+
+
+@pytest.mark.parametrize("n", [2_000_000, 5_000_000])
 @pytest.mark.parametrize("step,expect_no_redo", [(2.0 ** -12, True), (2.0 ** -8, True), (2.0 ** -6, True),
                                                    (2.0 ** -4, False)])
-def test_one_tensor_ties_at_the_threshold(step, expect_no_redo):
+def test_one_tensor_ties_at_the_threshold(step, expect_no_redo, n):
     """One large tensor whose values sit on a grid: from a dozen to thousands of elements share the
     threshold magnitude, so the tie cut (lowest indices win) decides; up to a few thousand ties the
     one-tensor kernel has to settle it without the exact redo."""
-    n = 2_000_000
     grads = [synth.quantised_gradient(n, 70 + s, step=step) for s in range(2)]
     seen = []
     check_topk_against_oracle([n], 0.01, grads, expect_counters=seen.append)
+    assert all((c[0] > n // 100) == (n > DIRECT_MAX) for c in seen), seen          # (which of the two kernels ran)
     if expect_no_redo:
         assert all(c[1] == 0 and c[2] == 0 for c in seen), seen
 
@@ -178,8 +182,8 @@ PATHS = {
 }
 
 
-@pytest.mark.parametrize("sizes", [[300_000, 5, 1_500_001, 131_072, 64, 131_071, 2_000_003], [3_000_001]],
-                         ids=["many_tensors", "one_tensor"])
+@pytest.mark.parametrize("sizes", [[300_000, 5, 1_500_001, 131_072, 64, 131_071, 2_000_003], [3_000_001], [4_500_001]],
+                         ids=["many_tensors", "one_tensor", "one_tensor_candidates"])
 @pytest.mark.parametrize("path", list(PATHS))
 def test_every_route_gives_the_same_bits(path, sizes):
     n = sum(sizes)
@@ -349,14 +353,14 @@ def test_large_sparse_bfloat16_gradient():
     assert torch.equal(r, a)
 
 
+@pytest.mark.parametrize("n", [3_000_001, 4_500_001])
 @pytest.mark.parametrize("options", [{}, {api.GC_OPT_SAMPLE_RANK_PERMILLE: 30}, {api.GC_OPT_CANDIDATE_CAPACITY: 4}],
                          ids=["plain", "starved", "overflow"])
-def test_private_workspace_skips_the_clearing_launch_and_stays_exact(options):
+def test_private_workspace_skips_the_clearing_launch_and_stays_exact(options, n):
     """GC_OPT_WORKSPACE_PRIVATE: from the second call on a workspace, the one-tensor kernel runs
     without the clearing launch in front of it (one launch per call) because it leaves the control
     block clean itself -- also when the safety net ran.  Five error-feedback steps, alternating two
     workspaces, every step against the oracle."""
-    n = 3_000_001
     plan = api.Plan([n], 0.01, device=0)
     plan.set_option(api.GC_OPT_WORKSPACE_PRIVATE, 1)
     for opt, value in options.items():
@@ -438,11 +442,11 @@ def test_private_workspace_many_tensors_and_workers_call(options):
         check(w, gs2[w])
 
 
-def test_private_workspace_broken_promise_is_caught():
+@pytest.mark.parametrize("n", [1_000_003, 4_500_001])
+def test_private_workspace_broken_promise_is_caught(n):
     """The caller overwrites a workspace it promised to leave alone: the next call must end at once
     with GC_E_INVALID in the device status (no barrier is entered on counters that cannot be
     trusted), and the call after that -- cleared again -- is exact."""
-    n = 1_000_003
     plan = api.Plan([n], 0.01, device=0)
     plan.set_option(api.GC_OPT_WORKSPACE_PRIVATE, 1)
     k = plan.total_cap
@@ -468,18 +472,18 @@ def test_private_workspace_broken_promise_is_caught():
         assert np.array_equal(to_np_u32(idx[:k]), oi) and np.array_equal(to_np_u32(r), bits(r_cpu))
 
 
-def test_candidate_path_needs_no_redo_in_error_feedback_steady_state():
+@pytest.mark.parametrize("n", [3_000_000, 6_000_000])
+def test_candidate_path_needs_no_redo_in_error_feedback_steady_state(n):
     """Re-using a few gradients makes unsent entries pile up just below the threshold (a cliff in
     the magnitude distribution).  The sampled threshold is an exact order statistic, so the
     candidate set must still come out large enough -- and small enough -- at every step."""
-    n = 3_000_000
     base = [randn(n, 300 + s) for s in range(2)]
     grads = [base[s % 2] for s in range(10)]
     seen = []
     check_topk_against_oracle([n], 0.01, grads, expect_counters=seen.append)
     assert all(c[1] == 0 and c[2] == 0 for c in seen), seen
-    k = 30_000
-    assert all(k <= c[0] <= 4 * k + 600_000 for c in seen), seen
+    k = n // 100
+    assert all(k <= c[0] <= 4 * k + 600_000 and (c[0] > k) == (n > DIRECT_MAX) for c in seen), seen
 
 
 @pytest.mark.parametrize("density", [0.0001, 0.0004])
@@ -502,10 +506,10 @@ def test_large_sparse_plans_of_several_tensors_need_no_redo(density):
         assert plan.last_counters(wk.ws)[1:] == (0, 0), step
 
 
-def test_sample_blind_spot_falls_back_and_stays_exact():
+@pytest.mark.parametrize("n", [1 << 21, 5 << 20])
+def test_sample_blind_spot_falls_back_and_stays_exact(n):
     """All large values sit where the sample never looks (groups that are not a multiple of the
     stride), so the sampled threshold is far too low or too high; the result must not care."""
-    n = 1 << 21
     g = randn(n, 77) * 1e-3
     grp = torch.arange(n) // 4
     hidden = (grp % 64) != 0
@@ -597,7 +601,7 @@ def test_random_plans_match_the_oracle(seed):
     check_topk_against_oracle(sizes, density, grads)
 
 
-@pytest.mark.parametrize("sizes,density", [([3_000_001], 0.01), ([70_001], 0.001),
+@pytest.mark.parametrize("sizes,density", [([3_000_001], 0.01), ([70_001], 0.001), ([4_500_001], 0.01), ([4_500_001], 0.03),
                                            ([300_000, 5, 1_500_001, 131_072, 64, 131_071, 4093, 0, 2_000_003], 0.001),
                                            ([5, 3, 1000, 7], 0.3)])
 def test_bf16_gradient_matches_the_oracle_on_the_widened_values(sizes, density):
@@ -721,7 +725,12 @@ def test_one_tensor_plans_around_the_grid_rule(tiles):
     both sides of that rule and where a CTA's share of tiles changes (296 CTAs), with a ragged
     last tile, two steps each against the oracle."""
     n = tiles * 4096 - 5
-    check_topk_against_oracle([n], 0.004, [randn(n, 9100 + tiles), randn(n, 9200 + tiles)])
+    grads = [randn(n, 9100 + tiles), randn(n, 9200 + tiles)]
+    check_topk_against_oracle([n], 0.004, grads)
+    if n <= DIRECT_MAX:                                    # (one slot less than there are steers to the candidate kernel)
+        slots, seen = api.Plan([n], 0.004, device=0).query(api.GC_Q_CANDIDATE_CAPACITY) - 1, []
+        check_topk_against_oracle([n], 0.004, grads, options={api.GC_OPT_CANDIDATE_CAPACITY: slots}, expect_counters=seen.append)
+        assert all(c[0] > n * 0.004 + 1 and c[1:] == (0, 0) for c in seen), seen
 
 
 def test_calls_on_a_side_stream():
@@ -766,7 +775,7 @@ def test_calls_on_a_side_stream():
     assert np.array_equal(to_np_u32(param), bits(p_cpu)) and np.array_equal(to_np_u32(vel), bits(v_cpu))
 
 
-@pytest.mark.parametrize("sizes", [[1_300_001], [200_000, 3, 0, 900_001, 4096]], ids=["one", "many"])
+@pytest.mark.parametrize("sizes", [[1_300_001], [4_600_001], [200_000, 3, 0, 900_001, 4096]], ids=["one", "one_candidates", "many"])
 def test_step_captured_in_a_cuda_graph(sizes):
     """A compress + decode step captured once in a CUDA graph (cooperative launch included) and
     replayed on fresh gradients copied into the captured buffer: every replay against the oracle.
