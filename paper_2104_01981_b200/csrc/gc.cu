@@ -72,7 +72,7 @@ struct gc_plan_s : DeviceFacts {
     // single-tensor shared-memory-pool kernel
     SingleGeom single[2];                   // k_topk_single for fp32 and for bfloat16 gradients
     uint32_t single_grid = 0;               // CTAs of the first (0 = plan does not qualify)
-    size_t off_hist5 = 0, off_rowseg = 0, off_mid = 0, off_fine = 0, off_age = 0;
+    size_t off_hist5 = 0, off_rowseg = 0, off_mid = 0, off_fine = 0, off_start = 0;
     uint32_t single_srank_hi = 0, single_srank_mid = 0;
     uint32_t thr_grid = 0, thr_maxt = 0, thr_pool = 0, thr_rounds = 0;    // one-tensor threshold kernel (0 = no)
     size_t thr_smem = 0;
@@ -123,6 +123,7 @@ constexpr double kDenseFrom = 0.02;          // density from which the forms wit
 constexpr uint32_t kMultiMaxTab = 1024;      // tensors whose tile tables k_topk_multi keeps in shared memory
 constexpr size_t kMultiMaxPer = 224;         // most tiles one CTA of k_topk_multi may own
 constexpr size_t kMultiRowBytes = (2 * kWarps + kSegWords) * sizeof(uint32_t);   // shared memory per owned tile
+constexpr uint32_t kSingleMaxG = 640;        // most CTAs of the one-tensor kernels
 constexpr size_t kSingleMaxT = 341;          // most tiles one CTA of k_topk_single may own
 
 inline uint64_t k_rule(uint64_t n, double density) {
@@ -220,7 +221,7 @@ void finish_layout(gc_plan_s* p) {
     p->reg_ids.clear();
     for (uint32_t t = 0; t < p->T; ++t) {
         TensorDesc& d = p->desc[t];
-        d.kind = kKindRegular; d.pad = 0;
+        d.kind = kKindRegular; d.reg = 0;
         uint64_t ccap = d.n;
         if (p->mode == GC_TOPK) {
             // (many tensors: the bracket is a histogram bin edge, up to twice the candidates)
@@ -252,7 +253,7 @@ void finish_layout(gc_plan_s* p) {
         d.stile0 = (uint32_t)stile0; d.nstiles = (uint32_t)nst;
         d.group0 = (uint32_t)group0; d.ngroups = (d.ntiles + kWarps - 1) / kWarps;
         if (d.kind == kKindSmall && d.n > 0) p->small_ids.push_back(t);
-        if (d.kind != kKindSmall && d.n > 0) p->reg_ids.push_back(t);
+        if (d.kind != kKindSmall && d.n > 0) { d.reg = (uint32_t)p->reg_ids.size(); p->reg_ids.push_back(t); }
         stile0 += nst; group0 += d.ngroups; ccap_total += ccap;
     }
     p->nstiles = (uint32_t)stile0;
@@ -292,15 +293,14 @@ void finish_layout(gc_plan_s* p) {
     p->control_bytes = align_up(p->off_rowseg + (T == 1 ? sizeof(uint32_t) * kSingleMaxT * 20 * 2 : 0), 256);
     p->off_fine = p->control_bytes;
     p->control_bytes = align_up(p->off_fine + (T == 1 ? sizeof(uint32_t) * (size_t)kFineBins : 0), 256);
-    p->off_age = p->control_bytes;                                   // CTAs arrived per SM (one-tensor kernels)
-    p->control_bytes = align_up(p->off_age + (T == 1 ? sizeof(uint32_t) * 1024 : 0), 256);
-    // many-tensor kernel: sample and band histogram per tensor, short-list lengths
-    const size_t multi_hist = T >= 2 ? sizeof(uint32_t) * (size_t)kHistBins * T : 0;
+    // many-tensor kernel: sample and band histogram per tensor that is not small, short-list lengths
+    const size_t multi_hist = T >= 2 ? sizeof(uint32_t) * (size_t)kHistBins * std::max<size_t>(p->reg_ids.size(), 1) : 0;
     p->off_shist = p->control_bytes;
     p->off_bhist = align_up(p->off_shist + multi_hist, 256);
     p->off_midn = align_up(p->off_bhist + multi_hist, 256);
     p->control_bytes = align_up(p->off_midn + (multi_hist ? sizeof(uint32_t) * T : 0), 256);
-    p->off_tinfo = p->control_bytes;
+    p->off_start = p->control_bytes;                                 // where and when the CTAs started (one-tensor kernel)
+    p->off_tinfo = align_up(p->off_start + (T == 1 ? sizeof(uint2) * kSingleMaxG : 0), 256);
     p->off_cidx = align_up(p->off_tinfo + sizeof(uint2) * (size_t)p->ntiles * kWarps, 256);
     p->off_mid = align_up(p->off_cidx + sizeof(uint2) * (size_t)p->cand_cap_alloc, 256);
     p->off_mmid = align_up(p->off_mid + (T == 1 ? sizeof(uint2) * (size_t)kSingleMidCap : 0), 256);
@@ -358,7 +358,7 @@ void plan_single(gc_plan_s* p) {
         if (d.ntiles <= 3000u || (bf16 == 0 && p->density <= kSparseUpTo && d.ntiles <= two * (uint32_t)kSingleMaxT)) g.G = std::min(g.G, two);
         g.maxt = (d.ntiles + g.G - 1) / g.G;
         g.rows = make_row_map(p, d.ntiles, g.G, g.maxt, g.votes ? 0.0 : p->density >= 0.005 ? kSingleSkew : kSingleSkewSparse);
-        if (g.maxt > kSingleMaxT || g.G > 640) return;               // chunk records and totals must stay small
+        if (g.maxt > kSingleMaxT || g.G > kSingleMaxG) return;               // chunk records and totals must stay small
         // region per CTA; one bit per slot has to fit in shared memory beside the chunk records
         g.pool = std::min<uint32_t>(p->cand_cap_alloc / g.G, kSinglePoolMax);
         g.smem = (size_t)g.maxt * kSingleRowBytes + sizeof(uint32_t) * ((g.pool + 31) / 32);
@@ -386,7 +386,7 @@ void plan_thr_single(gc_plan_s* p) {
     if (d.ntiles <= 2500u) G = std::min<uint32_t>(G, 2u * (uint32_t)p->sm_count);    // small tensors: as in plan_single (2M: 28.9 against 33.1 us)
     const uint32_t maxt = (d.ntiles + G - 1) / G;     // equal shares (unequal ones as in the top-k kernel: 268.5 us
                                                       // against 262.5 us on the 110M-element workload)
-    if (maxt > kSingleMaxT || G > 640) return;
+    if (maxt > kSingleMaxT || G > kSingleMaxG) return;
     const uint32_t pool = std::min<uint32_t>(p->cand_cap_alloc / G, kSinglePoolMax);
     if ((double)pool < 1.25 * (double)d.k / (double)G + 256.0) return;
     const uint64_t groups = ((uint64_t)d.n + 3) / 4, nsg = (groups + d.sstride - 1) / d.sstride;
@@ -834,7 +834,7 @@ static int fill_plan(gc_plan_s* p, int device, uint32_t n_tensors, const uint64_
         d.off = (uint32_t)off; d.n = (uint32_t)n; d.k = (uint32_t)k; d.cap = (uint32_t)cap;
         d.out_off = (uint32_t)out_off; d.tile0 = (uint32_t)tile0; d.ntiles = (uint32_t)nt;
         d.stride = n <= 65536 ? 1u : sample_stride;
-        d.kind = kKindRegular; d.pad = 0;
+        d.kind = kKindRegular; d.reg = 0;
         off += n; out_off += cap; tile0 += nt;
     }
     p->total_cap = out_off;
@@ -955,8 +955,8 @@ static bool takes_direct(const gc_plan_s* p) {
            p->cand_cap == p->cand_cap_alloc;
 }
 
-// The control block as the self-cleaning kernels see it (see CleanArgs): up to three early sections.
-static CleanArgs clean_args(const gc_plan_s* p, void* workspace, int route, bool expect_clean) {
+// The control block as the fused kernels see it (see CleanArgs): up to two early sections.
+static CleanArgs clean_args(const gc_plan_s* p, void* workspace, int route, uint32_t mode) {
     CleanArgs c{};
     c.ctrl = reinterpret_cast<uint4*>(workspace);
     c.ctrl_units = (uint32_t)(p->control_bytes / 16);
@@ -964,13 +964,13 @@ static CleanArgs clean_args(const gc_plan_s* p, void* workspace, int route, bool
     if (route == GC_ROUTE_TOPK_ONE) {
         range(0, p->off_hist5, sizeof(uint32_t) * kHistBins);                 // coarse sample histogram
         range(1, p->off_fine, sizeof(uint32_t) * (size_t)kFineBins);          // fine sample histogram
-        range(2, p->off_age, sizeof(uint32_t) * 1024);                        // arrivals per SM
     } else {
-        range(0, p->off_shist, sizeof(uint32_t) * (size_t)kHistBins * p->T);  // coarse sample histogram per tensor
+        range(0, p->off_shist, p->off_bhist - p->off_shist);                  // coarse sample histogram per tensor
     }
+    c.redo[0] = (uint32_t)(p->off_hist / 16); c.redo[1] = (uint32_t)(p->off_hist5 / 16);      // histograms, look-back words
     c.mark = 0xC1EA9B10C5ull ^ ((unsigned long long)p->control_bytes << 24) ^ ((unsigned long long)route << 56) ^
              (unsigned long long)p->total_n;
-    c.expect_clean = expect_clean ? 1u : 0u;
+    c.mode = mode;
     return c;
 }
 
@@ -1005,7 +1005,7 @@ static int compress_route(const gc_plan_s* p) {
 
 // Argument block of the many-tensor kernel for one worker's buffers and a given geometry.
 static MultiArgs multi_args(const gc_plan_s* p, const MultiGeom& mg, const void* grad, float* residual,
-                            uint32_t* out_idx, float* out_val, uint32_t* out_count, void* workspace, bool expect_clean) {
+                            uint32_t* out_idx, float* out_val, uint32_t* out_count, void* workspace, uint32_t clean_mode) {
     char* wb = static_cast<char*>(workspace);
     WsView ws = view(p, workspace);
     WsView gws = ws;                 // redo of failed tensors: own records, gated by the main ones
@@ -1028,7 +1028,7 @@ static MultiArgs multi_args(const gc_plan_s* p, const MultiGeom& mg, const void*
     ma.tile_cnt = reinterpret_cast<uint32_t*>(wb + p->off_tinfo);
     ma.skeys = reinterpret_cast<uint4*>(wb + p->off_skeys);
     ma.ws = ws; ma.gws = gws;
-    ma.cl = clean_args(p, workspace, GC_ROUTE_TOPK_MANY, expect_clean);
+    ma.cl = clean_args(p, workspace, GC_ROUTE_TOPK_MANY, clean_mode);
     return ma;
 }
 
@@ -1051,6 +1051,7 @@ static ThrMultiArgs thr_multi_args(const gc_plan_s* p, const MultiGeom& mg, cons
     ta.tile_cnt = reinterpret_cast<uint32_t*>(wb + p->off_tinfo);
     ta.tsel = reinterpret_cast<TensorSel*>(wb + p->off_ssel);
     ta.ws = view(p, workspace);
+    ta.cl = clean_args(p, workspace, GC_ROUTE_THRESHOLD_MANY, kCleanSelf);
     return ta;
 }
 
@@ -1074,14 +1075,18 @@ static int compress_impl(gc_plan_t* p, const void* grad_any, bool bf16, float* r
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     WsView ws = view(p, workspace);
     const int route = compress_route(p);
-    // The one-tensor top-k kernel leaves the control block as the next launch needs it; when the
-    // caller has promised that nobody else touches the workspace, the clearing launch is skipped
-    // for a workspace that kernel ran on last (the kernel checks a mark in the header and leaves
-    // with GC_E_INVALID if the promise was broken).
+    // The fused top-k kernels leave the control block as the next launch needs it; when the
+    // caller has promised that nobody else touches the workspace, a workspace that such a kernel ran
+    // on last is not cleared at all (the kernel checks a mark in the header and leaves with
+    // GC_E_INVALID if the promise was broken).  Without the promise the fused kernels, those of
+    // threshold mode included, clear the block themselves; a clearing launch is left in front of a private
+    // workspace's first call and of the other routes.
     const bool self_cleaning = route == GC_ROUTE_TOPK_ONE || route == GC_ROUTE_TOPK_MANY;
     const bool direct = route == GC_ROUTE_TOPK_ONE && takes_direct(p);
     const bool kept_clean = take_clean(p, workspace) && p->ws_private && self_cleaning;
-    if (!kept_clean) {
+    const bool clears_itself = (self_cleaning && !p->ws_private) || route == GC_ROUTE_THRESHOLD_ONE || route == GC_ROUTE_THRESHOLD_MANY;
+    const uint32_t clean_mode = kept_clean ? kCleanExpected : clears_itself ? kCleanSelf : kCleanDone;
+    if (clean_mode == kCleanDone) {
         Timed tm(p, s, GC_K_CLEAR_CTRL);
         const size_t n16 = (direct ? offsetof(DirectScratch, list) : p->control_bytes) / 16;             // (multiples of 256)
         const int gc = (int)std::min<size_t>((n16 + kBlock - 1) / kBlock, (size_t)p->sm_count * 8);
@@ -1110,6 +1115,7 @@ static int compress_impl(gc_plan_t* p, const void* grad_any, bool bf16, float* r
         ta.tile_cnt = reinterpret_cast<uint32_t*>(wb + p->off_tinfo);
         ta.seg_tot = reinterpret_cast<uint32_t*>(wb + p->off_rowseg);
         ta.ws = ws;
+        ta.cl = clean_args(p, workspace, GC_ROUTE_THRESHOLD_ONE, clean_mode);
         void* args[] = {&ta};
         Timed tm(p, s, GC_K_FUSED);
         GC_CUDA(p, cudaLaunchCooperativeKernel((const void*)k_threshold_single, dim3(p->thr_grid), dim3(kBlock),
@@ -1175,7 +1181,8 @@ static int compress_impl(gc_plan_t* p, const void* grad_any, bool bf16, float* r
         DirectArgs da{};
         da.g = grad_any; da.r = residual; da.n = (uint32_t)p->total_n; da.k = p->desc[0].k; da.out_idx = out_idx; da.out_val = out_val;
         da.out_count = out_count; da.s = reinterpret_cast<DirectScratch*>(workspace);
-        da.mark = clean_args(p, workspace, GC_ROUTE_TOPK_ONE, false).mark + 1u; da.expect_clean = kept_clean ? 1u : 0u;
+        da.mark = clean_args(p, workspace, GC_ROUTE_TOPK_ONE, kCleanDone).mark + 1u; da.expect_clean = kept_clean ? 1u : 0u;
+        da.clear_first = clean_mode == kCleanSelf ? 1u : 0u;
         const DirectGeom dg = direct_geometry(da.n, p->sm_count);
         note_clean(p, workspace);
         void* args[] = {&da};
@@ -1197,12 +1204,12 @@ static int compress_impl(gc_plan_t* p, const void* grad_any, bool bf16, float* r
         sa.srank_hi = p->single_srank_hi; sa.srank_mid = p->single_srank_mid; sa.mid_cap = (uint32_t)kSingleMidCap;
         sa.mid = reinterpret_cast<uint2*>(wb + p->off_mid);
         sa.fine = reinterpret_cast<uint32_t*>(wb + p->off_fine);
-        sa.age = reinterpret_cast<uint32_t*>(wb + p->off_age);
+        sa.start = reinterpret_cast<uint2*>(wb + p->off_start);
         sa.tile_cnt = reinterpret_cast<uint32_t*>(wb + p->off_tinfo);
         sa.seg_tot = reinterpret_cast<uint32_t*>(wb + p->off_rowseg);
         sa.tile_eq = sa.tile_cnt + nt; sa.seg_eq = sa.seg_tot + kSingleMaxT * 20;
         sa.ws = ws; sa.gws = gws;
-        sa.cl = clean_args(p, workspace, GC_ROUTE_TOPK_ONE, kept_clean);
+        sa.cl = clean_args(p, workspace, GC_ROUTE_TOPK_ONE, clean_mode);
         note_clean(p, workspace);
         void* args[] = {&sa};
         Timed tm(p, s, GC_K_FUSED);
@@ -1218,7 +1225,7 @@ static int compress_impl(gc_plan_t* p, const void* grad_any, bool bf16, float* r
         MultiGeom mg;
         mg.G = p->multi_grid; mg.per = p->multi_per; mg.pool = p->multi_pool; mg.full = p->multi_full;
         mg.ntab = p->multi_ntab; mg.smem = p->multi_smem;
-        MultiArgs ma = multi_args(p, mg, grad_any, residual, out_idx, out_val, out_count, workspace, kept_clean);
+        MultiArgs ma = multi_args(p, mg, grad_any, residual, out_idx, out_val, out_count, workspace, clean_mode);
         note_clean(p, workspace);
         void* args[] = {&ma};
         Timed tm(p, s, GC_K_FUSED);
@@ -1368,15 +1375,16 @@ int gc_compress_workers(gc_plan_t* p, uint32_t W, const float* const* grads, flo
         WorkersArgs wa;
         ThrWorkersArgs ta;
         wa.W = ta.W = wn; wa.G = ta.G = mg.G;
-        // the clearing launch is skipped only if every workspace of this launch was left clean
+        // private workspaces: a clearing launch in front unless every workspace of this launch was left clean
         bool kept_clean = p->ws_private && topk_multi;
         for (uint32_t i = 0; i < wn; ++i) kept_clean = take_clean(p, workspaces[w0 + i]) && kept_clean;
+        const uint32_t clean_mode = kept_clean ? kCleanExpected : topk_multi && p->ws_private ? kCleanDone : kCleanSelf;
         for (uint32_t i = 0; i < wn; ++i) {
             const uint32_t w = w0 + i;
             cm.p[i] = reinterpret_cast<uint4*>(workspaces[w]);
             uint32_t* const oc = out_count ? out_count[w] : nullptr;
             if (topk_multi) {
-                wa.per[i] = multi_args(p, mg, grads[w], residuals[w], out_idx[w], out_val[w], oc, workspaces[w], kept_clean);
+                wa.per[i] = multi_args(p, mg, grads[w], residuals[w], out_idx[w], out_val[w], oc, workspaces[w], clean_mode);
                 note_clean(p, workspaces[w]);
             }
             if (!topk_multi) ta.per[i] = thr_multi_args(p, mg, grads[w], residuals[w], out_idx[w], out_val[w], oc, workspaces[w]);
@@ -1389,7 +1397,7 @@ int gc_compress_workers(gc_plan_t* p, uint32_t W, const float* const* grads, flo
             cm.p[i] = nullptr;
             if (topk_multi) wa.per[i] = wa.per[0]; else ta.per[i] = ta.per[0];
         }
-        if (!kept_clean) {
+        if (clean_mode == kCleanDone) {
             Timed tm(p, s, GC_K_CLEAR_CTRL);
             const size_t n16 = p->control_bytes / 16;
             const unsigned gx = (unsigned)std::min<size_t>((n16 + kBlock - 1) / kBlock, (size_t)p->sm_count * 8 / wn + 1);

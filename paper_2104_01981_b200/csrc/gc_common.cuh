@@ -1,8 +1,11 @@
 // Shared device-side definitions of libgc: tensor table, workspace layout, tile geometry,
 // warp/block scan helpers and the ordered-tile prefix exchange ("look-back").
 #pragma once
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include <utility>
 
 namespace gc {
 
@@ -46,7 +49,7 @@ struct TensorDesc {          // one per tensor, immutable, plan-owned device mem
     uint32_t ngroups;        // compaction groups of this tensor
     uint32_t kind;           // kKindRegular, or kKindSmall: the candidate path hands the whole tensor
                              // to one CTA that selects exactly on its own (no sample, no candidates)
-    uint32_t pad;
+    uint32_t reg;            // number among the tensors that are not small (and not empty)
 };
 constexpr uint32_t kKindRegular = 0u, kKindSmall = 1u;
 constexpr uint32_t kSmallMax = kTile - 3;     // tensors below this many elements always lie inside one tile,
@@ -399,41 +402,70 @@ __device__ __forceinline__ bool grid_barrier(WsHeader* hdr, uint32_t& passed, in
 // (the writers come after the barrier, so there is no ordering problem); the sections written
 // before the first barrier ("early": at most three ranges) are zeroed right after the barrier that
 // follows their last reader; the barrier counter is reset by the CTA that leaves last (an exit
-// counter in the header), which then sets a 64-bit mark.  When the host has skipped the clearing
-// launch (on the caller's promise that nobody else writes to the workspace), the kernel first
-// checks the mark and leaves at once if it is missing: no barrier is entered on a counter that
-// cannot be trusted.  G CTAs share the block, this is CTA b of them.
+// counter in the header), which then sets a 64-bit mark.  When the host relies on that (on the
+// caller's promise that nobody else writes to the workspace), the kernel first checks the mark and
+// leaves at once if it is missing: no barrier is entered on a counter that cannot be trusted.
+// Without the promise the launch clears the whole block itself, a slice per CTA, and nobody touches
+// it before all slices are done: that barrier cannot count in the block, so it is the cooperative
+// launch's own; the arrival stands here, the wait behind the loads of the sample (ClearWait).
+// Against a clearing launch in front: 161 tensors of 25.6M elements in all 102.4 -> 99.1 us, 110M in 199 tensors at 5 % 350.5 ->
+// 345.1, 1M elements with their decode 30.7 -> 28.8, threshold mode 110M 258.7 -> 256.4, eight 161-tensor workers 541.6 -> 536.4.
+// The sections that only the exact redo uses are left alone; the redo zeroes them before its barrier.
+// G CTAs share the block, this is CTA b of them.
+enum : uint32_t { kCleanDone = 0u,       // a launch in front has cleared the block
+                  kCleanExpected = 1u,   // the last launch left it clean: check the mark
+                  kCleanSelf = 2u };     // whatever is in it: this launch clears it
 struct CleanArgs {
     uint4* ctrl;                     // the control block (= the workspace), in 16-byte units
     uint32_t ctrl_units;             // its length
-    uint32_t early[3][2];            // [begin, end) in units of the sections written before the first barrier
+    uint32_t early[2][2];            // [begin, end) in units of the sections written before the first barrier
+    uint32_t redo[2];                // [begin, end) in units of the sections of the exact redo
     unsigned long long mark;         // what the header's mark reads after a launch that left the block clean
-    uint32_t expect_clean;           // the host skipped the clearing launch
+    uint32_t mode;                   // kClean...
+};
+// The wait that belongs to the arrival at the launch's barrier; the whole CTA calls, once or more often.
+struct ClearWait {
+    cooperative_groups::grid_group::arrival_token token{};
+    bool pending = false;            // (the same in every thread)
+    __device__ __forceinline__ void operator()() {
+        if (!pending) return;
+        cooperative_groups::this_grid().barrier_wait(std::move(token));
+        pending = false;
+    }
 };
 __device__ __forceinline__ unsigned long long* clean_mark_ptr(WsHeader* hdr) {
     return reinterpret_cast<unsigned long long*>(reinterpret_cast<uint32_t*>(hdr) + kHdrSigWord);
 }
 // First thing in the kernel (after anything that must see the CTAs in their order of arrival).
-// Returns false if the launch must end here.  Contains a block-wide barrier for CTA 0.
-__device__ __forceinline__ bool clean_begin(const CleanArgs& c, WsHeader* hdr, uint32_t G, uint32_t b, int tid) {
-    if (c.expect_clean != 0u && ld_cg(clean_mark_ptr(hdr)) != c.mark) {
+// Returns false if the launch must end here.  Contains a block-wide barrier for CTA 0, or (kCleanSelf) for
+// every CTA; `cleared` has to be waited for before anything else of the block is read or written.
+__device__ __forceinline__ bool clean_begin(const CleanArgs& c, WsHeader* hdr, uint32_t G, uint32_t b, int tid, ClearWait& cleared) {
+    if (c.mode == kCleanExpected && ld_cg(clean_mark_ptr(hdr)) != c.mark) {
         if (b == 0 && tid == 0) record_status(hdr, -1 /*GC_E_INVALID*/, 0xC1EA0000ull);
         return false;                // every CTA sees the same word
     }
+    const bool self = c.mode == kCleanSelf;
     const uint32_t per = (c.ctrl_units + G - 1) / G;
     const uint32_t u0 = max(b * per, 16u), u1 = min(c.ctrl_units, (b + 1u) * per);     // (the header is 16 units)
     for (uint32_t u = u0 + (uint32_t)tid; u < u1; u += kBlock) {
-        const bool is_early = (u >= c.early[0][0] && u < c.early[0][1]) || (u >= c.early[1][0] && u < c.early[1][1]) ||
-                              (u >= c.early[2][0] && u < c.early[2][1]);
-        if (!is_early) c.ctrl[u] = make_uint4(0u, 0u, 0u, 0u);
+        const bool is_early = (u >= c.early[0][0] && u < c.early[0][1]) || (u >= c.early[1][0] && u < c.early[1][1]);
+        if ((self || !is_early) && !(u >= c.redo[0] && u < c.redo[1])) c.ctrl[u] = make_uint4(0u, 0u, 0u, 0u);
     }
     if (b == 0) {                    // the header: all but the barrier's, the exit counter's and the mark's words
-        if (tid < 64 && tid != (int)kHdrBarrierWord && tid != (int)kHdrExitWord && tid != (int)kHdrSigWord &&
-            tid != (int)kHdrSigWord + 1)
+        if (tid < 64 && (self || (tid != (int)kHdrBarrierWord && tid != (int)kHdrExitWord && tid != (int)kHdrSigWord &&
+                                  tid != (int)kHdrSigWord + 1)))
             reinterpret_cast<uint32_t*>(hdr)[tid] = 0u;
         __syncthreads();
     }
+    if (self) {
+        cleared.token = cooperative_groups::this_grid().barrier_arrive();      // (a barrier of the block as well)
+        cleared.pending = true;
+    }
     return true;
+}
+// The sections of the exact redo; a grid barrier follows before they are used.
+__device__ __forceinline__ void clean_redo(const CleanArgs& c, uint32_t G, uint32_t b, int tid) {
+    for (uint32_t u = c.redo[0] + b * kBlock + (uint32_t)tid; u < c.redo[1]; u += G * kBlock) c.ctrl[u] = make_uint4(0u, 0u, 0u, 0u);
 }
 // After the first barrier: every CTA has read the mark, the block is in use.
 __device__ __forceinline__ void clean_in_use(WsHeader* hdr, uint32_t b, int tid) {
@@ -442,7 +474,7 @@ __device__ __forceinline__ void clean_in_use(WsHeader* hdr, uint32_t b, int tid)
 // After the barrier that follows the last reader of the early sections.
 __device__ __forceinline__ void clean_early(const CleanArgs& c, uint32_t G, uint32_t b, int tid) {
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
+    for (int q = 0; q < 2; ++q) {
         const uint32_t len = c.early[q][1] - c.early[q][0], per = (len + G - 1) / G;
         for (uint32_t u = c.early[q][0] + b * per + (uint32_t)tid; u < min(c.early[q][1], c.early[q][0] + (b + 1u) * per); u += kBlock)
             c.ctrl[u] = make_uint4(0u, 0u, 0u, 0u);

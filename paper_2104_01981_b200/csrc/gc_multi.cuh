@@ -53,8 +53,8 @@ struct MultiArgs {
     uint2* cand;                     // [gridDim.x * pool_cap]
     uint2* mid;                      // [T][kMultiMidCap] candidates inside the band bin of the threshold
     uint32_t* mid_n;                 // [T] their number (zeroed)
-    uint32_t* shist;                 // [T][kHistBins] coarse sample histogram (zeroed)
-    uint32_t* bhist;                 // [T][kHistBins] band histogram (zeroed)
+    uint32_t* shist;                 // [n_reg][kHistBins] coarse sample histogram (zeroed)
+    uint32_t* bhist;                 // [n_reg][kHistBins] band histogram (zeroed)
     uint32_t* tile_cnt;              // [ntiles] candidates above the band bin, per tile
     uint4* skeys;                    // [nstiles * kBlock] the sampled keys, one group of four per entry
     WsView ws, gws;
@@ -116,7 +116,8 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     WsHeader* hdr = a.ws.hdr;
     uint32_t passed = 0, n_stamp = 0;
-    if (!clean_begin(a.cl, hdr, G, b, tid)) return;
+    ClearWait cleared;
+    if (!clean_begin(a.cl, hdr, G, b, tid, cleared)) return;
     // The CTAs launched last are the youngest on their SMs and advance the slowest (see RowMap in
     // the one-tensor kernel), so whatever the full runs leave over is spread evenly over them.
     uint32_t first, last;
@@ -156,7 +157,7 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
         TensorDesc d;
         for (uint32_t st = sfirst; st < slast;) {
             if (t == 0xFFFFFFFFu || st >= d.stile0 + d.nstiles) {
-                if (t != 0xFFFFFFFFu) flush_hist(sm, a.shist + (size_t)t * kHistBins, 1 << level_bits(0));
+                if (t != 0xFFFFFFFFu) { cleared(); flush_hist(sm, a.shist + (size_t)d.reg * kHistBins, 1 << level_bits(0)); }
                 __syncthreads();
                 t = a.ntab ? owner(tab_stile0, st) : find_tensor<SampleSpace>(a.desc, a.T, st);
                 d = a.desc[t];
@@ -214,8 +215,10 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
             }
             st += nb;
         }
-        if (t != 0xFFFFFFFFu) flush_hist(sm, a.shist + (size_t)t * kHistBins, 1 << level_bits(0));
+        cleared();
+        if (t != 0xFFFFFFFFu) flush_hist(sm, a.shist + (size_t)d.reg * kHistBins, 1 << level_bits(0));
     }
+    cleared();
     grid_arrive(hdr);
     // small tensors need nothing from anyone: they fill the wait (CTAs from the top take them)
     for (uint32_t q8 = G - 1u - b; q8 * kWarps < a.n_tiny; q8 += G) {        // tiny ones: a warp each, eight at a time
@@ -259,7 +262,7 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
                 // (a sample too small for that margin: the largest sampled key bounds the band instead)
                 const uint32_t want[3] = {d.srank, hi >= 1.0f ? (uint32_t)hi : 1u, max(1u, (uint32_t)ceilf(ks))};
                 Picked pk[3];
-                block_select_multi<(1 << level_bits(0)), 3>(sm, a.shist + (size_t)cur * kHistBins, want, pk);
+                block_select_multi<(1 << level_bits(0)), 3>(sm, a.shist + (size_t)d.reg * kHistBins, want, pk);
                 if (pk[0].ok) tau = pk[0].bin << level_shift(0);
                 if (pk[0].ok && d.nstiles <= kRefineTiles) {
                     // second radix level of the lower bracket and of the guess over the kept sample keys:
@@ -322,7 +325,7 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
         for (uint32_t tile = first; tile < last; ++tile) {
             const uint32_t i = tile - first;
             if (cur == 0xFFFFFFFFu || tile >= d.tile0 + d.ntiles) {
-                if (open) flush_hist(sm, a.bhist + (size_t)cur * kHistBins, 2048);
+                if (open) flush_hist(sm, a.bhist + (size_t)d.reg * kHistBins, 2048);
                 open = false;
                 cur = a.ntab ? owner(tab_tile0, tile) : find_tensor(a.desc, a.T, tile);
                 d = a.desc[cur];
@@ -338,6 +341,7 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
                         s[SG_BASE0] = (d.off & ~3u) + (tile - d.tile0) * (uint32_t)kTile; s[SG_BEGIN] = tg0.lo;
                         s[SG_TAU] = tau; s[SG_TAUZ] = tau_z; s[SG_SHIFT] = (uint32_t)shift;
                         s[SG_OK] = 1u; s[SG_OUT] = d.out_off; s[SG_K] = d.k;
+                        s[SG_A] = d.reg;               // (until the band bin is known)
                     }
                     ++nseg;
                     open = true;
@@ -454,7 +458,7 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
                 }
             }
         }
-        if (open) flush_hist(sm, a.bhist + (size_t)cur * kHistBins, 2048);
+        if (open) flush_hist(sm, a.bhist + (size_t)d.reg * kHistBins, 2048);
         if (__syncthreads_or(block_overflow ? 1 : 0)) {
             if (tid == 0) atomicExch(&hdr->overflow, 1u);
         }
@@ -481,7 +485,7 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
         for (uint32_t sidx = (uint32_t)warp; sidx < nseg; sidx += kWarps) {      // a warp per segment, all at once
             uint32_t* s = seg + (size_t)sidx * kSegWords;
             const uint32_t t = s[SG_T];
-            const Picked pa = warp_select_2048(a.bhist + (size_t)t * kHistBins, s[SG_K], lane);
+            const Picked pa = warp_select_2048(a.bhist + (size_t)s[SG_A] * kHistBins, s[SG_K], lane);
             const bool ok = pa.ok && pa.count <= kMultiMidCap;
             if (lane == 0) {
                 s[SG_A] = pa.bin; s[SG_ABOVE] = pa.above; s[SG_M] = pa.count; s[SG_OK] = ok ? 1u : 0u;
@@ -770,6 +774,7 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
 
     // ---------------------------------------------------------------- exact redo (rare)
     // of the flagged tensors, or of all of them after an overflow: r holds a = g + r for them again
+    clean_redo(a.cl, G, b, tid);
     if (!grid_barrier(hdr, passed, &sm.ok, G)) return;
     phase_stamp(hdr, n_stamp, b);
     hist_body<0, SRC_RESID>(sm, a.desc, a.T, a.ntiles, nullptr, a.r, a.gws, G, b);

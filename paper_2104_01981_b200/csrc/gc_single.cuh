@@ -75,22 +75,35 @@ struct RowMap {
     }
 };
 
-// This CTA's arrival number on its SM (0 = it got there first) and the SM's number; the counters
-// are zeroed before the launch.
-__device__ __forceinline__ uint32_t note_age(uint32_t* per_sm, uint32_t& smid) {
-    asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
-    return atomicAdd(per_sm + (smid & 1023u), 1u);
+// Where and when this CTA started: the SM's number and the SM's cycle counter.
+__device__ __forceinline__ uint2 note_start() {
+    uint2 s;
+    asm volatile("mov.u32 %0, %%smid;" : "=r"(s.x));
+    asm volatile("mov.u32 %0, %%clock;" : "=r"(s.y));
+    return s;
 }
-// Column of this CTA once every CTA has called note_age (after a grid barrier): by age, oldest
-// first, column = age x gA + SM number.  That is a one-to-one assignment only if SMs 0..gA-1
-// hold three CTAs each; every CTA checks the same counters and otherwise keeps column b.
-// Called by the whole CTA (contains a block-wide vote).
-__device__ __forceinline__ uint32_t aged_column(const RowMap& rm, const uint32_t* per_sm, uint32_t age, uint32_t smid,
-                                                uint32_t G, uint32_t b, int tid) {
-    const bool fits = (uint32_t)tid >= rm.gA || ld_cg(per_sm + tid) == 3u;
-    const bool none_beyond = (uint32_t)tid < rm.gA || tid >= 1024 || ld_cg(per_sm + tid) == 0u;
-    const bool aged = __syncthreads_and(fits && none_beyond) && rm.gA * 3u == G && rm.gA <= (uint32_t)kBlock;
-    return aged ? min(age, 2u) * rm.gA + smid : b;
+// Column of this CTA once every CTA has written down its start (before a grid barrier): its age is the number
+// of CTAs of its SM that started before it, and column = age x gA + SM number, oldest first.  That is a
+// one-to-one assignment only if SMs 0..gA-1 hold three CTAs each; every CTA checks the same table and
+// otherwise keeps column b.  Called by the whole CTA; count[] (1024 words of shared memory) is zero before and after.
+__device__ __forceinline__ uint32_t aged_column(const RowMap& rm, const uint2* start, uint2 mine, uint32_t G, uint32_t b,
+                                                uint32_t* count, uint32_t* s_age, int tid) {
+    if (rm.gA * 3u != G || rm.gA > (uint32_t)kBlock) return b;           // one class of columns
+    if (tid == 0) *s_age = 0u;
+    __syncthreads();
+    for (uint32_t c = tid; c < G; c += kBlock) {
+        const uint2 s = ld_cg(start + c);
+        atomicAdd(&count[s.x & 1023u], 1u);
+        const int later = (int)(mine.y - s.y);                           // (the counter wraps)
+        if (s.x == mine.x && c != b && (later > 0 || (later == 0 && c < b))) atomicAdd(s_age, 1u);
+    }
+    __syncthreads();
+    const bool aged = __syncthreads_and((uint32_t)tid >= rm.gA || count[tid] == 3u);      // (3 gA = G: none beyond)
+    const uint32_t age = *s_age;
+    __syncthreads();
+    for (uint32_t i = tid; i < 1024u; i += kBlock) count[i] = 0u;
+    __syncthreads();
+    return aged ? min(age, 2u) * rm.gA + mine.x : b;
 }
 
 struct SingleArgs {
@@ -110,7 +123,7 @@ struct SingleArgs {
     uint2* mid;                      // [mid_cap] candidates inside the band bin of the threshold
     uint32_t* hist5;                 // [0] coarse sample histogram, [2] band histogram,
                                      // [3][0] short-list length, [4] keys inside a counted band (all zeroed)
-    uint32_t* age;                   // [1024] CTAs that have arrived on every SM (zeroed)
+    uint2* start;                    // [gridDim.x] SM and cycle at which every CTA started
     uint32_t* fine;                  // [kFineBins] fine sample histogram (zeroed)
     uint32_t* tile_cnt;              // [ntiles] candidates above the band bin, per tile
     uint32_t* seg_tot;               // [maxt][ceil(G/32)] the same summed over each run of 32 CTAs of a row (zeroed)
@@ -419,13 +432,14 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
     WsHeader* hdr = a.ws.hdr;
     uint32_t passed = 0, n_stamp = 0;
     const RowMap& rm = a.rows;
-    __shared__ uint32_t s_age[2];
-    // This CTA's age among the CTAs of its SM = its arrival number at the SM's counter, taken
-    // first thing: the number has to reflect the order in which the CTAs really started (a load
-    // in front of it was measured to cost the fold pass 10 us: the shares no longer matched).
-    uint32_t my_age = 0, my_sm = 0;
-    if (tid == 0) my_age = note_age(a.age, my_sm);
-    if (!clean_begin(a.cl, hdr, G, b, tid)) return;
+    __shared__ uint32_t s_age;
+    __shared__ uint2 s_start;
+    // When this CTA started, taken first thing: the ages have to reflect the order in which the CTAs really
+    // started (taken behind a load they were measured to cost the fold pass 10 us: the shares no longer matched).
+    uint2 my_start = make_uint2(0u, 0u);
+    if (tid == 0) my_start = note_start();
+    ClearWait cleared;
+    if (!clean_begin(a.cl, hdr, G, b, tid, cleared)) return;
     for (int i = tid; i < 2048; i += kBlock) sm.hist[i] = 0u;
     for (uint32_t i = tid; i < a.maxt * kWarps; i += kBlock) rec2[i] = 0u;
     for (uint32_t i = tid; i < a.maxt; i += kBlock) row_mid[i] = 0u;
@@ -463,7 +477,8 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
 #pragma unroll
             for (int e = 0; e < 4; ++e) skey[q][e] = key_of(__fadd_rn(gv[e], rv[e]));
         }
-        if (tid == 0) { s_age[0] = my_age; s_age[1] = my_sm; }
+        if (tid == 0) { s_start = my_start; a.start[b] = my_start; }
+        cleared();                                       // (the loads above are under way meanwhile)
         __syncthreads();
 #pragma unroll
         for (int q = 0; q < kMaxOwn; ++q)
@@ -489,7 +504,7 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
         phase_stamp(hdr, n_stamp);
         clean_in_use(hdr, b, tid);
         {
-            col = aged_column(rm, a.age, s_age[0], s_age[1], G, b, tid);
+            col = aged_column(rm, a.start, s_start, G, b, sm.hist, &s_age, tid);
             n_own = rm.rows_of(col);
             while (n_own > 0u && rm.tile_of(n_own - 1u, col) >= a.ntiles) --n_own;
             myseg = col / 32u;
@@ -664,7 +679,7 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
     flush_hist(sm, a.hist5 + 2 * kHistBins, 2048);
     if (!grid_barrier(hdr, passed, &sm.ok)) return;
     phase_stamp(hdr, n_stamp);
-    // the three early sections have had their last reader (the bracket, right after the first
+    // the early sections have had their last reader (the bracket, right after the first
     // barrier): they are zeroed for the next launch
     clean_early(a.cl, G, b, tid);
 
@@ -1016,6 +1031,7 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
             a.r[pr.x] = __uint_as_float(pr.y);
         }
     }
+    clean_redo(a.cl, G, b, tid);
     if (!grid_barrier(hdr, passed, &sm.ok)) return;
     phase_stamp(hdr, n_stamp);
     hist_body<0, SRC_RESID>(sm, a.desc, 1u, a.ntiles, nullptr, a.r, a.gws);

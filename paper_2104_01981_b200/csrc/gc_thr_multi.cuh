@@ -36,11 +36,12 @@ struct ThrMultiArgs {
     float* out_val;
     uint32_t* out_count;
     uint2* cand;                     // [gridDim.x * pool_cap]
-    uint32_t* shist;                 // [T][kHistBins] coarse sample histogram (zeroed)
+    uint32_t* shist;                 // [n_reg][kHistBins] coarse sample histogram (zeroed)
     uint4* skeys;                    // [nstiles * kBlock] the sampled keys
     uint32_t* tile_cnt;              // [ntiles] hits per tile
     TensorSel* tsel;                 // [T] .T receives tau
     WsView ws;
+    CleanArgs cl;                    // (the launch clears the control block itself)
 };
 
 // A tiny tensor (at most kTinyMaxN elements, sampled in full, rank at most kTinyMaxK) by one warp:
@@ -231,6 +232,8 @@ static __device__ __forceinline__ void threshold_multi_body(const ThrMultiArgs& 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     WsHeader* hdr = a.ws.hdr;
     uint32_t passed = 0, n_stamp = 0;
+    ClearWait cleared;
+    if (!clean_begin(a.cl, hdr, G, b, tid, cleared)) return;
     const uint32_t first = min(a.ntiles, b * a.per), last = min(a.ntiles, first + a.per);
     const uint32_t ntl = last - first;
     for (int i = tid; i < 2048; i += kBlock) sm.hist[i] = 0u;
@@ -259,7 +262,7 @@ static __device__ __forceinline__ void threshold_multi_body(const ThrMultiArgs& 
         TensorDesc d;
         for (uint32_t st = sfirst; st < slast;) {
             if (t == 0xFFFFFFFFu || st >= d.stile0 + d.nstiles) {
-                if (t != 0xFFFFFFFFu) flush_hist(sm, a.shist + (size_t)t * kHistBins, 1 << level_bits(0));
+                if (t != 0xFFFFFFFFu) { cleared(); flush_hist(sm, a.shist + (size_t)d.reg * kHistBins, 1 << level_bits(0)); }
                 __syncthreads();
                 t = a.ntab ? owner(tab_stile0, st) : find_tensor<SampleSpace>(a.desc, a.T, st);
                 d = a.desc[t];
@@ -311,8 +314,10 @@ static __device__ __forceinline__ void threshold_multi_body(const ThrMultiArgs& 
             }
             st += nb;
         }
-        if (t != 0xFFFFFFFFu) flush_hist(sm, a.shist + (size_t)t * kHistBins, 1 << level_bits(0));
+        cleared();
+        if (t != 0xFFFFFFFFu) flush_hist(sm, a.shist + (size_t)d.reg * kHistBins, 1 << level_bits(0));
     }
+    cleared();
     grid_arrive(hdr);
     for (uint32_t q8 = G - 1u - b; q8 * kWarps < a.n_tiny; q8 += G) {        // tiny tensors: a warp each, eight at a time
         const uint32_t q = q8 * kWarps + (uint32_t)warp;
@@ -340,7 +345,7 @@ static __device__ __forceinline__ void threshold_multi_body(const ThrMultiArgs& 
         uint32_t tau = 0xFFFFFFFFu;
         const uint32_t want[1] = {d.srank};
         Picked p0[1];
-        block_select_multi<(1 << level_bits(0)), 1>(sm, a.shist + (size_t)t * kHistBins, want, p0);
+        block_select_multi<(1 << level_bits(0)), 1>(sm, a.shist + (size_t)d.reg * kHistBins, want, p0);
         bool ok = p0[0].ok;
         const uint4* sk = a.skeys + (size_t)d.stile0 * kBlock;
         const uint32_t nk = d.nstiles * kBlock;
@@ -610,6 +615,7 @@ static __device__ __forceinline__ void threshold_multi_body(const ThrMultiArgs& 
             a.r[pr.x] = __uint_as_float(pr.y);
         }
     }
+    clean_redo(a.cl, G, b, tid);
     if (!grid_barrier(hdr, passed, &sm.ok, G)) return;
     phase_stamp(hdr, n_stamp, b);
     threshold_emit_body<false, true>(a.desc, a.T, a.ntiles, nullptr, a.r, a.out_idx, a.out_val, a.out_count, a.ws,

@@ -44,6 +44,7 @@ struct ThrSingleArgs {
     uint32_t* tile_cnt;              // [ntiles] hits per tile
     uint32_t* seg_tot;               // [maxt][ceil(G/32)] hits per run of 32 CTAs of a row (zeroed)
     WsView ws;
+    CleanArgs cl;                    // (the launch clears the control block itself)
 };
 
 // (three CTAs per SM: 80 registers and no spills beat four at 64 registers, see k_topk_single)
@@ -63,6 +64,8 @@ k_threshold_single(const __grid_constant__ ThrSingleArgs a) {
     const TensorDesc& d = a.d;
     WsHeader* hdr = a.ws.hdr;
     uint32_t passed = 0, n_stamp = 0;
+    ClearWait cleared;
+    if (!clean_begin(a.cl, hdr, G, b, tid, cleared)) return;
     const uint32_t n_own = b < a.ntiles ? (a.ntiles - b + G - 1) / G : 0u;
     const uint32_t nseg = (G + 31u) / 32u, myseg = b / 32u;
     for (int i = tid; i < 2048; i += kBlock) sm.hist[i] = 0u;
@@ -115,6 +118,7 @@ k_threshold_single(const __grid_constant__ ThrSingleArgs a) {
     // counts what lies in the bin of its own sample that holds four times the rank's share, or above (with
     // every key counted the phase takes 10 us longer on 110M elements).  Should the rank's bin turn out to
     // lie below the highest floor of any CTA, what the CTAs left out of that bin is counted after the barrier.
+    cleared();
     uint32_t floor_bin = 0;
     if (a.sample_rounds > 1u) {                            // (a short sample: finding the floor takes longer than it saves)
         __syncthreads();
@@ -429,6 +433,7 @@ k_threshold_single(const __grid_constant__ ThrSingleArgs a) {
             a.r[pr.x] = __uint_as_float(pr.y);
         }
     }
+    clean_redo(a.cl, G, b, tid);
     if (!grid_barrier(hdr, passed, &sm.ok)) return;
     phase_stamp(hdr, n_stamp);
     threshold_emit_body<false>(a.desc, 1u, a.ntiles, nullptr, a.r, a.out_idx, a.out_val, a.out_count, a.ws,
