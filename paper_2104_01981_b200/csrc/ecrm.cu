@@ -1,7 +1,7 @@
 // Erasure-coded embedding-table hot path: summation encoder / subtraction decoder over whole
 // shards, the optimizer step that emits entry and state differences, the parity host's
 // scatter-add of those differences, and degraded reads.  Everything is bound by HBM traffic:
-// rows are 512-byte (dim = 128) contiguous runs, one warp moves one row with 128-bit accesses.
+// rows are contiguous runs (512 bytes at dim = 128) moved with 128-bit accesses by a group of lanes.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -10,7 +10,6 @@
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kWarpsPerCta = kThreads / 32;
 
 struct PtrTable { const float* p[ECRM_MAX_K]; };
 struct RowTable { const uint32_t* p[ECRM_MAX_K]; };
@@ -58,20 +57,45 @@ __global__ void __launch_bounds__(kThreads) k_ecrm_combine(PtrTable t, uint32_t 
     }
 }
 
-// One warp per updated row.  OPT: ECRM_ADAGRAD or ECRM_MOMENTUM.
+// Rows are dealt out to groups of LPR lanes, a float4 per lane: a whole warp for rows of more than 64
+// floats, 16 or 8 lanes for shorter ones, so that two or four rows are in flight per warp and no lane idles
+// (a warp per row whatever its length left three lanes of four without work at 32 floats; step + parity of
+// 200,003 rows: 32 floats 85.7 -> 49.7 us, 64 floats 100.9 -> 80.9, 128 floats 157.1 -> 155.5 = 5.9 TB/s;
+// degraded reads of 200,000 rows of 32 floats 48.8 -> 27.3).  HBM bounds it; the number of the next row is asked
+// for under the current one, so a row costs one round trip to memory instead of two.
+template <int LPR>
+struct RowGroups {
+    uint32_t first, step, lane;
+    __device__ __forceinline__ RowGroups()
+        : first((blockIdx.x * kThreads + threadIdx.x) / LPR), step(gridDim.x * (kThreads / LPR)), lane(threadIdx.x % LPR) {}
+};
+
 template <int OPT>
+__device__ __forceinline__ void optimizer_step(float g, float e, float s, float lr, float hyper, float& en, float& sn) {
+    if (OPT == ECRM_ADAGRAD) {
+        sn = __fadd_rn(s, __fmul_rn(g, g));
+        const float step = __fdiv_rn(lr, __fsqrt_rn(__fadd_rn(sn, hyper)));
+        en = __fsub_rn(e, __fmul_rn(step, g));
+    } else {
+        sn = __fadd_rn(__fmul_rn(hyper, s), g);
+        en = __fsub_rn(e, __fmul_rn(lr, sn));
+    }
+}
+
+// OPT: ECRM_ADAGRAD or ECRM_MOMENTUM.
+template <int OPT, int LPR>
 __global__ void __launch_bounds__(kThreads) k_ecrm_rows_step(uint32_t m, const uint32_t* __restrict__ rows,
                                                               const float* __restrict__ grad, float* __restrict__ entry,
                                                               float* __restrict__ state, uint64_t n_rows, uint32_t dim4,
                                                               float lr, float hyper, float* __restrict__ d_entry,
                                                               float* __restrict__ d_state, uint32_t* bad_rows) {
-    const int lane = threadIdx.x & 31;
-    const uint64_t warp = (uint64_t)blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5);
-    const uint64_t nwarps = (uint64_t)gridDim.x * kWarpsPerCta;
-    for (uint64_t j = warp; j < m; j += nwarps) {
-        const uint32_t row = __ldg(rows + j);
+    const RowGroups<LPR> rg;
+    uint32_t next = rg.first < m ? __ldg(rows + rg.first) : 0u;
+    for (uint64_t j = rg.first; j < m; j += rg.step) {
+        const uint32_t row = next;
+        if (j + rg.step < m) next = __ldg(rows + j + rg.step);
         if (row >= n_rows) {
-            if (lane == 0 && bad_rows != nullptr) atomicAdd(bad_rows, 1u);
+            if (rg.lane == 0 && bad_rows != nullptr) atomicAdd(bad_rows, 1u);
             continue;
         }
         const float4* g4 = reinterpret_cast<const float4*>(grad) + j * dim4;
@@ -79,7 +103,8 @@ __global__ void __launch_bounds__(kThreads) k_ecrm_rows_step(uint32_t m, const u
         float4* s4 = reinterpret_cast<float4*>(state) + (uint64_t)row * dim4;
         float4* de4 = reinterpret_cast<float4*>(d_entry) + j * dim4;
         float4* ds4 = reinterpret_cast<float4*>(d_state) + j * dim4;
-        for (uint32_t c = lane; c < dim4; c += 32) {
+#pragma unroll 1
+        for (uint32_t c = rg.lane; c < dim4; c += LPR) {
             const float4 g = __ldcs(g4 + c);
             const float4 e = e4[c];
             const float4 s = s4[c];
@@ -87,14 +112,7 @@ __global__ void __launch_bounds__(kThreads) k_ecrm_rows_step(uint32_t m, const u
             float en[4], sn[4], de[4], ds[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                if (OPT == ECRM_ADAGRAD) {
-                    sn[q] = __fadd_rn(sv[q], __fmul_rn(gv[q], gv[q]));
-                    const float step = __fdiv_rn(lr, __fsqrt_rn(__fadd_rn(sn[q], hyper)));
-                    en[q] = __fsub_rn(ev[q], __fmul_rn(step, gv[q]));
-                } else {
-                    sn[q] = __fadd_rn(__fmul_rn(hyper, sv[q]), gv[q]);
-                    en[q] = __fsub_rn(ev[q], __fmul_rn(lr, sn[q]));
-                }
+                optimizer_step<OPT>(gv[q], ev[q], sv[q], lr, hyper, en[q], sn[q]);
                 de[q] = __fsub_rn(en[q], ev[q]);
                 ds[q] = __fsub_rn(sn[q], sv[q]);
             }
@@ -107,8 +125,8 @@ __global__ void __launch_bounds__(kThreads) k_ecrm_rows_step(uint32_t m, const u
 }
 
 // The optimizer step and the parity update of the same rows in one pass, for a data shard whose
-// parity lives on the same GPU: the two differences stay in registers.  One warp per row.
-template <int OPT>
+// parity lives on the same GPU: the two differences stay in registers.
+template <int OPT, int LPR>
 __global__ void __launch_bounds__(kThreads) k_ecrm_rows_step_parity(uint32_t m, const uint32_t* __restrict__ rows,
                                                                      const uint32_t* __restrict__ prow,
                                                                      const float* __restrict__ grad, float* __restrict__ entry,
@@ -116,13 +134,14 @@ __global__ void __launch_bounds__(kThreads) k_ecrm_rows_step_parity(uint32_t m, 
                                                                      float* __restrict__ p_entry, float* __restrict__ p_state,
                                                                      uint64_t n_prows, uint32_t dim4, float lr, float hyper,
                                                                      uint32_t* bad_rows) {
-    const int lane = threadIdx.x & 31;
-    const uint64_t warp = (uint64_t)blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5);
-    const uint64_t nwarps = (uint64_t)gridDim.x * kWarpsPerCta;
-    for (uint64_t j = warp; j < m; j += nwarps) {
-        const uint32_t row = __ldg(rows + j), pr = __ldg(prow + j);
+    const RowGroups<LPR> rg;
+    uint32_t next = 0u, pnext = 0u;
+    if (rg.first < m) { next = __ldg(rows + rg.first); pnext = __ldg(prow + rg.first); }
+    for (uint64_t j = rg.first; j < m; j += rg.step) {
+        const uint32_t row = next, pr = pnext;
+        if (j + rg.step < m) { next = __ldg(rows + j + rg.step); pnext = __ldg(prow + j + rg.step); }
         if (row >= n_rows || pr >= n_prows) {
-            if (lane == 0 && bad_rows != nullptr) atomicAdd(bad_rows, 1u);
+            if (rg.lane == 0 && bad_rows != nullptr) atomicAdd(bad_rows, 1u);
             continue;
         }
         const float4* g4 = reinterpret_cast<const float4*>(grad) + j * dim4;
@@ -130,7 +149,8 @@ __global__ void __launch_bounds__(kThreads) k_ecrm_rows_step_parity(uint32_t m, 
         float4* s4 = reinterpret_cast<float4*>(state) + (uint64_t)row * dim4;
         float4* pe4 = reinterpret_cast<float4*>(p_entry) + (uint64_t)pr * dim4;
         float4* ps4 = reinterpret_cast<float4*>(p_state) + (uint64_t)pr * dim4;
-        for (uint32_t c = lane; c < dim4; c += 32) {
+#pragma unroll 1
+        for (uint32_t c = rg.lane; c < dim4; c += LPR) {
             const float4 g = __ldcs(g4 + c);
             const float4 e = e4[c], s = s4[c], pe = pe4[c], ps = ps4[c];
             const float gv[4] = {g.x, g.y, g.z, g.w}, ev[4] = {e.x, e.y, e.z, e.w}, sv[4] = {s.x, s.y, s.z, s.w};
@@ -138,14 +158,7 @@ __global__ void __launch_bounds__(kThreads) k_ecrm_rows_step_parity(uint32_t m, 
             float en[4], sn[4], pen[4], psn[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                if (OPT == ECRM_ADAGRAD) {
-                    sn[q] = __fadd_rn(sv[q], __fmul_rn(gv[q], gv[q]));
-                    const float step = __fdiv_rn(lr, __fsqrt_rn(__fadd_rn(sn[q], hyper)));
-                    en[q] = __fsub_rn(ev[q], __fmul_rn(step, gv[q]));
-                } else {
-                    sn[q] = __fadd_rn(__fmul_rn(hyper, sv[q]), gv[q]);
-                    en[q] = __fsub_rn(ev[q], __fmul_rn(lr, sn[q]));
-                }
+                optimizer_step<OPT>(gv[q], ev[q], sv[q], lr, hyper, en[q], sn[q]);
                 pen[q] = __fadd_rn(pev[q], __fsub_rn(en[q], ev[q]));      // parity += fl(new - old), as the two calls do
                 psn[q] = __fadd_rn(psv[q], __fsub_rn(sn[q], sv[q]));
             }
@@ -157,22 +170,24 @@ __global__ void __launch_bounds__(kThreads) k_ecrm_rows_step_parity(uint32_t m, 
     }
 }
 
-// One warp per parity row: p += d (entry and, if given, state).
+// Parity rows: p += d (entry and, if given, state).
+template <int LPR>
 __global__ void __launch_bounds__(kThreads) k_ecrm_parity_add(uint32_t m, const uint32_t* __restrict__ prow,
                                                                const float* __restrict__ d_entry,
                                                                const float* __restrict__ d_state,
                                                                float* __restrict__ p_entry, float* __restrict__ p_state,
                                                                uint64_t n_prows, uint32_t dim4, uint32_t* bad_rows) {
-    const int lane = threadIdx.x & 31;
-    const uint64_t warp = (uint64_t)blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5);
-    const uint64_t nwarps = (uint64_t)gridDim.x * kWarpsPerCta;
-    for (uint64_t j = warp; j < m; j += nwarps) {
-        const uint32_t row = __ldg(prow + j);
+    const RowGroups<LPR> rg;
+    uint32_t next = rg.first < m ? __ldg(prow + rg.first) : 0u;
+    for (uint64_t j = rg.first; j < m; j += rg.step) {
+        const uint32_t row = next;
+        if (j + rg.step < m) next = __ldg(prow + j + rg.step);
         if (row >= n_prows) {
-            if (lane == 0 && bad_rows != nullptr) atomicAdd(bad_rows, 1u);
+            if (rg.lane == 0 && bad_rows != nullptr) atomicAdd(bad_rows, 1u);
             continue;
         }
-        for (uint32_t c = lane; c < dim4; c += 32) {
+#pragma unroll 1
+        for (uint32_t c = rg.lane; c < dim4; c += LPR) {
             float4* pe = reinterpret_cast<float4*>(p_entry) + (uint64_t)row * dim4 + c;
             const float4 d = __ldcs(reinterpret_cast<const float4*>(d_entry) + j * dim4 + c);
             float4 p = *pe;
@@ -189,33 +204,39 @@ __global__ void __launch_bounds__(kThreads) k_ecrm_parity_add(uint32_t m, const 
     }
 }
 
-// One warp per requested row: parity row minus the surviving rows, in shard order.
+// Requested rows: parity row minus the surviving rows, in shard order, four of them in flight.
+template <int LPR>
 __global__ void __launch_bounds__(kThreads) k_ecrm_degraded_read(uint32_t k_avail, uint32_t m,
-                                                                  const uint32_t* __restrict__ prow, RowTable srow,
-                                                                  PtrTable shards, const float* __restrict__ parity,
+                                                                  const uint32_t* __restrict__ prow, const __grid_constant__ RowTable srow,
+                                                                  const __grid_constant__ PtrTable shards, const float* __restrict__ parity,
                                                                   uint64_t n_rows, uint32_t dim4,
                                                                   float* __restrict__ out, uint32_t* bad_rows) {
-    const int lane = threadIdx.x & 31;
-    const uint64_t warp = (uint64_t)blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5);
-    const uint64_t nwarps = (uint64_t)gridDim.x * kWarpsPerCta;
-    for (uint64_t j = warp; j < m; j += nwarps) {
-        const uint32_t pr = __ldg(prow + j);
+    const RowGroups<LPR> rg;
+    uint32_t next = rg.first < m ? __ldg(prow + rg.first) : 0u;
+    for (uint64_t j = rg.first; j < m; j += rg.step) {
+        const uint32_t pr = next;
+        if (j + rg.step < m) next = __ldg(prow + j + rg.step);
+        auto row_of = [&](uint32_t s) { return srow.p[s] != nullptr ? __ldg(srow.p[s] + j) : pr; };
         bool ok = pr < n_rows;
-        uint32_t sr[ECRM_MAX_K];
-        for (uint32_t s = 0; s < k_avail; ++s) {
-            sr[s] = srow.p[s] != nullptr ? __ldg(srow.p[s] + j) : pr;
-            ok = ok && sr[s] < n_rows;
-        }
+        for (uint32_t s = 0; s < k_avail; ++s) ok = ok && row_of(s) < n_rows;
         if (!ok) {
-            if (lane == 0 && bad_rows != nullptr) atomicAdd(bad_rows, 1u);
+            if (rg.lane == 0 && bad_rows != nullptr) atomicAdd(bad_rows, 1u);
             continue;
         }
-        for (uint32_t c = lane; c < dim4; c += 32) {
+#pragma unroll 1
+        for (uint32_t c = rg.lane; c < dim4; c += LPR) {
             float4 acc = reinterpret_cast<const float4*>(parity)[(uint64_t)pr * dim4 + c];
-            for (uint32_t s = 0; s < k_avail; ++s) {
-                const float4 v = reinterpret_cast<const float4*>(shards.p[s])[(uint64_t)sr[s] * dim4 + c];
-                acc.x = __fsub_rn(acc.x, v.x); acc.y = __fsub_rn(acc.y, v.y);
-                acc.z = __fsub_rn(acc.z, v.z); acc.w = __fsub_rn(acc.w, v.w);
+            for (uint32_t s = 0; s < k_avail; s += 4) {
+                float4 v[4];
+#pragma unroll
+                for (uint32_t u = 0; u < 4; ++u)
+                    if (s + u < k_avail) v[u] = reinterpret_cast<const float4*>(shards.p[s + u])[(uint64_t)row_of(s + u) * dim4 + c];
+#pragma unroll
+                for (uint32_t u = 0; u < 4; ++u) {
+                    if (s + u >= k_avail) continue;
+                    acc.x = __fsub_rn(acc.x, v[u].x); acc.y = __fsub_rn(acc.y, v[u].y);
+                    acc.z = __fsub_rn(acc.z, v[u].z); acc.w = __fsub_rn(acc.w, v[u].w);
+                }
             }
             __stcs(reinterpret_cast<float4*>(out) + j * dim4 + c, acc);
         }
@@ -224,10 +245,12 @@ __global__ void __launch_bounds__(kThreads) k_ecrm_degraded_read(uint32_t k_avai
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-int grid_for_rows(uint32_t m) {
+// Lanes per row, and the grid for m rows.
+int lanes_for(uint32_t dim4) { return dim4 <= 8 ? 8 : dim4 <= 16 ? 16 : 32; }
+int grid_for_rows(uint32_t m, int lpr) {
     int dev = 0, sms = 148;
     if (cudaGetDevice(&dev) == cudaSuccess) (void)cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const uint64_t want = ((uint64_t)m + kWarpsPerCta - 1) / kWarpsPerCta;
+    const uint64_t per = (uint64_t)(kThreads / lpr), want = ((uint64_t)m + per - 1) / per;
     const uint64_t cap = (uint64_t)sms * 8 * 4;          // a few waves of resident CTAs, then a row loop
     return (int)(want < cap ? (want ? want : 1) : cap);
 }
@@ -285,13 +308,11 @@ int ecrm_rows_step(int optimizer, uint32_t m, const uint32_t* rows, const float*
     if (!aligned16(grad) || !aligned16(entry) || !aligned16(state) || !aligned16(d_entry) || !aligned16(d_state))
         return ECRM_E_INVALID;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const int grid = grid_for_rows(m);
-    if (optimizer == ECRM_ADAGRAD)
-        k_ecrm_rows_step<ECRM_ADAGRAD><<<grid, kThreads, 0, s>>>(m, rows, grad, entry, state, n_rows, dim / 4, lr,
-                                                                  hyper, d_entry, d_state, bad_rows);
-    else
-        k_ecrm_rows_step<ECRM_MOMENTUM><<<grid, kThreads, 0, s>>>(m, rows, grad, entry, state, n_rows, dim / 4, lr,
-                                                                   hyper, d_entry, d_state, bad_rows);
+    const int lpr = lanes_for(dim / 4);
+    auto k = optimizer == ECRM_ADAGRAD
+                 ? (lpr == 8 ? k_ecrm_rows_step<ECRM_ADAGRAD, 8> : lpr == 16 ? k_ecrm_rows_step<ECRM_ADAGRAD, 16> : k_ecrm_rows_step<ECRM_ADAGRAD, 32>)
+                 : (lpr == 8 ? k_ecrm_rows_step<ECRM_MOMENTUM, 8> : lpr == 16 ? k_ecrm_rows_step<ECRM_MOMENTUM, 16> : k_ecrm_rows_step<ECRM_MOMENTUM, 32>);
+    k<<<grid_for_rows(m, lpr), kThreads, 0, s>>>(m, rows, grad, entry, state, n_rows, dim / 4, lr, hyper, d_entry, d_state, bad_rows);
     return launched();
 }
 
@@ -309,13 +330,11 @@ int ecrm_rows_step_parity(int optimizer, uint32_t m, const uint32_t* rows, const
         return ECRM_E_INVALID;
     if (p_entry == entry || p_state == state || p_entry == state || p_state == entry) return ECRM_E_INVALID;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const int grid = grid_for_rows(m);
-    if (optimizer == ECRM_ADAGRAD)
-        k_ecrm_rows_step_parity<ECRM_ADAGRAD><<<grid, kThreads, 0, s>>>(m, rows, prow, grad, entry, state, n_rows, p_entry,
-                                                                         p_state, n_prows, dim / 4, lr, hyper, bad_rows);
-    else
-        k_ecrm_rows_step_parity<ECRM_MOMENTUM><<<grid, kThreads, 0, s>>>(m, rows, prow, grad, entry, state, n_rows, p_entry,
-                                                                          p_state, n_prows, dim / 4, lr, hyper, bad_rows);
+    const int lpr = lanes_for(dim / 4);
+    auto k = optimizer == ECRM_ADAGRAD
+                 ? (lpr == 8 ? k_ecrm_rows_step_parity<ECRM_ADAGRAD, 8> : lpr == 16 ? k_ecrm_rows_step_parity<ECRM_ADAGRAD, 16> : k_ecrm_rows_step_parity<ECRM_ADAGRAD, 32>)
+                 : (lpr == 8 ? k_ecrm_rows_step_parity<ECRM_MOMENTUM, 8> : lpr == 16 ? k_ecrm_rows_step_parity<ECRM_MOMENTUM, 16> : k_ecrm_rows_step_parity<ECRM_MOMENTUM, 32>);
+    k<<<grid_for_rows(m, lpr), kThreads, 0, s>>>(m, rows, prow, grad, entry, state, n_rows, p_entry, p_state, n_prows, dim / 4, lr, hyper, bad_rows);
     return launched();
 }
 
@@ -326,8 +345,9 @@ int ecrm_parity_add(uint32_t m, const uint32_t* prow, const float* d_entry, cons
     if (prow == nullptr || d_entry == nullptr || p_entry == nullptr || (d_state == nullptr) != (p_state == nullptr))
         return ECRM_E_INVALID;
     if (!aligned16(d_entry) || !aligned16(p_entry) || !aligned16(d_state) || !aligned16(p_state)) return ECRM_E_INVALID;
-    k_ecrm_parity_add<<<grid_for_rows(m), kThreads, 0, static_cast<cudaStream_t>(stream)>>>(
-        m, prow, d_entry, d_state, p_entry, p_state, n_prows, dim / 4, bad_rows);
+    const int lpr = lanes_for(dim / 4);
+    auto k = lpr == 8 ? k_ecrm_parity_add<8> : lpr == 16 ? k_ecrm_parity_add<16> : k_ecrm_parity_add<32>;
+    k<<<grid_for_rows(m, lpr), kThreads, 0, static_cast<cudaStream_t>(stream)>>>(m, prow, d_entry, d_state, p_entry, p_state, n_prows, dim / 4, bad_rows);
     return launched();
 }
 
@@ -347,8 +367,9 @@ int ecrm_degraded_read(uint32_t k_avail, uint32_t m, const uint32_t* prow, const
         t.p[s] = shards[s];
         rt.p[s] = srow != nullptr ? srow[s] : nullptr;
     }
-    k_ecrm_degraded_read<<<grid_for_rows(m), kThreads, 0, static_cast<cudaStream_t>(stream)>>>(
-        k_avail, m, prow, rt, t, parity, n_rows, dim / 4, out, bad_rows);
+    const int lpr = lanes_for(dim / 4);
+    auto k = lpr == 8 ? k_ecrm_degraded_read<8> : lpr == 16 ? k_ecrm_degraded_read<16> : k_ecrm_degraded_read<32>;
+    k<<<grid_for_rows(m, lpr), kThreads, 0, static_cast<cudaStream_t>(stream)>>>(k_avail, m, prow, rt, t, parity, n_rows, dim / 4, out, bad_rows);
     return launched();
 }
 
