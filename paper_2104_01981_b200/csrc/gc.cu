@@ -23,7 +23,7 @@ using namespace gc;
 
 // Geometry of k_topk_single; votes: see its template argument.
 struct SingleGeom { uint32_t G = 0, maxt = 0, pool = 0; size_t smem = 0; RowMap rows = {}; bool votes = false; };
-struct MultiGeom { uint32_t G = 0, per = 0, pool = 0, full = 0, ntab = 0; size_t smem = 0; };   // see multi_geometry
+struct MultiGeom { uint32_t G = 0, per = 0, pool = 0, ntab = 0; RunMap runs = {}; size_t smem = 0; };   // see multi_geometry
 
 // How many CTAs of every kernel are resident on a device (the dynamic shared memory raised where a kernel
 // needs it): asked once per device, copied into every plan.
@@ -82,9 +82,7 @@ struct gc_plan_s : DeviceFacts {
     std::vector<const void*> clean_ws;      // workspaces the one-tensor top-k kernel ran on last (and left clean), if private
     uint32_t wk_W = 0, wk_batch = 0;        // gc_compress_workers: workers per launch chosen for the last W seen
     MultiGeom wk_geom;
-    uint32_t multi_ntab = 0;
-    uint32_t multi_grid = 0, multi_per = 0, multi_pool = 0, multi_full = 0;       // 0 = plan does not qualify
-    size_t multi_smem = 0;
+    MultiGeom multi;                        // k_topk_multi (G = 0: plan does not qualify)
     size_t off_shist = 0, off_bhist = 0, off_midn = 0, off_mmid = 0, off_skeys = 0;
     uint32_t n_empty = 0;                   // tensors without elements
     unsigned long long launches = 0;
@@ -420,7 +418,7 @@ MultiGeom thr_multi_geometry(const gc_plan_s* p, uint32_t G) {
         worst = std::max(worst, e);
     }
     if ((double)pool < 2.0 * worst + 512.0) return mg;
-    mg.G = G; mg.per = per; mg.pool = pool; mg.full = G;
+    mg.G = G; mg.per = per; mg.pool = pool;
     mg.ntab = p->T <= kMultiMaxTab ? p->T : 0u;
     mg.smem = (size_t)per * kMultiRowBytes + 2 * sizeof(uint32_t) * (size_t)mg.ntab;
     return mg;
@@ -438,14 +436,28 @@ void plan_thr_multi(gc_plan_s* p) {
 // Geometry of the many-tensor kernel when G CTAs share one worker's tiles: MultiGeom.
 
 // Decides whether G CTAs can run the many-tensor kernel on this plan (G = 0 in the result: no).
-// `age_skew`: the CTA index follows the CTAs' age on their SMs (a launch that fills the device
-// with this plan alone), so the leftover tiles go to the youngest third.
-MultiGeom multi_geometry(const gc_plan_s* p, uint32_t G, bool age_skew) {
+// `workers`: how many such groups share the launch.  In a launch that fills the device the CTA index follows
+// the CTAs' age on their SMs: what the full runs of a lone worker leave over goes to the youngest third; several
+// workers, whose CTAs have a hundred tiles and more, take unequal shares (eight 161-tensor workers, equal
+// shares: the three ages were through with the fold after 351, 362 and 380 us; step 559 -> 533 us, three workers
+// of 110M elements in 199 tensors 796 -> 738).
+MultiGeom multi_geometry(const gc_plan_s* p, uint32_t G, uint32_t workers) {
     MultiGeom mg;
     if (p->mode != GC_TOPK || p->T < 2 || G == 0 || p->ntiles == 0) return mg;
     G = std::min<uint32_t>(G, p->ntiles);
-    const uint32_t per = (p->ntiles + G - 1) / G;
+    uint32_t per = (p->ntiles + G - 1) / G;
     if (per > kMultiMaxPer) return mg;
+    RunMap runs{G, per, G, per};
+    const uint32_t third = (uint32_t)p->sm_count / workers, over = (uint32_t)(((uint64_t)p->ntiles * 37u) / (1000u * G));
+    if (workers == 1u && p->ntiles >= (uint32_t)p->grid_multi_max && per >= 8u) {
+        const uint32_t fc = (uint32_t)((uint64_t)G * 2u / 3u);
+        if ((uint64_t)fc * per < p->ntiles) runs = RunMap{fc, per, fc, per};
+    } else if (workers > 1u && p->grid_multi_max == 3 * p->sm_count && G == (uint32_t)p->grid_multi_max / workers && third >= 4u &&
+               over >= 2u && per + over <= kMultiMaxPer) {
+        const uint32_t mean = p->ntiles / G;
+        runs = RunMap{third, mean + over, 2u * third, mean + over / 8u};
+        per = mean + over;
+    }
     const uint32_t pool = std::min<uint32_t>(p->cand_cap_alloc / G, kMultiPoolMax);
     // expected candidates of the busiest CTA (bracket rank over sample size, times two where tau is a
     // bin edge), with head-room
@@ -458,25 +470,11 @@ MultiGeom multi_geometry(const gc_plan_s* p, uint32_t G, bool age_skew) {
         const double edge = d.nstiles <= kRefineTiles ? 1.02 : 2.0;      // tau is exact to 21 bits, or a bin edge
         per_tile[t] = std::min<double>(kTile, edge * (double)kTile * (double)d.srank / (4.0 * (double)nsg));
     }
-    // runs: `per` tiles for the first two thirds of a full grid, the rest spread over the last third
-    // (the youngest CTAs of their SMs, which advance the slowest); every CTA `per` tiles otherwise
-    uint32_t full_ctas = G;
-    if (age_skew && per >= 8) {
-        const uint32_t fc = (uint32_t)((uint64_t)G * 2u / 3u);
-        if ((uint64_t)fc * per < p->ntiles) full_ctas = fc;
-    }
-    auto run_of = [&](uint32_t b, uint32_t& f, uint32_t& l) {
-        if (b < full_ctas) { f = std::min<uint32_t>(p->ntiles, b * per); l = std::min<uint32_t>(p->ntiles, f + per); return; }
-        const uint32_t s0 = std::min<uint32_t>(p->ntiles, full_ctas * per), rest = p->ntiles - s0, nb = G - full_ctas;
-        f = s0 + (uint32_t)(((uint64_t)(b - full_ctas) * rest) / nb);
-        l = s0 + (uint32_t)(((uint64_t)(b - full_ctas + 1) * rest) / nb);
-    };
     double worst = 0.0;
     uint32_t t = 0;
     for (uint32_t b = 0; b < G; ++b) {
         double e = 0.0;
-        uint32_t f, l;
-        run_of(b, f, l);
+        const uint32_t f = runs.begin(b, G, p->ntiles), l = runs.begin(b + 1u, G, p->ntiles);
         if (l - f > per) return mg;
         for (uint32_t tile = f; tile < l; ++tile) {
             while (t + 1 < p->T && (p->desc[t].ntiles == 0 || tile >= p->desc[t].tile0 + p->desc[t].ntiles)) ++t;
@@ -485,7 +483,7 @@ MultiGeom multi_geometry(const gc_plan_s* p, uint32_t G, bool age_skew) {
         worst = std::max(worst, e);
     }
     if ((double)pool < 1.5 * worst + 512.0) return mg;
-    mg.G = G; mg.per = per; mg.pool = pool; mg.full = full_ctas;
+    mg.G = G; mg.per = per; mg.pool = pool; mg.runs = runs;
     mg.ntab = p->T <= kMultiMaxTab ? p->T : 0u;
     mg.smem = (size_t)per * kMultiRowBytes + sizeof(uint32_t) * ((pool + 31) / 32) + 2 * sizeof(uint32_t) * (size_t)mg.ntab;
     return mg;
@@ -493,12 +491,8 @@ MultiGeom multi_geometry(const gc_plan_s* p, uint32_t G, bool age_skew) {
 
 // Decides whether the plan can use the many-tensor kernel and with which geometry.
 void plan_multi(gc_plan_s* p) {
-    p->multi_grid = 0;
-    if (p->grid_multi_max <= 0) return;
-    const MultiGeom mg = multi_geometry(p, (uint32_t)p->grid_multi_max, p->ntiles >= (uint32_t)p->grid_multi_max);
-    if (mg.G == 0) return;
-    p->multi_grid = mg.G; p->multi_per = mg.per; p->multi_pool = mg.pool; p->multi_full = mg.full;
-    p->multi_ntab = mg.ntab; p->multi_smem = mg.smem;
+    p->multi = MultiGeom{};
+    if (p->grid_multi_max > 0) p->multi = multi_geometry(p, (uint32_t)p->grid_multi_max, 1u);
 }
 
 int upload_table(gc_plan_s* p) {
@@ -998,7 +992,7 @@ static int compress_route(const gc_plan_s* p) {
     }
     if (p->path == GC_PATH_EXACT) return GC_ROUTE_EXACT;
     if (p->path == GC_PATH_AUTO && p->single_grid > 0) return GC_ROUTE_TOPK_ONE;
-    if (p->path == GC_PATH_AUTO && p->multi_grid > 0) return GC_ROUTE_TOPK_MANY;
+    if (p->path == GC_PATH_AUTO && p->multi.G > 0) return GC_ROUTE_TOPK_MANY;
     if (p->path == GC_PATH_AUTO && p->grid_fused > 0) return GC_ROUTE_TOPK_GENERAL;
     return GC_ROUTE_TOPK_STAGED;
 }
@@ -1013,7 +1007,7 @@ static MultiArgs multi_args(const gc_plan_s* p, const MultiGeom& mg, const void*
     gws.gate = ws.sel;
     MultiArgs ma;
     ma.desc = p->d_desc; ma.T = p->T; ma.ntiles = p->ntiles; ma.nstiles = p->nstiles;
-    ma.per = mg.per; ma.full_ctas = mg.full;
+    ma.per = mg.per; ma.runs = mg.runs;
     ma.pool_cap = std::min<uint32_t>(mg.pool, p->cand_cap / mg.G);     // each CTA's share
     ma.pool_smem_words = (mg.pool + 31) / 32; ma.ntab = mg.ntab;
     ma.small_ids = p->d_small; ma.n_small = (uint32_t)p->small_ids.size(); ma.n_tiny = p->n_tiny;
@@ -1062,7 +1056,7 @@ static int compress_impl(gc_plan_t* p, const void* grad_any, bool bf16, float* r
     if (p->device < 0) return GC_E_UNSUPPORTED;
     if (!on_plan_device(p)) return GC_E_INVALID;
     // a bf16 gradient is read by the two fused top-k kernels only
-    if (bf16 && !(p->mode == GC_TOPK && p->path == GC_PATH_AUTO && (p->single_grid > 0 || p->multi_grid > 0)))
+    if (bf16 && !(p->mode == GC_TOPK && p->path == GC_PATH_AUTO && (p->single_grid > 0 || p->multi.G > 0)))
         return GC_E_UNSUPPORTED;
     if (p->total_n == 0) return GC_OK;
     if (grad == nullptr || residual == nullptr || out_idx == nullptr || out_val == nullptr ||
@@ -1222,9 +1216,7 @@ static int compress_impl(gc_plan_t* p, const void* grad_any, bool bf16, float* r
     }
     if (route == GC_ROUTE_TOPK_MANY) {
         // many tensors: one cooperative launch, four grid barriers
-        MultiGeom mg;
-        mg.G = p->multi_grid; mg.per = p->multi_per; mg.pool = p->multi_pool; mg.full = p->multi_full;
-        mg.ntab = p->multi_ntab; mg.smem = p->multi_smem;
+        const MultiGeom& mg = p->multi;
         MultiArgs ma = multi_args(p, mg, grad_any, residual, out_idx, out_val, out_count, workspace, clean_mode);
         note_clean(p, workspace);
         void* args[] = {&ma};
@@ -1232,7 +1224,7 @@ static int compress_impl(gc_plan_t* p, const void* grad_any, bool bf16, float* r
         const bool dense = p->density >= kDenseFrom;
         const void* kfn = bf16 ? (dense ? (const void*)k_topk_multi<GradBF16, true, true> : (const void*)k_topk_multi<GradBF16, false, true>)
                                : (dense ? (const void*)k_topk_multi<GradF32, true, true> : (const void*)k_topk_multi<GradF32, false, true>);
-        GC_CUDA(p, cudaLaunchCooperativeKernel(kfn, dim3(p->multi_grid), dim3(kBlock), args, p->multi_smem, s));
+        GC_CUDA(p, cudaLaunchCooperativeKernel(kfn, dim3(mg.G), dim3(kBlock), args, mg.smem, s));
         return GC_OK;
     }
     if (route == GC_ROUTE_TOPK_GENERAL) {
@@ -1338,14 +1330,14 @@ int gc_compress_workers(gc_plan_t* p, uint32_t W, const float* const* grads, flo
     // share must still satisfy the kernel's limits (tiles and candidates per CTA)
     uint32_t batch = 0;
     MultiGeom mg;
-    const bool topk_multi = p->mode == GC_TOPK && p->path == GC_PATH_AUTO && p->multi_grid > 0;
+    const bool topk_multi = p->mode == GC_TOPK && p->path == GC_PATH_AUTO && p->multi.G > 0;
     const bool thr_multi = p->mode == GC_THRESHOLD && p->path == GC_PATH_AUTO && p->thrm_grid > 0;
     if ((topk_multi || thr_multi) && W >= 2) {
         if (p->wk_W != W) {                      // (kept for the next call; options that change the layout reset it)
             p->wk_W = W; p->wk_batch = 0;
             try {
                 for (uint32_t wb = std::min<uint32_t>(W, kWorkersPerLaunch); wb >= 2 && p->wk_batch == 0; --wb) {
-                    const MultiGeom g2 = topk_multi ? multi_geometry(p, (uint32_t)p->grid_multi_max / wb, false)
+                    const MultiGeom g2 = topk_multi ? multi_geometry(p, (uint32_t)p->grid_multi_max / wb, wb)
                                                     : thr_multi_geometry(p, (uint32_t)p->grid_thr_multi_max / wb);
                     if (g2.G > 0 && g2.smem <= (topk_multi ? p->multi_smem_max : p->thrm_smem_max)) {
                         p->wk_batch = wb; p->wk_geom = g2;

@@ -1,15 +1,15 @@
 // Threshold-estimation variant for MANY tensors in one cooperative launch.
 //
 //   sample   per tensor: coarse histogram (top 11 key bits) of the strided sample, the sampled
-//            keys are kept.  Tensors that fit one tile are finished here by one CTA each,
-//            between the arrival at and the wait on the barrier       | grid barrier
+//            keys are kept                                            | grid barrier
 //   tau      one CTA per remaining tensor: coarse bin from the histogram, then two more radix
 //            levels over that tensor's kept keys in shared memory: the EXACT k_s-th largest
 //            sampled key (it is part of the result's definition)      | grid barrier
 //   fold     CTA b walks its contiguous run of tiles, segment by segment (a segment = one
 //            tensor's tiles inside the run): a = g + r, every element with key >= tau is a hit,
 //            goes to the CTA's region of the hit list and leaves +0 in the residual; per-tile
-//            hit counts are published                                  | grid barrier
+//            hit counts are published.  Tensors that fit one tile are finished by the CTAs
+//            that are through first, before they wait                  | grid barrier
 //   emit     slot of a hit = hits of the tensor's earlier tiles + hits before it in its tile;
 //            hits whose slot reaches the tensor's capacity get their value written back.
 // A full hit-list region restores the listed values and hands over to the ticket-ordered
@@ -318,24 +318,7 @@ static __device__ __forceinline__ void threshold_multi_body(const ThrMultiArgs& 
         if (t != 0xFFFFFFFFu) flush_hist(sm, a.shist + (size_t)d.reg * kHistBins, 1 << level_bits(0));
     }
     cleared();
-    grid_arrive(hdr);
-    for (uint32_t q8 = G - 1u - b; q8 * kWarps < a.n_tiny; q8 += G) {        // tiny tensors: a warp each, eight at a time
-        const uint32_t q = q8 * kWarps + (uint32_t)warp;
-        if (q < a.n_tiny) {
-            const uint32_t t = a.small_ids[q];
-            const TensorDesc d = a.desc[t];
-            tiny_threshold_warp(d, t, a.T, a.g, a.r, a.out_idx, a.out_val, a.out_count, hdr, lane);
-        }
-    }
-    // (the other small ones start with the CTAs next to those that took the tiny ones)
-    for (uint32_t q = a.n_tiny + (2u * G - 1u - b - ((a.n_tiny + kWarps - 1u) / kWarps) % G) % G; q < a.n_small; q += G) {
-        const uint32_t t = a.small_ids[q];
-        const TensorDesc d = a.desc[t];
-        small_threshold_body(sm, d, t, a.T, a.g, a.r, a.out_idx, a.out_val, a.out_count, hdr);
-    }
-    __syncthreads();
-    for (int i = tid; i < 2048; i += kBlock) sm.hist[i] = 0u;
-    if (!grid_wait(hdr, passed, &sm.ok, G)) return;
+    if (!grid_barrier(hdr, passed, &sm.ok, G)) return;
     phase_stamp(hdr, n_stamp, b);
 
     // ---------------------------------------------------------------- exact tau, one CTA per tensor
@@ -528,7 +511,29 @@ static __device__ __forceinline__ void threshold_multi_body(const ThrMultiArgs& 
         for (int w = 0; w < kWarps; ++w) tot += rec[i * kWarps + w] & 1023u;
         a.tile_cnt[first + i] = tot;
     }
-    if (!grid_barrier(hdr, passed, &sm.ok, G)) return;
+    // small tensors: by the CTAs that are through with their fold first (see the top-k kernel)
+    if (a.n_small != 0u) {
+        const uint32_t tiny = (a.n_tiny + kWarps - 1u) / kWarps, units = tiny + a.n_small - a.n_tiny;
+        for (uint32_t u = grid_arrive(hdr, passed, &sm.tile, G); u < units; u += G) {
+            if (u < tiny) {                                  // tiny ones: a warp each, eight at a time
+                const uint32_t q = u * kWarps + (uint32_t)warp;
+                if (q < a.n_tiny) {
+                    const uint32_t t = a.small_ids[q];
+                    const TensorDesc d = a.desc[t];
+                    tiny_threshold_warp(d, t, a.T, a.g, a.r, a.out_idx, a.out_val, a.out_count, hdr, lane);
+                }
+                continue;
+            }
+            const uint32_t t = a.small_ids[a.n_tiny + u - tiny];
+            const TensorDesc d = a.desc[t];
+            small_threshold_body(sm, d, t, a.T, a.g, a.r, a.out_idx, a.out_val, a.out_count, hdr);
+            __syncthreads();
+            for (int i = tid; i < 2048; i += kBlock) sm.hist[i] = 0u;
+        }
+        if (!grid_wait(hdr, passed, &sm.ok, G)) return;
+    } else if (!grid_barrier(hdr, passed, &sm.ok, G)) {
+        return;
+    }
     phase_stamp(hdr, n_stamp, b);
 
     if (ld_cg(&hdr->overflow) == 0u) {
