@@ -29,7 +29,12 @@ namespace gc {
 constexpr uint32_t kMultiMidCap = 4u * kMidFast; // short list per tensor (the first kMidFast entries stay in registers)
 constexpr uint32_t kSegWords = 16;               // shared-memory words per segment record
 constexpr uint32_t kRefineTiles = 32;            // samples of up to this many sample tiles are ranked a second time
-constexpr uint32_t kWarpMid = 128;               // short lists up to this length are settled by one warp
+// Short lists up to kWarpMid entries are settled by one warp (a CTA with many segments has eight at a time), up
+// to kRankMid by the whole CTA, every entry against all others; longer ones by radix select.  A warp alone
+// takes 4 us for 100 entries, radix select 10 us whatever the length, and the CTAs of large tensors came that much
+// later: 161 tensors of 25.6M elements at 0.1 % 100 -> 91 us, a dozen of 30M at 0.4 % 125 -> 113, 199 of 110M at 1 % 286 -> 279.
+constexpr uint32_t kWarpMid = 32;
+constexpr uint32_t kRankMid = 512;
 
 // Contiguous runs of tiles: CTAs below c1 take n1 tiles each, those from there below c2 take n2, the others share
 // the rest evenly.  The CTAs launched last are the youngest on their SMs and advance the slowest (see RowMap in
@@ -490,8 +495,9 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
     };
     auto chunk_of = [&](const uint32_t* s, uint32_t idx) -> uint32_t {
         const uint32_t rel = idx - s[SG_BASE0];
-        return (s[SG_TILE0] + (rel >> 12)) * kWarps + ((rel >> 9) & (kWarps - 1u));
+        return s[SG_TILE0] * kWarps + (rel >> 9);
     };
+    static_assert(kWarpChunk == 512 && kWarps * kWarpChunk == kTile, "chunks side by side");
 
     const bool overflowed = ld_cg(&hdr->overflow) != 0u, by_chunk = DENSE && used >= kChunkWalk * ntl * kWarps;
     if (!overflowed && nseg != 0u) {
@@ -617,10 +623,59 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
                 }
             }
             __syncthreads();
-            // longer short lists: the whole CTA, one segment after the other (radix select in shared memory)
+            // longer short lists: the whole CTA, one segment after the other
             for (uint32_t sidx = 0; sidx < nseg; ++sidx) {
                 uint32_t* s = seg + (size_t)sidx * kSegWords;
-                if (s[SG_OK] == 0u || s[SG_M] <= kWarpMid) continue;
+                const uint32_t m = s[SG_M];
+                if (s[SG_OK] == 0u || m <= kWarpMid || m > kRankMid) continue;
+                const uint32_t t = s[SG_T];
+                const TensorDesc d = a.desc[t];
+                const uint2* mid = a.mid + (size_t)t * kMultiMidCap;
+                uint2* const list = reinterpret_cast<uint2*>(sm.hist);
+                static_assert(kRankMid <= 1024u, "the list fits in the histogram");
+                for (uint32_t i = tid; i < m; i += kBlock) { const uint2 pr = ld_cg(mid + i); list[i] = make_uint2(pr.x, pr.y & kKeyMask); }
+                // candidates above the band bin in the tensor's tiles before this segment
+                const uint32_t nbefore = first + s[SG_TILE0] - d.tile0;
+                uint32_t before = 0;
+                for (uint32_t q = tid; q < nbefore; q += kBlock) before += ld_cg(a.tile_cnt + d.tile0 + q);
+                if (tid == 0) { s_cnt = 0u; sm.scratch[2] = 0u; }
+                __syncthreads();
+                const uint32_t krem = s[SG_K] - s[SG_ABOVE];             // entries of the short list that are sent (1 .. m)
+                const uint32_t seg_end = s[SG_BASE0] + s[SG_NTILE] * (uint32_t)kTile;
+                for (uint32_t i = tid; i < m; i += kBlock) {
+                    const uint2 mine = list[i];
+                    uint32_t place = 0;                                  // entries in front: key descending, index ascending
+#pragma unroll 4
+                    for (uint32_t j = 0; j < m; ++j) {
+                        const uint2 o = list[j];
+                        place += (o.y > mine.y || (o.y == mine.y && o.x < mine.x)) ? 1u : 0u;
+                    }
+                    if (place == krem - 1u) { sm.scratch[0] = mine.y; sm.scratch[1] = mine.x; sm.scratch[2] = 1u; }
+                    if (place < krem) {
+                        if (mine.x < s[SG_BEGIN]) ++before;
+                        else if (mine.x < seg_end) atomicAdd(&rec2[chunk_of(s, mine.x)], 1u);
+                    }
+                }
+                before = __reduce_add_sync(0xFFFFFFFFu, before);
+                if (lane == 0 && before) atomicAdd(&s_cnt, before);
+                __syncthreads();
+                if (tid == 0) {
+                    s[SG_TKEY] = sm.scratch[0]; s[SG_CUT] = sm.scratch[1];
+                    s[SG_OUT] = d.out_off + s_cnt;                     // slot of the segment's first sent entry
+                    if (sm.scratch[2] == 0u) {  // cannot happen unless the list changed under us: report, send nothing
+                        s[SG_OK] = 0u;
+                        record_status(hdr, -1 /*GC_E_INVALID*/, 0xE0000000ull + t);
+                    } else if (a.out_count != nullptr && first + s[SG_TILE0] == d.tile0) {
+                        a.out_count[t] = d.k; a.out_count[a.T + t] = d.k;
+                    }
+                }
+                for (uint32_t i = tid; i < 2u * m; i += kBlock) sm.hist[i] = 0u;
+                __syncthreads();
+            }
+            // (radix select in shared memory)
+            for (uint32_t sidx = 0; sidx < nseg; ++sidx) {
+                uint32_t* s = seg + (size_t)sidx * kSegWords;
+                if (s[SG_OK] == 0u || s[SG_M] <= kRankMid) continue;
                 const uint32_t t = s[SG_T], m = s[SG_M];
                 const TensorDesc d = a.desc[t];
                 const uint2* mid = a.mid + (size_t)t * kMultiMidCap;
