@@ -384,12 +384,17 @@ __device__ __forceinline__ bool fold_tail_votes(BlockSmem& sm, const float (&av)
             const float v = (m & 3u) ? v01 : v23;
             const uint32_t e = (uint32_t)__ffs((int)m) - 1u;
             to[pos] = make_uint2(at0 + j * 128u + e, __float_as_uint(v));
-            atomicAdd(&sm.hist[min((key_of(v) - tau) >> shift, 2047u)], 1u);
+            if (!staged) atomicAdd(&sm.hist[min((key_of(v) - tau) >> shift, 2047u)], 1u);
         }
     }
+    // (counted here, where the lanes are side by side: 355M at 0.1 % 954 -> 953 us with the decode, bfloat16 110M 225 -> 224)
     if (staged) {
         __syncwarp();
-        for (uint32_t q = lane; q < cr.total; q += 32) pool[off + q] = sm.emit[warp][q];
+        for (uint32_t q = lane; q < cr.total; q += 32) {
+            const uint2 pr = sm.emit[warp][q];
+            pool[off + q] = pr;
+            atomicAdd(&sm.hist[min(((pr.y & kKeyMask) - tau) >> shift, 2047u)], 1u);
+        }
         __syncwarp();
     }
     return true;
