@@ -788,20 +788,22 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
             e[u] = !counted && u * kBlock + tid < m ? ld_cg(a.mid + u * kBlock + tid) : make_uint2(0u, 0u);
         // while those loads fly: per row, the candidates above the bin in the whole row and in
         // the tiles of lower CTAs (whole 32-CTA segments below this CTA's + the lower CTAs of
-        // its own segment): two loads per lane and row, two rows per step
-        for (uint32_t i0 = warp * 2u; i0 < n_own; i0 += kWarps * 2u) {
-            uint32_t sv[2], tv[2];
+        // its own segment): two loads per lane and row, eight rows per warp and step (two: 355M elements
+        // with 293 rows 11.8 -> 8.2 us, 110M with 61 6.3 -> 5.6)
+        constexpr uint32_t kRows = 8;
+        for (uint32_t i0 = warp; i0 < n_own; i0 += kWarps * kRows) {
+            uint32_t sv[kRows], tv[kRows];
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const uint32_t i = i0 + u, q = myseg * 32u + (uint32_t)lane;
+            for (uint32_t u = 0; u < kRows; ++u) {
+                const uint32_t i = i0 + u * kWarps, q = myseg * 32u + (uint32_t)lane;
                 sv[u] = (i < n_own && (uint32_t)lane < nseg) ? ld_cg(a.seg_tot + (size_t)i * nseg + lane) : 0u;
                 tv[u] = (i < n_own && q < col) ? ld_cg(a.tile_cnt + rm.tile_of(i, q)) : 0u;
             }
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
+            for (uint32_t u = 0; u < kRows; ++u) {
                 const uint32_t row = __reduce_add_sync(0xFFFFFFFFu, sv[u]);
                 const uint32_t low = __reduce_add_sync(0xFFFFFFFFu, tv[u] + ((uint32_t)lane < myseg ? sv[u] : 0u));
-                if (lane == 0 && i0 + u < n_own) { row_sum[i0 + u] = row; tile_base[i0 + u] = low; }
+                if (lane == 0 && i0 + u * kWarps < n_own) { row_sum[i0 + u * kWarps] = row; tile_base[i0 + u * kWarps] = low; }
             }
         }
         if (counted) {                                    // the same for the candidates at the threshold key

@@ -354,19 +354,20 @@ k_threshold_single(const __grid_constant__ ThrSingleArgs a) {
 
     if (ld_cg(&hdr->overflow) == 0u) {
         // ------------------------------------------------------------ slots and emission
-        for (uint32_t i0 = warp * 2u; i0 < n_own; i0 += kWarps * 2u) {
-            uint32_t sv[2], tv[2];
+        constexpr uint32_t kRows = 8;                      // (see the top-k kernel)
+        for (uint32_t i0 = warp; i0 < n_own; i0 += kWarps * kRows) {
+            uint32_t sv[kRows], tv[kRows];
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const uint32_t i = i0 + u, q = myseg * 32u + (uint32_t)lane;
+            for (uint32_t u = 0; u < kRows; ++u) {
+                const uint32_t i = i0 + u * kWarps, q = myseg * 32u + (uint32_t)lane;
                 sv[u] = (i < n_own && (uint32_t)lane < nseg) ? ld_cg(a.seg_tot + (size_t)i * nseg + lane) : 0u;
                 tv[u] = (i < n_own && q < b) ? ld_cg(a.tile_cnt + (size_t)i * G + q) : 0u;
             }
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
+            for (uint32_t u = 0; u < kRows; ++u) {
                 const uint32_t row = __reduce_add_sync(0xFFFFFFFFu, sv[u]);
                 const uint32_t low = __reduce_add_sync(0xFFFFFFFFu, tv[u] + ((uint32_t)lane < myseg ? sv[u] : 0u));
-                if (lane == 0 && i0 + u < n_own) { row_sum[i0 + u] = row; tile_base[i0 + u] = low; }
+                if (lane == 0 && i0 + u * kWarps < n_own) { row_sum[i0 + u * kWarps] = row; tile_base[i0 + u * kWarps] = low; }
             }
         }
         __syncthreads();
