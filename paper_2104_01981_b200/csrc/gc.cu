@@ -764,6 +764,18 @@ static bool device_facts(int device, DeviceFacts& out) {
     return true;
 }
 
+// Decode kernels start while the kernel in front of them ends (see launch_wait).
+template <typename... P, typename... A>
+static void launch_behind(void (*kernel)(P...), int grid, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t c{};
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.gridDim = dim3((unsigned)grid); c.blockDim = dim3(kDecBlock); c.dynamicSmemBytes = smem; c.stream = s;
+    c.attrs = &at; c.numAttrs = 1;
+    (void)cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);      // (the caller asks for the error)
+}
+
 extern "C" {
 
 static int compress_route(const gc_plan_s* p);
@@ -1445,11 +1457,10 @@ int gc_decompress_accumulate(gc_plan_t* p, uint32_t W, const uint32_t* const* id
             const uint32_t nt8 = (uint32_t)((p->total_n + 8u * g.T - 1) / (8u * g.T));
             auto kr = zero_first ? (W > 32 ? k_decode_rings<false, false, true> : k_decode_rings<false, false, false>)
                                  : (W > 32 ? k_decode_rings<false, true, true> : k_decode_rings<false, true, false>);
-            kr<<<std::min<uint32_t>(nt8, (uint32_t)(p->sm_count * g.ctas)), kDecBlock, g.smem, s>>>(
+            launch_behind(kr, (int)std::min<uint32_t>(nt8, (uint32_t)(p->sm_count * g.ctas)), g.smem, s, 
                 ls, W, (uint32_t)p->total_cap, (uint32_t)p->total_n, g.T, g.RS, dense_out, use_bulk, ws.hdr, ApplyArgs{});
         } else {
-            k_decode_tiles<false><<<grid, kDecBlock, nbuf * kDecTileBytes, s>>>(
-                ls, W, (uint32_t)p->total_cap, (uint32_t)p->total_n, dense_out, zero_first ? 1 : 0, use_bulk, nbuf, ws.hdr,
+            launch_behind(k_decode_tiles<false>, grid, nbuf * kDecTileBytes, s, ls, W, (uint32_t)p->total_cap, (uint32_t)p->total_n, dense_out, zero_first ? 1 : 0, use_bulk, nbuf, ws.hdr,
                 ApplyArgs{});
         }
         GC_CUDA(p, cudaGetLastError());
@@ -1467,8 +1478,7 @@ int gc_decompress_accumulate(gc_plan_t* p, uint32_t W, const uint32_t* const* id
         const int grid = (int)std::min<uint32_t>(ntl, (uint32_t)p->grid_decode_seg[nbuf - 1]);
         const int use_bulk = (reinterpret_cast<uintptr_t>(dense_out) & 15u) == 0 ? 1 : 0;
         Timed tm(p, s, GC_K_DECODE_TILES);
-        k_decode_segments<false><<<grid, kDecBlock, nbuf * kDecTileBytes, s>>>(
-            ls, W, p->d_desc, p->T, p->d_dectile, (uint32_t)p->total_n, dense_out, zero_first ? 1 : 0, use_bulk, nbuf,
+        launch_behind(k_decode_segments<false>, grid, nbuf * kDecTileBytes, s, ls, W, p->d_desc, p->T, p->d_dectile, (uint32_t)p->total_n, dense_out, zero_first ? 1 : 0, use_bulk, nbuf,
             ws.hdr, ApplyArgs{});
         GC_CUDA(p, cudaGetLastError());
         return GC_OK;
@@ -1521,22 +1531,20 @@ int gc_decompress_apply_momentum(gc_plan_t* p, uint32_t W, const uint32_t* const
     ApplyArgs ap{param, velocity, lr, momentum, scale};
     Timed tm(p, s, GC_K_DECODE_TILES);
     if (segmented && W > 0) {
-        k_decode_segments<true><<<(int)std::min<uint32_t>(ntl, (uint32_t)p->grid_decode_seg_apply), kDecBlock,
-                                  kDecTileBytes, s>>>(ls, W, p->d_desc, p->T, p->d_dectile, (uint32_t)p->total_n,
+        launch_behind(k_decode_segments<true>, (int)std::min<uint32_t>(ntl, (uint32_t)p->grid_decode_seg_apply), kDecTileBytes, s, ls, W, p->d_desc, p->T, p->d_dectile, (uint32_t)p->total_n,
                                                       nullptr, 1, 0, 1, ws.hdr, ap);
         GC_CUDA(p, cudaGetLastError());
         return GC_OK;
     }
     if (!takes_rings(p, W, true, true)) {
-        k_decode_tiles<true><<<(int)std::min<uint32_t>(ntl, (uint32_t)p->grid_decode_apply), kDecBlock, kDecTileBytes, s>>>(
-            ls, W, (uint32_t)p->total_cap, (uint32_t)p->total_n, nullptr, 1, 0, 1, ws.hdr, ap);
+        launch_behind(k_decode_tiles<true>, (int)std::min<uint32_t>(ntl, (uint32_t)p->grid_decode_apply), kDecTileBytes, s, ls, W, (uint32_t)p->total_cap, (uint32_t)p->total_n, nullptr, 1, 0, 1, ws.hdr, ap);
         GC_CUDA(p, cudaGetLastError());
         return GC_OK;
     }
     const RingGeom g = ring_geometry(p, W, true);
     const uint32_t nt8 = (uint32_t)((p->total_n + 8u * g.T - 1) / (8u * g.T));
     auto kr = W > 32 ? k_decode_rings<true, false, true> : k_decode_rings<true, false, false>;
-    kr<<<std::min<uint32_t>(nt8, (uint32_t)(p->sm_count * g.ctas)), kDecBlock, g.smem, s>>>(
+    launch_behind(kr, (int)std::min<uint32_t>(nt8, (uint32_t)(p->sm_count * g.ctas)), g.smem, s, 
         ls, W, (uint32_t)p->total_cap, (uint32_t)p->total_n, g.T, g.RS, nullptr, 0, ws.hdr, ap);
     GC_CUDA(p, cudaGetLastError());
     return GC_OK;

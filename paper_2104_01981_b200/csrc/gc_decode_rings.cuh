@@ -43,7 +43,7 @@ __device__ __forceinline__ void warp_lower_bounds(const uint32_t* const (&idx)[Q
         for (int q = 0; q < Q; ++q) {
             const uint32_t span = hi[q] - lo[q];
             const uint32_t p = lo[q] + (uint32_t)(((unsigned long long)span * (uint32_t)(lane + 1)) / 33u);
-            ge[q] = span == 0u || __ldg(idx[q] + p) >= key;
+            ge[q] = span == 0u || __ldcg(idx[q] + p) >= key;
         }
         more = false;
 #pragma unroll
@@ -75,6 +75,7 @@ k_decode_rings(const __grid_constant__ DecodeLists ls, uint32_t W, uint32_t cnt,
     constexpr int kW8 = kDecBlock / 32, U = WIDE ? 2 : 1;
     extern __shared__ __align__(128) float s_dyn_rings[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    launch_wait();
     // rings [W][2][RS] (indices, values), then the sub-tiles
     const uint32_t Wb = (W + kRingBatch - 1u) / kRingBatch * kRingBatch;
     uint32_t* const rings = reinterpret_cast<uint32_t*>(s_dyn_rings);
@@ -109,7 +110,7 @@ k_decode_rings(const __grid_constant__ DecodeLists ls, uint32_t W, uint32_t cnt,
         for (uint32_t q = lane; q < T / 4; q += 32) reinterpret_cast<float4*>(s_tile)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
 
     // where every list enters this CTA's run of tiles
-    if (tid < 64) s_len[tid] = (uint32_t)tid >= W ? 0u : ls.len[tid] != nullptr ? min(__ldg(ls.len[tid]), cnt) : cnt;
+    if (tid < 64) s_len[tid] = (uint32_t)tid >= W ? 0u : ls.len[tid] != nullptr ? min(__ldcg(ls.len[tid]), cnt) : cnt;
     __syncthreads();
     for (uint32_t w0 = (uint32_t)warp; w0 < W; w0 += 4u * kW8) {
         const uint32_t* ip[4];
