@@ -148,8 +148,9 @@ int gc_plan(gc_plan_t **out, int device, uint32_t n_tensors, const uint64_t *siz
  *                                GC_ORDER_ANY: the caller would accept any order, i.e. results within
  *                                (hits - 1) x 2^-24 x sum |values| of the fixed-order ones.  The fixed
  *                                order is the faster one in every kernel, so both values give it.
- *   GC_OPT_WORKSPACE_PRIVATE     0 (default): every gc_compress starts with a launch that clears the
- *                                control block of the workspace, so a workspace may be shared by
+ *   GC_OPT_WORKSPACE_PRIVATE     0 (default): every gc_compress clears the control block of the
+ *                                workspace (the fused kernels inside their own launch, the other
+ *                                routes in a launch in front), so a workspace may be shared by
  *                                plans or refilled by the caller between calls.  1: the caller
  *                                promises that between two gc_compress calls of THIS plan on a
  *                                workspace nothing else writes to it (the decode calls of this plan
@@ -158,7 +159,8 @@ int gc_plan(gc_plan_t **out, int device, uint32_t n_tensors, const uint64_t *siz
  *                                shared launch of gc_compress_workers) clean the control block as
  *                                they go (each section right after the grid barrier that follows its
  *                                last reader, the rest at the start of the next launch), so their
- *                                calls then do without the clearing launch.  A broken promise is
+ *                                calls then need no clearing at all (but for a launch in front of a
+ *                                workspace's first call).  A broken promise is
  *                                caught by a mark in the workspace header: the kernel leaves at once
  *                                and GC_E_INVALID is recorded in the device status; after any error
  *                                status read through gc_last_status the next call clears again.

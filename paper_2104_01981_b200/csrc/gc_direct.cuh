@@ -9,7 +9,7 @@
 // sample, no candidate list, no capacity that data could overflow: if more entries share the 21 bits than
 // the list takes, the last 10 bits get a global histogram and the shares are counted (one more barrier),
 // and nothing is ever redone.  The scratch is 29 KB and the launch leaves it clean.  Without a plan, six
-// launches over the whole tensor took 55 us at 2.4M elements and 31 us at 20,000; this takes 29 and 16 us.
+// launches over the whole tensor took 55 us at 2.4M elements; this takes 26.7, and 15.2 us at 200,000.
 #pragma once
 #include <cstddef>
 
@@ -39,7 +39,7 @@ struct DirectArgs {
     DirectScratch* s;
     unsigned long long mark;                     // what the header's mark reads after a launch that left the scratch clean
     uint32_t expect_clean;                       // the host relies on that mark (see CleanArgs)
-    uint32_t clear_first;                        // the launch clears the scratch itself, whatever is in it
+    uint32_t clear_first;                        // the launch clears the scratch itself, whatever is in it, and leaves it as it is
 };
 
 // Grid barrier: release by the arrival, acquire by the poll (see grid_barrier for the bounded wait).
@@ -125,8 +125,8 @@ k_topk_direct(const __grid_constant__ DirectArgs a) {
     const uint32_t w0 = (uint32_t)(((unsigned long long)warp * len) / kWarps), w1 = (uint32_t)(((unsigned long long)(warp + 1) * len) / kWarps);
     for (int i = tid; i < 2048; i += kBlock) sm.hist[i] = 0u;
     // A launch that clears for itself: the clearing ends at a barrier of the launch, since the scratch's own
-    // counter is among what is cleared.  Arrival here, wait behind the fold (2.4M elements: 28.7 us; 29.1 with
-    // the whole barrier behind the fold, 30.1 with a clearing launch in front, 26.8 without clearing).
+    // counter is among what is cleared.  Arrival here, wait behind the fold (2.4M elements, still with an exit count:
+    // 28.7 us; 29.1 with the whole barrier behind the fold, 30.1 with a clearing launch in front).
     const auto grid = cooperative_groups::this_grid();
     cooperative_groups::grid_group::arrival_token cleared{};
     if (a.clear_first != 0u) {
@@ -138,7 +138,14 @@ k_topk_direct(const __grid_constant__ DirectArgs a) {
         if (b == 0 && tid < 62 && tid != (int)kHdrBarrierWord && tid != (int)kHdrExitWord) reinterpret_cast<uint32_t*>(hdr)[tid] = 0u;
         __syncthreads();
     }
-    if (b == 0 && tid == 0) hdr->cand_total = a.k;
+    if (b == 0 && tid == 0) {
+        hdr->cand_total = a.k;
+        if (a.clear_first != 0u && a.status_out != nullptr) *a.status_out = 0 /*GC_OK*/;      // (an error is written over it)
+    }
+    auto report = [&](unsigned long long detail) {
+        record_status(hdr, -1 /*GC_E_INVALID*/, detail);
+        if (a.clear_first != 0u && a.status_out != nullptr) *a.status_out = -1;
+    };
     phase_stamp(hdr, n_stamp);
     auto flush = [&](uint32_t* dst, int nb) {
         __syncthreads();
@@ -228,7 +235,7 @@ k_topk_direct(const __grid_constant__ DirectArgs a) {
         // Somebody else's counts in the scratch: nothing is sent (the residual keeps g + r), the scratch is
         // cleaned on the way out.  Every CTA sees the same sum.
         if (direct_select<2048>(sm, a.s->hist0, a.k, tid, lane, warp) != a.n) {
-            if (b == 0 && tid == 0) { record_status(hdr, -1 /*GC_E_INVALID*/, 0xC1EA0001ull); atomicExch(&hdr->abort, 1u); }
+            if (b == 0 && tid == 0) { report(0xC1EA0001ull); atomicExch(&hdr->abort, 1u); }
             live = false;
         }
     }
@@ -314,7 +321,8 @@ k_topk_direct(const __grid_constant__ DirectArgs a) {
     if (live) {
         // ------------------------------------------------------------ emission
         // the histograms have had their last readers (of hist2: before the barrier that followed)
-        for (uint32_t i = b * kBlock + tid; i < 4096u; i += G * kBlock) a.s->hist0[i] = 0u;        // (hist0, hist1, hist2 in a row)
+        if (a.clear_first == 0u)
+            for (uint32_t i = b * kBlock + tid; i < 4096u; i += G * kBlock) a.s->hist0[i] = 0u;    // (hist0, hist1, hist2 in a row)
         unsigned long long before = (unsigned long long)eq_before << 32 | gt_before;
         for (uint32_t c = tid; c < b; c += kBlock) before += ld_cg(&a.s->tot[c]);
         before = warp_sum64(before);
@@ -357,7 +365,7 @@ k_topk_direct(const __grid_constant__ DirectArgs a) {
                             a.out_val[slot] = xe[e];
                             a.r[i] = 0.0f;
                         } else {
-                            record_status(hdr, -1 /*GC_E_INVALID*/, i);
+                            report(i);
                         }
                     }
                 }
@@ -367,9 +375,15 @@ k_topk_direct(const __grid_constant__ DirectArgs a) {
         // (counted and emitted entries agree and add up to k, unless others wrote to the scratch)
         if (lane == 0 && (gt_at != gt_end || eq_at != eq_end ||
                           (b == G - 1u && warp == kWarps - 1 && gt_at + min(eq_at, m_eq) != a.k)))
-            record_status(hdr, -1 /*GC_E_INVALID*/, 0xC1EA0002ull);
+            report(0xC1EA0002ull);
         if (a.out_count != nullptr && b == 0 && tid == 0) { a.out_count[0] = a.k; a.out_count[1] = a.k; }
         phase_stamp(hdr, n_stamp);
+    }
+    if (a.clear_first != 0u) {
+        // (nothing to be left clean; a wait that ran out is the one error that is not reported above)
+        if (!live && tid == 0 && a.status_out != nullptr && *reinterpret_cast<volatile int32_t*>(&hdr->status) != 0)
+            *a.status_out = *reinterpret_cast<volatile int32_t*>(&hdr->status);
+        return;
     }
     // The CTA that leaves last resets what the others may still have been reading; after a wait that ran
     // out, or counts that do not add up, it cleans everything and sets no mark (the next call on a private
