@@ -76,6 +76,11 @@ struct gc_plan_s : DeviceFacts {
     uint32_t single_srank_hi = 0, single_srank_mid = 0;
     uint32_t thr_grid = 0, thr_maxt = 0, thr_pool = 0, thr_rounds = 0;    // one-tensor threshold kernel (0 = no)
     size_t thr_smem = 0;
+    // threshold mode, several tensors, fold first (k_topk_multi with THR): the table with the bracket's sample
+    std::vector<TensorDesc> tdesc;          // (empty: the plan does not qualify)
+    TensorDesc* d_tdesc = nullptr;          // (behind d_desc)
+    uint32_t tnstiles = 0;
+    MultiGeom thrf;
     uint32_t thrm_grid = 0, thrm_per = 0, thrm_pool = 0, thrm_ntab = 0;   // many-tensor threshold kernel (0 = no)
     size_t thrm_smem = 0;
     bool ws_private = false;                // GC_OPT_WORKSPACE_PRIVATE
@@ -118,6 +123,8 @@ constexpr double kSingleSkew = 0.08, kSingleSkewSparse = 0.04;
 constexpr size_t kSingleRowBytes = (2 * kWarps + 4) * sizeof(uint32_t);   // shared memory per owned tile
 constexpr double kSparseUpTo = 0.002;        // density up to which most chunks are empty (see VOTES of k_topk_single)
 constexpr double kDenseFrom = 0.02;          // density from which the forms with emission by chunk are taken (12 candidates per chunk)
+constexpr double kThrFoldUpTo = 0.005;       // density up to which, and elements from which threshold plans of several tensors are
+constexpr uint64_t kThrFoldFrom = 12u << 20; // taken fold first (see plan_thr_fold)
 constexpr uint32_t kMultiMaxTab = 1024;      // tensors whose tile tables k_topk_multi keeps in shared memory
 constexpr size_t kMultiMaxPer = 224;         // most tiles one CTA of k_topk_multi may own
 constexpr size_t kMultiRowBytes = (2 * kWarps + kSegWords) * sizeof(uint32_t);   // shared memory per owned tile
@@ -211,6 +218,21 @@ void sample_params(TensorDesc& d, double density, uint32_t rank_permille, uint64
     *ccap = cap >= (double)n ? n : (uint64_t)cap;
 }
 
+// Threshold plans of several tensors, fold first: the sample that sets a tensor's bracket (kept keys, so at most 32,000
+// elements), one group of four in `stride`, and the rank of its lower end, six standard deviations of both samples' noise
+// above the expected one.
+struct ThrBracket { uint64_t stride, groups; double rank; };
+ThrBracket thr_bracket(const TensorDesc& d, uint32_t rank_permille) {
+    ThrBracket b;
+    const uint64_t groups = ((uint64_t)d.n + 3) / 4, target = std::min<uint64_t>(32000, std::max<uint64_t>(d.n / 128, std::min<uint64_t>(8192, d.n / 2)));
+    b.stride = std::max<uint64_t>(1, d.n / target);
+    b.groups = (groups + b.stride - 1) / b.stride;
+    const double m = 4.0 * (double)b.groups, among = 4.0 * (double)((groups + d.stride - 1) / d.stride), ks = (double)d.srank * m / among;
+    b.rank = std::max(1.0, std::ceil(ks + 6.0 * std::sqrt(ks + ks * ks / (double)d.srank) + 8.0) * (double)rank_permille / 1000.0);
+    if (b.rank >= 0.9 * m) b.rank = 0.0;                   // (nearly everything would be a candidate: not this way)
+    return b;
+}
+
 // Fills the derived fields of the tensor table and the workspace layout.
 void finish_layout(gc_plan_s* p) {
     uint64_t stile0 = 0, group0 = 0, ccap_total = 0, stiles_worst = 0;
@@ -239,6 +261,7 @@ void finish_layout(gc_plan_s* p) {
                 m = (nsg - 1) * 4 + std::min<uint64_t>(4, d.n - last_first);
             }
             d.srank = (uint32_t)k_rule(m, p->density);
+            if (d.ntiles > 1) stiles_worst += kRefineTiles;       // (the bracket's sample, see plan_thr_fold)
             if (d.n > 0 && d.ntiles == 1 && p->T >= 2) d.kind = kKindSmall;    // one CTA finishes it (many-tensor kernel)
         }
         uint64_t nst = 0;
@@ -275,6 +298,13 @@ void finish_layout(gc_plan_s* p) {
         ccap_total = 0;
         if (p->T >= 1 && p->total_cap > 0)
             ccap_total = std::min<uint64_t>(0x7FFFFFFFull, (uint64_t)(1.25 * (double)p->total_cap) + (1u << 20));
+        double fold = 0.0;                 // the candidates between the brackets, twice over
+        for (const TensorDesc& d : p->desc) {
+            if (p->T < 2 || d.kind == kKindSmall || d.n == 0) continue;
+            const ThrBracket b = thr_bracket(d, 1000);
+            fold += b.rank > 0.0 ? std::min<double>(d.n, 2.5 * (double)d.n * (b.rank + 6.0 * std::sqrt(b.rank)) / (4.0 * (double)b.groups) + 4096.0) : 0.0;
+        }
+        ccap_total = std::min<uint64_t>(0x7FFFFFFFull, std::max<uint64_t>(ccap_total, (uint64_t)fold));
     }
     if (p->cand_cap_alloc == 0) p->cand_cap_alloc = (uint32_t)ccap_total;   // fixed at plan creation
     p->cand_cap = (uint32_t)std::min<uint64_t>(ccap_total, p->cand_cap_alloc);
@@ -441,9 +471,10 @@ void plan_thr_multi(gc_plan_s* p) {
 // workers, whose CTAs have a hundred tiles and more, take unequal shares (eight 161-tensor workers, equal
 // shares: the three ages were through with the fold after 351, 362 and 380 us; step 559 -> 533 us, three workers
 // of 110M elements in 199 tensors 796 -> 738).
-MultiGeom multi_geometry(const gc_plan_s* p, uint32_t G, uint32_t workers) {
+// `desc`: the table whose samples set the brackets.
+MultiGeom multi_geometry(const gc_plan_s* p, const std::vector<TensorDesc>& desc, uint32_t G, uint32_t workers) {
     MultiGeom mg;
-    if (p->mode != GC_TOPK || p->T < 2 || G == 0 || p->ntiles == 0) return mg;
+    if (desc.size() != p->T || p->T < 2 || G == 0 || p->ntiles == 0) return mg;
     G = std::min<uint32_t>(G, p->ntiles);
     uint32_t per = (p->ntiles + G - 1) / G;
     if (per > kMultiMaxPer) return mg;
@@ -463,7 +494,7 @@ MultiGeom multi_geometry(const gc_plan_s* p, uint32_t G, uint32_t workers) {
     // bin edge), with head-room
     std::vector<double> per_tile(p->T, 0.0);
     for (uint32_t t = 0; t < p->T; ++t) {
-        const TensorDesc& d = p->desc[t];
+        const TensorDesc& d = desc[t];
         if (d.kind == kKindSmall || d.ntiles == 0) continue;
         if (d.sstride == 0) { per_tile[t] = (double)kTile; continue; }
         const uint64_t groups = ((uint64_t)d.n + 3) / 4, nsg = (groups + d.sstride - 1) / d.sstride;
@@ -477,7 +508,7 @@ MultiGeom multi_geometry(const gc_plan_s* p, uint32_t G, uint32_t workers) {
         const uint32_t f = runs.begin(b, G, p->ntiles), l = runs.begin(b + 1u, G, p->ntiles);
         if (l - f > per) return mg;
         for (uint32_t tile = f; tile < l; ++tile) {
-            while (t + 1 < p->T && (p->desc[t].ntiles == 0 || tile >= p->desc[t].tile0 + p->desc[t].ntiles)) ++t;
+            while (t + 1 < p->T && (desc[t].ntiles == 0 || tile >= desc[t].tile0 + desc[t].ntiles)) ++t;
             e += per_tile[t];
         }
         worst = std::max(worst, e);
@@ -492,7 +523,37 @@ MultiGeom multi_geometry(const gc_plan_s* p, uint32_t G, uint32_t workers) {
 // Decides whether the plan can use the many-tensor kernel and with which geometry.
 void plan_multi(gc_plan_s* p) {
     p->multi = MultiGeom{};
-    if (p->grid_multi_max > 0) p->multi = multi_geometry(p, (uint32_t)p->grid_multi_max, 1u);
+    if (p->grid_multi_max > 0 && p->mode == GC_TOPK) p->multi = multi_geometry(p, p->desc, (uint32_t)p->grid_multi_max, 1u);
+}
+
+// Decides whether a threshold plan of several tensors is taken fold first (k_topk_multi with THR), and makes the table
+// with the bracket's samples.
+// Fold first costs a lighter sample, but more candidates than hits and one more pass over them, so it pays for sparse
+// plans (sample-first / fold-first, us): 161 tensors of 25.6M elements at 0.1 % 101 / 97, 0.5 % 103.3 / 102.3, 1 % 104.6 / 106,
+// 5 % 113 / 117; eight such workers 498 / 461, 500 / 485, 505 / 506, 560 / 636; a dozen of 30M 120 / 108, 116 / 110.5, 118 / 112, 127 / 128
+// (eight workers 571 / 531, 567 / 554, 575 / 578, 635 / 736); of 3M at 0.1 % 39.5 / 39.0, eight workers 92.1 / 93.3.  Plans with samples of more than
+// 128 sample tiles, which no fused kernel took, always go this way: 110M in 199 tensors at 1 % 882 -> 271, at 5 % 330.
+void plan_thr_fold(gc_plan_s* p) {
+    p->thrf = MultiGeom{};
+    p->tdesc.clear();
+    if (p->mode != GC_THRESHOLD || p->T < 2 || p->grid_multi_max <= 0) return;
+    if (p->thrm_grid > 0 && (p->density > kThrFoldUpTo || p->total_n < kThrFoldFrom)) return;
+    std::vector<TensorDesc> td = p->desc;
+    uint64_t stile0 = 0;
+    for (TensorDesc& d : td) {
+        d.k = d.srank;
+        d.stile0 = (uint32_t)stile0; d.nstiles = 0;
+        if (d.kind == kKindSmall || d.n == 0) continue;
+        const ThrBracket b = thr_bracket(d, p->rank_permille);
+        d.nstiles = (uint32_t)((b.groups + (uint64_t)kSampleTile - 1) / (uint64_t)kSampleTile);
+        if (b.rank <= 0.0 || d.nstiles > kRefineTiles) return;
+        d.sstride = (uint32_t)b.stride; d.srank = (uint32_t)b.rank;
+        stile0 += d.nstiles;
+    }
+    p->tnstiles = (uint32_t)stile0;
+    p->tdesc = std::move(td);
+    p->thrf = multi_geometry(p, p->tdesc, (uint32_t)p->grid_multi_max, 1u);
+    if (p->thrf.G == 0) p->tdesc.clear();
 }
 
 int upload_table(gc_plan_s* p) {
@@ -505,6 +566,8 @@ int upload_table(gc_plan_s* p) {
     if (e == cudaSuccess && !p->reg_ids.empty())
         e = cudaMemcpy(p->d_small + p->T, p->reg_ids.data(), sizeof(uint32_t) * p->reg_ids.size(),
                        cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && !p->tdesc.empty())
+        e = cudaMemcpy(p->d_tdesc, p->tdesc.data(), sizeof(TensorDesc) * (size_t)p->T, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) { p->last_cuda_error = (int)e; (void)cudaGetLastError(); return GC_E_CUDA; }
     return GC_OK;
 }
@@ -684,7 +747,9 @@ static bool ask_device(int device, DeviceFacts* p) {
             const std::initializer_list<const void*> forms = {
                 (const void*)k_topk_multi<GradF32, false, true>, (const void*)k_topk_multi<GradF32, true, true>,
                 (const void*)k_topk_multi<GradBF16, false, true>, (const void*)k_topk_multi<GradBF16, true, true>,
-                (const void*)k_topk_workers<GradF32, false>, (const void*)k_topk_workers<GradF32, true>};
+                (const void*)k_topk_workers<GradF32, false>, (const void*)k_topk_workers<GradF32, true>,
+                (const void*)k_topk_multi<GradF32, false, true, true>, (const void*)k_topk_multi<GradF32, true, true, true>,
+                (const void*)k_topk_workers<GradF32, false, true>, (const void*)k_topk_workers<GradF32, true, true>};
             if (allow_smem(forms, p->multi_smem_max)) {
                 nb = 1 << 20;
                 for (const void* fn : forms) {
@@ -856,7 +921,8 @@ static int fill_plan(gc_plan_s* p, int device, uint32_t n_tensors, const uint64_
     } restore_device{caller_device};
     cudaError_t e = cudaSetDevice(device);
     if (e == cudaSuccess && n_tensors > 0) {
-        e = cudaMalloc(reinterpret_cast<void**>(&p->d_desc), sizeof(TensorDesc) * (size_t)n_tensors);
+        e = cudaMalloc(reinterpret_cast<void**>(&p->d_desc), sizeof(TensorDesc) * (size_t)n_tensors * (p->mode == GC_THRESHOLD ? 2u : 1u));
+        p->d_tdesc = p->d_desc + n_tensors;
         if (e == cudaSuccess)
             e = cudaMalloc(reinterpret_cast<void**>(&p->d_small), sizeof(uint32_t) * 2 * (size_t)n_tensors);
         if (e == cudaSuccess) e = upload_table(p) == GC_OK ? cudaSuccess : cudaErrorUnknown;
@@ -882,7 +948,8 @@ static int fill_plan(gc_plan_s* p, int device, uint32_t n_tensors, const uint64_
     plan_thr_single(p);
     plan_thr_multi(p);
     plan_multi(p);
-    return GC_OK;
+    plan_thr_fold(p);
+    return p->tdesc.empty() ? GC_OK : upload_table(p);
 }
 
 int gc_plan_set_option(gc_plan_t* p, int option, uint64_t value) {
@@ -903,6 +970,7 @@ int gc_plan_set_option(gc_plan_t* p, int option, uint64_t value) {
                 finish_layout(p);                      // workspace size stays as planned (see skeys_tiles_alloc)
                 plan_single(p);
                 plan_multi(p);
+                plan_thr_fold(p);
             } catch (...) { return GC_E_INVALID; }     // out of host memory
             return upload_table(p);
         case GC_OPT_CANDIDATE_CAPACITY:
@@ -999,7 +1067,7 @@ static int compress_route(const gc_plan_s* p) {
     if (p->device < 0 || p->total_n == 0) return GC_ROUTE_NONE;
     if (p->mode == GC_THRESHOLD) {
         if (p->path == GC_PATH_AUTO && p->thr_grid > 0) return GC_ROUTE_THRESHOLD_ONE;
-        if (p->path == GC_PATH_AUTO && p->thrm_grid > 0) return GC_ROUTE_THRESHOLD_MANY;
+        if (p->path == GC_PATH_AUTO && (p->thrm_grid > 0 || p->thrf.G > 0)) return GC_ROUTE_THRESHOLD_MANY;
         return GC_ROUTE_THRESHOLD_STAGED;
     }
     if (p->path == GC_PATH_EXACT) return GC_ROUTE_EXACT;
@@ -1034,7 +1102,9 @@ static MultiArgs multi_args(const gc_plan_s* p, const MultiGeom& mg, const void*
     ma.tile_cnt = reinterpret_cast<uint32_t*>(wb + p->off_tinfo);
     ma.skeys = reinterpret_cast<uint4*>(wb + p->off_skeys);
     ma.ws = ws; ma.gws = gws;
-    ma.cl = clean_args(p, workspace, GC_ROUTE_TOPK_MANY, clean_mode);
+    ma.cl = clean_args(p, workspace, p->mode == GC_TOPK ? GC_ROUTE_TOPK_MANY : GC_ROUTE_THRESHOLD_MANY, clean_mode);
+    ma.nstiles_def = p->nstiles;
+    if (p->mode == GC_THRESHOLD) { ma.desc = p->d_tdesc; ma.nstiles = p->tnstiles; }
     return ma;
 }
 
@@ -1126,6 +1196,15 @@ static int compress_impl(gc_plan_t* p, const void* grad_any, bool bf16, float* r
         Timed tm(p, s, GC_K_FUSED);
         GC_CUDA(p, cudaLaunchCooperativeKernel((const void*)k_threshold_single, dim3(p->thr_grid), dim3(kBlock),
                                                args, p->thr_smem, s));
+        return GC_OK;
+    }
+    if (route == GC_ROUTE_THRESHOLD_MANY && p->thrf.G > 0) {
+        // several tensors: bracket, fold + candidates, exact thresholds and emission in one cooperative launch
+        MultiArgs ma = multi_args(p, p->thrf, grad, residual, out_idx, out_val, out_count, workspace, clean_mode);
+        void* args[] = {&ma};
+        Timed tm(p, s, GC_K_FUSED);
+        GC_CUDA(p, cudaLaunchCooperativeKernel(p->density >= kDenseFrom ? (const void*)k_topk_multi<GradF32, true, true, true> : (const void*)k_topk_multi<GradF32, false, true, true>,
+                                               dim3(p->thrf.G), dim3(kBlock), args, p->thrf.smem, s));
         return GC_OK;
     }
     if (route == GC_ROUTE_THRESHOLD_MANY) {
@@ -1343,15 +1422,17 @@ int gc_compress_workers(gc_plan_t* p, uint32_t W, const float* const* grads, flo
     uint32_t batch = 0;
     MultiGeom mg;
     const bool topk_multi = p->mode == GC_TOPK && p->path == GC_PATH_AUTO && p->multi.G > 0;
+    const bool thr_fold = p->mode == GC_THRESHOLD && p->path == GC_PATH_AUTO && p->thrf.G > 0;
     const bool thr_multi = p->mode == GC_THRESHOLD && p->path == GC_PATH_AUTO && p->thrm_grid > 0;
-    if ((topk_multi || thr_multi) && W >= 2) {
+    const bool fold_first = topk_multi || thr_fold;               // (the kernels of gc_multi.cuh)
+    if ((fold_first || thr_multi) && W >= 2) {
         if (p->wk_W != W) {                      // (kept for the next call; options that change the layout reset it)
             p->wk_W = W; p->wk_batch = 0;
             try {
                 for (uint32_t wb = std::min<uint32_t>(W, kWorkersPerLaunch); wb >= 2 && p->wk_batch == 0; --wb) {
-                    const MultiGeom g2 = topk_multi ? multi_geometry(p, (uint32_t)p->grid_multi_max / wb, wb)
+                    const MultiGeom g2 = fold_first ? multi_geometry(p, topk_multi ? p->desc : p->tdesc, (uint32_t)p->grid_multi_max / wb, wb)
                                                     : thr_multi_geometry(p, (uint32_t)p->grid_thr_multi_max / wb);
-                    if (g2.G > 0 && g2.smem <= (topk_multi ? p->multi_smem_max : p->thrm_smem_max)) {
+                    if (g2.G > 0 && g2.smem <= (fold_first ? p->multi_smem_max : p->thrm_smem_max)) {
                         p->wk_batch = wb; p->wk_geom = g2;
                     }
                 }
@@ -1387,11 +1468,11 @@ int gc_compress_workers(gc_plan_t* p, uint32_t W, const float* const* grads, flo
             const uint32_t w = w0 + i;
             cm.p[i] = reinterpret_cast<uint4*>(workspaces[w]);
             uint32_t* const oc = out_count ? out_count[w] : nullptr;
-            if (topk_multi) {
+            if (fold_first) {
                 wa.per[i] = multi_args(p, mg, grads[w], residuals[w], out_idx[w], out_val[w], oc, workspaces[w], clean_mode);
-                note_clean(p, workspaces[w]);
+                if (topk_multi) note_clean(p, workspaces[w]);
             }
-            if (!topk_multi) ta.per[i] = thr_multi_args(p, mg, grads[w], residuals[w], out_idx[w], out_val[w], oc, workspaces[w]);
+            if (!fold_first) ta.per[i] = thr_multi_args(p, mg, grads[w], residuals[w], out_idx[w], out_val[w], oc, workspaces[w]);
             if (oc != nullptr && p->n_empty > 0) {
                 Timed tm(p, s, GC_K_CLEAR_CTRL);
                 GC_CUDA(p, cudaMemsetAsync(oc, 0, sizeof(uint32_t) * 2 * (size_t)p->T, s));
@@ -1399,7 +1480,7 @@ int gc_compress_workers(gc_plan_t* p, uint32_t W, const float* const* grads, flo
         }
         for (uint32_t i = wn; i < kWorkersPerLaunch; ++i) {
             cm.p[i] = nullptr;
-            if (topk_multi) wa.per[i] = wa.per[0]; else ta.per[i] = ta.per[0];
+            if (fold_first) wa.per[i] = wa.per[0]; else ta.per[i] = ta.per[0];
         }
         if (clean_mode == kCleanDone) {
             Timed tm(p, s, GC_K_CLEAR_CTRL);
@@ -1407,9 +1488,10 @@ int gc_compress_workers(gc_plan_t* p, uint32_t W, const float* const* grads, flo
             const unsigned gx = (unsigned)std::min<size_t>((n16 + kBlock - 1) / kBlock, (size_t)p->sm_count * 8 / wn + 1);
             k_clear_many<<<dim3(gx, wn), kBlock, 0, s>>>(cm, n16);
         }
-        void* args[] = {topk_multi ? (void*)&wa : (void*)&ta};
+        void* args[] = {fold_first ? (void*)&wa : (void*)&ta};
         Timed tm(p, s, GC_K_FUSED);
         GC_CUDA(p, cudaLaunchCooperativeKernel(topk_multi ? (p->density >= kDenseFrom ? (const void*)k_topk_workers<GradF32, true> : (const void*)k_topk_workers<GradF32, false>)
+                                                          : thr_fold ? (p->density >= kDenseFrom ? (const void*)k_topk_workers<GradF32, true, true> : (const void*)k_topk_workers<GradF32, false, true>)
                                                           : thr_list(p) ? (const void*)k_threshold_workers<true> : (const void*)k_threshold_workers<false>,
                                                dim3(mg.G * wn), dim3(kBlock), args, mg.smem, s));
     }

@@ -227,13 +227,15 @@ static __global__ void __launch_bounds__(kBlock) k_clear_many(const __grid_const
 //   SRC_SAMPLE:           walks the tensor's sample (one 4-element group out of `sstride`),
 //                         a = g + r is computed but not stored; rank = the tensor's srank
 // At levels above 0 only keys under the prefix fixed so far are counted.
-constexpr int SRC_FOLD = 0, SRC_RESID = 1, SRC_SAMPLE = 2;
+//   SRC_RSAMPLE:          the same where r holds a = g + r already
+constexpr int SRC_FOLD = 0, SRC_RESID = 1, SRC_SAMPLE = 2, SRC_RSAMPLE = 3;
+__host__ __device__ constexpr bool src_is_sample(int src) { return src == SRC_SAMPLE || src == SRC_RSAMPLE; }
 
 template <int LEVEL, int SRC>
 __device__ void hist_body(BlockSmem& sm, const TensorDesc* __restrict__ desc, uint32_t T, uint32_t ntiles,
                           const float* __restrict__ g, float* __restrict__ r, const WsView& ws,
                           uint32_t G, uint32_t b_in_group) {       // G CTAs share the work, this is CTA b of them
-    using S = typename std::conditional<SRC == SRC_SAMPLE, SampleSpace, FullSpace>::type;
+    using S = typename std::conditional<src_is_sample(SRC), SampleSpace, FullSpace>::type;
     constexpr int NB = 1 << level_bits(LEVEL);
     constexpr int SH = level_shift(LEVEL);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -262,7 +264,7 @@ __device__ void hist_body(BlockSmem& sm, const TensorDesc* __restrict__ desc, ui
             prefix = level_is_first(LEVEL) ? 0u : ld_cg(&ws.sel[t].prefix);
         }
         if (!active) continue;
-        if (SRC == SRC_SAMPLE) {
+        if (src_is_sample(SRC)) {
             // sample tile: kSampleTile sample groups, one per thread; all loads are issued
             // before any of them is used
             const uint32_t ngroups = (d.n + 3u) >> 2;
@@ -274,13 +276,13 @@ __device__ void hist_body(BlockSmem& sm, const TensorDesc* __restrict__ desc, ui
             for (int e = 0; e < 4; ++e) {
                 bool v = gi < ngroups && i0 + e < d.n;
                 uint32_t f = d.off + (v ? i0 + e : 0u);
-                gv[e] = v ? __ldg(g + f) : 0.f;
+                gv[e] = SRC == SRC_SAMPLE && v ? __ldg(g + f) : 0.f;
                 rv[e] = v ? ld_cg(r + f) : 0.f;
                 ok |= (uint32_t)v << e;
             }
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                uint32_t key = key_of(__fadd_rn(gv[e], rv[e]));
+                uint32_t key = key_of(SRC == SRC_RSAMPLE ? rv[e] : __fadd_rn(gv[e], rv[e]));
                 bool in = (ok >> e) & 1u;
                 if (!level_is_first(LEVEL)) in = in && ((key >> (SH + level_bits(LEVEL))) == prefix);
                 if (in) atomicAdd(&sm.hist[(key >> SH) & (NB - 1)], 1u);

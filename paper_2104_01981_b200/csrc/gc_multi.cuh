@@ -23,6 +23,7 @@
 //     if a CTA's candidate region overflows, everything is redone.
 #pragma once
 #include "gc_single.cuh"
+#include "gc_threshold.cuh"
 
 namespace gc {
 
@@ -57,6 +58,9 @@ struct MultiArgs {
     uint32_t pool_cap;               // candidate slots per CTA
     uint32_t pool_smem_words;        // words of shared memory reserved for one bit per candidate slot
     uint32_t ntab;                   // T if the tile tables fit in shared memory, else 0
+    // threshold mode (see topk_multi_body): `desc` holds the bracket's sample and, as k, the rank in the definition's; the
+    // table with the definition's sample stands in front of it (desc - T) and has so many sample tiles
+    uint32_t nstiles_def;
     const uint32_t* small_ids;       // the tensors that fit one tile, the tiny ones (one warp each) first
     uint32_t n_small, n_tiny;
     const uint32_t* reg_ids;         // the tensors that are not small (and not empty)
@@ -81,7 +85,8 @@ struct MultiArgs {
 // segment record (one per tensor a CTA's tile run touches), kSegWords words in shared memory
 enum : uint32_t {
     SG_T = 0, SG_TILE0, SG_NTILE, SG_BASE0, SG_BEGIN, SG_TAU, SG_TAUZ, SG_SHIFT,
-    SG_A, SG_ABOVE, SG_M, SG_TKEY, SG_CUT, SG_OK, SG_OUT, SG_K
+    SG_A, SG_ABOVE, SG_M, SG_TKEY, SG_CUT, SG_OK, SG_OUT, SG_K,
+    SG_END = SG_CUT                  // threshold mode: end of the tensor's slots (there is no tie cut)
 };
 
 // First half of a barrier; returns this CTA's place in the order of arrival (0 = first).
@@ -119,10 +124,156 @@ __device__ __forceinline__ bool grid_wait(WsHeader* hdr, uint32_t& passed, int* 
     return grid_wait(hdr, passed, s_ok, gridDim.x);
 }
 
+// Threshold mode: is the element at `idx` of a tensor that starts at `off` in the definition's sample?
+struct InSample {
+    uint32_t off, stride;
+    __device__ __forceinline__ bool operator()(uint32_t idx) const {
+        const uint32_t q = (idx - off) >> 2;
+        return (stride & (stride - 1u)) == 0u ? (q & (stride - 1u)) == 0u : q % stride == 0u;
+    }
+};
+// (gc_thr_multi.cuh)
+static __device__ void tiny_threshold_warp(const TensorDesc& d, uint32_t t, uint32_t T, const float* __restrict__ g, float* __restrict__ r,
+                                           uint32_t* __restrict__ out_idx, float* __restrict__ out_val, uint32_t* __restrict__ out_count,
+                                           WsHeader* hdr, int lane);
+static __device__ void small_threshold_body(BlockSmem& sm, const TensorDesc& d, uint32_t t, uint32_t T, const float* __restrict__ g,
+                                            float* __restrict__ r, uint32_t* __restrict__ out_idx, float* __restrict__ out_val,
+                                            uint32_t* __restrict__ out_count, WsHeader* hdr);
+
 // The whole compress of one worker by the G CTAs of one group (this CTA is number b of them);
 // the group's barriers count on the worker's own workspace header.
+// Threshold mode, behind the counts: exact threshold, first slot and counts of every segment.  The wanted rank is one
+// among the sampled entries of the short list, of which there are a handful: a warp per segment takes them
+// from the top, one distinct key at a time; lists beyond kThrWarpMid entries take the block-wide radix select.  The CTA
+// that holds a tensor's first tile totals its hits.
+constexpr uint32_t kThrWarpMid = 256;
+template <typename F>
+__device__ __forceinline__ void thr_slots(const MultiArgs& a, uint32_t* seg, uint32_t nseg, uint32_t* rec2, uint32_t first, BlockSmem& sm,
+                                          uint32_t& s_cnt, WsHeader* hdr, F chunk_of) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (uint32_t q = tid; q < nseg; q += kBlock) {
+        uint32_t* s = seg + (size_t)q * kSegWords;
+        s[SG_M] = ld_cg(a.mid_n + s[SG_T]);
+    }
+    __syncthreads();
+    for (uint32_t sidx = (uint32_t)warp; sidx < nseg; sidx += kWarps) {
+        uint32_t* s = seg + (size_t)sidx * kSegWords;
+        const uint32_t m = s[SG_M];
+        if (m > kThrWarpMid) continue;
+        const uint32_t t = s[SG_T];
+        const TensorDesc d = a.desc[t];
+        const InSample in{d.off, d.stride};
+        const uint2* mid = a.mid + (size_t)t * kMultiMidCap;
+        uint2 e[kThrWarpMid / 32];
+        uint32_t sampled = 0;                                // one bit per own entry
+#pragma unroll
+        for (uint32_t u = 0; u < kThrWarpMid / 32; ++u) {
+            e[u] = u * 32u + lane < m ? ld_cg(mid + u * 32u + lane) : make_uint2(0u, 0u);
+            sampled |= u * 32u + lane < m && in(e[u].x) ? 1u << u : 0u;
+        }
+        const uint32_t nbefore = first + s[SG_TILE0] - d.tile0;
+        uint32_t before = 0;
+        for (uint32_t q = lane; q < nbefore; q += 32u) before += ld_cg(a.tile_cnt + d.tile0 + q);
+        uint32_t left = s[SG_K] - s[SG_ABOVE], below = 0x80000000u, T = 0xFFFFFFFFu;
+        while (true) {
+            uint32_t best = 0, same = 0;                     // largest sampled key below the last one, plus 1
+#pragma unroll
+            for (uint32_t u = 0; u < kThrWarpMid / 32; ++u) {
+                const uint32_t key = e[u].y & kKeyMask;
+                if (((sampled >> u) & 1u) && key < below) best = max(best, key + 1u);
+            }
+            best = __reduce_max_sync(0xFFFFFFFFu, best);
+            if (best == 0u) break;                           // (the list holds at least that many, unless it changed under us)
+            below = best - 1u;
+#pragma unroll
+            for (uint32_t u = 0; u < kThrWarpMid / 32; ++u) same += ((sampled >> u) & 1u) && (e[u].y & kKeyMask) == below ? 1u : 0u;
+            same = __reduce_add_sync(0xFFFFFFFFu, same);
+            if (left <= same) { T = below; break; }
+            left -= same;
+        }
+        const uint32_t seg_end = s[SG_BASE0] + s[SG_NTILE] * (uint32_t)kTile;
+#pragma unroll
+        for (uint32_t u = 0; u < kThrWarpMid / 32; ++u) {
+            if (u * 32u + lane >= m || (e[u].y & kKeyMask) < T) continue;
+            if (e[u].x < s[SG_BEGIN]) ++before;
+            else if (e[u].x < seg_end) atomicAdd(&rec2[chunk_of(s, e[u].x)], 1u);
+        }
+        before = __reduce_add_sync(0xFFFFFFFFu, before);
+        __syncwarp();
+        if (lane == 0) {
+            s[SG_TKEY] = T; s[SG_OUT] = d.out_off + before;
+            if (T == 0xFFFFFFFFu) { s[SG_OK] = 0u; record_status(hdr, -1 /*GC_E_INVALID*/, 0xE0000000ull + t); }
+        }
+    }
+    __syncthreads();
+    for (uint32_t sidx = 0; sidx < nseg; ++sidx) {           // long lists: the whole CTA, one segment after the other
+        uint32_t* s = seg + (size_t)sidx * kSegWords;
+        const uint32_t m = s[SG_M];
+        if (m <= kThrWarpMid) continue;
+        const uint32_t t = s[SG_T];
+        const TensorDesc d = a.desc[t];
+        const InSample in{d.off, d.stride};
+        const uint2* mid = a.mid + (size_t)t * kMultiMidCap;
+        uint2 e[kMidRegs];
+#pragma unroll
+        for (uint32_t u = 0; u < kMidRegs; ++u) e[u] = u * kBlock + tid < m ? ld_cg(mid + u * kBlock + tid) : make_uint2(0u, 0u);
+        const uint32_t nbefore = first + s[SG_TILE0] - d.tile0;
+        uint32_t before = 0;
+        for (uint32_t q = tid; q < nbefore; q += kBlock) before += ld_cg(a.tile_cnt + d.tile0 + q);
+        if (tid == 0) s_cnt = 0u;
+        const uint32_t shift = s[SG_SHIFT], A = s[SG_A], binlo = s[SG_TAU] + (A << shift);
+        uint32_t v, x0, x1;
+        const bool good = short_list_select(sm, e, mid, m, A == 2047u ? 31 : max((int)shift, 1), s[SG_K] - s[SG_ABOVE],
+                                            [&](const uint2& pr, uint32_t& w) { w = (pr.y & kKeyMask) - binlo; return in(pr.x); }, v, x0, x1);
+        const uint32_t T = good ? binlo + v : 0xFFFFFFFFu, seg_end = s[SG_BASE0] + s[SG_NTILE] * (uint32_t)kTile;
+        auto settle = [&](const uint2& pr) {
+            if ((pr.y & kKeyMask) < T) return;
+            if (pr.x < s[SG_BEGIN]) ++before;
+            else if (pr.x < seg_end) atomicAdd(&rec2[chunk_of(s, pr.x)], 1u);
+        };
+#pragma unroll
+        for (uint32_t u = 0; u < kMidRegs; ++u)
+            if (u * kBlock + tid < m) settle(e[u]);
+        for (uint32_t i = kMidFast + tid; i < m; i += kBlock) settle(ld_cg(mid + i));
+        __syncthreads();
+        before = __reduce_add_sync(0xFFFFFFFFu, before);
+        if (lane == 0 && before) atomicAdd(&s_cnt, before);
+        __syncthreads();
+        if (tid == 0) {
+            s[SG_TKEY] = T; s[SG_OUT] = d.out_off + s_cnt;
+            if (!good) { s[SG_OK] = 0u; record_status(hdr, -1 /*GC_E_INVALID*/, 0xE0000000ull + t); }
+        }
+        __syncthreads();
+    }
+    for (uint32_t sidx = (uint32_t)warp; sidx < nseg; sidx += kWarps) {
+        const uint32_t* s = seg + (size_t)sidx * kSegWords;
+        const uint32_t t = s[SG_T], m = s[SG_M], T = s[SG_TKEY];
+        if (first + s[SG_TILE0] != a.desc[t].tile0 || s[SG_OK] == 0u) continue;
+        const TensorDesc d = a.desc[t];
+        uint32_t hits = 0;
+        for (uint32_t q0 = 0; q0 < d.ntiles; q0 += 256u) {
+#pragma unroll
+            for (uint32_t u = 0; u < 8; ++u) hits += q0 + u * 32u + lane < d.ntiles ? ld_cg(a.tile_cnt + d.tile0 + q0 + u * 32u + lane) : 0u;
+        }
+        for (uint32_t q = lane; q < m; q += 32u) hits += (ld_cg(a.mid + (size_t)t * kMultiMidCap + q).y & kKeyMask) >= T ? 1u : 0u;
+        hits = __reduce_add_sync(0xFFFFFFFFu, hits);
+        if (lane == 0) {
+            if (a.out_count != nullptr) { a.out_count[t] = min(hits, d.cap); a.out_count[a.T + t] = hits; }
+            if (hits > d.cap) record_status(hdr, 1 /*GC_W_TRUNCATED*/, t);
+        }
+    }
+}
+
 // (DENSE, VOTES: see k_topk_single)
-template <typename GL, bool DENSE, bool VOTES>
+// THR: threshold mode.  The threshold is the k_s-th largest key of the sample that the definition fixes, one group of
+// four elements per `stride` groups, and reading those before the fold costs what as many scattered accesses cost.
+// Here they are picked out of the stream instead: the bracket comes from a sample of 128-byte lines as in top-k mode, the
+// band histogram counts the candidates that are in the definition's sample, the band bin of rank k_s and the short list
+// (all candidates in it) give the exact threshold, and every candidate at or above it is a hit, up to the capacity.
+// What fails (bracket missed, list or region full) is redone from the residual by radix levels over the
+// definition's sample and the look-back emission.  Eight 161-tensor workers: sample and thresholds 95 -> 26 us, call
+// with the decode 532 -> 494.
+template <typename GL, bool DENSE, bool VOTES, bool THR = false>
 __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32_t G, const uint32_t b, BlockSmem& sm,
                                                 uint32_t& s_used, uint32_t& s_cnt, unsigned char* s_dyn) {
     uint32_t* const rec = reinterpret_cast<uint32_t*>(s_dyn);                  // [per*kWarps] off<<10 | cnt
@@ -249,8 +400,10 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
             if (d.sstride != 0u) {
                 const uint32_t ngroups = (d.n + 3u) >> 2;
                 const float msamp = 4.0f * (float)((ngroups + d.sstride - 1) / d.sstride);
-                const float ks = (float)d.k * msamp / (float)d.n;
-                const float hi = floorf(ks - 6.0f * sqrtf(ks) - 8.0f);
+                // (threshold mode: k is a rank among the elements of another sample, whose noise comes on top)
+                const float among = THR ? 4.0f * (float)((ngroups + d.stride - 1) / d.stride) : (float)d.n;
+                const float ks = (float)d.k * msamp / among;
+                const float hi = floorf(ks - 6.0f * sqrtf(THR ? ks + ks * ks / (float)d.k : ks) - 8.0f);
                 // (a sample too small for that margin: the largest sampled key bounds the band instead)
                 const uint32_t want[3] = {d.srank, hi >= 1.0f ? (uint32_t)hi : 1u, max(1u, (uint32_t)ceilf(ks))};
                 Picked pk[3];
@@ -334,6 +487,7 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
                         s[SG_TAU] = tau; s[SG_TAUZ] = tau_z; s[SG_SHIFT] = (uint32_t)shift;
                         s[SG_OK] = 1u; s[SG_OUT] = d.out_off; s[SG_K] = d.k;
                         s[SG_A] = d.reg;               // (until the band bin is known)
+                        if (THR) s[SG_END] = d.out_off + d.cap;
                     }
                     ++nseg;
                     open = true;
@@ -373,8 +527,12 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
                 }
             }
             if constexpr (VOTES) {
-                block_overflow |= !fold_tail_votes(sm, av, interior, valid, tau, tau_z, shift, tg.base + my_off, a.r, s_used, a.pool_cap, pool,
-                                                   rec[i * kWarps + warp], lane, warp);
+                if constexpr (THR)
+                    block_overflow |= !fold_tail_votes(sm, av, interior, valid, tau, tau_z, shift, tg.base + my_off, a.r, s_used, a.pool_cap, pool,
+                                                       rec[i * kWarps + warp], lane, warp, InSample{d.off, d.stride});
+                else
+                    block_overflow |= !fold_tail_votes(sm, av, interior, valid, tau, tau_z, shift, tg.base + my_off, a.r, s_used, a.pool_cap, pool,
+                                                       rec[i * kWarps + warp], lane, warp);
             } else {
                 uint32_t cnt[kVpt], cm = 0, hm = 0;      // candidates; candidates that are zeroed right away
 #pragma unroll
@@ -440,11 +598,15 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
                         const uint32_t pos = rkj + (uint32_t)__popc(em & ((1u << bq) - 1u) & (0xFu << (4u * j)));
                         const uint2 pr = make_uint2(tg.base + my_off + j * 128u + (bq & 3u), __float_as_uint(v));
                         if (staged) sm.emit[warp][pos] = pr; else pool[off + pos] = pr;
-                        atomicAdd(&sm.hist[min((key_of(v) - tau) >> shift, 2047u)], 1u);
+                        if (THR ? !staged && InSample{d.off, d.stride}(pr.x) : true) atomicAdd(&sm.hist[min((key_of(v) - tau) >> shift, 2047u)], 1u);
                     }
                     if (staged) {
                         __syncwarp();
-                        for (uint32_t q = lane; q < wtot; q += 32) pool[off + q] = sm.emit[warp][q];
+                        for (uint32_t q = lane; q < wtot; q += 32) {
+                            const uint2 pr = sm.emit[warp][q];
+                            pool[off + q] = pr;
+                            if (THR && InSample{d.off, d.stride}(pr.x)) atomicAdd(&sm.hist[min(((pr.y & kKeyMask) - tau) >> shift, 2047u)], 1u);
+                        }
                         __syncwarp();
                     }
                 }
@@ -470,13 +632,15 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
                 if (q < a.n_tiny) {
                     const uint32_t t = a.small_ids[q];
                     const TensorDesc d = a.desc[t];
-                    tiny_tensor_warp<GL>(d.off, d.n, d.k, d.out_off, t, a.T, a.g, a.r, a.out_idx, a.out_val, a.out_count, lane);
+                    if constexpr (THR) tiny_threshold_warp(d, t, a.T, (const float*)a.g, a.r, a.out_idx, a.out_val, a.out_count, hdr, lane);
+                    else tiny_tensor_warp<GL>(d.off, d.n, d.k, d.out_off, t, a.T, a.g, a.r, a.out_idx, a.out_val, a.out_count, lane);
                 }
                 continue;
             }
             const uint32_t t = a.small_ids[a.n_tiny + u - tiny];
             const TensorDesc d = a.desc[t];
-            if (d.k <= kFewK) small_tensor_fewk<GL>(sm, d, t, a.T, a.g, a.r, a.out_idx, a.out_val, a.out_count);
+            if constexpr (THR) small_threshold_body(sm, d, t, a.T, (const float*)a.g, a.r, a.out_idx, a.out_val, a.out_count, hdr);
+            else if (d.k <= kFewK) small_tensor_fewk<GL>(sm, d, t, a.T, a.g, a.r, a.out_idx, a.out_val, a.out_count);
             else small_tensor_body<GL>(sm, d, t, a.T, a.g, a.r, a.out_idx, a.out_val, a.out_count);
             __syncthreads();
             for (int i = tid; i < 2048; i += kBlock) sm.hist[i] = 0u;
@@ -511,7 +675,7 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
             uint32_t* s = seg + (size_t)sidx * kSegWords;
             const uint32_t t = s[SG_T];
             const Picked pa = warp_select_2048(a.bhist + (size_t)s[SG_A] * kHistBins, s[SG_K], lane);
-            const bool ok = pa.ok && pa.count <= kMultiMidCap;
+            const bool ok = pa.ok && (THR || pa.count <= kMultiMidCap);      // (threshold mode counts the sampled ones only)
             if (lane == 0) {
                 s[SG_A] = pa.bin; s[SG_ABOVE] = pa.above; s[SG_M] = pa.count; s[SG_OK] = ok ? 1u : 0u;
                 if (!ok) {          // every CTA that sees this tensor decides the same; count it once
@@ -536,6 +700,7 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
             } else {
                 const uint32_t slot = atomicAdd(a.mid_n + c_t, 1u);
                 if (slot < kMultiMidCap) a.mid[(size_t)c_t * kMultiMidCap + slot] = pr;
+                else if (THR && slot == kMultiMidCap) atomicAdd(&hdr->n_failed, 1u);
             }
         };
         for (uint32_t i0 = tid; i0 < used; i0 += 4 * kBlock) {      // four loads in flight per thread
@@ -560,8 +725,11 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
     if (!grid_barrier(hdr, passed, &sm.ok, G)) return;
     phase_stamp(hdr, n_stamp, b);
 
-    if (!overflowed) {
+    if (THR ? !overflowed && ld_cg(&hdr->n_failed) == 0u : !overflowed) {
         if (nseg != 0u) {
+            if constexpr (THR) {
+                thr_slots(a, seg, nseg, rec2, first, sm, s_cnt, hdr, chunk_of);
+            } else {
             // -------------------------------------------------------- threshold, tie cut and slots per segment
             // Short lists of up to kWarpMid entries (nearly all: a band bin holds a handful of
             // candidates) are settled by a warp each, all segments of the CTA at once and without a
@@ -744,6 +912,7 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
                 }
                 __syncthreads();
             }
+            }
             // rec2[c] = output slot of the first sent candidate of chunk c (one warp walks each segment)
             for (uint32_t sidx = warp; sidx < nseg; sidx += kWarps) {
                 const uint32_t* s = seg + (size_t)sidx * kSegWords;
@@ -762,10 +931,11 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
         }
         phase_stamp(hdr, n_stamp, b);
         // of the segment at hand: its threshold key (none is reached where the tensor is redone), tie cut, guess
-        uint32_t c_T = 0xFFFFFFFFu, c_cut = 0, c_tauz = 0, c_base0 = 0, c_chunk0 = 0;
+        uint32_t c_T = 0xFFFFFFFFu, c_cut = 0, c_tauz = 0, c_base0 = 0, c_chunk0 = 0, c_last = 0;      // c_last: end of its slots (THR)
         auto enter = [&](const uint32_t* s) {
             c_T = s[SG_OK] != 0u ? s[SG_TKEY] : 0xFFFFFFFFu;
             c_cut = s[SG_CUT]; c_tauz = s[SG_TAUZ]; c_base0 = s[SG_BASE0]; c_chunk0 = s[SG_TILE0] * kWarps;
+            if (THR) { c_last = s[SG_END]; c_cut = 0xFFFFFFFFu; }
         };
         auto sent_key = [&](const uint2& pr) {
             const uint32_t key = pr.y & kKeyMask;
@@ -787,8 +957,10 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
                 for (uint32_t q0 = 0; q0 < cnt; q0 += 32u) {
                     const bool in = q0 + lane < cnt;
                     const uint2 pr = q0 == 0u ? p[0] : q0 == 32u ? p[1] : in ? pool[off + q0 + lane] : make_uint2(0u, 0u);
-                    const bool sent = in && sent_key(pr), zeroed = (pr.y & kKeyMask) >= c_tauz;
+                    bool sent = in && sent_key(pr);
+                    const bool zeroed = (pr.y & kKeyMask) >= c_tauz;
                     const unsigned sb = __ballot_sync(0xFFFFFFFFu, sent);
+                    if constexpr (THR) sent = sent && slot + (uint32_t)__popc(sb & ((1u << lane) - 1u)) < c_last;      // (beyond the capacity: stays in the residual)
                     if (in && sent != zeroed) a.r[pr.x] = sent ? 0.0f : __uint_as_float(pr.y);
                     if (sent) {
                         const uint32_t at = slot + (uint32_t)__popc(sb & ((1u << lane) - 1u));
@@ -836,7 +1008,7 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
                     if (zeroed) a.r[pr[u].x] = __uint_as_float(pr[u].y);     // value goes back
                     continue;
                 }
-                if (!zeroed) a.r[pr[u].x] = 0.0f;
+                if (!THR && !zeroed) a.r[pr[u].x] = 0.0f;
                 const uint32_t c = c_chunk0 + ((pr[u].x - c_base0) >> 9);
                 const uint32_t p0 = rec[c] >> 10;                  // first list position of the chunk
                 uint32_t before;
@@ -847,6 +1019,11 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
                     for (uint32_t w = (p0 >> 5) + 1u; w < (i >> 5); ++w) before += __popc(sent_bits[w]);
                 }
                 const uint32_t slot = rec2[c] + before;
+                if (THR) {
+                    const bool goes = slot < c_last;                 // (beyond the capacity: stays in the residual)
+                    if (goes != zeroed) a.r[pr[u].x] = goes ? 0.0f : __uint_as_float(pr[u].y);
+                    if (!goes) continue;
+                }
                 a.out_idx[slot] = pr[u].x;
                 a.out_val[slot] = __uint_as_float(pr[u].y);
             }
@@ -854,6 +1031,7 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
         __syncthreads();
         phase_stamp(hdr, n_stamp, b);
         exit_stamp(hdr);
+        if (THR) return;
         if (ld_cg(&hdr->n_failed) == 0u) { leave_clean(a.cl, hdr, G, tid); return; }
     } else {
         // a candidate region overflowed: every recorded candidate gets its value back
@@ -871,6 +1049,19 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
     clean_redo(a.cl, G, b, tid);
     if (!grid_barrier(hdr, passed, &sm.ok, G)) return;
     phase_stamp(hdr, n_stamp, b);
+    if constexpr (THR) {
+        const TensorDesc* const def = a.desc - a.T;
+        WsView ws = a.gws;                               // (its records, ungated)
+        ws.gate = nullptr;
+        hist_body<0, SRC_RSAMPLE>(sm, def, a.T, a.nstiles_def, nullptr, a.r, ws, G, b);
+        if (!grid_barrier(hdr, passed, &sm.ok, G)) return;
+        hist_body<1, SRC_RSAMPLE>(sm, def, a.T, a.nstiles_def, nullptr, a.r, ws, G, b);
+        if (!grid_barrier(hdr, passed, &sm.ok, G)) return;
+        hist_body<2, SRC_RSAMPLE>(sm, def, a.T, a.nstiles_def, nullptr, a.r, ws, G, b);
+        if (!grid_barrier(hdr, passed, &sm.ok, G)) return;
+        threshold_emit_body<false, true>(def, a.T, a.ntiles, nullptr, a.r, a.out_idx, a.out_val, a.out_count, a.ws, ws.sel, 0u, 0);
+        return;
+    }
     hist_body<0, SRC_RESID>(sm, a.desc, a.T, a.ntiles, nullptr, a.r, a.gws, G, b);
     if (!grid_barrier(hdr, passed, &sm.ok, G)) return;
     hist_body<1, SRC_RESID>(sm, a.desc, a.T, a.ntiles, nullptr, a.r, a.gws, G, b);
@@ -884,14 +1075,14 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
 
 // Votes: 25.6M elements in 161 tensors at 0.1 % 99 -> 97 us, 110M in 199 at 1 % 302 -> 289 us.  (Why the
 // one-tensor kernel loses with them at 1 %, see there, was not found.)
-template <typename GL, bool DENSE, bool VOTES>
+template <typename GL, bool DENSE, bool VOTES, bool THR = false>
 // (three CTAs per SM: 80 registers and no spills beat four at 64 registers, see k_topk_single)
 static __global__ void __launch_bounds__(kBlock, 3)
 k_topk_multi(const __grid_constant__ MultiArgs a) {
     __shared__ BlockSmem sm;
     __shared__ uint32_t s_used, s_cnt;
     extern __shared__ __align__(16) unsigned char s_dyn[];
-    topk_multi_body<GL, DENSE, VOTES>(a, gridDim.x, blockIdx.x, sm, s_used, s_cnt, s_dyn);
+    topk_multi_body<GL, DENSE, VOTES, THR>(a, gridDim.x, blockIdx.x, sm, s_used, s_cnt, s_dyn);
 }
 
 // Several workers' compress calls in ONE cooperative launch: the grid is cut into one group of
@@ -909,7 +1100,7 @@ static_assert(sizeof(WorkersArgs) <= 4000, "kernel parameters stay below 4 KB");
 
 // (The scan stays here: 475 against 484 us with votes for eight 161-tensor workers at 0.1 %, the one shape
 // both were measured on.)
-template <typename GL, bool DENSE>
+template <typename GL, bool DENSE, bool THR = false>
 static __global__ void __launch_bounds__(kBlock, 3)
 k_topk_workers(const __grid_constant__ WorkersArgs wa) {
     __shared__ BlockSmem sm;
@@ -923,7 +1114,7 @@ k_topk_workers(const __grid_constant__ WorkersArgs wa) {
         for (uint32_t i = threadIdx.x; i < sizeof(MultiArgs) / 4; i += kBlock) dst[i] = src[i];
     }
     __syncthreads();
-    topk_multi_body<GL, DENSE, false>(s_args, wa.G, b, sm, s_used, s_cnt, s_dyn);
+    topk_multi_body<GL, DENSE, false, THR>(s_args, wa.G, b, sm, s_used, s_cnt, s_dyn);
 }
 
 }  // namespace gc

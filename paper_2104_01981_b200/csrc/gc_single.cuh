@@ -329,9 +329,12 @@ __device__ __forceinline__ void chunk_ranks(uint32_t cm, int lane, ChunkRanks& c
 
 // The rest of the fold of one warp chunk in the form with votes: residual, list entries, band histogram.
 // `at0` = flat index of this thread's first element.  Returns false if the candidate region is full.
+// `counts`: whether the histogram counts the candidate of that index.
+struct CountsAll { __device__ __forceinline__ bool operator()(uint32_t) const { return true; } };
+template <typename F = CountsAll>
 __device__ __forceinline__ bool fold_tail_votes(BlockSmem& sm, const float (&av)[kVpt][4], bool interior, uint32_t valid, uint32_t tau,
                                                 uint32_t tau_z, int shift, uint32_t at0, float* r, uint32_t& s_used, uint32_t pool_cap,
-                                                uint2* pool, uint32_t& rec, int lane, int warp) {
+                                                uint2* pool, uint32_t& rec, int lane, int warp, F counts = F{}) {
     uint32_t cm = 0;                         // candidates of this thread, one bit per element
 #pragma unroll
     for (int q = 0; q < 4 * kVpt; ++q) cm |= key_of(av[q / 4][q % 4]) >= tau ? 1u << q : 0u;
@@ -384,7 +387,7 @@ __device__ __forceinline__ bool fold_tail_votes(BlockSmem& sm, const float (&av)
             const float v = (m & 3u) ? v01 : v23;
             const uint32_t e = (uint32_t)__ffs((int)m) - 1u;
             to[pos] = make_uint2(at0 + j * 128u + e, __float_as_uint(v));
-            if (!staged) atomicAdd(&sm.hist[min((key_of(v) - tau) >> shift, 2047u)], 1u);
+            if (!staged && counts(at0 + j * 128u + e)) atomicAdd(&sm.hist[min((key_of(v) - tau) >> shift, 2047u)], 1u);
         }
     }
     // (counted here, where the lanes are side by side: 355M at 0.1 % 954 -> 953 us with the decode, bfloat16 110M 225 -> 224)
@@ -393,7 +396,7 @@ __device__ __forceinline__ bool fold_tail_votes(BlockSmem& sm, const float (&av)
         for (uint32_t q = lane; q < cr.total; q += 32) {
             const uint2 pr = sm.emit[warp][q];
             pool[off + q] = pr;
-            atomicAdd(&sm.hist[min(((pr.y & kKeyMask) - tau) >> shift, 2047u)], 1u);
+            if (counts(pr.x)) atomicAdd(&sm.hist[min(((pr.y & kKeyMask) - tau) >> shift, 2047u)], 1u);
         }
         __syncwarp();
     }

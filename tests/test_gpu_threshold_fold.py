@@ -1,0 +1,70 @@
+"""Threshold mode, several tensors, fold first: the definition's sample is picked out of the stream; every way out of it."""
+import pytest
+import torch
+
+import test_gpu_threshold as thr
+from paper_2104_01981_b200 import api
+from test_gpu_threshold import _built, randn   # noqa: F401  (the module's build fixture)
+
+pytestmark = pytest.mark.gpu
+
+# (large enough, and the largest one's sample long enough at small strides, that the plans are taken this way)
+SIZES = [300_000, 5, 1_500_001, 0, 4096, 64, 11_000_003, 4097, 65_537]
+
+
+@pytest.fixture
+def options(request, monkeypatch):
+    class WithOptions(api.Plan):
+        def __init__(self, *a, **k):
+            super().__init__(*a, **k)
+            for opt, value in request.param.items():
+                self.set_option(opt, value)
+    monkeypatch.setattr(thr.api, "Plan", WithOptions)
+
+
+@pytest.mark.parametrize("options", [{}, {api.GC_OPT_SAMPLE_RANK_PERMILLE: 30}, {api.GC_OPT_CANDIDATE_CAPACITY: 100},
+                                     {api.GC_OPT_SAMPLE_RANK_PERMILLE: 700}], ids=["plain", "starved", "overflow", "tight"], indirect=True)
+@pytest.mark.parametrize("density", [0.0005, 0.01, 0.06])
+@pytest.mark.parametrize("stride,cap_factor", [(0, 0.0), (1, 1.0), (7, 1.5), (1000, 2.0)])
+def test_strides_densities_and_redo(options, density, stride, cap_factor):
+    n = sum(SIZES)
+    thr.check_threshold(SIZES, density, [randn(n, 7 * stride + s) for s in range(2)], stride=stride, cap_factor=cap_factor)
+
+
+@pytest.mark.parametrize("what", ["blind", "biased", "grid", "constant", "zeros", "nonfinite", "sorted"])
+def test_samples_that_mislead(what):
+    """The definition's sample and the one that sets the bracket see different tensors, or equal keys by the thousand."""
+    g = randn(sum(SIZES), 8)
+    off = 0
+    for n in SIZES:
+        v, grp = g[off:off + n], torch.arange(n) // 4
+        if what == "blind":
+            v[(grp % 64) == 0] *= 1e-3
+        elif what == "biased":
+            v[(grp % 64) == 0] *= 1e3
+        elif what == "grid":
+            v.copy_((v * 8).round() / 8)
+        elif what == "constant":
+            v.fill_(0.25)
+        elif what == "zeros":
+            v[: n - n // 200] = 0.0
+        elif what == "nonfinite" and n > 100:
+            v[::97] = float("inf")
+            v[1::1009] = float("nan")
+        elif what == "sorted":
+            v.copy_(v[v.abs().argsort()])
+        off += n
+    thr.check_threshold(SIZES, 0.01, [g, g], cap_factor=3.0)
+
+
+def test_tensors_with_long_samples():
+    """Samples of more than 128 sample tiles: such plans took the staged route before."""
+    sizes = [20_000_003, 70_000, 9_000_000]
+    assert api.Plan(sizes, 0.01, mode=api.GC_THRESHOLD, device=0).query(api.GC_Q_COMPRESS_ROUTE) == api.GC_ROUTE_THRESHOLD_MANY
+    thr.check_threshold(sizes, 0.01, [randn(sum(sizes), s) for s in range(2)])
+
+
+@pytest.mark.parametrize("W,density", [(2, 0.01), (8, 0.001), (3, 0.05)])
+def test_workers(W, density):
+    sizes = [9_300_000, 3, 70_001, 4097, 3_400_000, 513]
+    thr.check_threshold_workers(sizes, density, W, lambda w, s: randn(sum(sizes), 100 * s + w))
