@@ -32,10 +32,11 @@ constexpr uint32_t kSegWords = 16;               // shared-memory words per segm
 constexpr uint32_t kRefineTiles = 32;            // samples of up to this many sample tiles are ranked a second time
 // Short lists up to kWarpMid entries are settled by one warp (a CTA with many segments has eight at a time), up
 // to kRankMid by the whole CTA, every entry against all others; longer ones by radix select.  A warp alone
-// takes 4 us for 100 entries, radix select 10 us whatever the length, and the CTAs of large tensors came that much
+// takes 4 us for 100 entries and radix select 3 us or more, and the CTAs of large tensors came that much
 // later: 161 tensors of 25.6M elements at 0.1 % 100 -> 91 us, a dozen of 30M at 0.4 % 125 -> 113, 199 of 110M at 1 % 286 -> 279.
+// (direct ranking up to 512 entries instead of 128: 110M in 199 tensors at 5 % 324.5 / 316.7, the dozen 111.8 / 109.3.)
 constexpr uint32_t kWarpMid = 32;
-constexpr uint32_t kRankMid = 512;
+constexpr uint32_t kRankMid = 128;
 
 // Contiguous runs of tiles: CTAs below c1 take n1 tiles each, those from there below c2 take n2, the others share
 // the rest evenly.  The CTAs launched last are the youngest on their SMs and advance the slowest (see RowMap in
