@@ -74,6 +74,9 @@ struct gc_plan_s : DeviceFacts {
     uint32_t single_grid = 0;               // CTAs of the first (0 = plan does not qualify)
     size_t off_hist5 = 0, off_rowseg = 0, off_mid = 0, off_fine = 0, off_start = 0;
     uint32_t single_srank_hi = 0, single_srank_mid = 0;
+    SingleGeom thr_single;                  // one-tensor threshold plan, fold first (k_topk_single with THR; G = 0: no)
+    TensorDesc thr_d = {};                  // its tensor with the bracket's sample
+    uint32_t thr_srank_hi = 0, thr_srank_mid = 0;
     uint32_t thr_grid = 0, thr_maxt = 0, thr_pool = 0, thr_rounds = 0;    // one-tensor threshold kernel (0 = no)
     size_t thr_smem = 0;
     // threshold mode, several tensors, fold first (k_topk_multi with THR): the table with the bracket's sample
@@ -123,6 +126,8 @@ constexpr double kSingleSkew = 0.08, kSingleSkewSparse = 0.04;
 constexpr size_t kSingleRowBytes = (2 * kWarps + 4) * sizeof(uint32_t);   // shared memory per owned tile
 constexpr double kSparseUpTo = 0.002;        // density up to which most chunks are empty (see VOTES of k_topk_single)
 constexpr double kDenseFrom = 0.02;          // density from which the forms with emission by chunk are taken (12 candidates per chunk)
+constexpr double kThrOneFoldUpTo = 0.02;     // one tensor: the same, and the elements from which (see plan_thr_single_fold)
+constexpr uint32_t kThrOneFoldFrom = 12u << 20;
 constexpr double kThrFoldUpTo = 0.005;       // density up to which, and elements from which threshold plans of several tensors are
 constexpr uint64_t kThrFoldFrom = 12u << 20; // taken fold first (see plan_thr_fold)
 constexpr uint32_t kMultiMaxTab = 1024;      // tensors whose tile tables k_topk_multi keeps in shared memory
@@ -364,6 +369,33 @@ static RowMap make_row_map(const gc_plan_s* p, uint32_t ntiles, uint32_t G, uint
     return rm;
 }
 
+// Geometry of k_topk_single for tensor d with the bracket's sample in it (G = 0: no).
+SingleGeom single_geometry(const gc_plan_s* p, const TensorDesc& d, bool bf16) {
+    SingleGeom g;
+    const uint64_t groups = ((uint64_t)d.n + 3) / 4, nsg = (groups + d.sstride - 1) / d.sstride;
+    g.votes = bf16 || p->mode == GC_THRESHOLD || p->density <= kSparseUpTo;
+    g.G = std::min<uint32_t>((uint32_t)p->grid_single_max, d.ntiles);
+    // Small tensors are all latency (a CTA has a handful of tiles and five phases to walk through):
+    // there two CTAs per SM get through the phases sooner than three (2M-10M elements: 31-49 us
+    // against 37-51 us).  From about 12M elements on the third CTA pays for itself, except on sparse
+    // plans of fp32 gradients (see VOTES); below 300 tiles there is a CTA per tile anyway (fewer were
+    // no faster).  Sparse plans of more tiles than two CTAs per SM may own (413M elements) keep the
+    // third: 420M at 0.1 % 836 us against 1103 us on the general kernel, which reads no bfloat16 at all.
+    const uint32_t two = 2u * (uint32_t)p->sm_count;
+    if (d.ntiles <= 3000u || (!bf16 && p->density <= kSparseUpTo && d.ntiles <= two * (uint32_t)kSingleMaxT)) g.G = std::min(g.G, two);
+    g.maxt = (d.ntiles + g.G - 1) / g.G;
+    g.rows = make_row_map(p, d.ntiles, g.G, g.maxt, g.votes ? 0.0 : p->density >= 0.005 ? kSingleSkew : kSingleSkewSparse);
+    if (g.maxt > kSingleMaxT || g.G > kSingleMaxG) return SingleGeom{};               // chunk records and totals must stay small
+    // region per CTA; one bit per slot has to fit in shared memory beside the chunk records
+    g.pool = std::min<uint32_t>(p->cand_cap_alloc / g.G, kSinglePoolMax);
+    g.smem = (size_t)g.maxt * kSingleRowBytes + sizeof(uint32_t) * ((g.pool + 31) / 32);
+    // expected candidates per CTA (sample rank over sample size, times n), with head-room
+    if (nsg > (uint64_t)2 * g.G * kBlock) return SingleGeom{};                // a thread owns at most two sample groups
+    const double expect = (double)d.n * (double)d.srank / (4.0 * (double)nsg) / (double)g.G;
+    if ((double)g.pool < 1.5 * expect + 512.0) return SingleGeom{};
+    return g;
+}
+
 // Decides whether the plan can use the single-tensor kernel and with which geometries.
 void plan_single(gc_plan_s* p) {
     p->single_grid = 0;
@@ -373,27 +405,8 @@ void plan_single(gc_plan_s* p) {
     if (d.ntiles >= (1u << 20)) return;                              // (the row arithmetic divides by multiplication)
     const uint64_t groups = ((uint64_t)d.n + 3) / 4, nsg = (groups + d.sstride - 1) / d.sstride;
     for (int bf16 = 0; bf16 < 2; ++bf16) {
-        SingleGeom g;
-        g.votes = bf16 != 0 || p->density <= kSparseUpTo;
-        g.G = std::min<uint32_t>((uint32_t)p->grid_single_max, d.ntiles);
-        // Small tensors are all latency (a CTA has a handful of tiles and five phases to walk through):
-        // there two CTAs per SM get through the phases sooner than three (2M-10M elements: 31-49 us
-        // against 37-51 us).  From about 12M elements on the third CTA pays for itself, except on sparse
-        // plans of fp32 gradients (see VOTES); below 300 tiles there is a CTA per tile anyway (fewer were
-        // no faster).  Sparse plans of more tiles than two CTAs per SM may own (413M elements) keep the
-        // third: 420M at 0.1 % 836 us against 1103 us on the general kernel, which reads no bfloat16 at all.
-        const uint32_t two = 2u * (uint32_t)p->sm_count;
-        if (d.ntiles <= 3000u || (bf16 == 0 && p->density <= kSparseUpTo && d.ntiles <= two * (uint32_t)kSingleMaxT)) g.G = std::min(g.G, two);
-        g.maxt = (d.ntiles + g.G - 1) / g.G;
-        g.rows = make_row_map(p, d.ntiles, g.G, g.maxt, g.votes ? 0.0 : p->density >= 0.005 ? kSingleSkew : kSingleSkewSparse);
-        if (g.maxt > kSingleMaxT || g.G > kSingleMaxG) return;               // chunk records and totals must stay small
-        // region per CTA; one bit per slot has to fit in shared memory beside the chunk records
-        g.pool = std::min<uint32_t>(p->cand_cap_alloc / g.G, kSinglePoolMax);
-        g.smem = (size_t)g.maxt * kSingleRowBytes + sizeof(uint32_t) * ((g.pool + 31) / 32);
-        // expected candidates per CTA (sample rank over sample size, times n), with head-room
-        if (nsg > (uint64_t)2 * g.G * kBlock) return;                // a thread owns at most two sample groups
-        const double expect = (double)d.n * (double)d.srank / (4.0 * (double)nsg) / (double)g.G;
-        if ((double)g.pool < 1.5 * expect + 512.0) return;
+        const SingleGeom g = single_geometry(p, d, bf16 != 0);
+        if (g.G == 0) return;
         p->single[bf16] = g;
     }
     // upper bracket: the sample rank that stays below the expected one by the same margin
@@ -402,6 +415,29 @@ void plan_single(gc_plan_s* p) {
     p->single_srank_hi = hi >= 1.0 ? (uint32_t)hi : 1u;    // small sample: the largest sampled key bounds the band
     p->single_srank_mid = (uint32_t)std::max(1.0, std::ceil(ks));
     p->single_grid = p->single[0].G;
+}
+
+// The same for a threshold plan that is taken fold first.
+// Sample-first / fold-first, us: 14M elements at 0.1 % 55.3 / 53.7, 1 % 57.0 / 55.7, 2 % 59.2 / 57.7, 5 % 60.0 / 62.8; 40M 109 / 103,
+// 110.3 / 108.0, 113.7 / 113.8, 122 / 125; 110M 255 / 229, 264 / 244, 273 / 254, 291 / 285; 355M at 0.1 % 768 / 679, 1 % 819 / 715.  At 5M the
+// two are equal up to 1 % (39.0 / 38.7) and the sample first is ahead above (2 % 39.5 / 40.8).
+void plan_thr_single_fold(gc_plan_s* p) {
+    p->thr_single = SingleGeom{};
+    if (p->mode != GC_THRESHOLD || p->T != 1 || p->grid_single_max <= 0) return;
+    TensorDesc d = p->desc[0];
+    if (d.srank == 0 || d.ntiles == 0 || d.off != 0 || d.ntiles >= (1u << 20)) return;
+    if (p->thr_grid > 0 && (p->density > kThrOneFoldUpTo || d.n < kThrOneFoldFrom)) return;
+    const uint64_t groups = ((uint64_t)d.n + 3) / 4, stride = std::max<uint64_t>(1, d.n / std::min<uint64_t>(kSampleMaxSingle, std::max<uint64_t>(d.n / 128, 8192)));
+    const double m = 4.0 * (double)((groups + stride - 1) / stride), among = 4.0 * (double)((groups + d.stride - 1) / d.stride);
+    const double ks = (double)d.srank * m / among, sd = std::sqrt(ks + ks * ks / (double)d.srank);
+    const double rank = std::max(1.0, std::ceil(ks + 6.0 * sd + 8.0) * (double)p->rank_permille / 1000.0), hi = std::floor(ks - 6.0 * sd - 8.0);
+    if (rank >= 0.9 * m) return;
+    d.k = d.srank;
+    d.sstride = (uint32_t)stride; d.srank = (uint32_t)rank;
+    p->thr_d = d;
+    p->thr_srank_hi = hi >= 1.0 ? (uint32_t)hi : 1u;
+    p->thr_srank_mid = (uint32_t)std::max(1.0, std::ceil(ks));
+    p->thr_single = single_geometry(p, d, false);
 }
 
 // Decides whether a threshold plan can use the one-tensor kernel and with which geometry.
@@ -690,7 +726,8 @@ static bool ask_device(int device, DeviceFacts* p) {
             int nb = 1 << 20;
             for (const void* fn : {(const void*)k_topk_single<GradF32, false, false>, (const void*)k_topk_single<GradF32, true, false>,
                                    (const void*)k_topk_single<GradF32, false, true>, (const void*)k_topk_single<GradBF16, false, true>,
-                                   (const void*)k_topk_single<GradBF16, true, true>}) {
+                                   (const void*)k_topk_single<GradBF16, true, true>, (const void*)k_topk_single<GradF32, false, true, true>,
+                                   (const void*)k_topk_single<GradF32, true, true, true>}) {
                 int n1 = 0;
                 if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n1, fn, kBlock, smem_max) != cudaSuccess) n1 = 0;
                 nb = std::min(nb, n1);
@@ -948,6 +985,7 @@ static int fill_plan(gc_plan_s* p, int device, uint32_t n_tensors, const uint64_
     plan_thr_single(p);
     plan_thr_multi(p);
     plan_multi(p);
+    plan_thr_single_fold(p);
     plan_thr_fold(p);
     return p->tdesc.empty() ? GC_OK : upload_table(p);
 }
@@ -970,6 +1008,7 @@ int gc_plan_set_option(gc_plan_t* p, int option, uint64_t value) {
                 finish_layout(p);                      // workspace size stays as planned (see skeys_tiles_alloc)
                 plan_single(p);
                 plan_multi(p);
+                plan_thr_single_fold(p);
                 plan_thr_fold(p);
             } catch (...) { return GC_E_INVALID; }     // out of host memory
             return upload_table(p);
@@ -1035,7 +1074,7 @@ static CleanArgs clean_args(const gc_plan_s* p, void* workspace, int route, uint
     c.ctrl = reinterpret_cast<uint4*>(workspace);
     c.ctrl_units = (uint32_t)(p->control_bytes / 16);
     auto range = [&](int q, size_t off, size_t bytes) { c.early[q][0] = (uint32_t)(off / 16); c.early[q][1] = (uint32_t)((off + bytes) / 16); };
-    if (route == GC_ROUTE_TOPK_ONE) {
+    if (p->T == 1) {
         range(0, p->off_hist5, sizeof(uint32_t) * kHistBins);                 // coarse sample histogram
         range(1, p->off_fine, sizeof(uint32_t) * (size_t)kFineBins);          // fine sample histogram
     } else {
@@ -1066,7 +1105,7 @@ static void note_clean(gc_plan_s* p, const void* workspace) {
 static int compress_route(const gc_plan_s* p) {
     if (p->device < 0 || p->total_n == 0) return GC_ROUTE_NONE;
     if (p->mode == GC_THRESHOLD) {
-        if (p->path == GC_PATH_AUTO && p->thr_grid > 0) return GC_ROUTE_THRESHOLD_ONE;
+        if (p->path == GC_PATH_AUTO && (p->thr_grid > 0 || p->thr_single.G > 0)) return GC_ROUTE_THRESHOLD_ONE;
         if (p->path == GC_PATH_AUTO && (p->thrm_grid > 0 || p->thrf.G > 0)) return GC_ROUTE_THRESHOLD_MANY;
         return GC_ROUTE_THRESHOLD_STAGED;
     }
@@ -1176,7 +1215,7 @@ static int compress_impl(gc_plan_t* p, const void* grad_any, bool bf16, float* r
     const int gh = (int)std::min<uint32_t>(nt, (uint32_t)p->grid_hist);
     const int gcp = (int)std::min<uint32_t>(nt, (uint32_t)p->grid_compact);
     char* wb = static_cast<char*>(workspace);
-    if (route == GC_ROUTE_THRESHOLD_ONE) {
+    if (route == GC_ROUTE_THRESHOLD_ONE && p->thr_single.G == 0) {
         // one large tensor: sample, exact threshold, fold + hits and emission in one cooperative launch
         ThrSingleArgs ta;
         ta.d = p->desc[0]; ta.desc = p->d_desc; ta.ntiles = nt; ta.maxt = p->thr_maxt; ta.pool_cap = p->thr_pool;
@@ -1277,16 +1316,17 @@ static int compress_impl(gc_plan_t* p, const void* grad_any, bool bf16, float* r
         GC_CUDA(p, cudaLaunchCooperativeKernel(kfn, dim3(dg.G), dim3(kBlock), args, dg.smem, s));
         return GC_OK;
     }
-    if (route == GC_ROUTE_TOPK_ONE) {
-        // one large tensor: candidates stay in shared memory
-        const SingleGeom& sg = p->single[bf16 ? 1 : 0];
+    if (route == GC_ROUTE_TOPK_ONE || route == GC_ROUTE_THRESHOLD_ONE) {
+        // one large tensor (threshold mode: fold first)
+        const bool thr = route == GC_ROUTE_THRESHOLD_ONE;
+        const SingleGeom& sg = thr ? p->thr_single : p->single[bf16 ? 1 : 0];
         SingleArgs sa;
-        sa.d = p->desc[0]; sa.desc = p->d_desc; sa.ntiles = nt; sa.maxt = sg.maxt; sa.rows = sg.rows;
+        sa.d = thr ? p->thr_d : p->desc[0]; sa.nstiles_def = p->nstiles; sa.desc = p->d_desc; sa.ntiles = nt; sa.maxt = sg.maxt; sa.rows = sg.rows;
         sa.pool_cap = std::min<uint32_t>(sg.pool, p->cand_cap);
         sa.cand = reinterpret_cast<uint2*>(wb + p->off_cidx);
         sa.g = grad_any; sa.r = residual; sa.out_idx = out_idx; sa.out_val = out_val; sa.out_count = out_count;
         sa.hist5 = reinterpret_cast<uint32_t*>(wb + p->off_hist5);
-        sa.srank_hi = p->single_srank_hi; sa.srank_mid = p->single_srank_mid; sa.mid_cap = (uint32_t)kSingleMidCap;
+        sa.srank_hi = thr ? p->thr_srank_hi : p->single_srank_hi; sa.srank_mid = thr ? p->thr_srank_mid : p->single_srank_mid; sa.mid_cap = (uint32_t)kSingleMidCap;
         sa.mid = reinterpret_cast<uint2*>(wb + p->off_mid);
         sa.fine = reinterpret_cast<uint32_t*>(wb + p->off_fine);
         sa.start = reinterpret_cast<uint2*>(wb + p->off_start);
@@ -1295,11 +1335,12 @@ static int compress_impl(gc_plan_t* p, const void* grad_any, bool bf16, float* r
         sa.tile_eq = sa.tile_cnt + nt; sa.seg_eq = sa.seg_tot + kSingleMaxT * 20;
         sa.ws = ws; sa.gws = gws;
         sa.cl = clean_args(p, workspace, GC_ROUTE_TOPK_ONE, clean_mode);
-        note_clean(p, workspace);
+        if (!thr) note_clean(p, workspace);
         void* args[] = {&sa};
         Timed tm(p, s, GC_K_FUSED);
         const bool dense = p->density >= kDenseFrom;
-        const void* kfn = bf16 ? (dense ? (const void*)k_topk_single<GradBF16, true, true> : (const void*)k_topk_single<GradBF16, false, true>)
+        const void* kfn = thr  ? (dense ? (const void*)k_topk_single<GradF32, true, true, true> : (const void*)k_topk_single<GradF32, false, true, true>)
+                        : bf16 ? (dense ? (const void*)k_topk_single<GradBF16, true, true> : (const void*)k_topk_single<GradBF16, false, true>)
                         : sg.votes ? (const void*)k_topk_single<GradF32, false, true>
                                    : (dense ? (const void*)k_topk_single<GradF32, true, false> : (const void*)k_topk_single<GradF32, false, false>);
         GC_CUDA(p, cudaLaunchCooperativeKernel(kfn, dim3(sg.G), dim3(kBlock), args, sg.smem, s));

@@ -23,7 +23,6 @@
 //     if a CTA's candidate region overflows, everything is redone.
 #pragma once
 #include "gc_single.cuh"
-#include "gc_threshold.cuh"
 
 namespace gc {
 
@@ -125,14 +124,6 @@ __device__ __forceinline__ bool grid_wait(WsHeader* hdr, uint32_t& passed, int* 
     return grid_wait(hdr, passed, s_ok, gridDim.x);
 }
 
-// Threshold mode: is the element at `idx` of a tensor that starts at `off` in the definition's sample?
-struct InSample {
-    uint32_t off, stride;
-    __device__ __forceinline__ bool operator()(uint32_t idx) const {
-        const uint32_t q = (idx - off) >> 2;
-        return (stride & (stride - 1u)) == 0u ? (q & (stride - 1u)) == 0u : q % stride == 0u;
-    }
-};
 // (gc_thr_multi.cuh)
 static __device__ void tiny_threshold_warp(const TensorDesc& d, uint32_t t, uint32_t T, const float* __restrict__ g, float* __restrict__ r,
                                            uint32_t* __restrict__ out_idx, float* __restrict__ out_val, uint32_t* __restrict__ out_count,

@@ -32,6 +32,7 @@
 // misses (or a list overflows) the exact multi-pass kernels redo the tensor.
 #pragma once
 #include "gc_fast.cuh"
+#include "gc_threshold.cuh"
 
 namespace gc {
 
@@ -111,6 +112,8 @@ struct SingleArgs {
     const TensorDesc* desc;          // device table (for the redo phases)
     uint32_t ntiles, maxt, pool_cap; // tiles, max tiles per CTA, pool slots per CTA
     RowMap rows;                     // which tile is row i of column c
+    uint32_t nstiles_def;            // threshold mode: sample tiles of the definition's sample (`d` holds the bracket's, and as
+                                     // k the rank in the definition's; `desc` the definition's)
     uint32_t srank_hi;               // sample rank of the upper bracket (at least 1)
     uint32_t srank_mid;              // sample rank that estimates the threshold itself
     uint32_t mid_cap;                // capacity of the short list
@@ -327,6 +330,14 @@ __device__ __forceinline__ void chunk_ranks(uint32_t cm, int lane, ChunkRanks& c
     }
 }
 
+// Threshold mode: is the element at `idx` of a tensor that starts at `off` in the definition's sample?
+struct InSample {
+    uint32_t off, stride;
+    __device__ __forceinline__ bool operator()(uint32_t idx) const {
+        const uint32_t q = (idx - off) >> 2;
+        return (stride & (stride - 1u)) == 0u ? (q & (stride - 1u)) == 0u : q % stride == 0u;
+    }
+};
 // The rest of the fold of one warp chunk in the form with votes: residual, list entries, band histogram.
 // `at0` = flat index of this thread's first element.  Returns false if the candidate region is full.
 // `counts`: whether the histogram counts the candidate of that index.
@@ -416,7 +427,9 @@ __device__ __forceinline__ bool fold_tail_votes(BlockSmem& sm, const float (&av)
 // DENSE (plans of 2 % and more) has the emission by chunk, the bfloat16 form the counted band: the other
 // forms do without their code.  Many tensors, without / with DENSE: 110M elements at 2 % 305 / 310 us, 5 %
 // 359 / 346; 25.6M at 5 % 134 / 131; one tensor: 110M at 2 % 268 / 267, 5 % 312 / 311, 8M at 2 % 49 / 51.
-template <typename GL, bool DENSE, bool VOTES>
+// THR: threshold mode, fold first (see the many-tensor kernel; the exact threshold is a rank among the sampled entries
+// of the short list; always with votes: with the shuffle scan the fold of 110M elements at 1 % takes 331 us, with votes 206).
+template <typename GL, bool DENSE, bool VOTES, bool THR = false>
 static __global__ void __launch_bounds__(kBlock, 3)
 k_topk_single(const __grid_constant__ SingleArgs a) {
     __shared__ BlockSmem sm;
@@ -598,8 +611,12 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
             }
         }
         if constexpr (VOTES) {
-            block_overflow |= !fold_tail_votes(sm, av, interior, valid, tau, tau_z, shift, tg.base + my_off, a.r, s_used, a.pool_cap, pool,
-                                               rec[i * kWarps + warp], lane, warp);
+            if constexpr (THR)
+                block_overflow |= !fold_tail_votes(sm, av, interior, valid, tau, tau_z, shift, tg.base + my_off, a.r, s_used, a.pool_cap, pool,
+                                                   rec[i * kWarps + warp], lane, warp, InSample{d.off, d.stride});
+            else
+                block_overflow |= !fold_tail_votes(sm, av, interior, valid, tau, tau_z, shift, tg.base + my_off, a.r, s_used, a.pool_cap, pool,
+                                                   rec[i * kWarps + warp], lane, warp);
         } else {
             uint32_t cnt[kVpt], cm = 0, hm = 0;      // candidates; candidates that are zeroed right away
 #pragma unroll
@@ -702,14 +719,15 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
     const uint32_t want_k[1] = {d.k};
     Picked pa[1];
     block_select_multi<2048, 1>(sm, a.hist5 + 2 * kHistBins, want_k, pa);
-    const uint32_t A = pa[0].bin, aboveA = pa[0].above, m = pa[0].count;      // m = candidates inside the band bin
+    const uint32_t A = pa[0].bin, aboveA = pa[0].above;
+    uint32_t m = pa[0].count;                  // candidates inside the band bin (THR: the sampled ones, until all are listed)
     // A band bin with thousands of candidates (bfloat16 gradients on a residual of zero, or of few values as
     // when one gradient is folded again and again, tie by the thousands) is counted: its keys are histogrammed one by one (at most 2048 of them), which gives the threshold
     // key after the barrier; then every CTA counts its candidates above and at that key per tile, and
     // after one more barrier the candidates at the key in the tiles before a tile say how many of its own
     // are sent.  110M elements, bfloat16, 60,000 ties: counts + threshold + slots 15 us, 41 us as a list.
     const bool counted = GL::kManyTies && overflowed == 0u && pa[0].ok && m > kMidCounted && A < 2047u && shift <= 11;
-    bool good = overflowed == 0u && pa[0].ok && (m <= a.mid_cap || counted);
+    bool good = overflowed == 0u && pa[0].ok && (THR || m <= a.mid_cap || counted);
     const uint32_t binlo = tau + (A << shift);
 
     const bool by_chunk = DENSE && used >= kChunkWalk * n_own * kWarps;
@@ -727,6 +745,7 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
                 if (counted) { atomicAdd(&sm.hist[(pr.y & kKeyMask) - binlo], 1u); return; }
                 const uint32_t slot = atomicAdd(a.hist5 + 3 * kHistBins, 1u);
                 if (slot < a.mid_cap) a.mid[slot] = pr;
+                else if (THR && slot == a.mid_cap) atomicAdd(&hdr->n_failed, 1u);
             }
         };
 #pragma unroll
@@ -780,6 +799,10 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
         }
         if (!grid_barrier(hdr, passed, &sm.ok)) return;
         phase_stamp(hdr, n_stamp);
+        if constexpr (THR) {
+            m = ld_cg(a.hist5 + 3 * kHistBins);
+            good = m <= a.mid_cap;
+        }
 
         // ------------------------------------------------------------ exact threshold from the short list
         // Every CTA ranks the same m entries: Tkey = the (k - aboveA)-th largest key among them.
@@ -788,7 +811,7 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
         uint2 e[kMidRegs];
 #pragma unroll
         for (uint32_t u = 0; u < kMidRegs; ++u)
-            e[u] = !counted && u * kBlock + tid < m ? ld_cg(a.mid + u * kBlock + tid) : make_uint2(0u, 0u);
+            e[u] = good && !counted && u * kBlock + tid < m ? ld_cg(a.mid + u * kBlock + tid) : make_uint2(0u, 0u);
         // while those loads fly: per row, the candidates above the bin in the whole row and in
         // the tiles of lower CTAs (whole 32-CTA segments below this CTA's + the lower CTAs of
         // its own segment): two loads per lane and row, eight rows per warp and step (two: 355M elements
@@ -820,12 +843,12 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
             }
         }
         uint32_t v_sel, mid_gt, n_eq = 0, cut_end = 0xFFFFFFFFu;      // candidates at Tkey are sent below index cut_end
-        if (!counted) {
+        if (!counted && good) {
         good = short_list_select(sm, e, a.mid, m, A == 2047u ? 31 : max(shift, 1), d.k - aboveA,
-                                 [&](const uint2& pr, uint32_t& v) { v = (pr.y & kKeyMask) - binlo; return true; },
+                                 [&](const uint2& pr, uint32_t& v) { v = (pr.y & kKeyMask) - binlo; return !THR || InSample{d.off, d.stride}(pr.x); },
                                  v_sel, mid_gt, n_eq);
         Tkey = binlo + v_sel;
-        m_eq = d.k - aboveA - mid_gt;      // entries equal to Tkey that are sent
+        m_eq = THR ? 0xFFFFFFFFu : d.k - aboveA - mid_gt;      // entries equal to Tkey that are sent
         }
         if (good && n_eq > m_eq && n_eq <= (uint32_t)kBlock) {
             // a few entries tie at the threshold: list their indices, rank them directly
@@ -881,6 +904,21 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
             for (uint32_t i = kMidFast + tid; !counted && i < m; i += kBlock) below(ld_cg(a.mid + i));
             if (tid == 0) { sm.scratch[0] = 0u; sm.scratch[1] = 0xFFFFFFFFu; }
             __syncthreads();
+            if (THR && col == 0u) {            // (this column has a tile in every row: the rows' totals are the tensor's)
+                uint32_t hits = 0;
+                for (uint32_t i = tid; i < n_own; i += kBlock) hits += row_sum[i];
+#pragma unroll
+                for (uint32_t u = 0; u < kMidRegs; ++u) hits += u * kBlock + tid < m && sent_key(e[u]) ? 1u : 0u;
+                for (uint32_t i = kMidFast + tid; i < m; i += kBlock) hits += sent_key(ld_cg(a.mid + i)) ? 1u : 0u;
+                hits = __reduce_add_sync(0xFFFFFFFFu, hits);
+                if (lane == 0 && hits) atomicAdd(&sm.scratch[0], hits);
+                __syncthreads();
+                if (tid == 0) {
+                    hits = sm.scratch[0];
+                    if (a.out_count != nullptr) { a.out_count[0] = min(hits, d.cap); a.out_count[1] = hits; }
+                    if (hits > d.cap) record_status(hdr, 1 /*GC_W_TRUNCATED*/, 0);
+                }
+            }
             if (warp == 0) {
                 // tile_base[i] = rows before i + lower CTAs of row i + sent short-list entries before the tile
                 // (counted band: + the candidates at the threshold key in the tiles before it, as far as sent)
@@ -963,8 +1001,10 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
                     for (uint32_t q0 = 0; q0 < cnt; q0 += 32u) {
                         const bool in = q0 + lane < cnt;
                         const uint2 pr = q0 == 0u ? p[0] : q0 == 32u ? p[1] : in ? pool[off + q0 + lane] : make_uint2(0u, 0u);
-                        const bool sent = in && sent_key(pr), zeroed = (pr.y & kKeyMask) >= tau_z;
+                        bool sent = in && sent_key(pr);
+                        const bool zeroed = (pr.y & kKeyMask) >= tau_z;
                         const unsigned sb = __ballot_sync(0xFFFFFFFFu, sent);
+                        if constexpr (THR) sent = sent && slot + (uint32_t)__popc(sb & ((1u << lane) - 1u)) < d.cap;      // (beyond the capacity: stays in the residual)
                         if (in && sent != zeroed) a.r[pr.x] = sent ? 0.0f : __uint_as_float(pr.y);
                         if (sent) emit(pr, slot + (uint32_t)__popc(sb & ((1u << lane) - 1u)));
                         slot += (uint32_t)__popc(sb);
@@ -1007,7 +1047,7 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
                         if (zeroed) a.r[pr[u].x] = __uint_as_float(pr[u].y);     // value goes back
                         continue;
                     }
-                    if (!zeroed) a.r[pr[u].x] = 0.0f;
+                    if (!THR && !zeroed) a.r[pr[u].x] = 0.0f;
                     const uint32_t rel = pr[u].x - base0;
                     const uint32_t c = rm.row_of(rel >> 12) * kWarps + ((rel >> 9) & (kWarps - 1u));
                     const uint32_t s = rec[c] >> 10;                   // first list position of the chunk
@@ -1018,10 +1058,15 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
                         before = __popc(sent_bits[s >> 5] >> (s & 31u)) + __popc(sent_bits[i >> 5] & ((1u << (i & 31u)) - 1u));
                         for (uint32_t w = (s >> 5) + 1u; w < (i >> 5); ++w) before += __popc(sent_bits[w]);
                     }
+                    if constexpr (THR) {
+                        const bool goes = rec2[c] + before < d.cap;          // (beyond the capacity: stays in the residual)
+                        if (goes != zeroed) a.r[pr[u].x] = goes ? 0.0f : __uint_as_float(pr[u].y);
+                        if (!goes) continue;
+                    }
                     emit(pr[u], rec2[c] + before);
                 }
             }
-            if (a.out_count != nullptr && b == 0 && tid == 0) { a.out_count[0] = d.k; a.out_count[1] = d.k; }
+            if (!THR && a.out_count != nullptr && b == 0 && tid == 0) { a.out_count[0] = d.k; a.out_count[1] = d.k; }
             __syncthreads();
             phase_stamp(hdr, n_stamp);
             exit_stamp(hdr);
@@ -1033,7 +1078,7 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
     // ---------------------------------------------------------------- safety net (rare)
     // The pool overflowed or the candidate set was smaller than k: give every pooled candidate
     // its value back, then run the exact multi-pass kernels on r (= a everywhere again).
-    if (b == 0 && tid == 0) { a.ws.sel[0].flags = kSelFailed; atomicAdd(&hdr->n_failed, 1u); }
+    if (!THR && b == 0 && tid == 0) { a.ws.sel[0].flags = kSelFailed; atomicAdd(&hdr->n_failed, 1u); }
     for (uint32_t c = tid; c < n_own * kWarps; c += kBlock) {      // only chunks that were stored
         const uint32_t rc = rec[c], off = rc >> 10, cnt = rc & 1023u;
         for (uint32_t j = 0; j < cnt; ++j) {
@@ -1044,6 +1089,18 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
     clean_redo(a.cl, G, b, tid);
     if (!grid_barrier(hdr, passed, &sm.ok)) return;
     phase_stamp(hdr, n_stamp);
+    if constexpr (THR) {
+        WsView ws = a.gws;                     // (its records, ungated)
+        ws.gate = nullptr;
+        hist_body<0, SRC_RSAMPLE>(sm, a.desc, 1u, a.nstiles_def, nullptr, a.r, ws, G, b);
+        if (!grid_barrier(hdr, passed, &sm.ok)) return;
+        hist_body<1, SRC_RSAMPLE>(sm, a.desc, 1u, a.nstiles_def, nullptr, a.r, ws, G, b);
+        if (!grid_barrier(hdr, passed, &sm.ok)) return;
+        hist_body<2, SRC_RSAMPLE>(sm, a.desc, 1u, a.nstiles_def, nullptr, a.r, ws, G, b);
+        if (!grid_barrier(hdr, passed, &sm.ok)) return;
+        threshold_emit_body<false>(a.desc, 1u, a.ntiles, nullptr, a.r, a.out_idx, a.out_val, a.out_count, a.ws, ws.sel, 0u, 0);
+        return;
+    }
     hist_body<0, SRC_RESID>(sm, a.desc, 1u, a.ntiles, nullptr, a.r, a.gws);
     if (!grid_barrier(hdr, passed, &sm.ok)) return;
     hist_body<1, SRC_RESID>(sm, a.desc, 1u, a.ntiles, nullptr, a.r, a.gws);
