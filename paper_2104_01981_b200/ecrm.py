@@ -43,13 +43,14 @@ def lib() -> ctypes.CDLL:
     return l
 
 
+# Marshalling bounds the calls on a few thousand rows (their kernels take 4-5 us), so addresses travel as plain
+# numbers and tables as arrays, which the declared argument types turn into pointers.
 def _ptr(t: Optional[torch.Tensor]):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else ctypes.c_void_p(0)
+    return t.data_ptr() if t is not None else None
 
 
 def _table(ts: Sequence[Optional[torch.Tensor]]):
-    arr = (ctypes.c_void_p * max(len(ts), 1))(*[(t.data_ptr() if t is not None else 0) for t in ts])
-    return ctypes.cast(arr, ctypes.POINTER(ctypes.c_void_p)), arr
+    return (ctypes.c_void_p * max(len(ts), 1))(*[(t.data_ptr() if t is not None else 0) for t in ts])
 
 
 def _stream(stream):
@@ -63,13 +64,11 @@ def _check(fn: str, rc: int) -> int:
 
 
 def encode(shards: Sequence[torch.Tensor], parity: torch.Tensor, stream=None) -> int:
-    tab, keep = _table(shards)
-    return _check("ecrm_encode", lib().ecrm_encode(len(shards), tab, _ptr(parity), parity.numel(), _stream(stream)))
+    return _check("ecrm_encode", lib().ecrm_encode(len(shards), _table(shards), _ptr(parity), parity.numel(), _stream(stream)))
 
 
 def decode(survivors: Sequence[torch.Tensor], parity: torch.Tensor, out: torch.Tensor, stream=None) -> int:
-    tab, keep = _table(survivors)
-    return _check("ecrm_decode", lib().ecrm_decode(len(survivors), tab, _ptr(parity), _ptr(out), out.numel(),
+    return _check("ecrm_decode", lib().ecrm_decode(len(survivors), _table(survivors), _ptr(parity), _ptr(out), out.numel(),
                                                    _stream(stream)))
 
 
@@ -104,9 +103,8 @@ def degraded_read(prow: torch.Tensor, srows: Optional[Sequence[Optional[torch.Te
                   shards: Sequence[torch.Tensor], parity: torch.Tensor, out: torch.Tensor,
                   bad_rows: Optional[torch.Tensor] = None, stream=None) -> int:
     n_rows, dim = parity.shape
-    stab, keep1 = _table(shards)
-    rtab, keep2 = _table(list(srows) if srows is not None else [None] * len(shards))
-    return _check("ecrm_degraded_read", lib().ecrm_degraded_read(len(shards), prow.numel(), _ptr(prow), rtab, stab,
+    rows = _table(srows) if srows is not None else None
+    return _check("ecrm_degraded_read", lib().ecrm_degraded_read(len(shards), prow.numel(), _ptr(prow), rows, _table(shards),
                                                                  _ptr(parity), n_rows, dim, _ptr(out),
                                                                  _ptr(bad_rows), _stream(stream)))
 
