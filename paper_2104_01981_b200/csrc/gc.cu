@@ -121,10 +121,12 @@ constexpr uint32_t kSinglePoolMax = 65536, kMultiPoolMax = 98304;   // most cand
 // best between 6 and 10 % on the 110M-element workload at 1 % density.  Sparser plans have fewer
 // candidates to handle in the fold loop and compete less for issue slots: below 0.5 % the smaller
 // one (4 % did better than 8 % at 0.1 %, where 8 % let the oldest CTAs of the 355M-element workload
-// finish last).  Forms with votes (up to kSparseUpTo, bfloat16) take equal shares.
+// finish last).  Forms with votes take equal shares.
 constexpr double kSingleSkew = 0.08, kSingleSkewSparse = 0.04;
 constexpr size_t kSingleRowBytes = (2 * kWarps + 4) * sizeof(uint32_t);   // shared memory per owned tile
 constexpr double kSparseUpTo = 0.002;        // density up to which most chunks are empty (see VOTES of k_topk_single)
+constexpr double kVotesFrom = 0.009;         // one-tensor fp32 plans between these densities and from so many tiles on rank by
+constexpr uint32_t kVotesBelow = 16000;      // the shuffle scan (see VOTES of k_topk_single)
 constexpr double kDenseFrom = 0.02;          // density from which the forms with emission by chunk are taken (12 candidates per chunk)
 constexpr double kThrOneFoldUpTo = 0.02;     // one tensor: the same, and the elements from which (see plan_thr_single_fold)
 constexpr uint32_t kThrOneFoldFrom = 12u << 20;
@@ -373,7 +375,7 @@ static RowMap make_row_map(const gc_plan_s* p, uint32_t ntiles, uint32_t G, uint
 SingleGeom single_geometry(const gc_plan_s* p, const TensorDesc& d, bool bf16) {
     SingleGeom g;
     const uint64_t groups = ((uint64_t)d.n + 3) / 4, nsg = (groups + d.sstride - 1) / d.sstride;
-    g.votes = bf16 || p->mode == GC_THRESHOLD || p->density <= kSparseUpTo;
+    g.votes = bf16 || p->mode == GC_THRESHOLD || p->density <= kSparseUpTo || p->density >= kVotesFrom || d.ntiles < kVotesBelow;
     g.G = std::min<uint32_t>((uint32_t)p->grid_single_max, d.ntiles);
     // Small tensors are all latency (a CTA has a handful of tiles and five phases to walk through):
     // there two CTAs per SM get through the phases sooner than three (2M-10M elements: 31-49 us
@@ -724,7 +726,7 @@ static bool ask_device(int device, DeviceFacts* p) {
             // sized for the largest chunk-record block the kernel may be given; the form that fits least counts
             const size_t smem_max = kSingleMaxT * kSingleRowBytes + kSinglePoolMax / 8;
             int nb = 1 << 20;
-            for (const void* fn : {(const void*)k_topk_single<GradF32, false, false>, (const void*)k_topk_single<GradF32, true, false>,
+            for (const void* fn : {(const void*)k_topk_single<GradF32, false, false>, (const void*)k_topk_single<GradF32, true, true>,
                                    (const void*)k_topk_single<GradF32, false, true>, (const void*)k_topk_single<GradBF16, false, true>,
                                    (const void*)k_topk_single<GradBF16, true, true>, (const void*)k_topk_single<GradF32, false, true, true>,
                                    (const void*)k_topk_single<GradF32, true, true, true>}) {
@@ -1341,8 +1343,8 @@ static int compress_impl(gc_plan_t* p, const void* grad_any, bool bf16, float* r
         const bool dense = p->density >= kDenseFrom;
         const void* kfn = thr  ? (dense ? (const void*)k_topk_single<GradF32, true, true, true> : (const void*)k_topk_single<GradF32, false, true, true>)
                         : bf16 ? (dense ? (const void*)k_topk_single<GradBF16, true, true> : (const void*)k_topk_single<GradBF16, false, true>)
-                        : sg.votes ? (const void*)k_topk_single<GradF32, false, true>
-                                   : (dense ? (const void*)k_topk_single<GradF32, true, false> : (const void*)k_topk_single<GradF32, false, false>);
+                        : sg.votes ? (dense ? (const void*)k_topk_single<GradF32, true, true> : (const void*)k_topk_single<GradF32, false, true>)
+                                   : (const void*)k_topk_single<GradF32, false, false>;
         GC_CUDA(p, cudaLaunchCooperativeKernel(kfn, dim3(sg.G), dim3(kBlock), args, sg.smem, s));
         return GC_OK;
     }

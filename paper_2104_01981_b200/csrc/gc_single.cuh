@@ -422,8 +422,10 @@ __device__ __forceinline__ bool fold_tail_votes(BlockSmem& sm, const float (&av)
 // most chunks are empty (fp32 up to 0.2 %, with two CTAs per SM, since a loop that hardly waits for itself
 // keeps the memory busier than it likes with three: 110M elements at 0.1 % 252 -> 231 us, 355M 710 -> 680 us;
 // bfloat16 at five sixths of the bytes wants the third: 0.2 % 227 -> 208 us and 655 -> 598 us).
-// Between, fp32 is bound by memory and the slower loop with unequal shares does better (0.5 %: 245 against
-// 249-254 us; 355M at 0.3 %: 697 against 714).
+// From 0.9 % on, and at any density below 65M elements, the votes win as well (scan / votes, us: 5M at 1 % 40.5 / 39.1, 14M
+// 61.6 / 59.5, 40M at 0.3 % 109.7 / 108.7, 2 % 119 / 115, 110M at 1 % 251.5 / 250, 2 % 262 / 257, 5 % 300 / 285).  Large plans between 0.2 and
+// 0.9 % are bound by memory, and the slower loop with unequal shares does better (110M at 0.3 % 245 / 253, 0.5 % 246 / 252-254;
+// 355M at 0.3 % 705 / 716).  Several workers in one launch keep the scan (see k_topk_workers).
 // DENSE (plans of 2 % and more) has the emission by chunk, the bfloat16 form the counted band: the other
 // forms do without their code.  Many tensors, without / with DENSE: 110M elements at 2 % 305 / 310 us, 5 %
 // 359 / 346; 25.6M at 5 % 134 / 131; one tensor: 110M at 2 % 268 / 267, 5 % 312 / 311, 8M at 2 % 49 / 51.
