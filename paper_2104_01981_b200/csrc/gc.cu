@@ -225,19 +225,31 @@ void sample_params(TensorDesc& d, double density, uint32_t rank_permille, uint64
     *ccap = cap >= (double)n ? n : (uint64_t)cap;
 }
 
-// Threshold plans of several tensors, fold first: the sample that sets a tensor's bracket (kept keys, so at most 32,000
-// elements), one group of four in `stride`, and the rank of its lower end, six standard deviations of both samples' noise
-// above the expected one.
-struct ThrBracket { uint64_t stride, groups; double rank; };
-ThrBracket thr_bracket(const TensorDesc& d, uint32_t rank_permille) {
-    ThrBracket b;
-    const uint64_t groups = ((uint64_t)d.n + 3) / 4, target = std::min<uint64_t>(32000, std::max<uint64_t>(d.n / 128, std::min<uint64_t>(8192, d.n / 2)));
-    b.stride = std::max<uint64_t>(1, d.n / target);
-    b.groups = (groups + b.stride - 1) / b.stride;
-    const double m = 4.0 * (double)b.groups, among = 4.0 * (double)((groups + d.stride - 1) / d.stride), ks = (double)d.srank * m / among;
-    b.rank = std::max(1.0, std::ceil(ks + 6.0 * std::sqrt(ks + ks * ks / (double)d.srank) + 8.0) * (double)rank_permille / 1000.0);
-    if (b.rank >= 0.9 * m) b.rank = 0.0;                   // (nearly everything would be a candidate: not this way)
+// Threshold plans taken fold first: the sample that sets the bracket of tensor d -- about `target` groups of the definition's
+// (see BracketSample), at most `most` -- and the ranks of its ends in that sample, six standard deviations of drawing a
+// part without putting back around the expected one.  Among the sample's keys at most k_s - 1 lie above the k_s-th
+// largest of the whole, so the lower end is never below rank k_s; where the whole is read the ends are exact.
+struct ThrBracket { uint32_t step, groups, hi, mid; double rank; };
+ThrBracket thr_bracket(const TensorDesc& d, uint32_t rank_permille, uint64_t target, uint64_t most) {
+    const uint64_t unit = BracketSample(d.n, d.stride, 1).unit, units = BracketSample(d.n, d.stride, 1).units();
+    ThrBracket b{};
+    b.step = (uint32_t)std::max<uint64_t>({1, units * unit / target, (units * unit + most - 1) / most});
+    const BracketSample s(d.n, d.stride, b.step);
+    b.groups = s.count();
+    const double part = std::min(1.0, (double)b.groups / (double)s.of), ks = (double)d.srank * part, sd = std::sqrt(ks * (1.0 - part));
+    b.rank = std::max(1.0, std::min<double>(d.srank, std::ceil(ks + 6.0 * sd + 8.0)) * (double)rank_permille / 1000.0);
+    b.hi = (uint32_t)std::max(1.0, std::floor(ks - 6.0 * sd - 8.0));      // (a sample too small for that margin: its largest key bounds the band)
+    b.mid = (uint32_t)std::max(1.0, std::ceil(ks));
+    if (b.rank >= 0.9 * 4.0 * (double)b.groups) b.rank = 0.0;             // (nearly everything would be a candidate: not this way)
     return b;
+}
+// Of several tensors each: a quarter of what the default stride gives, at least 1024 groups; where everything is sampled,
+// lines, which cost an eighth of the accesses; as many as have their keys kept.  (Fewer scattered reads or fewer candidates:
+// at least 1024 / 512 groups, us: 110M elements in 199 tensors at 0.5 % 269 / 273, 1 % 274 / 281, eight 161-tensor workers at 0.1 %
+// 458 / 455, 0.5 % 483 / 484; an eighth and 256 groups: 282, 293, 464, 502.)
+ThrBracket thr_bracket(const TensorDesc& d, uint32_t rank_permille) {
+    const uint64_t target = d.stride == 1u ? std::max<uint64_t>(d.n / 512, 2048) : std::max<uint64_t>(d.n / 1024, 1024);
+    return thr_bracket(d, rank_permille, target, kRefineTiles * kSampleTile);
 }
 
 // Fills the derived fields of the tensor table and the workspace layout.
@@ -371,10 +383,9 @@ static RowMap make_row_map(const gc_plan_s* p, uint32_t ntiles, uint32_t G, uint
     return rm;
 }
 
-// Geometry of k_topk_single for tensor d with the bracket's sample in it (G = 0: no).
-SingleGeom single_geometry(const gc_plan_s* p, const TensorDesc& d, bool bf16) {
+// Geometry of k_topk_single for tensor d with the bracket's sample, of nsg groups, in it (G = 0: no).
+SingleGeom single_geometry(const gc_plan_s* p, const TensorDesc& d, uint64_t nsg, bool bf16) {
     SingleGeom g;
-    const uint64_t groups = ((uint64_t)d.n + 3) / 4, nsg = (groups + d.sstride - 1) / d.sstride;
     g.votes = bf16 || p->mode == GC_THRESHOLD || p->density <= kSparseUpTo || p->density >= kVotesFrom || d.ntiles < kVotesBelow;
     g.G = std::min<uint32_t>((uint32_t)p->grid_single_max, d.ntiles);
     // Small tensors are all latency (a CTA has a handful of tiles and five phases to walk through):
@@ -407,7 +418,7 @@ void plan_single(gc_plan_s* p) {
     if (d.ntiles >= (1u << 20)) return;                              // (the row arithmetic divides by multiplication)
     const uint64_t groups = ((uint64_t)d.n + 3) / 4, nsg = (groups + d.sstride - 1) / d.sstride;
     for (int bf16 = 0; bf16 < 2; ++bf16) {
-        const SingleGeom g = single_geometry(p, d, bf16 != 0);
+        const SingleGeom g = single_geometry(p, d, nsg, bf16 != 0);
         if (g.G == 0) return;
         p->single[bf16] = g;
     }
@@ -420,26 +431,24 @@ void plan_single(gc_plan_s* p) {
 }
 
 // The same for a threshold plan that is taken fold first.
-// Sample-first / fold-first, us: 14M elements at 0.1 % 55.3 / 53.7, 1 % 57.0 / 55.7, 2 % 59.2 / 57.7, 5 % 60.0 / 62.8; 40M 109 / 103,
-// 110.3 / 108.0, 113.7 / 113.8, 122 / 125; 110M 255 / 229, 264 / 244, 273 / 254, 291 / 285; 355M at 0.1 % 768 / 679, 1 % 819 / 715.  At 5M the
-// two are equal up to 1 % (39.0 / 38.7) and the sample first is ahead above (2 % 39.5 / 40.8).
+// Sample-first / fold-first, us: 14M elements at 0.1 % 55.2 / 52.9, 1 % 58.3 / 56.7, 2 % 59.0 / 58.1, 5 % 60.0 / 62.8; 40M 110 / 104,
+// 114.8 / 109.7, 116.0 / 115.0, 122 / 125; 110M 256 / 232, 262 / 246, 269 / 258, 291 / 285; 355M at 0.1 % 774 / 695, 1 % 774 / 723.  At 5M the
+// two are equal up to 1 % (39.0 / 38.7) and the sample first is ahead above (2 % 39.5 / 40.8).  With a log-normal scale of spread 0.1
+// or 0.4 per column of 768, 15M at 1 % 61.0 and 60.6 / 57.4 and 57.4, 110M 263 and 262 / 246 and 246 (with the bracket from
+// lines anywhere, which is redone at times, 245 and 451).
 void plan_thr_single_fold(gc_plan_s* p) {
     p->thr_single = SingleGeom{};
     if (p->mode != GC_THRESHOLD || p->T != 1 || p->grid_single_max <= 0) return;
     TensorDesc d = p->desc[0];
     if (d.srank == 0 || d.ntiles == 0 || d.off != 0 || d.ntiles >= (1u << 20)) return;
     if (p->thr_grid > 0 && (p->density > kThrOneFoldUpTo || d.n < kThrOneFoldFrom)) return;
-    const uint64_t groups = ((uint64_t)d.n + 3) / 4, stride = std::max<uint64_t>(1, d.n / std::min<uint64_t>(kSampleMaxSingle, std::max<uint64_t>(d.n / 128, 8192)));
-    const double m = 4.0 * (double)((groups + stride - 1) / stride), among = 4.0 * (double)((groups + d.stride - 1) / d.stride);
-    const double ks = (double)d.srank * m / among, sd = std::sqrt(ks + ks * ks / (double)d.srank);
-    const double rank = std::max(1.0, std::ceil(ks + 6.0 * sd + 8.0) * (double)p->rank_permille / 1000.0), hi = std::floor(ks - 6.0 * sd - 8.0);
-    if (rank >= 0.9 * m) return;
+    const ThrBracket br = thr_bracket(d, p->rank_permille, std::max<uint64_t>(d.n / 1024, 2048), kSampleMaxSingle / 4);
+    if (br.rank <= 0.0) return;
     d.k = d.srank;
-    d.sstride = (uint32_t)stride; d.srank = (uint32_t)rank;
+    d.sstride = br.step; d.srank = (uint32_t)br.rank;
     p->thr_d = d;
-    p->thr_srank_hi = hi >= 1.0 ? (uint32_t)hi : 1u;
-    p->thr_srank_mid = (uint32_t)std::max(1.0, std::ceil(ks));
-    p->thr_single = single_geometry(p, d, false);
+    p->thr_srank_hi = br.hi; p->thr_srank_mid = br.mid;
+    p->thr_single = single_geometry(p, d, br.groups, false);
 }
 
 // Decides whether a threshold plan can use the one-tensor kernel and with which geometry.
@@ -535,7 +544,8 @@ MultiGeom multi_geometry(const gc_plan_s* p, const std::vector<TensorDesc>& desc
         const TensorDesc& d = desc[t];
         if (d.kind == kKindSmall || d.ntiles == 0) continue;
         if (d.sstride == 0) { per_tile[t] = (double)kTile; continue; }
-        const uint64_t groups = ((uint64_t)d.n + 3) / 4, nsg = (groups + d.sstride - 1) / d.sstride;
+        const uint64_t groups = ((uint64_t)d.n + 3) / 4;
+        const uint64_t nsg = p->mode == GC_THRESHOLD ? BracketSample(d.n, d.stride, d.sstride).count() : (groups + d.sstride - 1) / d.sstride;
         const double edge = d.nstiles <= kRefineTiles ? 1.02 : 2.0;      // tau is exact to 21 bits, or a bin edge
         per_tile[t] = std::min<double>(kTile, edge * (double)kTile * (double)d.srank / (4.0 * (double)nsg));
     }
@@ -567,10 +577,12 @@ void plan_multi(gc_plan_s* p) {
 // Decides whether a threshold plan of several tensors is taken fold first (k_topk_multi with THR), and makes the table
 // with the bracket's samples.
 // Fold first costs a lighter sample, but more candidates than hits and one more pass over them, so it pays for sparse
-// plans (sample-first / fold-first, us): 161 tensors of 25.6M elements at 0.1 % 101 / 97, 0.5 % 103.3 / 102.3, 1 % 104.6 / 106,
-// 5 % 113 / 117; eight such workers 498 / 461, 500 / 485, 505 / 506, 560 / 636; a dozen of 30M 120 / 108, 116 / 110.5, 118 / 112, 127 / 128
-// (eight workers 571 / 531, 567 / 554, 575 / 578, 635 / 736); of 3M at 0.1 % 39.5 / 39.0, eight workers 92.1 / 93.3.  Plans with samples of more than
-// 128 sample tiles, which no fused kernel took, always go this way: 110M in 199 tensors at 1 % 882 -> 271, at 5 % 330.
+// plans (sample-first / fold-first, us): 161 tensors of 25.6M elements at 0.1 % 102 / 96, 0.5 % 104.5 / 99.9, 1 % 104.6 / 106,
+// 5 % 113 / 117; eight such workers 504 / 460, 503 / 483, 505 / 506, 560 / 636; a dozen of 30M 119 / 109, 119 / 109, 118 / 112, 127 / 128
+// (eight workers 574 / 528, 568 / 557, 575 / 578, 635 / 736); of 3M at 0.1 % 39.5 / 39.0, eight workers 92.1 / 93.3.  Plans with samples of more than
+// 128 sample tiles, which no fused kernel took, always go this way: 110M in 199 tensors at 1 % 871 -> 274, at 5 % 329.  With a
+// log-normal scale of spread 0.4 per column or channel, the eight workers 508 / 462 at 0.1 % and 504 / 487 at 0.5 %, the 199 tensors 872 -> 269 at
+// 0.5 % (with the bracket from lines anywhere 1665, 1465 and 333).
 void plan_thr_fold(gc_plan_s* p) {
     p->thrf = MultiGeom{};
     p->tdesc.clear();
@@ -583,9 +595,9 @@ void plan_thr_fold(gc_plan_s* p) {
         d.stile0 = (uint32_t)stile0; d.nstiles = 0;
         if (d.kind == kKindSmall || d.n == 0) continue;
         const ThrBracket b = thr_bracket(d, p->rank_permille);
-        d.nstiles = (uint32_t)((b.groups + (uint64_t)kSampleTile - 1) / (uint64_t)kSampleTile);
+        d.nstiles = (b.groups + (uint32_t)kSampleTile - 1u) / (uint32_t)kSampleTile;
         if (b.rank <= 0.0 || d.nstiles > kRefineTiles) return;
-        d.sstride = (uint32_t)b.stride; d.srank = (uint32_t)b.rank;
+        d.sstride = b.step; d.srank = (uint32_t)b.rank;
         stile0 += d.nstiles;
     }
     p->tnstiles = (uint32_t)stile0;

@@ -265,6 +265,25 @@ __device__ __forceinline__ uint64_t sample_group(uint64_t sg, uint32_t sstride) 
     return (sg >> 3) * (8ull * sstride) + (sg & 7ull);
 }
 
+// Which groups set the bracket of a threshold plan that is taken fold first: groups of the definition's own sample (one
+// in `stride` of the tensor's), one unit out of `step`, each at a place of its own inside its run of `step` units.
+// Entries at other places say nothing about that sample where magnitudes vary along rows: one group in 64 always meets
+// the same columns of a tensor whose rows are a multiple of 256 long or a few such steps (15M and 60M elements, a log-normal scale per
+// column of 768: a bracket from lines anywhere missed 0 of 8 times at equal scales, 3 of 8 at a spread of 0.1, 5 of 8 at 0.4).
+// The place inside the run follows no period of the rows either (the golden ratio's multiples).  A unit is one
+// group, or a 128-byte line of eight where the definition samples everything.
+struct BracketSample {
+    uint32_t of, unit, step;         // groups of the definition's sample, groups per unit
+    __host__ __device__ BracketSample(uint32_t n, uint32_t stride, uint32_t step_)
+        : of(((n >> 2) + ((n & 3u) != 0u) + stride - 1u) / stride), unit(stride == 1u ? 8u : 1u), step(step_) {}
+    __host__ __device__ uint32_t units() const { return (of + unit - 1u) / unit; }
+    __host__ __device__ uint32_t count() const { return (units() + step - 1u) / step * unit; }      // groups, the last ones perhaps beyond the end
+    __device__ __forceinline__ uint64_t group(uint32_t i, uint32_t stride) const {                   // (one beyond the end is beyond the tensor)
+        const uint32_t u = unit == 1u ? i : i >> 3, in = unit == 1u ? 0u : i & 7u;
+        return (((uint64_t)u * step + __umulhi(u * 0x9E3779B1u, step)) * unit + in) * stride;
+    }
+};
+
 // One count per lane into a shared-memory histogram, aggregated over the warp first: lanes that
 // hit the same bin elect one of them to add their number (keys of one tensor crowd into a
 // handful of coarse bins, and 32 atomics on one shared-memory word are served one after the

@@ -324,7 +324,8 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
             constexpr uint32_t kSampleBatch = 4;
             const uint32_t nb = min(kSampleBatch, min(slast, d.stile0 + d.nstiles) - st);
             const uint32_t ngroups = (d.n + 3u) >> 2;
-            const uint32_t nsg = (ngroups + d.sstride - 1) / d.sstride;
+            const BracketSample def(d.n, d.stride, d.sstride);             // (threshold mode)
+            const uint32_t nsg = THR ? def.count() : (ngroups + d.sstride - 1) / d.sstride;
             const bool vec_ok = (d.off & 3u) == 0u;           // the tensor's groups are 16-byte aligned in the flat buffers
             float gv[kSampleBatch][4], rv[kSampleBatch][4];
             uint32_t i0[kSampleBatch];
@@ -332,7 +333,7 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
 #pragma unroll
             for (uint32_t u = 0; u < kSampleBatch; ++u) {
                 const uint64_t sg = (uint64_t)(st + u - d.stile0) * kBlock + tid;
-                const uint64_t gi = sample_group(sg, d.sstride);
+                const uint64_t gi = THR ? def.group((uint32_t)sg, d.stride) : sample_group(sg, d.sstride);
                 live[u] = u < nb && sg < nsg && gi < ngroups;
                 i0[u] = live[u] ? (uint32_t)gi * 4u : 0u;
                 if (vec_ok && live[u] && i0[u] + 3u < d.n) {
@@ -391,11 +392,15 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
             uint32_t tau_hi = 0x80000000u;
             if (d.sstride != 0u) {
                 const uint32_t ngroups = (d.n + 3u) >> 2;
-                const float msamp = 4.0f * (float)((ngroups + d.sstride - 1) / d.sstride);
-                // (threshold mode: k is a rank among the elements of another sample, whose noise comes on top)
-                const float among = THR ? 4.0f * (float)((ngroups + d.stride - 1) / d.stride) : (float)d.n;
-                const float ks = (float)d.k * msamp / among;
-                const float hi = floorf(ks - 6.0f * sqrtf(THR ? ks + ks * ks / (float)d.k : ks) - 8.0f);
+                float ks, sd;                              // expected rank of the threshold in the sample, its noise
+                if constexpr (THR) {                       // (k is a rank in the definition's sample, this one a part of it: see thr_bracket)
+                    const BracketSample def(d.n, d.stride, d.sstride);
+                    const float part = fminf(1.0f, (float)def.count() / (float)def.of);
+                    ks = (float)d.k * part; sd = sqrtf(ks * (1.0f - part));
+                } else {
+                    ks = (float)d.k * (4.0f * (float)((ngroups + d.sstride - 1) / d.sstride)) / (float)d.n; sd = sqrtf(ks);
+                }
+                const float hi = floorf(ks - 6.0f * sd - 8.0f);
                 // (a sample too small for that margin: the largest sampled key bounds the band instead)
                 const uint32_t want[3] = {d.srank, hi >= 1.0f ? (uint32_t)hi : 1u, max(1u, (uint32_t)ceilf(ks))};
                 Picked pk[3];

@@ -471,7 +471,7 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
     phase_stamp(hdr, n_stamp);
 
     // ---------------------------------------------------------------- sample
-    // One 4-element group out of d.sstride.  Two histograms of the sampled keys are built in one
+    // One 4-element group out of d.sstride (threshold mode: see BracketSample).  Two histograms of the sampled keys are built in one
     // pass: a coarse one (top 11 bits, via shared memory) and a fine one (top 16 bits, straight
     // into global memory; few samples share a fine bin).  tau = the srank-th largest sampled
     // key cut to 16 bits; tau_hi = upper edge of the 16-bit cell of the srank_hi-th largest.
@@ -479,23 +479,31 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
     uint32_t col = b, n_own = 0, myseg = 0;      // set after the first barrier
     {
         const uint32_t ngroups = (d.n + 3u) >> 2;
-        const uint32_t nsg = (ngroups + d.sstride - 1) / d.sstride;
+        const BracketSample def(d.n, d.stride, d.sstride);                // (threshold mode)
+        const uint32_t nsg = THR ? def.count() : (ngroups + d.sstride - 1) / d.sstride;
         constexpr int kMaxOwn = 2;                       // sample groups a thread may own
         uint32_t skey[kMaxOwn][4], sok = 0;
 #pragma unroll
         for (int q = 0; q < kMaxOwn; ++q) {
             const uint64_t sg = (uint64_t)q * G * kBlock + (uint64_t)b * kBlock + tid;
-            const uint64_t gi = sample_group(sg, d.sstride);
+            const uint64_t gi = THR ? def.group((uint32_t)sg, d.stride) : sample_group(sg, d.sstride);
             const bool in = sg < nsg && gi < ngroups;
             const uint32_t i0 = in ? (uint32_t)gi * 4u : 0u;
             float gv[4], rv[4];
+            if (THR && in && i0 + 3u < d.n) {            // (scattered: a whole group per access; the tensor starts at 0)
+                const float4 g4 = GL::ld4(a.g, i0), r4 = ld_cg(reinterpret_cast<const float4*>(a.r + i0));
+                gv[0] = g4.x; gv[1] = g4.y; gv[2] = g4.z; gv[3] = g4.w;
+                rv[0] = r4.x; rv[1] = r4.y; rv[2] = r4.z; rv[3] = r4.w;
+                sok |= 0xFu << (4 * q);
+            } else {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const bool v = in && i0 + e < d.n;
-                const uint32_t f = d.off + (v ? i0 + e : 0u);
-                gv[e] = v ? GL::ld1(a.g, f) : 0.f;
-                rv[e] = v ? ld_cg(a.r + f) : 0.f;
-                sok |= (uint32_t)v << (4 * q + e);
+                for (int e = 0; e < 4; ++e) {
+                    const bool v = in && i0 + e < d.n;
+                    const uint32_t f = d.off + (v ? i0 + e : 0u);
+                    gv[e] = v ? GL::ld1(a.g, f) : 0.f;
+                    rv[e] = v ? ld_cg(a.r + f) : 0.f;
+                    sok |= (uint32_t)v << (4 * q + e);
+                }
             }
 #pragma unroll
             for (int e = 0; e < 4; ++e) skey[q][e] = key_of(__fadd_rn(gv[e], rv[e]));
@@ -747,7 +755,6 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
                 if (counted) { atomicAdd(&sm.hist[(pr.y & kKeyMask) - binlo], 1u); return; }
                 const uint32_t slot = atomicAdd(a.hist5 + 3 * kHistBins, 1u);
                 if (slot < a.mid_cap) a.mid[slot] = pr;
-                else if (THR && slot == a.mid_cap) atomicAdd(&hdr->n_failed, 1u);
             }
         };
 #pragma unroll
@@ -1080,7 +1087,7 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
     // ---------------------------------------------------------------- safety net (rare)
     // The pool overflowed or the candidate set was smaller than k: give every pooled candidate
     // its value back, then run the exact multi-pass kernels on r (= a everywhere again).
-    if (!THR && b == 0 && tid == 0) { a.ws.sel[0].flags = kSelFailed; atomicAdd(&hdr->n_failed, 1u); }
+    if (b == 0 && tid == 0) { a.ws.sel[0].flags = kSelFailed; atomicAdd(&hdr->n_failed, 1u); }
     for (uint32_t c = tid; c < n_own * kWarps; c += kBlock) {      // only chunks that were stored
         const uint32_t rc = rec[c], off = rc >> 10, cnt = rc & 1023u;
         for (uint32_t j = 0; j < cnt; ++j) {
