@@ -146,12 +146,13 @@ __device__ __forceinline__ void thr_slots(const MultiArgs& a, uint32_t* seg, uin
     for (uint32_t q = tid; q < nseg; q += kBlock) {
         uint32_t* s = seg + (size_t)q * kSegWords;
         s[SG_M] = ld_cg(a.mid_n + s[SG_T]);
+        if (s[SG_M] > kMultiMidCap) s[SG_OK] = 0u;               // (flagged by the thread that came too late for the list)
     }
     __syncthreads();
     for (uint32_t sidx = (uint32_t)warp; sidx < nseg; sidx += kWarps) {
         uint32_t* s = seg + (size_t)sidx * kSegWords;
         const uint32_t m = s[SG_M];
-        if (m > kThrWarpMid) continue;
+        if (s[SG_OK] == 0u || m > kThrWarpMid) continue;
         const uint32_t t = s[SG_T];
         const TensorDesc d = a.desc[t];
         const InSample in{d.off, d.stride};
@@ -201,7 +202,7 @@ __device__ __forceinline__ void thr_slots(const MultiArgs& a, uint32_t* seg, uin
     for (uint32_t sidx = 0; sidx < nseg; ++sidx) {           // long lists: the whole CTA, one segment after the other
         uint32_t* s = seg + (size_t)sidx * kSegWords;
         const uint32_t m = s[SG_M];
-        if (m <= kThrWarpMid) continue;
+        if (s[SG_OK] == 0u || m <= kThrWarpMid) continue;
         const uint32_t t = s[SG_T];
         const TensorDesc d = a.desc[t];
         const InSample in{d.off, d.stride};
@@ -262,8 +263,9 @@ __device__ __forceinline__ void thr_slots(const MultiArgs& a, uint32_t* seg, uin
 // Here they are picked out of the stream instead: the bracket comes from a sample of 128-byte lines as in top-k mode, the
 // band histogram counts the candidates that are in the definition's sample, the band bin of rank k_s and the short list
 // (all candidates in it) give the exact threshold, and every candidate at or above it is a hit, up to the capacity.
-// What fails (bracket missed, list or region full) is redone from the residual by radix levels over the
-// definition's sample and the look-back emission.  Eight 161-tensor workers: sample and thresholds 95 -> 26 us, call
+// A tensor that fails (bracket missed, list full) is redone from the residual by radix levels over the
+// definition's sample and the look-back emission, all are if a region is full (199 tensors of 110M elements rounded to
+// bfloat16, a list of ties too long in the largest: 1036 us with all of them redone, 658 with that one).  Eight 161-tensor workers: sample and thresholds 95 -> 26 us, call
 // with the decode 532 -> 494.
 template <typename GL, bool DENSE, bool VOTES, bool THR = false>
 __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32_t G, const uint32_t b, BlockSmem& sm,
@@ -697,7 +699,10 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
             } else {
                 const uint32_t slot = atomicAdd(a.mid_n + c_t, 1u);
                 if (slot < kMultiMidCap) a.mid[(size_t)c_t * kMultiMidCap + slot] = pr;
-                else if (THR && slot == kMultiMidCap) atomicAdd(&hdr->n_failed, 1u);
+                else if (THR && slot == kMultiMidCap) {      // (one thread per tensor gets here)
+                    atomicOr(&a.ws.sel[c_t].flags, kSelFailed);
+                    atomicAdd(&hdr->n_failed, 1u);
+                }
             }
         };
         for (uint32_t i0 = tid; i0 < used; i0 += 4 * kBlock) {      // four loads in flight per thread
@@ -722,7 +727,7 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
     if (!grid_barrier(hdr, passed, &sm.ok, G)) return;
     phase_stamp(hdr, n_stamp, b);
 
-    if (THR ? !overflowed && ld_cg(&hdr->n_failed) == 0u : !overflowed) {
+    if (!overflowed) {
         if (nseg != 0u) {
             if constexpr (THR) {
                 thr_slots(a, seg, nseg, rec2, first, sm, s_cnt, hdr, chunk_of);
@@ -1028,7 +1033,6 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
         __syncthreads();
         phase_stamp(hdr, n_stamp, b);
         exit_stamp(hdr);
-        if (THR) return;
         if (ld_cg(&hdr->n_failed) == 0u) { leave_clean(a.cl, hdr, G, tid); return; }
     } else {
         // a candidate region overflowed: every recorded candidate gets its value back
@@ -1048,15 +1052,15 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
     phase_stamp(hdr, n_stamp, b);
     if constexpr (THR) {
         const TensorDesc* const def = a.desc - a.T;
-        WsView ws = a.gws;                               // (its records, ungated)
-        ws.gate = nullptr;
-        hist_body<0, SRC_RSAMPLE>(sm, def, a.T, a.nstiles_def, nullptr, a.r, ws, G, b);
+        hist_body<0, SRC_RSAMPLE>(sm, def, a.T, a.nstiles_def, nullptr, a.r, a.gws, G, b);
         if (!grid_barrier(hdr, passed, &sm.ok, G)) return;
-        hist_body<1, SRC_RSAMPLE>(sm, def, a.T, a.nstiles_def, nullptr, a.r, ws, G, b);
+        hist_body<1, SRC_RSAMPLE>(sm, def, a.T, a.nstiles_def, nullptr, a.r, a.gws, G, b);
         if (!grid_barrier(hdr, passed, &sm.ok, G)) return;
-        hist_body<2, SRC_RSAMPLE>(sm, def, a.T, a.nstiles_def, nullptr, a.r, ws, G, b);
+        hist_body<2, SRC_RSAMPLE>(sm, def, a.T, a.nstiles_def, nullptr, a.r, a.gws, G, b);
         if (!grid_barrier(hdr, passed, &sm.ok, G)) return;
-        threshold_emit_body<false, true>(def, a.T, a.ntiles, nullptr, a.r, a.out_idx, a.out_val, a.out_count, a.ws, ws.sel, 0u, 0);
+        WsView ws = a.ws;
+        ws.gate = a.ws.sel;
+        threshold_emit_body<false, true>(def, a.T, a.ntiles, nullptr, a.r, a.out_idx, a.out_val, a.out_count, ws, a.gws.sel, 0u, 0);
         return;
     }
     hist_body<0, SRC_RESID>(sm, a.desc, a.T, a.ntiles, nullptr, a.r, a.gws, G, b);

@@ -10,7 +10,8 @@ namespace gc {
 // look-back exchange, so output slots are index-ordered and a truncated tensor keeps exactly
 // its first `cap` hits.  tau of tensor t = ssel[t].T, or `tau_fixed` when ssel is null.
 // FOLD: a = g + r is computed here (and stored); otherwise r already holds a.
-// SKIP_SMALL: tensors of kind "small" were finished elsewhere and are left alone.
+// SKIP_SMALL: tensors of kind "small" were finished elsewhere and are left alone, as are all that the view's gate (if
+// there is one) is closed for.
 template <bool FOLD, bool SKIP_SMALL = false>
 static __device__ void threshold_emit_body(const TensorDesc* __restrict__ desc, uint32_t T, uint32_t ntiles,
                                            const float* __restrict__ g, float* __restrict__ r,
@@ -36,7 +37,7 @@ static __device__ void threshold_emit_body(const TensorDesc* __restrict__ desc, 
         if (tile >= ntiles) break;
         const uint32_t t = find_tensor(desc, T, tile);
         const TensorDesc d = desc[t];
-        if (SKIP_SMALL && d.kind == kKindSmall) continue;
+        if ((SKIP_SMALL && d.kind == kKindSmall) || !gate_open(ws, t, d)) continue;
         const uint32_t tau = ssel != nullptr ? ssel[t].T : tau_fixed;
         const TileGeom tg = tile_geom(d, tile - d.tile0);
         Tile tl;

@@ -68,3 +68,14 @@ def test_tensors_with_long_samples():
 def test_workers(W, density):
     sizes = [9_300_000, 3, 70_001, 4097, 3_400_000, 513]
     thr.check_threshold_workers(sizes, density, W, lambda w, s: randn(sum(sizes), 100 * s + w))
+
+
+@pytest.mark.parametrize("cap_factor", [8.0, 1.0], ids=["all", "truncated"])
+@pytest.mark.parametrize("bad", [0, 2, 6])
+def test_one_tensor_fails_and_the_others_do_not(bad, cap_factor):
+    """A tensor whose short list is too long is redone by itself, in front of, between or behind others that are not."""
+    g = randn(sum(SIZES), 9)
+    t = g[sum(SIZES[:bad]):sum(SIZES[:bad + 1])]
+    t[t.abs() > 2.0] = 2.0                             # equal keys from above the threshold to below it
+    plan, w = thr.check_threshold(SIZES, 0.01, [g], cap_factor=cap_factor)
+    assert plan.last_counters(w.ws)[1:] == (0, 1)
