@@ -426,7 +426,7 @@ __device__ __forceinline__ bool fold_tail_votes(BlockSmem& sm, const float (&av)
 // 61.6 / 59.5, 40M at 0.3 % 109.7 / 108.7, 2 % 119 / 115, 110M at 1 % 251.5 / 250, 2 % 262 / 257, 5 % 300 / 285).  Large plans between 0.2 and
 // 0.9 % are bound by memory, and the slower loop with unequal shares does better (110M at 0.3 % 245 / 253, 0.5 % 246 / 252-254;
 // 355M at 0.3 % 705 / 716).  Several workers in one launch keep the scan (see k_topk_workers).
-// DENSE (plans of 2 % and more) has the emission by chunk, the bfloat16 form the counted band: the other
+// DENSE (plans of 2 % and more) has the emission by chunk, the bfloat16 and threshold forms the counted band: the other
 // forms do without their code.  Many tensors, without / with DENSE: 110M elements at 2 % 305 / 310 us, 5 %
 // 359 / 346; 25.6M at 5 % 134 / 131; one tensor: 110M at 2 % 268 / 267, 5 % 312 / 311, 8M at 2 % 49 / 51.
 // THR: threshold mode, fold first (see the many-tensor kernel; the exact threshold is a rank among the sampled entries
@@ -736,7 +736,12 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
     // key after the barrier; then every CTA counts its candidates above and at that key per tile, and
     // after one more barrier the candidates at the key in the tiles before a tile say how many of its own
     // are sent.  110M elements, bfloat16, 60,000 ties: counts + threshold + slots 15 us, 41 us as a list.
-    const bool counted = GL::kManyTies && overflowed == 0u && pa[0].ok && m > kMidCounted && A < 2047u && shift <= 11;
+    // Threshold mode histograms the sampled ones and sends whatever reaches the key they give: no ties to settle (110M
+    // elements that were rounded to bfloat16, residual zero, 1 %: counts + threshold + slots 48 us as a list, 22 counted; beyond 65,536
+    // equal keys the list was full and the call redone).
+    const bool counted = (GL::kManyTies || THR) && overflowed == 0u && pa[0].ok && A < 2047u && shift <= 11 &&
+                         (unsigned long long)m * (THR ? d.stride : 1u) > kMidCounted;
+    const bool ties = !THR && counted;                   // of the candidates at the key the lowest indices are sent
     bool good = overflowed == 0u && pa[0].ok && (THR || m <= a.mid_cap || counted);
     const uint32_t binlo = tau + (A << shift);
 
@@ -752,7 +757,10 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
                 const uint32_t rel = pr.x - base0;
                 atomicAdd(&rec2[rm.row_of(rel >> 12) * kWarps + ((rel >> 9) & (kWarps - 1u))], 1u);
             } else if (bin == A) {
-                if (counted) { atomicAdd(&sm.hist[(pr.y & kKeyMask) - binlo], 1u); return; }
+                if (counted) {
+                    if (!THR || InSample{d.off, d.stride}(pr.x)) atomicAdd(&sm.hist[(pr.y & kKeyMask) - binlo], 1u);
+                    return;
+                }
                 const uint32_t slot = atomicAdd(a.hist5 + 3 * kHistBins, 1u);
                 if (slot < a.mid_cap) a.mid[slot] = pr;
             }
@@ -779,8 +787,8 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
             const uint32_t want_in[1] = {d.k - aboveA};
             Picked pt[1];
             block_select_multi<2048, 1>(sm, a.hist5 + 4 * kHistBins, want_in, pt);
-            Tkey = binlo + pt[0].bin; m_eq = d.k - aboveA - pt[0].above;
-            // per chunk: candidates above the threshold key in the low half, those at it in the high half
+            Tkey = binlo + pt[0].bin; m_eq = THR ? 0xFFFFFFFFu : d.k - aboveA - pt[0].above;
+            // per chunk: candidates above the threshold key in the low half, those at it in the high half (threshold mode: all in the low one)
             for (uint32_t i0 = tid; i0 < used; i0 += 8 * kBlock) {
                 uint2 pr[8];
 #pragma unroll
@@ -790,7 +798,7 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
                     const uint32_t key = pr[u].y & kKeyMask;
                     if (i0 + u * kBlock >= used || key < Tkey || min((key - tau) >> shift, 2047u) != A) continue;
                     const uint32_t rel = pr[u].x - base0;
-                    atomicAdd(&rec2[rm.row_of(rel >> 12) * kWarps + ((rel >> 9) & (kWarps - 1u))], key == Tkey ? 1u << 16 : 1u);
+                    atomicAdd(&rec2[rm.row_of(rel >> 12) * kWarps + ((rel >> 9) & (kWarps - 1u))], !THR && key == Tkey ? 1u << 16 : 1u);
                 }
             }
         }
@@ -801,7 +809,7 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
             for (int w = 0; w < kWarps; ++w) { tot += rec2[i * kWarps + w] & 0xFFFFu; eq += rec2[i * kWarps + w] >> 16; }
             a.tile_cnt[rm.tile_of(i, col)] = tot;
             atomicAdd(a.seg_tot + (size_t)i * nseg + myseg, tot);
-            if (counted) {
+            if (ties) {
                 a.tile_eq[rm.tile_of(i, col)] = eq;
                 atomicAdd(a.seg_eq + (size_t)i * nseg + myseg, eq);
             }
@@ -841,7 +849,7 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
                 if (lane == 0 && i0 + u * kWarps < n_own) { row_sum[i0 + u * kWarps] = row; tile_base[i0 + u * kWarps] = low; }
             }
         }
-        if (counted) {                                    // the same for the candidates at the threshold key
+        if (ties) {                                       // the same for the candidates at the threshold key
             for (uint32_t i = warp; i < n_own; i += kWarps) {
                 const uint32_t q = myseg * 32u + (uint32_t)lane;
                 const uint32_t sv = (uint32_t)lane < nseg ? ld_cg(a.seg_eq + (size_t)i * nseg + lane) : 0u;
@@ -936,7 +944,7 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
                     const uint32_t i = i0 + lane;
                     const uint32_t v = i < n_own ? row_sum[i] : 0u;
                     const uint32_t w = i < n_own ? row_mid[i] : 0u;
-                    if (counted) {
+                    if (ties) {
                         const uint32_t inc = warp_incl_scan(v, lane), inc_eq = warp_incl_scan(w, lane);
                         if (i < n_own) {
                             const uint32_t eq = row_eq[i] + run_eq + inc_eq - w;
@@ -953,7 +961,7 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
                 }
             }
             __syncthreads();
-            if (counted) {
+            if (ties) {
                 // what every chunk sends; this CTA's cut: the end of its last chunk that sends all its
                 // candidates at the key, or a place inside the one chunk (of the whole tensor) that sends some
                 for (uint32_t i = tid; i < n_own; i += kBlock) {

@@ -43,3 +43,13 @@ def test_samples_that_mislead(what):
     elif what == "sorted":
         g = g[g.abs().argsort()].contiguous()
     thr.check_threshold([N], 0.01, [g, g], cap_factor=3.0)
+
+
+@pytest.mark.parametrize("what,n,density", [("bfloat16", N, 0.01), ("bfloat16", N, 0.02), ("grid", 40_000_001, 0.01), ("grid", 40_000_001, 0.003)])
+@pytest.mark.parametrize("cap_factor", [8.0, 1.0], ids=["all", "truncated"])
+def test_ties_by_the_thousand_are_counted(what, n, density, cap_factor):
+    """More equal keys at the threshold than a short list is worth, or than it holds: no redo."""
+    g = randn(n, 5)
+    g = g.to(torch.bfloat16).float() if what == "bfloat16" else (g * 8).round() / 8
+    plan, w = thr.check_threshold([n], density, [g], cap_factor=cap_factor)
+    assert plan.last_counters(w.ws)[1:] == (0, 0)
