@@ -138,14 +138,7 @@ k_topk_direct(const __grid_constant__ DirectArgs a) {
         if (b == 0 && tid < 62 && tid != (int)kHdrBarrierWord && tid != (int)kHdrExitWord) reinterpret_cast<uint32_t*>(hdr)[tid] = 0u;
         __syncthreads();
     }
-    if (b == 0 && tid == 0) {
-        hdr->cand_total = a.k;
-        if (a.clear_first != 0u && a.status_out != nullptr) *a.status_out = 0 /*GC_OK*/;      // (an error is written over it)
-    }
-    auto report = [&](unsigned long long detail) {
-        record_status(hdr, -1 /*GC_E_INVALID*/, detail);
-        if (a.clear_first != 0u && a.status_out != nullptr) *a.status_out = -1;
-    };
+    if (b == 0 && tid == 0) hdr->cand_total = a.k;
     phase_stamp(hdr, n_stamp);
     auto flush = [&](uint32_t* dst, int nb) {
         __syncthreads();
@@ -235,7 +228,7 @@ k_topk_direct(const __grid_constant__ DirectArgs a) {
         // Somebody else's counts in the scratch: nothing is sent (the residual keeps g + r), the scratch is
         // cleaned on the way out.  Every CTA sees the same sum.
         if (direct_select<2048>(sm, a.s->hist0, a.k, tid, lane, warp) != a.n) {
-            if (b == 0 && tid == 0) { report(0xC1EA0001ull); atomicExch(&hdr->abort, 1u); }
+            if (b == 0 && tid == 0) { record_status(hdr, -1 /*GC_E_INVALID*/, 0xC1EA0001ull); atomicExch(&hdr->abort, 1u); }
             live = false;
         }
     }
@@ -365,7 +358,7 @@ k_topk_direct(const __grid_constant__ DirectArgs a) {
                             a.out_val[slot] = xe[e];
                             a.r[i] = 0.0f;
                         } else {
-                            report(i);
+                            record_status(hdr, -1 /*GC_E_INVALID*/, i);
                         }
                     }
                 }
@@ -375,14 +368,22 @@ k_topk_direct(const __grid_constant__ DirectArgs a) {
         // (counted and emitted entries agree and add up to k, unless others wrote to the scratch)
         if (lane == 0 && (gt_at != gt_end || eq_at != eq_end ||
                           (b == G - 1u && warp == kWarps - 1 && gt_at + min(eq_at, m_eq) != a.k)))
-            report(0xC1EA0002ull);
+            record_status(hdr, -1 /*GC_E_INVALID*/, 0xC1EA0002ull);
         if (a.out_count != nullptr && b == 0 && tid == 0) { a.out_count[0] = a.k; a.out_count[1] = a.k; }
         phase_stamp(hdr, n_stamp);
     }
     if (a.clear_first != 0u) {
-        // (nothing to be left clean; a wait that ran out is the one error that is not reported above)
-        if (!live && tid == 0 && a.status_out != nullptr && *reinterpret_cast<volatile int32_t*>(&hdr->status) != 0)
-            *a.status_out = *reinterpret_cast<volatile int32_t*>(&hdr->status);
+        // Nothing to be left clean; the caller's status word is written when the work is done, by the CTA that leaves last.
+        if (a.status_out == nullptr) return;
+        __syncthreads();
+        if (tid == 0) {
+            uint32_t gone;                                 // (the CTAs that left before, their writes done)
+            asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(gone) : "l"(&hdr->exit_count) : "memory");
+            if (gone == G - 1u) {
+                const int32_t st = *reinterpret_cast<volatile int32_t*>(&hdr->status);
+                asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(a.status_out), "r"(st) : "memory");
+            }
+        }
         return;
     }
     // The CTA that leaves last resets what the others may still have been reading; after a wait that ran

@@ -91,8 +91,8 @@ extern "C" int gc_compress_noalloc(const float* grad, float* residual, uint32_t 
     da.g = grad; da.r = residual; da.n = n; da.k = k; da.out_idx = out_idx; da.out_val = out_val;
     da.status_out = device_status; da.s = pd.scratch;
     const DirectGeom dg = direct_geometry(n, pd.sms);
-    // The kernel leaves the scratch clean, but no caller can replace this array: what two calls that
-    // overlapped against the rules left in it must not outlive them.
+    // No caller can replace this array, and what two calls that overlapped against the rules left in it must not
+    // outlive them: every launch clears it.
     da.clear_first = 1u;
     void* args[] = {&da};
     const void* fn = dg.resident ? (const void*)k_topk_direct<GradF32, true> : (const void*)k_topk_direct<GradF32, false>;

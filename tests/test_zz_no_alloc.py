@@ -202,3 +202,29 @@ def test_whatever_is_left_in_the_scratch_does_not_reach_the_next_call(fill):
         torch.cuda.synchronize()
         assert status.item() == api.GC_OK
         assert np.array_equal(u32(idx), o_idx) and np.array_equal(u32(val), o_val) and np.array_equal(u32(r), o_r)
+
+
+def test_status_is_written_when_the_work_is_done():
+    """Copies on another stream while the call runs: whoever sees the status sees everything that was sent."""
+    n, k, pairs = api.GC_NOALLOC_MAX_N, 4096, 24
+    g = torch.randn(n, device="cuda", generator=torch.Generator(device="cuda").manual_seed(5))
+    r, idx, val = torch.zeros(n, device="cuda"), torch.zeros(k, dtype=torch.int32, device="cuda"), torch.zeros(k, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    seen = [(torch.zeros(1, dtype=torch.int32).pin_memory(), torch.zeros(k, dtype=torch.int32).pin_memory()) for _ in range(pairs)]
+    side = torch.cuda.Stream()
+    done = 0
+    for _ in range(10):
+        r.zero_(); idx.fill_(-1); status.fill_(77)
+        torch.cuda.synchronize()
+        assert api.compress_noalloc(g, r, n, k, idx, val, status) == api.GC_OK
+        with torch.cuda.stream(side):
+            for st, ix in seen:
+                st.copy_(status, non_blocking=True)
+                ix.copy_(idx, non_blocking=True)
+        torch.cuda.synchronize()
+        for st, ix in seen:
+            assert int(st) in (77, api.GC_OK)
+            if int(st) == api.GC_OK:
+                done += 1
+                assert int(ix.min()) >= 0
+    assert done > 0 and int(status.cpu()) == api.GC_OK
