@@ -8,6 +8,7 @@
 #include <initializer_list>
 #include <mutex>
 #include <new>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -751,13 +752,15 @@ static bool ask_device(int device, DeviceFacts* p) {
         }
         (void)cudaGetLastError();
         p->direct_ok = coop != 0;
-        for (const void* fn : {(const void*)k_topk_direct<GradF32, true>, (const void*)k_topk_direct<GradBF16, true>}) {
+        for (const void* fn : {(const void*)k_topk_direct<GradF32, true, false>, (const void*)k_topk_direct<GradF32, true, true>,
+                               (const void*)k_topk_direct<GradBF16, true, false>, (const void*)k_topk_direct<GradBF16, true, true>}) {
             int nb = 0;
             if (!allow_smem({fn}, kDirectResident) ||
                 cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kBlock, kDirectResident) != cudaSuccess || nb < 2)
                 p->direct_ok = false;
         }
-        for (const void* fn : {(const void*)k_topk_direct<GradF32, false>, (const void*)k_topk_direct<GradBF16, false>}) {
+        for (const void* fn : {(const void*)k_topk_direct<GradF32, false, false>, (const void*)k_topk_direct<GradF32, false, true>,
+                               (const void*)k_topk_direct<GradBF16, false, false>, (const void*)k_topk_direct<GradBF16, false, true>}) {
             int nb = 0;
             if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kBlock, 0) != cudaSuccess || nb < 3) p->direct_ok = false;
         }
@@ -1320,13 +1323,16 @@ static int compress_impl(gc_plan_t* p, const void* grad_any, bool bf16, float* r
         da.g = grad_any; da.r = residual; da.n = (uint32_t)p->total_n; da.k = p->desc[0].k; da.out_idx = out_idx; da.out_val = out_val;
         da.out_count = out_count; da.s = reinterpret_cast<DirectScratch*>(workspace);
         da.mark = clean_args(p, workspace, GC_ROUTE_TOPK_ONE, kCleanDone).mark + 1u; da.expect_clean = kept_clean ? 1u : 0u;
-        da.clear_first = clean_mode == kCleanSelf ? 1u : 0u;
         const DirectGeom dg = direct_geometry(da.n, p->sm_count);
         note_clean(p, workspace);
         void* args[] = {&da};
         Timed tm(p, s, GC_K_FUSED);
-        const void* kfn = dg.resident ? (bf16 ? (const void*)k_topk_direct<GradBF16, true> : (const void*)k_topk_direct<GradF32, true>)
-                                      : (bf16 ? (const void*)k_topk_direct<GradBF16, false> : (const void*)k_topk_direct<GradF32, false>);
+        auto form = [&](auto self) {
+            constexpr bool S = decltype(self)::value;
+            return dg.resident ? (bf16 ? (const void*)k_topk_direct<GradBF16, true, S> : (const void*)k_topk_direct<GradF32, true, S>)
+                               : (bf16 ? (const void*)k_topk_direct<GradBF16, false, S> : (const void*)k_topk_direct<GradF32, false, S>);
+        };
+        const void* kfn = clean_mode == kCleanSelf ? form(std::true_type{}) : form(std::false_type{});
         GC_CUDA(p, cudaLaunchCooperativeKernel(kfn, dim3(dg.G), dim3(kBlock), args, dg.smem, s));
         return GC_OK;
     }

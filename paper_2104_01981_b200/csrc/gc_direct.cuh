@@ -8,8 +8,9 @@
 // them are counted | barrier | every CTA takes the threshold key from the list and emits its share.  No
 // sample, no candidate list, no capacity that data could overflow: if more entries share the 21 bits than
 // the list takes, the last 10 bits get a global histogram and the shares are counted (one more barrier),
-// and nothing is ever redone.  The scratch is 29 KB and the launch leaves it clean.  Without a plan, six
-// launches over the whole tensor took 55 us at 2.4M elements; this takes 26.7, and 15.2 us at 200,000.
+// and nothing is ever redone.  The scratch is 29 KB; on a private workspace the launch leaves it clean,
+// otherwise it clears it itself.  Without a plan, six launches over the whole tensor took 55 us at 2.4M elements; this takes
+// 26.7, and 16.4 us at 200,000.
 #pragma once
 #include <cstddef>
 
@@ -20,7 +21,7 @@ namespace gc {
 constexpr uint32_t kDirectList = 1024;           // entries sharing 21 key bits that travel as a list
 constexpr uint32_t kDirectMaxG = 512;            // most CTAs
 
-struct DirectScratch {                           // zero before a launch (see clear_first), except `list` and `tot`
+struct DirectScratch {                           // zero before a launch (see SELF), except `list` and `tot`
     WsHeader hdr;
     uint32_t hist0[2048], hist1[1024], hist2[1024];
     uint32_t list_n, pad[63];
@@ -39,7 +40,6 @@ struct DirectArgs {
     DirectScratch* s;
     unsigned long long mark;                     // what the header's mark reads after a launch that left the scratch clean
     uint32_t expect_clean;                       // the host relies on that mark (see CleanArgs)
-    uint32_t clear_first;                        // the launch clears the scratch itself, whatever is in it, and leaves it as it is
 };
 
 // Grid barrier: release by the arrival, acquire by the poll (see grid_barrier for the bounded wait).
@@ -106,7 +106,10 @@ __device__ __forceinline__ uint32_t direct_select(DirectSmem& sm, const uint32_t
 }
 
 // RES: the share of a CTA stays in (dynamic) shared memory; otherwise it is read back from r.
-template <typename GL, bool RES>
+// SELF: the launch clears the scratch itself, whatever is in it, and leaves it as it is.  A form of its own: with
+// both in one, chosen by an argument, each paid for the other's code (us, in one / apart: workspace left clean 0.3M elements 17.3 /
+// 16.6, 3.9M 36.8 / 35.6, 0.5M 18.5 / 18.5; cleared by the launch 0.5M 18.4 / 17.4, 3.9M 34.6 / 32.8).
+template <typename GL, bool RES, bool SELF>
 static __global__ void __launch_bounds__(kBlock, 3)
 k_topk_direct(const __grid_constant__ DirectArgs a) {
     __shared__ DirectSmem sm;
@@ -114,7 +117,7 @@ k_topk_direct(const __grid_constant__ DirectArgs a) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t G = gridDim.x, b = blockIdx.x;
     WsHeader* const hdr = &a.s->hdr;
-    if (a.expect_clean != 0u && ld_cg(reinterpret_cast<const unsigned long long*>(&hdr->clean_mark)) != a.mark) {
+    if (!SELF && a.expect_clean != 0u && ld_cg(reinterpret_cast<const unsigned long long*>(&hdr->clean_mark)) != a.mark) {
         if (b == 0 && tid == 0) record_status(hdr, -1 /*GC_E_INVALID*/, 0xC1EA0000ull);
         return;                                            // every CTA sees the same word
     }
@@ -128,8 +131,8 @@ k_topk_direct(const __grid_constant__ DirectArgs a) {
     // counter is among what is cleared.  Arrival here, wait behind the fold (2.4M elements, still with an exit count:
     // 28.7 us; 29.1 with the whole barrier behind the fold, 30.1 with a clearing launch in front).
     const auto grid = cooperative_groups::this_grid();
-    cooperative_groups::grid_group::arrival_token cleared{};
-    if (a.clear_first != 0u) {
+    [[maybe_unused]] cooperative_groups::grid_group::arrival_token cleared{};
+    if constexpr (SELF) {
         uint4* const w = reinterpret_cast<uint4*>(a.s);
         for (uint32_t i = b * kBlock + tid; i < (uint32_t)(offsetof(DirectScratch, list) / 16); i += G * kBlock) w[i] = make_uint4(0u, 0u, 0u, 0u);
         cleared = grid.barrier_arrive();                   // (a barrier of the block as well)
@@ -217,7 +220,7 @@ k_topk_direct(const __grid_constant__ DirectArgs a) {
                 if (e < ne[u]) atomicAdd(&sm.hist[key_of(se[e]) >> 20], 1u);
         }
     }
-    if (a.clear_first != 0u) grid.barrier_wait(std::move(cleared));
+    if constexpr (SELF) grid.barrier_wait(std::move(cleared));
     flush(a.s->hist0, 2048);
     bool live = direct_barrier(hdr, passed, &sm.ok);
     uint32_t prefix = 0, krem = 0, T = 0, m_eq = 0, gt_before = 0, eq_before = 0;
@@ -314,7 +317,7 @@ k_topk_direct(const __grid_constant__ DirectArgs a) {
     if (live) {
         // ------------------------------------------------------------ emission
         // the histograms have had their last readers (of hist2: before the barrier that followed)
-        if (a.clear_first == 0u)
+        if constexpr (!SELF)
             for (uint32_t i = b * kBlock + tid; i < 4096u; i += G * kBlock) a.s->hist0[i] = 0u;    // (hist0, hist1, hist2 in a row)
         unsigned long long before = (unsigned long long)eq_before << 32 | gt_before;
         for (uint32_t c = tid; c < b; c += kBlock) before += ld_cg(&a.s->tot[c]);
@@ -372,7 +375,7 @@ k_topk_direct(const __grid_constant__ DirectArgs a) {
         if (a.out_count != nullptr && b == 0 && tid == 0) { a.out_count[0] = a.k; a.out_count[1] = a.k; }
         phase_stamp(hdr, n_stamp);
     }
-    if (a.clear_first != 0u) {
+    if constexpr (SELF) {
         // Nothing to be left clean; the caller's status word is written when the work is done, by the CTA that leaves last.
         if (a.status_out == nullptr) return;
         __syncthreads();
@@ -401,7 +404,6 @@ k_topk_direct(const __grid_constant__ DirectArgs a) {
         if (failed) for (uint32_t i = tid; i < 4096u; i += kBlock) a.s->hist0[i] = 0u;
         if (tid == 0) {
             a.s->list_n = 0u; hdr->barrier = 0u; hdr->exit_count = 0u; hdr->abort = 0u;
-            if (a.status_out != nullptr) *a.status_out = *reinterpret_cast<volatile int32_t*>(&hdr->status);
             __threadfence();
             if (!failed) hdr->clean_mark = a.mark;
         }

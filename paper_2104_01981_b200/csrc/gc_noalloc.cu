@@ -74,10 +74,10 @@ extern "C" int gc_compress_noalloc(const float* grad, float* residual, uint32_t 
             if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
             if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
             if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k_topk_direct<GradF32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDirectResident);
+                e = cudaFuncSetAttribute(k_topk_direct<GradF32, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDirectResident);
             if (e == cudaSuccess)
-                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_topk_direct<GradF32, true>, kBlock, kDirectResident);
-            if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb2, k_topk_direct<GradF32, false>, kBlock, 0);
+                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_topk_direct<GradF32, true, true>, kBlock, kDirectResident);
+            if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb2, k_topk_direct<GradF32, false, true>, kBlock, 0);
             if (e != cudaSuccess || ptr == nullptr || sms < 1 || coop == 0 || nb < 2 || nb2 < 3) {
                 (void)cudaGetLastError();
                 return GC_E_CUDA;
@@ -92,10 +92,9 @@ extern "C" int gc_compress_noalloc(const float* grad, float* residual, uint32_t 
     da.status_out = device_status; da.s = pd.scratch;
     const DirectGeom dg = direct_geometry(n, pd.sms);
     // No caller can replace this array, and what two calls that overlapped against the rules left in it must not
-    // outlive them: every launch clears it.
-    da.clear_first = 1u;
+    // outlive them: the form that clears it.
     void* args[] = {&da};
-    const void* fn = dg.resident ? (const void*)k_topk_direct<GradF32, true> : (const void*)k_topk_direct<GradF32, false>;
+    const void* fn = dg.resident ? (const void*)k_topk_direct<GradF32, true, true> : (const void*)k_topk_direct<GradF32, false, true>;
     if (cudaLaunchCooperativeKernel(fn, dim3(dg.G), dim3(kBlock), args, dg.smem, s) != cudaSuccess) {
         (void)cudaGetLastError();
         return GC_E_CUDA;
