@@ -348,7 +348,7 @@ void finish_layout(gc_plan_s* p) {
     p->off_midn = align_up(p->off_bhist + multi_hist, 256);
     p->control_bytes = align_up(p->off_midn + (multi_hist ? sizeof(uint32_t) * T : 0), 256);
     p->off_start = p->control_bytes;                                 // where and when the CTAs started (one-tensor kernel)
-    p->off_tinfo = align_up(p->off_start + (T == 1 ? sizeof(uint2) * kSingleMaxG : 0), 256);
+    p->off_tinfo = align_up(p->off_start + (T == 1 ? sizeof(unsigned long long) * kSingleMaxG : 0), 256);
     p->off_cidx = align_up(p->off_tinfo + sizeof(uint2) * (size_t)p->ntiles * kWarps, 256);
     p->off_mid = align_up(p->off_cidx + sizeof(uint2) * (size_t)p->cand_cap_alloc, 256);
     p->off_mmid = align_up(p->off_mid + (T == 1 ? sizeof(uint2) * (size_t)kSingleMidCap : 0), 256);
@@ -1349,7 +1349,7 @@ static int compress_impl(gc_plan_t* p, const void* grad_any, bool bf16, float* r
         sa.srank_hi = thr ? p->thr_srank_hi : p->single_srank_hi; sa.srank_mid = thr ? p->thr_srank_mid : p->single_srank_mid; sa.mid_cap = (uint32_t)kSingleMidCap;
         sa.mid = reinterpret_cast<uint2*>(wb + p->off_mid);
         sa.fine = reinterpret_cast<uint32_t*>(wb + p->off_fine);
-        sa.start = reinterpret_cast<uint2*>(wb + p->off_start);
+        sa.start = reinterpret_cast<unsigned long long*>(wb + p->off_start);
         sa.tile_cnt = reinterpret_cast<uint32_t*>(wb + p->off_tinfo);
         sa.seg_tot = reinterpret_cast<uint32_t*>(wb + p->off_rowseg);
         sa.tile_eq = sa.tile_cnt + nt; sa.seg_eq = sa.seg_tot + kSingleMaxT * 20;

@@ -76,27 +76,27 @@ struct RowMap {
     }
 };
 
-// Where and when this CTA started: the SM's number and the SM's cycle counter.
-__device__ __forceinline__ uint2 note_start() {
-    uint2 s;
-    asm volatile("mov.u32 %0, %%smid;" : "=r"(s.x));
-    asm volatile("mov.u32 %0, %%clock;" : "=r"(s.y));
-    return s;
+// Where and when this CTA started.
+__device__ __forceinline__ unsigned long long note_start() {
+    uint32_t sm;
+    unsigned long long cycle;
+    asm volatile("mov.u32 %0, %%smid;" : "=r"(sm));
+    asm volatile("mov.u64 %0, %%clock64;" : "=l"(cycle));
+    return start_word(sm, cycle);
 }
 // Column of this CTA once every CTA has written down its start (before a grid barrier): its age is the number
 // of CTAs of its SM that started before it, and column = age x gA + SM number, oldest first.  That is a
 // one-to-one assignment only if SMs 0..gA-1 hold three CTAs each; every CTA checks the same table and
 // otherwise keeps column b.  Called by the whole CTA; count[] (1024 words of shared memory) is zero before and after.
-__device__ __forceinline__ uint32_t aged_column(const RowMap& rm, const uint2* start, uint2 mine, uint32_t G, uint32_t b,
+__device__ __forceinline__ uint32_t aged_column(const RowMap& rm, const unsigned long long* start, unsigned long long mine, uint32_t G, uint32_t b,
                                                 uint32_t* count, uint32_t* s_age, int tid) {
     if (rm.gA * 3u != G || rm.gA > (uint32_t)kBlock) return b;           // one class of columns
     if (tid == 0) *s_age = 0u;
     __syncthreads();
     for (uint32_t c = tid; c < G; c += kBlock) {
-        const uint2 s = ld_cg(start + c);
-        atomicAdd(&count[s.x & 1023u], 1u);
-        const int later = (int)(mine.y - s.y);                           // (the counter wraps)
-        if (s.x == mine.x && c != b && (later > 0 || (later == 0 && c < b))) atomicAdd(s_age, 1u);
+        const unsigned long long s = ld_cg(start + c);
+        atomicAdd(&count[start_sm(s)], 1u);
+        if (start_sm(s) == start_sm(mine) && c != b && started_before(s, c, mine, b)) atomicAdd(s_age, 1u);
     }
     __syncthreads();
     const bool aged = __syncthreads_and((uint32_t)tid >= rm.gA || count[tid] == 3u);      // (3 gA = G: none beyond)
@@ -104,7 +104,7 @@ __device__ __forceinline__ uint32_t aged_column(const RowMap& rm, const uint2* s
     __syncthreads();
     for (uint32_t i = tid; i < 1024u; i += kBlock) count[i] = 0u;
     __syncthreads();
-    return aged ? min(age, 2u) * rm.gA + mine.x : b;
+    return aged ? min(age, 2u) * rm.gA + start_sm(mine) : b;
 }
 
 struct SingleArgs {
@@ -126,7 +126,7 @@ struct SingleArgs {
     uint2* mid;                      // [mid_cap] candidates inside the band bin of the threshold
     uint32_t* hist5;                 // [0] coarse sample histogram, [2] band histogram,
                                      // [3][0] short-list length, [4] keys inside a counted band (all zeroed)
-    uint2* start;                    // [gridDim.x] SM and cycle at which every CTA started
+    unsigned long long* start;       // [gridDim.x] SM and cycle at which every CTA started
     uint32_t* fine;                  // [kFineBins] fine sample histogram (zeroed)
     uint32_t* tile_cnt;              // [ntiles] candidates above the band bin, per tile
     uint32_t* seg_tot;               // [maxt][ceil(G/32)] the same summed over each run of 32 CTAs of a row (zeroed)
@@ -456,10 +456,10 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
     uint32_t passed = 0, n_stamp = 0;
     const RowMap& rm = a.rows;
     __shared__ uint32_t s_age;
-    __shared__ uint2 s_start;
+    __shared__ unsigned long long s_start;
     // When this CTA started, taken first thing: the ages have to reflect the order in which the CTAs really
     // started (taken behind a load they were measured to cost the fold pass 10 us: the shares no longer matched).
-    uint2 my_start = make_uint2(0u, 0u);
+    unsigned long long my_start = 0ull;
     if (tid == 0) my_start = note_start();
     ClearWait cleared;
     if (!clean_begin(a.cl, hdr, G, b, tid, cleared)) return;
