@@ -133,6 +133,7 @@ constexpr double kThrOneFoldUpTo = 0.02;     // one tensor: the same, and the el
 constexpr uint32_t kThrOneFoldFrom = 12u << 20;
 constexpr double kThrFoldUpTo = 0.005;       // density up to which, and elements from which threshold plans of several tensors are
 constexpr uint64_t kThrFoldFrom = 12u << 20; // taken fold first (see plan_thr_fold)
+constexpr uint32_t kThrMaxTiles = 128;       // longest sample, in sample tiles, that a CTA of the sample-first kernel ranks
 constexpr uint32_t kMultiMaxTab = 1024;      // tensors whose tile tables k_topk_multi keeps in shared memory
 constexpr size_t kMultiMaxPer = 224;         // most tiles one CTA of k_topk_multi may own
 constexpr size_t kMultiRowBytes = (2 * kWarps + kSegWords) * sizeof(uint32_t);   // shared memory per owned tile
@@ -281,7 +282,8 @@ void finish_layout(gc_plan_s* p) {
                 m = (nsg - 1) * 4 + std::min<uint64_t>(4, d.n - last_first);
             }
             d.srank = (uint32_t)k_rule(m, p->density);
-            if (d.ntiles > 1) stiles_worst += kRefineTiles;       // (the bracket's sample, see plan_thr_fold)
+            if (d.ntiles > 1 && p->T >= 2)                        // (the bracket's sample, see plan_thr_fold; no option changes its size)
+                stiles_worst += (thr_bracket(d, 1000).groups + (uint32_t)kSampleTile - 1u) / (uint32_t)kSampleTile;
             if (d.n > 0 && d.ntiles == 1 && p->T >= 2) d.kind = kKindSmall;    // one CTA finishes it (many-tensor kernel)
         }
         uint64_t nst = 0;
@@ -318,9 +320,14 @@ void finish_layout(gc_plan_s* p) {
         ccap_total = 0;
         if (p->T >= 1 && p->total_cap > 0)
             ccap_total = std::min<uint64_t>(0x7FFFFFFFull, (uint64_t)(1.25 * (double)p->total_cap) + (1u << 20));
-        double fold = 0.0;                 // the candidates between the brackets, twice over
+        // Plans that may be taken fold first (by plan_thr_fold's rule, or since the sample-first kernel refuses samples that
+        // long or hit lists that full): the candidates between the brackets, twice over.
+        bool may_fold = p->density <= kThrFoldUpTo && p->total_n >= kThrFoldFrom;
+        double hits = 0.0, fold = 0.0;
+        for (const TensorDesc& d : p->desc) { may_fold |= d.nstiles > kThrMaxTiles; hits += (double)d.k; }
+        may_fold |= (double)ccap_total < 2.5 * hits + (1u << 19);
         for (const TensorDesc& d : p->desc) {
-            if (p->T < 2 || d.kind == kKindSmall || d.n == 0) continue;
+            if (!may_fold || p->T < 2 || d.kind == kKindSmall || d.n == 0) continue;
             const ThrBracket b = thr_bracket(d, 1000);
             fold += b.rank > 0.0 ? std::min<double>(d.n, 2.5 * (double)d.n * (b.rank + 6.0 * std::sqrt(b.rank)) / (4.0 * (double)b.groups) + 4096.0) : 0.0;
         }
@@ -481,7 +488,7 @@ MultiGeom thr_multi_geometry(const gc_plan_s* p, uint32_t G) {
     if (per > kMultiMaxPer) return mg;
     // one CTA ranks a whole tensor's kept sample keys: keep that bounded
     for (uint32_t t : p->reg_ids)
-        if (p->desc[t].nstiles > 128 || p->desc[t].sstride == 0) return mg;
+        if (p->desc[t].nstiles > kThrMaxTiles || p->desc[t].sstride == 0) return mg;
     const uint32_t pool = std::min<uint32_t>(p->cand_cap_alloc / G, kSinglePoolMax);
     // expected hits of the busiest CTA: about k per tensor, spread over its tiles
     double worst = 0.0;

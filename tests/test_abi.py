@@ -119,6 +119,13 @@ def test_workspace_size_survives_the_sample_rank_option(lib):
         p.destroy()
 
 
+@pytest.mark.parametrize("sizes,density,most", [([5000] * 2000, 0.001, 170e6), ([5000] * 2000, 0.05, 185e6), ([70_000] * 500, 0.01, 70e6),
+                                                ([2_500_000] * 12, 0.05, 42e6)])
+def test_workspace_of_threshold_plans_with_many_tensors(lib, sizes, density, most):
+    """No room is kept for samples and candidates that the plan cannot have."""
+    assert api.Plan(sizes, density, mode=api.GC_THRESHOLD, device=-1).query(api.GC_Q_WORKSPACE_BYTES) <= most
+
+
 def test_host_only_plan_refuses_compute(lib):
     p = api.Plan([16], 0.5, device=-1)
     assert p.compress_ptr(16, 16, 16, 16, None, 256, 0) == api.GC_E_UNSUPPORTED
