@@ -44,10 +44,31 @@ def test_threshold_from_a_dirty_workspace(dirty, sizes, ties):
     thr.check_threshold(sizes, 0.01, grads, cap_factor=2.0)
 
 
-@pytest.mark.parametrize("mode", [api.GC_TOPK, api.GC_THRESHOLD], ids=["topk", "threshold"])
-def test_workers_from_dirty_workspaces(mode):
+# (plans of these sizes are taken fold first; starved: the redo starts from whatever is in the workspace, too)
+FOLD_ONE, FOLD_MANY = [13_000_003], [300_000, 5, 1_500_001, 0, 64, 11_000_003, 4097]
+
+
+@pytest.mark.parametrize("sizes", [FOLD_ONE, FOLD_MANY], ids=["one", "many"])
+@pytest.mark.parametrize("opts", [{}, {api.GC_OPT_SAMPLE_RANK_PERMILLE: 30}, {api.GC_OPT_CANDIDATE_CAPACITY: 100}],
+                         ids=["plain", "starved", "overflow"])
+def test_threshold_fold_first_from_a_dirty_workspace(dirty, monkeypatch, sizes, opts):
+    class WithOptions(api.Plan):
+        def __init__(self, *a, **k):
+            super().__init__(*a, **k)
+            for opt, value in opts.items():
+                self.set_option(opt, value)
+    monkeypatch.setattr(thr.api, "Plan", WithOptions)
+    plan, w = thr.check_threshold(sizes, 0.002, [randn(sum(sizes), 41 + s) for s in range(2)])
+    assert (plan.last_counters(w.ws)[1:] == (0, 0)) == (not opts)
+
+
+@pytest.mark.parametrize("mode,MANY,starved", [(api.GC_TOPK, MANY, False), (api.GC_THRESHOLD, MANY, False), (api.GC_THRESHOLD, FOLD_MANY, False),
+                                               (api.GC_THRESHOLD, FOLD_MANY, True)], ids=["topk", "threshold", "fold_first", "fold_first_starved"])
+def test_workers_from_dirty_workspaces(mode, MANY, starved):
     """Three workers in one launch on dirty workspaces give what three calls on zeroed ones give."""
-    plan, n = api.Plan(MANY, 0.01, mode=mode, device=0), sum(MANY)
+    plan, n = api.Plan(MANY, 0.01 if MANY is not FOLD_MANY else 0.002, mode=mode, device=0), sum(MANY)
+    if starved:
+        plan.set_option(api.GC_OPT_SAMPLE_RANK_PERMILLE, 30)
     a, b = ([GpuWorker(plan) for _ in range(3)] for _ in range(2))
     for step in range(2):
         gs = [randn(n, 1000 * step + w).cuda() for w in range(3)]

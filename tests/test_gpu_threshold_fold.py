@@ -79,3 +79,11 @@ def test_one_tensor_fails_and_the_others_do_not(bad, cap_factor):
     t[t.abs() > 2.0] = 2.0                             # equal keys from above the threshold to below it
     plan, w = thr.check_threshold(SIZES, 0.01, [g], cap_factor=cap_factor)
     assert plan.last_counters(w.ws)[1:] == (0, 1)
+
+
+def test_more_tensors_than_the_tables_in_shared_memory_hold():
+    """Above 1024 tensors the owners of tiles and sample tiles are searched in the device tables."""
+    sizes = [9000] * 550 + [9_000_003] + [9001] * 550            # (the long sample: no other fused kernel takes the plan)
+    assert api.Plan(sizes, 0.002, mode=api.GC_THRESHOLD, device=0).query(api.GC_Q_COMPRESS_ROUTE) == api.GC_ROUTE_THRESHOLD_MANY
+    plan, w = thr.check_threshold(sizes, 0.002, [randn(sum(sizes), s) for s in range(2)])
+    assert plan.last_counters(w.ws)[1:] == (0, 0)

@@ -53,3 +53,12 @@ def test_ties_by_the_thousand_are_counted(what, n, density, cap_factor):
     g = g.to(torch.bfloat16).float() if what == "bfloat16" else (g * 8).round() / 8
     plan, w = thr.check_threshold([n], density, [g], cap_factor=cap_factor)
     assert plan.last_counters(w.ws)[1:] == (0, 0)
+
+
+@pytest.mark.parametrize("density", [0.001, 0.03])
+def test_samples_beyond_the_rounds_of_the_other_kernel(density):
+    """A definition that samples everything: more than 64 groups per thread, formerly four launches, now fold first at any density."""
+    n = 31_000_001
+    assert api.Plan([n], density, mode=api.GC_THRESHOLD, device=0, sample_stride=1).query(api.GC_Q_COMPRESS_ROUTE) == api.GC_ROUTE_THRESHOLD_ONE
+    plan, w = thr.check_threshold([n], density, [randn(n, s) for s in range(2)], stride=1)
+    assert plan.last_counters(w.ws)[1:] == (0, 0)
