@@ -73,7 +73,7 @@ struct gc_plan_s : DeviceFacts {
     // single-tensor shared-memory-pool kernel
     SingleGeom single[2];                   // k_topk_single for fp32 and for bfloat16 gradients
     uint32_t single_grid = 0;               // CTAs of the first (0 = plan does not qualify)
-    size_t off_hist5 = 0, off_rowseg = 0, off_mid = 0, off_fine = 0, off_start = 0;
+    size_t off_hist5 = 0, off_rowseg = 0, off_mid = 0, off_fine = 0;
     uint32_t single_srank_hi = 0, single_srank_mid = 0;
     SingleGeom thr_single;                  // one-tensor threshold plan, fold first (k_topk_single with THR; G = 0: no)
     TensorDesc thr_d = {};                  // its tensor with the bracket's sample
@@ -118,16 +118,12 @@ constexpr double kRefineFrom = 0.0005;         // plans of several tensors from 
 constexpr uint64_t kRefineLarge = 1u << 26;    // or this many elements on rank their sample twice (see sample_params)
 constexpr uint64_t kSampleMaxSingle = 262144;   // ... when the plan holds one tensor (the sample is read in one step)
 constexpr uint32_t kSinglePoolMax = 65536, kMultiPoolMax = 98304;   // most candidates one CTA of the fused kernels may hold
-// Share of the oldest CTA of an SM above (and of the youngest below) the middle one's: measured
-// best between 6 and 10 % on the 110M-element workload at 1 % density.  Sparser plans have fewer
-// candidates to handle in the fold loop and compete less for issue slots: below 0.5 % the smaller
-// one (4 % did better than 8 % at 0.1 %, where 8 % let the oldest CTAs of the 355M-element workload
-// finish last).  Forms with votes take equal shares.
-constexpr double kSingleSkew = 0.08, kSingleSkewSparse = 0.04;
 constexpr size_t kSingleRowBytes = (2 * kWarps + 4) * sizeof(uint32_t);   // shared memory per owned tile
 constexpr double kSparseUpTo = 0.002;        // density up to which most chunks are empty (see VOTES of k_topk_single)
-constexpr double kVotesFrom = 0.009;         // one-tensor fp32 plans between these densities and from so many tiles on rank by
-constexpr uint32_t kVotesBelow = 16000;      // the shuffle scan (see VOTES of k_topk_single)
+// One-tensor fp32 plans of so many tiles, up to the larger of the two densities (of still more tiles, the smaller one), rank
+// by the shuffle scan (see VOTES of k_topk_single).
+constexpr uint32_t kVotesBelow = 16000, kVotesLarge = 49152;
+constexpr double kVotesFrom = 0.0125, kVotesFromLarge = 0.0095;
 constexpr double kDenseFrom = 0.02;          // density from which the forms with emission by chunk are taken (12 candidates per chunk)
 constexpr double kThrOneFoldUpTo = 0.02;     // one tensor: the same, and the elements from which (see plan_thr_single_fold)
 constexpr uint32_t kThrOneFoldFrom = 12u << 20;
@@ -354,8 +350,7 @@ void finish_layout(gc_plan_s* p) {
     p->off_bhist = align_up(p->off_shist + multi_hist, 256);
     p->off_midn = align_up(p->off_bhist + multi_hist, 256);
     p->control_bytes = align_up(p->off_midn + (multi_hist ? sizeof(uint32_t) * T : 0), 256);
-    p->off_start = p->control_bytes;                                 // where and when the CTAs started (one-tensor kernel)
-    p->off_tinfo = align_up(p->off_start + (T == 1 ? sizeof(unsigned long long) * kSingleMaxG : 0), 256);
+    p->off_tinfo = p->control_bytes;
     p->off_cidx = align_up(p->off_tinfo + sizeof(uint2) * (size_t)p->ntiles * kWarps, 256);
     p->off_mid = align_up(p->off_cidx + sizeof(uint2) * (size_t)p->cand_cap_alloc, 256);
     p->off_mmid = align_up(p->off_mid + (T == 1 ? sizeof(uint2) * (size_t)kSingleMidCap : 0), 256);
@@ -366,35 +361,11 @@ void finish_layout(gc_plan_s* p) {
 }
 
 
-// Shares of a one-tensor plan's CTAs: equal, or - when the launch fills every SM three CTAs deep
-// and every column has at least twelve rows - in the proportion in which the oldest, middle and
-// youngest CTA of an SM advance.  `maxt` comes in as the rows of an equal share and goes out as
-// the rows of the largest one.
-static RowMap make_row_map(const gc_plan_s* p, uint32_t ntiles, uint32_t G, uint32_t& maxt, double skew) {
-    RowMap rm;
-    rm.G = G; rm.gA = G; rm.n0 = rm.n1 = rm.n2 = maxt; rm.s1 = rm.s2 = maxt * G;
-    if (skew > 0.0 && G == 3u * (uint32_t)p->sm_count && ntiles >= 12u * G) {
-        const uint32_t gA = (uint32_t)p->sm_count;
-        const uint32_t total = (ntiles + gA - 1) / gA;               // rows of the three classes together
-        const uint32_t n1 = maxt;
-        const uint32_t dd = std::max<uint32_t>(1u, (uint32_t)((double)ntiles / G * skew + 0.5));
-        const uint32_t n0 = n1 + dd;
-        if (total > n0 + n1 && total - n0 - n1 <= n1) {
-            rm.gA = gA; rm.n0 = n0; rm.n1 = n1; rm.n2 = total - n0 - n1;
-            rm.s1 = rm.n2 * G; rm.s2 = rm.s1 + (rm.n1 - rm.n2) * 2u * gA;
-            maxt = n0;
-        }
-    }
-    rm.mG = (uint32_t)((1ull << 32) / rm.G) + 1u;
-    rm.m2A = (uint32_t)((1ull << 32) / (2u * rm.gA)) + 1u;
-    rm.mA = (uint32_t)((1ull << 32) / rm.gA) + 1u;
-    return rm;
-}
-
 // Geometry of k_topk_single for tensor d with the bracket's sample, of nsg groups, in it (G = 0: no).
 SingleGeom single_geometry(const gc_plan_s* p, const TensorDesc& d, uint64_t nsg, bool bf16) {
     SingleGeom g;
-    g.votes = bf16 || p->mode == GC_THRESHOLD || p->density <= kSparseUpTo || p->density >= kVotesFrom || d.ntiles < kVotesBelow;
+    g.votes = bf16 || p->mode == GC_THRESHOLD || p->density <= kSparseUpTo || d.ntiles < kVotesBelow ||
+              p->density >= (d.ntiles < kVotesLarge ? kVotesFrom : kVotesFromLarge);
     g.G = std::min<uint32_t>((uint32_t)p->grid_single_max, d.ntiles);
     // Small tensors are all latency (a CTA has a handful of tiles and five phases to walk through):
     // there two CTAs per SM get through the phases sooner than three (2M-10M elements: 31-49 us
@@ -405,7 +376,7 @@ SingleGeom single_geometry(const gc_plan_s* p, const TensorDesc& d, uint64_t nsg
     const uint32_t two = 2u * (uint32_t)p->sm_count;
     if (d.ntiles <= 3000u || (!bf16 && p->density <= kSparseUpTo && d.ntiles <= two * (uint32_t)kSingleMaxT)) g.G = std::min(g.G, two);
     g.maxt = (d.ntiles + g.G - 1) / g.G;
-    g.rows = make_row_map(p, d.ntiles, g.G, g.maxt, g.votes ? 0.0 : p->density >= 0.005 ? kSingleSkew : kSingleSkewSparse);
+    g.rows = RowMap{g.G, (uint32_t)((1ull << 32) / g.G) + 1u};
     if (g.maxt > kSingleMaxT || g.G > kSingleMaxG) return SingleGeom{};               // chunk records and totals must stay small
     // region per CTA; one bit per slot has to fit in shared memory beside the chunk records
     g.pool = std::min<uint32_t>(p->cand_cap_alloc / g.G, kSinglePoolMax);
@@ -1356,7 +1327,6 @@ static int compress_impl(gc_plan_t* p, const void* grad_any, bool bf16, float* r
         sa.srank_hi = thr ? p->thr_srank_hi : p->single_srank_hi; sa.srank_mid = thr ? p->thr_srank_mid : p->single_srank_mid; sa.mid_cap = (uint32_t)kSingleMidCap;
         sa.mid = reinterpret_cast<uint2*>(wb + p->off_mid);
         sa.fine = reinterpret_cast<uint32_t*>(wb + p->off_fine);
-        sa.start = reinterpret_cast<unsigned long long*>(wb + p->off_start);
         sa.tile_cnt = reinterpret_cast<uint32_t*>(wb + p->off_tinfo);
         sa.seg_tot = reinterpret_cast<uint32_t*>(wb + p->off_rowseg);
         sa.tile_eq = sa.tile_cnt + nt; sa.seg_eq = sa.seg_tot + kSingleMaxT * 20;

@@ -254,18 +254,6 @@ __device__ __forceinline__ void warp_rank(const uint32_t (&c)[kVpt], int lane,
     total = run;
 }
 
-// Where and when a CTA started, in one word: the SM's number in the upper 10 bits, that SM's cycle counter in the others.
-// Of two CTAs of one SM (numbers ca and cb): did the first start before the second?  An order as long as the starts lie
-// within 2^53 cycles (the counter may wrap between them), so the CTAs of an SM have ages that differ.
-__host__ __device__ __forceinline__ unsigned long long start_word(uint32_t sm, unsigned long long cycle) {
-    return (unsigned long long)(sm & 1023u) << 54 | (cycle & ((1ull << 54) - 1ull));
-}
-__host__ __device__ __forceinline__ uint32_t start_sm(unsigned long long s) { return (uint32_t)(s >> 54); }
-__host__ __device__ __forceinline__ bool started_before(unsigned long long a, uint32_t ca, unsigned long long b, uint32_t cb) {
-    const long long d = (long long)((b - a) << 10);
-    return d > 0 || (d == 0 && ca < cb);
-}
-
 // Where the top-k kernels look for their sample (the sample only steers the candidate bracket;
 // no result depends on it).  Sample group number sg -> 4-element group of the tensor: runs of
 // eight consecutive groups, i.e. one 128-byte line, every 8 x sstride groups.  The same number

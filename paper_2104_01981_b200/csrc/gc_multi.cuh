@@ -38,8 +38,8 @@ constexpr uint32_t kWarpMid = 32;
 constexpr uint32_t kRankMid = 128;
 
 // Contiguous runs of tiles: CTAs below c1 take n1 tiles each, those from there below c2 take n2, the others share
-// the rest evenly.  The CTAs launched last are the youngest on their SMs and advance the slowest (see RowMap in
-// the one-tensor kernel).
+// the rest evenly.  The CTAs launched last are the youngest on their SMs and advance the slowest
+// (the oldest get the most issue slots).
 struct RunMap {
     uint32_t c1, n1, c2, n2;
     __host__ __device__ __forceinline__ uint32_t begin(uint32_t b, uint32_t G, uint32_t ntiles) const {
@@ -1074,8 +1074,7 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
     leave_clean(a.cl, hdr, G, tid);
 }
 
-// Votes: 25.6M elements in 161 tensors at 0.1 % 99 -> 97 us, 110M in 199 at 1 % 302 -> 289 us.  (Why the
-// one-tensor kernel loses with them at 1 %, see there, was not found.)
+// Votes: 25.6M elements in 161 tensors at 0.1 % 99 -> 97 us, 110M in 199 at 1 % 302 -> 289 us.
 template <typename GL, bool DENSE, bool VOTES, bool THR = false>
 // (three CTAs per SM: 80 registers and no spills beat four at 64 registers, see k_topk_single)
 static __global__ void __launch_bounds__(kBlock, 3)

@@ -3,8 +3,7 @@
 //
 // Same idea as the general candidate path (sample -> fold + candidates -> select on the
 // candidates -> index-ordered emission, exact multi-pass redo as the safety net), specialised:
-//   * a CTA owns one column of a row map over the tiles (in the simplest case tiles c, c + G,
-//     c + 2G, ... for column c; see RowMap for the unequal shares of large tensors): every CTA
+//   * a CTA owns one column of a row map over the tiles (tiles b, b + G, b + 2G, ...): every CTA
 //     sees every region of the tensor, so candidate counts stay balanced even when magnitudes
 //     differ between layers;
 //   * a CTA appends the candidates of its own tiles to a private, contiguous region of the
@@ -51,61 +50,18 @@ constexpr uint32_t kMidFast = kMidRegs * kBlock;       // short lists up to this
 // ranking a list costs every CTA five passes over it, counting costs one more grid barrier.
 constexpr uint32_t kMidCounted = 4096;
 
-// Rows of tiles.  A column is one CTA's share of the tensor: row i of column c is one tile, and
-// the tiles are numbered row by row.  The three CTAs that share an SM do not advance at the same
-// speed (the oldest one gets the most issue slots: with equal shares the first finished its fold
-// pass at 182 us, the third at 209 us on the 110M-element workload), so the columns come in
-// three classes of gA each with n0 >= n1 >= n2 rows, and every CTA takes a column of the class
-// that matches its age on its SM.  Row i is G wide below n2, 2 gA wide below n1, gA wide below
-// n0.  Plans that do not fill the GPU three CTAs deep use one class (gA = G, n0 = n1 = n2).
+// Rows of tiles: CTA b owns tiles b, b + G, b + 2G, ... -- column b of rows that are G tiles wide.  (Unequal shares, more
+// rows for the CTA that is the oldest on its SM and fewer for the youngest, are no longer worth their column by age and row arithmetic.
+// Where the shuffle scan ranks the candidates (see VOTES), 4 % more below 0.5 % and 8 % more above / equal, us: 70M elements at 0.3 % 169 / 165,
+// 110M at 0.3 % 246 / 241, 0.6 % 245 / 241, 160M at 0.5 % 338 / 335, 290M at 0.8 % 602 / 591, 355M at 0.5 % 709 / 706; better by up to 0.9 % on 220M to
+// 355M at 0.25 and 0.4 %, 446 / 449 and 697 / 702.)
 struct RowMap {
-    uint32_t G, gA, n0, n1, n2;
-    uint32_t s1, s2;                 // first tile of row n2 and of row n1
-    uint32_t mG, m2A, mA;            // floor(2^32 / d) + 1 for d = G, 2 gA, gA: t / d = mulhi(t, m) for t < 2^20
-    __device__ __forceinline__ uint32_t rows_of(uint32_t c) const { return c < gA ? n0 : c < 2u * gA ? n1 : n2; }
-    __device__ __forceinline__ uint32_t tile_of(uint32_t i, uint32_t c) const {
-        return i < n2 ? i * G + c : i < n1 ? s1 + (i - n2) * 2u * gA + c : s2 + (i - n1) * gA + c;
-    }
-    __device__ __forceinline__ void locate(uint32_t t, uint32_t& row, uint32_t& col) const {
-        if (t < s1) { row = __umulhi(t, mG); col = t - row * G; }
-        else if (t < s2) { const uint32_t q = __umulhi(t - s1, m2A); row = n2 + q; col = t - s1 - q * 2u * gA; }
-        else { const uint32_t q = __umulhi(t - s2, mA); row = n1 + q; col = t - s2 - q * gA; }
-    }
-    __device__ __forceinline__ uint32_t row_of(uint32_t t) const {
-        return t < s1 ? __umulhi(t, mG) : t < s2 ? n2 + __umulhi(t - s1, m2A) : n1 + __umulhi(t - s2, mA);
-    }
+    uint32_t G, mG;                  // mG = floor(2^32 / G) + 1: t / G = mulhi(t, mG) for t < 2^20
+    __device__ __forceinline__ uint32_t rows_of(uint32_t c, uint32_t ntiles) const { return c < ntiles ? row_of(ntiles - c + G - 1u) : 0u; }
+    __device__ __forceinline__ uint32_t tile_of(uint32_t i, uint32_t c) const { return i * G + c; }
+    __device__ __forceinline__ uint32_t row_of(uint32_t t) const { return __umulhi(t, mG); }
+    __device__ __forceinline__ void locate(uint32_t t, uint32_t& row, uint32_t& col) const { row = row_of(t); col = t - row * G; }
 };
-
-// Where and when this CTA started.
-__device__ __forceinline__ unsigned long long note_start() {
-    uint32_t sm;
-    unsigned long long cycle;
-    asm volatile("mov.u32 %0, %%smid;" : "=r"(sm));
-    asm volatile("mov.u64 %0, %%clock64;" : "=l"(cycle));
-    return start_word(sm, cycle);
-}
-// Column of this CTA once every CTA has written down its start (before a grid barrier): its age is the number
-// of CTAs of its SM that started before it, and column = age x gA + SM number, oldest first.  That is a
-// one-to-one assignment only if SMs 0..gA-1 hold three CTAs each; every CTA checks the same table and
-// otherwise keeps column b.  Called by the whole CTA; count[] (1024 words of shared memory) is zero before and after.
-__device__ __forceinline__ uint32_t aged_column(const RowMap& rm, const unsigned long long* start, unsigned long long mine, uint32_t G, uint32_t b,
-                                                uint32_t* count, uint32_t* s_age, int tid) {
-    if (rm.gA * 3u != G || rm.gA > (uint32_t)kBlock) return b;           // one class of columns
-    if (tid == 0) *s_age = 0u;
-    __syncthreads();
-    for (uint32_t c = tid; c < G; c += kBlock) {
-        const unsigned long long s = ld_cg(start + c);
-        atomicAdd(&count[start_sm(s)], 1u);
-        if (start_sm(s) == start_sm(mine) && c != b && started_before(s, c, mine, b)) atomicAdd(s_age, 1u);
-    }
-    __syncthreads();
-    const bool aged = __syncthreads_and((uint32_t)tid >= rm.gA || count[tid] == 3u);      // (3 gA = G: none beyond)
-    const uint32_t age = *s_age;
-    __syncthreads();
-    for (uint32_t i = tid; i < 1024u; i += kBlock) count[i] = 0u;
-    __syncthreads();
-    return aged ? min(age, 2u) * rm.gA + start_sm(mine) : b;
-}
 
 struct SingleArgs {
     TensorDesc d;                    // the tensor (by value)
@@ -126,7 +82,6 @@ struct SingleArgs {
     uint2* mid;                      // [mid_cap] candidates inside the band bin of the threshold
     uint32_t* hist5;                 // [0] coarse sample histogram, [2] band histogram,
                                      // [3][0] short-list length, [4] keys inside a counted band (all zeroed)
-    unsigned long long* start;       // [gridDim.x] SM and cycle at which every CTA started
     uint32_t* fine;                  // [kFineBins] fine sample histogram (zeroed)
     uint32_t* tile_cnt;              // [ntiles] candidates above the band bin, per tile
     uint32_t* seg_tot;               // [maxt][ceil(G/32)] the same summed over each run of 32 CTAs of a row (zeroed)
@@ -417,15 +372,16 @@ __device__ __forceinline__ bool fold_tail_votes(BlockSmem& sm, const float (&av)
 // Three CTAs per SM (80 registers, no spills): measured 15 us faster on the 110M-element workload
 // than four CTAs at 64 registers with spills, and than two.
 // VOTES: how the fold ranks a chunk's candidates -- votes, the residual stored first, chunks without
-// candidates left early, equal shares -- or the shuffle scan.  The votes are a fifth fewer instructions,
+// candidates left early -- or the shuffle scan.  The votes are a fifth fewer instructions,
 // which pays where instructions bound the loop (bfloat16, 110M elements at 1 %: 241 -> 224 us) and where
 // most chunks are empty (fp32 up to 0.2 %, with two CTAs per SM, since a loop that hardly waits for itself
 // keeps the memory busier than it likes with three: 110M elements at 0.1 % 252 -> 231 us, 355M 710 -> 680 us;
 // bfloat16 at five sixths of the bytes wants the third: 0.2 % 227 -> 208 us and 655 -> 598 us).
-// From 0.9 % on, and at any density below 65M elements, the votes win as well (scan / votes, us: 5M at 1 % 40.5 / 39.1, 14M
-// 61.6 / 59.5, 40M at 0.3 % 109.7 / 108.7, 2 % 119 / 115, 110M at 1 % 251.5 / 250, 2 % 262 / 257, 5 % 300 / 285).  Large plans between 0.2 and
-// 0.9 % are bound by memory, and the slower loop with unequal shares does better (110M at 0.3 % 245 / 253, 0.5 % 246 / 252-254;
-// 355M at 0.3 % 705 / 716).  Several workers in one launch keep the scan (see k_topk_workers).
+// Below 65M elements at any density, and on larger plans from about 1 % on, the votes win as well (scan / votes, us: 5M at 1 %
+// 40.5 / 39.1, 14M 61.6 / 59.5, 40M at 0.3 % 109.4 / 109.6, 2 % 119 / 115).  Large plans above 0.2 % are bound by memory, and
+// the slower loop does better: 70M at 0.25 % 164 / 174, 0.9 % 168 / 174, 1.2 % 170.2 / 170.3, 1.5 % 173 / 172; 110M at 0.3 % 241 / 253,
+// 1 % 246 / 250, 1.2 % 252 / 254, 2 % 262 / 257, 5 % 300 / 285; but 220M at 0.9 % 462 / 467, 1 % 476 / 466; 355M at 0.25 % 698 / 717,
+// 0.8 % 720 / 727, 0.9 % 735 / 724, 1 % 752 / 727.  Several workers in one launch keep the scan (see k_topk_workers).
 // DENSE (plans of 2 % and more) has the emission by chunk, the bfloat16 and threshold forms the counted band: the other
 // forms do without their code.  Many tensors, without / with DENSE: 110M elements at 2 % 305 / 310 us, 5 %
 // 359 / 346; 25.6M at 5 % 134 / 131; one tensor: 110M at 2 % 268 / 267, 5 % 312 / 311, 8M at 2 % 49 / 51.
@@ -455,12 +411,6 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
     WsHeader* hdr = a.ws.hdr;
     uint32_t passed = 0, n_stamp = 0;
     const RowMap& rm = a.rows;
-    __shared__ uint32_t s_age;
-    __shared__ unsigned long long s_start;
-    // When this CTA started, taken first thing: the ages have to reflect the order in which the CTAs really
-    // started (taken behind a load they were measured to cost the fold pass 10 us: the shares no longer matched).
-    unsigned long long my_start = 0ull;
-    if (tid == 0) my_start = note_start();
     ClearWait cleared;
     if (!clean_begin(a.cl, hdr, G, b, tid, cleared)) return;
     for (int i = tid; i < 2048; i += kBlock) sm.hist[i] = 0u;
@@ -476,7 +426,7 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
     // into global memory; few samples share a fine bin).  tau = the srank-th largest sampled
     // key cut to 16 bits; tau_hi = upper edge of the 16-bit cell of the srank_hi-th largest.
     uint32_t tau = 0, tau_hi = 0x80000000u, tau_z = 0;
-    uint32_t col = b, n_own = 0, myseg = 0;      // set after the first barrier
+    uint32_t col = 0, n_own = 0, myseg = 0;               // column, own tiles, run of 32 CTAs: set after the first barrier
     {
         const uint32_t ngroups = (d.n + 3u) >> 2;
         const BracketSample def(d.n, d.stride, d.sstride);                // (threshold mode)
@@ -508,7 +458,6 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
 #pragma unroll
             for (int e = 0; e < 4; ++e) skey[q][e] = key_of(__fadd_rn(gv[e], rv[e]));
         }
-        if (tid == 0) { s_start = my_start; a.start[b] = my_start; }
         cleared();                                       // (the loads above are under way meanwhile)
         __syncthreads();
 #pragma unroll
@@ -534,12 +483,11 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
         if (!grid_barrier(hdr, passed, &sm.ok)) return;
         phase_stamp(hdr, n_stamp);
         clean_in_use(hdr, b, tid);
-        {
-            col = aged_column(rm, a.start, s_start, G, b, sm.hist, &s_age, tid);
-            n_own = rm.rows_of(col);
-            while (n_own > 0u && rm.tile_of(n_own - 1u, col) >= a.ntiles) --n_own;
-            myseg = col / 32u;
-        }
+        // (Read here and not taken from b: what the compiler derives from a column it knows at the start is carried through
+        // the kernel, 80 registers and spills instead of 72; threshold mode, 110M elements at 1 %: 252 us instead of 246.)
+        asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(col));
+        n_own = rm.rows_of(col, a.ntiles);
+        myseg = col / 32u;
         // both brackets from one read of the coarse histogram, then the kFineBits finer bits of
         // each from the 2^kFineBits fine bins under its coarse bin (one warp per bracket)
         const uint32_t want[3] = {d.srank, a.srank_hi, a.srank_mid};
@@ -921,7 +869,7 @@ k_topk_single(const __grid_constant__ SingleArgs a) {
             for (uint32_t i = kMidFast + tid; !counted && i < m; i += kBlock) below(ld_cg(a.mid + i));
             if (tid == 0) { sm.scratch[0] = 0u; sm.scratch[1] = 0xFFFFFFFFu; }
             __syncthreads();
-            if (THR && col == 0u) {            // (this column has a tile in every row: the rows' totals are the tensor's)
+            if (THR && col == 0u) {              // (this column has a tile in every row: the rows' totals are the tensor's)
                 uint32_t hits = 0;
                 for (uint32_t i = tid; i < n_own; i += kBlock) hits += row_sum[i];
 #pragma unroll
