@@ -54,7 +54,9 @@ typedef struct gc_plan_s gc_plan_t;
 #define GC_E_UNSUPPORTED (-2)   /* not available in this build / on this device                        */
 #define GC_E_CUDA        (-3)   /* a CUDA runtime call failed; see gc_last_cuda_error                   */
 #define GC_E_TOO_LARGE   (-4)   /* size beyond a stated limit                                           */
-#define GC_E_TIMEOUT     (-5)   /* a bounded device-side wait gave up (device status only)              */
+#define GC_E_TIMEOUT     (-5)   /* a bounded device-side wait gave up (device status only; the wait for
+                                  the clearing of a workspace, a barrier of the cooperative launch, has no
+                                  limit of its own)                                                     */
 #define GC_W_TRUNCATED     1    /* threshold mode: more hits than capacity; the rest stayed in r       */
 
 /* selection modes */
@@ -110,12 +112,12 @@ typedef struct gc_plan_s gc_plan_t;
  *   density        in (0, 1]
  *   mode           GC_TOPK or GC_THRESHOLD
  *   sample_stride  threshold mode: sample one 4-element group out of this many (0 = 64);
- *                  tensors of <= 65,536 elements are always sampled in full.  Every sampled
- *                  group is a scattered 32-byte DRAM access in g and in r, and on tensors of
- *                  100M elements and more that is a tenth of the call at stride 64 (110M
- *                  elements: 262 us against 238 us at stride 512, whose sample still holds
- *                  214,000 elements); the stride is part of the result's definition, so the
- *                  library does not choose it
+ *                  tensors of <= 65,536 elements are always sampled in full.  Large sparse plans
+ *                  pick the sample out of the pass over the elements, where the stride hardly
+ *                  matters (110M elements at 1 %: 245, 245 and 242 us at strides 64, 512 and 4096);
+ *                  in the others every sampled group is a scattered 32-byte DRAM access in g and in r.
+ *                  The stride is part of the result's definition, so the library does not
+ *                  choose it
  *   cap_factor     threshold mode: per-tensor output capacity = min(n, ceil(cap_factor*k))
  *                  (0 = 2.0; must be >= 1)
  * Allocates a few KB of device memory for the tensor table (freed by gc_destroy).
@@ -234,10 +236,10 @@ int gc_compress_bf16(gc_plan_t *plan, const void *grad_bf16, float *residual,
  * to out_count[w]) and uses workspaces[w]; every result is exactly what W separate gc_compress
  * calls would give.  No counterpart in the source paper: the problem statement only says that
  * the 8-worker workload runs its workers on one GPU, and this call is how that is done without
- * paying a kernel's cold phases once per worker.  For top-k plans of several tensors on the
- * default route the workers share cooperative launches: the resident CTAs are dealt out evenly
- * among up to 12 workers per launch, each group of CTAs runs the many-tensor kernel on its own
- * worker and synchronises only with itself.  Every other plan (one tensor, threshold mode,
+ * paying a kernel's cold phases once per worker.  For plans of several tensors on the
+ * default route, in top-k and in threshold mode, the workers share cooperative launches: the resident CTAs are
+ * dealt out evenly among up to 12 workers per launch, each group of CTAs runs the many-tensor kernel on its own
+ * worker and synchronises only with itself.  Every other plan (one tensor,
  * GC_PATH_EXACT / GC_PATH_STAGED) is served by W consecutive gc_compress calls.
  *
  *   W            1..GC_MAX_WORKERS (0 does nothing)
@@ -409,7 +411,7 @@ int gc_compress_noalloc(const float *grad, float *residual, uint32_t n, uint32_t
  * three counters of the most recent gc_compress on this workspace to the host:
  *   counters[0] = candidates extracted by the one-pass path, counters[1] = 1 if the candidate
  *   list overflowed (every tensor was redone by the exact kernels), counters[2] = tensors
- *   whose candidate set was smaller than k (redone individually).
+ *   whose bracket missed the threshold or whose list of near-ties was full (redone individually).
  */
 int gc_last_counters(gc_plan_t *plan, const void *workspace, void *stream, uint32_t counters[3]);
 

@@ -489,8 +489,6 @@ void plan_thr_multi(gc_plan_s* p) {
     p->thrm_grid = mg.G; p->thrm_per = mg.per; p->thrm_pool = mg.pool; p->thrm_ntab = mg.ntab; p->thrm_smem = mg.smem;
 }
 
-// Geometry of the many-tensor kernel when G CTAs share one worker's tiles: MultiGeom.
-
 // Decides whether G CTAs can run the many-tensor kernel on this plan (G = 0 in the result: no).
 // `workers`: how many such groups share the launch.  In a launch that fills the device the CTA index follows
 // the CTAs' age on their SMs: what the full runs of a lone worker leave over goes to the youngest third; several

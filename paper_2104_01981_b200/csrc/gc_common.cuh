@@ -419,7 +419,7 @@ __device__ __forceinline__ bool grid_barrier(WsHeader* hdr, uint32_t& passed, in
 // find it, so that launch can do without the clearing launch in front of it.  Everything that is
 // first written after the first grid barrier is zeroed at the START of a launch, a slice per CTA
 // (the writers come after the barrier, so there is no ordering problem); the sections written
-// before the first barrier ("early": at most three ranges) are zeroed right after the barrier that
+// before the first barrier ("early": at most two ranges) are zeroed right after the barrier that
 // follows their last reader; the barrier counter is reset by the CTA that leaves last (an exit
 // counter in the header), which then sets a 64-bit mark.  When the host relies on that (on the
 // caller's promise that nobody else writes to the workspace), the kernel first checks the mark and

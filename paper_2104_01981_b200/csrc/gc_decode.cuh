@@ -22,7 +22,7 @@ constexpr size_t kDecTileBytes = kDecTile * sizeof(float);
 
 // The decode kernels are launched while the kernel in front of them still runs (programmatic dependent launch): its
 // CTAs take the SMs as they fall idle, and here they wait until all its writes are visible.  What that kernel
-// wrote is read through L2 from then on, never through the read-only path.  A decode behind a compress: 1M elements 28.9 ->
+// may have written is not read through the non-coherent read-only path.  A decode behind a compress: 1M elements 28.9 ->
 // 27.1 us for both, 300,000 24.6 -> 22.5; momentum on 25M 80.4 -> 78.3.  Triggers in the compress kernels (CTAs waiting on the
 // SMs under the emission) take it back: 30.1 and 24.8 us.
 __device__ __forceinline__ void launch_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

@@ -132,8 +132,6 @@ static __device__ void small_threshold_body(BlockSmem& sm, const TensorDesc& d, 
                                             float* __restrict__ r, uint32_t* __restrict__ out_idx, float* __restrict__ out_val,
                                             uint32_t* __restrict__ out_count, WsHeader* hdr);
 
-// The whole compress of one worker by the G CTAs of one group (this CTA is number b of them);
-// the group's barriers count on the worker's own workspace header.
 // Threshold mode, behind the counts: exact threshold, first slot and counts of every segment.  The wanted rank is one
 // among the sampled entries of the short list, of which there are a handful: a warp per segment takes them
 // from the top, one distinct key at a time; lists beyond kThrWarpMid entries take the block-wide radix select.  The CTA
@@ -257,6 +255,8 @@ __device__ __forceinline__ void thr_slots(const MultiArgs& a, uint32_t* seg, uin
     }
 }
 
+// The whole compress of one worker by the G CTAs of one group (this CTA is number b of them);
+// the group's barriers count on the worker's own workspace header.
 // (DENSE, VOTES: see k_topk_single)
 // THR: threshold mode.  The threshold is the k_s-th largest key of the sample that the definition fixes, one group of
 // four elements per `stride` groups, and reading those before the fold costs what as many scattered accesses cost.
