@@ -124,6 +124,18 @@ __device__ __forceinline__ bool grid_wait(WsHeader* hdr, uint32_t& passed, int* 
     return grid_wait(hdr, passed, s_ok, gridDim.x);
 }
 
+// Every listed candidate of the chunks [c0, c1) gets its value back in the residual, and the chunks are empty.  (Out of line:
+// rare, and its registers were spilled in the fold.)
+static __device__ __noinline__ void give_back_chunks(uint32_t* rec, uint32_t c0, uint32_t c1, const uint2* pool, float* r) {
+    for (uint32_t c = c0 + threadIdx.x; c < c1; c += kBlock) {
+        const uint32_t rc = rec[c];
+        for (uint32_t j = 0; j < (rc & 1023u); ++j) {
+            const uint2 pr = pool[(rc >> 10) + j];
+            r[pr.x] = __uint_as_float(pr.y);
+        }
+        rec[c] = 0u;
+    }
+}
 // (gc_thr_multi.cuh)
 static __device__ void tiny_threshold_warp(const TensorDesc& d, uint32_t t, uint32_t T, const float* __restrict__ g, float* __restrict__ r,
                                            uint32_t* __restrict__ out_idx, float* __restrict__ out_val, uint32_t* __restrict__ out_count,
@@ -263,9 +275,11 @@ __device__ __forceinline__ void thr_slots(const MultiArgs& a, uint32_t* seg, uin
 // Here they are picked out of the stream instead: the bracket comes from a sample of 128-byte lines as in top-k mode, the
 // band histogram counts the candidates that are in the definition's sample, the band bin of rank k_s and the short list
 // (all candidates in it) give the exact threshold, and every candidate at or above it is a hit, up to the capacity.
-// A tensor that fails (bracket missed, list full) is redone from the residual by radix levels over the
-// definition's sample and the look-back emission, all are if a region is full (199 tensors of 110M elements rounded to
-// bfloat16, a list of ties too long in the largest: 1036 us with all of them redone, 658 with that one).  Eight 161-tensor workers: sample and thresholds 95 -> 26 us, call
+// A tensor that fails (bracket missed, list full, no room in a region) is redone from the residual by radix levels over
+// the definition's sample and the look-back emission (199 tensors of 110M elements rounded to bfloat16, a list of ties too
+// long in the largest: 1036 us with all of them redone, 658 with that one; first calls on gradients with a log-normal scale of
+// spread 0.4 per channel, where the sample of a layer or two sees so small entries that a region fills: eight 161-tensor workers at
+// 0.1 % 696 -> 570 us, 0.5 % 994 -> 640, 199 tensors 926 -> 487).  Eight 161-tensor workers: sample and thresholds 95 -> 26 us, call
 // with the decode 532 -> 494.
 template <typename GL, bool DENSE, bool VOTES, bool THR = false>
 __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32_t G, const uint32_t b, BlockSmem& sm,
@@ -466,9 +480,23 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
         uint32_t cur = 0xFFFFFFFFu, tau = 0, tau_z = 0;
         int shift = 0;
         TensorDesc d;
+        // Threshold mode: the definition's sample may have met entries so small that many times k are hits.  A segment that
+        // does not fit the region then gives its candidates back and its room to the next one, and its tensor alone is redone.  (In
+        // top-k mode the number of candidates is a matter of the rank, and a full region has everything redone.)
+        auto give_back = [&](uint32_t end) {                    // the open segment ends in front of own tile `end`
+            if (!__syncthreads_or(block_overflow ? 1 : 0)) return;
+            block_overflow = false;
+            give_back_chunks(rec, seg[(size_t)(nseg - 1u) * kSegWords + SG_TILE0] * kWarps, end * kWarps, pool, a.r);
+            if (tid == 0) {
+                s_used = seg[(size_t)(nseg - 1u) * kSegWords + SG_ABOVE];
+                if ((atomicOr(&a.ws.sel[cur].flags, kSelFailed) & kSelFailed) == 0u) atomicAdd(&hdr->n_failed, 1u);
+            }
+            __syncthreads();
+        };
         for (uint32_t tile = first; tile < last; ++tile) {
             const uint32_t i = tile - first;
             if (cur == 0xFFFFFFFFu || tile >= d.tile0 + d.ntiles) {
+                if (THR && open) give_back(i);
                 if (open) flush_hist(sm, a.bhist + (size_t)d.reg * kHistBins, 2048);
                 open = false;
                 cur = a.ntab ? owner(tab_tile0, tile) : find_tensor(a.desc, a.T, tile);
@@ -486,8 +514,9 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
                         s[SG_TAU] = tau; s[SG_TAUZ] = tau_z; s[SG_SHIFT] = (uint32_t)shift;
                         s[SG_OK] = 1u; s[SG_OUT] = d.out_off; s[SG_K] = d.k;
                         s[SG_A] = d.reg;               // (until the band bin is known)
-                        if (THR) s[SG_END] = d.out_off + d.cap;
+                        if (THR) { s[SG_END] = d.out_off + d.cap; s[SG_ABOVE] = s_used; }      // (where its candidates begin)
                     }
+                    if (THR) __syncthreads();              // (before anyone adds to s_used again)
                     ++nseg;
                     open = true;
                 }
@@ -611,6 +640,7 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
                 }
             }
         }
+        if (THR && open) give_back(ntl);
         if (open) flush_hist(sm, a.bhist + (size_t)d.reg * kHistBins, 2048);
         if (__syncthreads_or(block_overflow ? 1 : 0)) {
             if (tid == 0) atomicExch(&hdr->overflow, 1u);
@@ -673,8 +703,10 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
         for (uint32_t sidx = (uint32_t)warp; sidx < nseg; sidx += kWarps) {      // a warp per segment, all at once
             uint32_t* s = seg + (size_t)sidx * kSegWords;
             const uint32_t t = s[SG_T];
+            const uint32_t flags = THR ? ld_cg(&a.ws.sel[t].flags) : 0u;
             const Picked pa = warp_select_2048(a.bhist + (size_t)s[SG_A] * kHistBins, s[SG_K], lane);
-            const bool ok = pa.ok && (THR || pa.count <= kMultiMidCap);      // (threshold mode counts the sampled ones only)
+            // (threshold mode counts the sampled ones only; some CTA may have had no room for the tensor)
+            const bool ok = pa.ok && (THR ? (flags & kSelFailed) == 0u : pa.count <= kMultiMidCap);
             if (lane == 0) {
                 s[SG_A] = pa.bin; s[SG_ABOVE] = pa.above; s[SG_M] = pa.count; s[SG_OK] = ok ? 1u : 0u;
                 if (!ok) {          // every CTA that sees this tensor decides the same; count it once

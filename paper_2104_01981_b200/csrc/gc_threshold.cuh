@@ -37,7 +37,11 @@ static __device__ void threshold_emit_body(const TensorDesc* __restrict__ desc, 
         if (tile >= ntiles) break;
         const uint32_t t = find_tensor(desc, T, tile);
         const TensorDesc d = desc[t];
-        if ((SKIP_SMALL && d.kind == kKindSmall) || !gate_open(ws, t, d)) continue;
+        if ((SKIP_SMALL && d.kind == kKindSmall) || !gate_open(ws, t, d)) {
+            // (all of its tiles at once: with a gate hardly any tensor is open)
+            if (tid == 0) atomicMax(&ws.hdr->ticket[ticket_slot], d.tile0 + d.ntiles);
+            continue;
+        }
         const uint32_t tau = ssel != nullptr ? ssel[t].T : tau_fixed;
         const TileGeom tg = tile_geom(d, tile - d.tile0);
         Tile tl;

@@ -72,13 +72,37 @@ def test_workers(W, density):
 
 @pytest.mark.parametrize("cap_factor", [8.0, 1.0], ids=["all", "truncated"])
 @pytest.mark.parametrize("bad", [0, 2, 6])
-def test_one_tensor_fails_and_the_others_do_not(bad, cap_factor):
-    """A tensor whose short list is too long is redone by itself, in front of, between or behind others that are not."""
+@pytest.mark.parametrize("what", ["ties", "blind"])
+def test_one_tensor_fails_and_the_others_do_not(what, bad, cap_factor):
+    """A tensor whose short list is too long, or that leaves no room in a region of the candidate list, is redone by itself,
+    in front of, between or behind others that are not."""
     g = randn(sum(SIZES), 9)
     t = g[sum(SIZES[:bad]):sum(SIZES[:bad + 1])]
-    t[t.abs() > 2.0] = 2.0                             # equal keys from above the threshold to below it
+    if what == "ties":
+        t[t.abs() > 2.0] = 2.0                         # equal keys from above the threshold to below it
+    else:
+        t[(torch.arange(t.numel()) // 4) % 64 == 0] *= 1e-3      # the sample meets small ones only: nearly every element is a hit
     plan, w = thr.check_threshold(SIZES, 0.01, [g], cap_factor=cap_factor)
-    assert plan.last_counters(w.ws)[1:] == (0, 1)
+    # (what such a tensor lists in a region that it shares may leave no room for the head of the next one)
+    assert plan.last_counters(w.ws)[1:] in ([(0, 1)] if what == "ties" else [(0, 1), (0, 2)])
+
+
+def test_workers_that_fail_in_one_tensor():
+    """The same in a launch that several workers share, another tensor for each of them; calls of their own give the same."""
+    plan = api.Plan(SIZES, 0.002, mode=api.GC_THRESHOLD, device=0)
+    a, b = ([thr.GpuWorker(plan) for _ in range(4)] for _ in range(2))
+    gs = [randn(sum(SIZES), 70 + w).cuda() for w in range(4)]
+    for w, bad in enumerate((0, 2, 6)):
+        t = gs[w][sum(SIZES[:bad]):sum(SIZES[:bad + 1])]
+        t[(torch.arange(t.numel(), device="cuda") // 4) % 64 == 0] *= 1e-3
+    plan.compress_workers(gs, [w.residual for w in a], [w.idx for w in a], [w.val for w in a], [w.count for w in a], [w.ws for w in a])
+    seen = [plan.last_counters(w.ws)[1:] for w in a]
+    assert all(c in ((0, 1), (0, 2)) for c in seen[:3]) and seen[3] == (0, 0)
+    for w in range(4):
+        b[w].step(gs[w])
+        assert torch.equal(a[w].count, b[w].count) and torch.equal(a[w].residual, b[w].residual)
+        for o, c in zip(plan.tensor_out_offset(), b[w].count.tolist()):
+            assert torch.equal(a[w].idx[o:o + c], b[w].idx[o:o + c]) and torch.equal(a[w].val[o:o + c], b[w].val[o:o + c])
 
 
 def test_more_tensors_than_the_tables_in_shared_memory_hold():
