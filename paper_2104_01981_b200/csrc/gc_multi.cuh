@@ -124,9 +124,11 @@ __device__ __forceinline__ bool grid_wait(WsHeader* hdr, uint32_t& passed, int* 
     return grid_wait(hdr, passed, s_ok, gridDim.x);
 }
 
-// Every listed candidate of the chunks [c0, c1) gets its value back in the residual, and the chunks are empty.  (Out of line:
-// rare, and its registers were spilled in the fold.)
-static __device__ __noinline__ void give_back_chunks(uint32_t* rec, uint32_t c0, uint32_t c1, const uint2* pool, float* r) {
+// A segment, chunks [c0, c1), that does not fit the CTA's region gives its candidates back to the residual and its room to
+// the next one (`used` = where it began), and its tensor is flagged.  The whole CTA calls.  (Out of line: rare, and its registers were
+// spilled in the fold.)
+static __device__ __noinline__ void give_back_segment(uint32_t* rec, uint32_t c0, uint32_t c1, const uint2* pool, float* r, uint32_t* s_used,
+                                                      uint32_t used, uint32_t* flags, WsHeader* hdr) {
     for (uint32_t c = c0 + threadIdx.x; c < c1; c += kBlock) {
         const uint32_t rc = rec[c];
         for (uint32_t j = 0; j < (rc & 1023u); ++j) {
@@ -135,6 +137,11 @@ static __device__ __noinline__ void give_back_chunks(uint32_t* rec, uint32_t c0,
         }
         rec[c] = 0u;
     }
+    if (threadIdx.x == 0) {
+        *s_used = used;
+        if ((atomicOr(flags, kSelFailed) & kSelFailed) == 0u) atomicAdd(&hdr->n_failed, 1u);
+    }
+    __syncthreads();
 }
 // (gc_thr_multi.cuh)
 static __device__ void tiny_threshold_warp(const TensorDesc& d, uint32_t t, uint32_t T, const float* __restrict__ g, float* __restrict__ r,
@@ -480,23 +487,19 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
         uint32_t cur = 0xFFFFFFFFu, tau = 0, tau_z = 0;
         int shift = 0;
         TensorDesc d;
-        // Threshold mode: the definition's sample may have met entries so small that many times k are hits.  A segment that
-        // does not fit the region then gives its candidates back and its room to the next one, and its tensor alone is redone.  (In
-        // top-k mode the number of candidates is a matter of the rank, and a full region has everything redone.)
-        auto give_back = [&](uint32_t end) {                    // the open segment ends in front of own tile `end`
-            if (!__syncthreads_or(block_overflow ? 1 : 0)) return;
-            block_overflow = false;
-            give_back_chunks(rec, seg[(size_t)(nseg - 1u) * kSegWords + SG_TILE0] * kWarps, end * kWarps, pool, a.r);
-            if (tid == 0) {
-                s_used = seg[(size_t)(nseg - 1u) * kSegWords + SG_ABOVE];
-                if ((atomicOr(&a.ws.sel[cur].flags, kSelFailed) & kSelFailed) == 0u) atomicAdd(&hdr->n_failed, 1u);
-            }
-            __syncthreads();
-        };
         for (uint32_t tile = first; tile < last; ++tile) {
             const uint32_t i = tile - first;
             if (cur == 0xFFFFFFFFu || tile >= d.tile0 + d.ntiles) {
-                if (THR && open) give_back(i);
+                // Threshold mode: the definition's sample may have met entries so small that many times k are hits.  A tensor that
+                // does not fit is redone alone.  (In top-k mode the number of candidates is a matter of the rank, and a full region
+                // has everything redone.)
+                if constexpr (THR) {
+                    if (open && __syncthreads_or(block_overflow ? 1 : 0)) {
+                        const uint32_t* q = seg + (size_t)(nseg - 1u) * kSegWords;
+                        give_back_segment(rec, q[SG_TILE0] * kWarps, i * kWarps, pool, a.r, &s_used, q[SG_ABOVE], &a.ws.sel[cur].flags, hdr);
+                        block_overflow = false;
+                    }
+                }
                 if (open) flush_hist(sm, a.bhist + (size_t)d.reg * kHistBins, 2048);
                 open = false;
                 cur = a.ntab ? owner(tab_tile0, tile) : find_tensor(a.desc, a.T, tile);
@@ -640,7 +643,13 @@ __device__ __forceinline__ void topk_multi_body(const MultiArgs& a, const uint32
                 }
             }
         }
-        if (THR && open) give_back(ntl);
+        if constexpr (THR) {
+            if (open && __syncthreads_or(block_overflow ? 1 : 0)) {
+                const uint32_t* q = seg + (size_t)(nseg - 1u) * kSegWords;
+                give_back_segment(rec, q[SG_TILE0] * kWarps, ntl * kWarps, pool, a.r, &s_used, q[SG_ABOVE], &a.ws.sel[cur].flags, hdr);
+                block_overflow = false;
+            }
+        }
         if (open) flush_hist(sm, a.bhist + (size_t)d.reg * kHistBins, 2048);
         if (__syncthreads_or(block_overflow ? 1 : 0)) {
             if (tid == 0) atomicExch(&hdr->overflow, 1u);
